@@ -391,10 +391,10 @@ int gl_profile_read(gl_ctx *ctx, gl_profile_data *out);
  * bwd_ms[d], the summed milliseconds of that level's forward and backward
  * sweep launches; fronts[d], its fronts over all subdomains; nonzeros[d],
  * their factor entries (sum of p(p+1)/2 + p q, what each sweep reads and
- * multiplies once); padded[d], the entries of the 32-column block panels
- * the kernels multiply (sum over blocks of 32 x the rows from the block
- * down: the diagonal blocks' upper triangles and the last block's missing
- * columns count as zeros); max_front[d], the rows of its largest front.
+ * multiplies once); padded[d], the entries of its panels rounded up to whole
+ * 32-column blocks (sum over blocks of 32 x the rows from the block down: the
+ * diagonal blocks' upper triangles and the last block's missing columns
+ * count); max_front[d], the rows of its largest front.
  * *n_levels = number of levels, *calls = timed
  * applications.  Every output pointer is host memory and may be NULL.
  * Errors: GL_ERR_STATE before gl_setup, GL_ERR_INVALID_ARG for

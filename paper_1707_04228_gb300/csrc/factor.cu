@@ -12,14 +12,15 @@
 //   4. blocked right-looking partial Cholesky of the p pivot columns:
 //      diagonal block (POTRF), panel below (TRSM), trailing lower triangle
 //      (SYRK/GEMM) -- the trailing update also forms the update matrix;
-//   5. copy the f x p panel into the factor array.
-// After all levels the stored factor is put in partitioned-inverse form
-// (k_block_inverse: inverted 32x32 diagonal blocks, rows below multiplied by
-// them).  The solves walk the same levels: forward (leaves to root) and
-// backward, each block step a plain product with that form.
+//   5. write the front's panel to the factor array in inverse form:
+//      L11^{-1} over W = L21 L11^{-1} (k_diag_inverse, k_tri_inverse, k_wpanel).
+// The solves walk the same levels, forward (leaves to root) and backward.  With
+// the pivot block's inverse stored, a front's step is one product with its
+// panel and no row of it waits for another.
 #include <algorithm>
 #include <cstdio>
 #include <mutex>
+#include <type_traits>
 
 #include "factor.h"
 #include "q2.cuh"
@@ -31,8 +32,6 @@ constexpr int NB = 32;        // pivot block
 constexpr int TILE = 64;      // trailing-update tile
 
 // ----------------------------------------------------------------- plan
-
-void sweep_smem_for_plan(int max_f);
 
 void build_plan(const std::vector<SubSymbolic> &subs, FactorPlan &P, cudaStream_t s) {
     P.n_sub = (int)subs.size();
@@ -121,7 +120,6 @@ void build_plan(const std::vector<SubSymbolic> &subs, FactorPlan &P, cudaStream_
     P.d_gdof.upload(P.h_gdof, s);
     P.d_vec_off.upload(P.vec_off, s);
     P.d_vec_len.upload(P.vec_len, s);
-    sweep_smem_for_plan(P.max_f);
     GL_CUDA(cudaStreamSynchronize(s));
 }
 
@@ -409,20 +407,6 @@ __global__ void __launch_bounds__(256) k_syrk(const int *__restrict__ fronts, co
         }
 }
 
-template <class T>
-__global__ void k_copy_panel(const int *__restrict__ fronts, const FrontDesc *__restrict__ D,
-                             const T *__restrict__ ws, T *__restrict__ L) {
-    const FrontDesc d = D[fronts[blockIdx.x]];
-    const int f = d.p + d.q;
-    const int64_t n = (int64_t)f * d.p;
-    const T *F = ws + d.front_off;
-    T *out = L + d.l_off;
-    for (int64_t idx = blockIdx.y * (int64_t)blockDim.x + threadIdx.x; idx < n; idx += (int64_t)gridDim.y * blockDim.x) {
-        int64_t j = idx / f, i = idx % f;
-        out[idx] = i >= j ? F[i + j * f] : T(0);
-    }
-}
-
 // Blocked right-looking partial Cholesky of the p pivot columns of every front
 // of a level.  FP64 (and FP32 with tc = false): blocks of NB = 32 pivots, each
 // followed by the rank-32 update of the whole trailing lower triangle.  FP32
@@ -472,56 +456,174 @@ static void partial_cholesky_level(const int *d_fronts, int n_fronts, const Fron
     }
 }
 
-// Partitioned-inverse form of the stored factor, used by the sweeps.  For
-// every block B of 32 consecutive pivots of a front (the last one may be
-// shorter): L[B,B] <- L[B,B]^{-1} (lower triangular) and, for every row i
-// below B in the front (later pivots and structure rows),
-// L[i,B] <- W[i,B] = L[i,B] L[B,B]^{-1}.  A forward step is then
-// y_B = L[B,B]^{-1} x_B and x_i -= W[i,B] x_B, a backward step
-// x_B = L[B,B]^{-T} y_B - W[i,B]^T x_i: plain products with no serial
-// triangular solve.  Computed in FP64 whatever the storage type.  One CTA per
-// (front, block); blocks are independent of one another.
+// ----------------------------------------------------------------- inverse form of the panels
+
+// The sweeps read a front's panel as [L11^{-1}; W], W = L21 L11^{-1}, so that a
+// forward step is y_1 = L11^{-1} x_1, x_2 -= W x_1 and a backward step
+// x_1 = L11^{-T} y_1 - W^T x_2: products without a triangular solve, as many
+// entries as the factor itself.  Both sweeps read the same numbers, so the
+// preconditioner stays symmetric positive definite whatever their rounding.
+// Computed in FP64 whatever the storage type.
+constexpr int INV_THREADS = 256;
+
+// Diagonal blocks: out[B, B] = L[B, B]^{-1}, the strict upper triangle zero.
+// One warp per (front, 32-pivot block): lane j solves for column j.
 template <class T>
-__global__ void __launch_bounds__(256) k_block_inverse(const FrontDesc *__restrict__ D, T *__restrict__ L) {
-    const FrontDesc d = D[blockIdx.x];
+__global__ void __launch_bounds__(32) k_diag_inverse(const int *__restrict__ fronts, const FrontDesc *__restrict__ D,
+                                                     const T *__restrict__ ws, T *__restrict__ out) {
+    const FrontDesc d = D[fronts[blockIdx.x]];
     const int jb = blockIdx.y * 32;
     if (jb >= d.p) return;
-    const int kb = min(32, d.p - jb), f = d.p + d.q;
-    T *Lp = L + d.l_off;
+    const int kb = min(32, d.p - jb), f = d.p + d.q, j = threadIdx.x;
+    const T *A = ws + d.front_off + jb + (int64_t)jb * f;
     __shared__ double Dk[32][33], Li[32][33];
-    for (int idx = threadIdx.x; idx < 1024; idx += blockDim.x) {
-        const int i = idx & 31, j = idx >> 5;
-        Dk[i][j] = (i < kb && j < kb && i >= j) ? (double)Lp[(jb + i) + (int64_t)(jb + j) * f] : 0.0;
-        Li[i][j] = 0.0;
-    }
-    __syncthreads();
-    if (threadIdx.x < kb) {
-        // column j of the inverse by forward substitution on e_j
-        const int j = threadIdx.x;
-        Li[j][j] = 1.0 / Dk[j][j];
-        for (int i = j + 1; i < kb; ++i) {
-            double acc = 0.0;
-            for (int k = j; k < i; ++k) acc += Dk[i][k] * Li[k][j];
-            Li[i][j] = -acc / Dk[i][i];
+    for (int c = 0; c < kb; ++c) Dk[j][c] = j < kb && j >= c ? (double)A[j + (int64_t)c * f] : 0.0;
+    __syncwarp();
+    const double rd = j < kb ? 1.0 / Dk[j][j] : 0.0;
+    for (int i = 0; i < kb; ++i) {
+        double a0 = i == j ? 1.0 : 0.0, a1 = 0.0;
+        int k = 0;
+        for (; k + 1 < i; k += 2) {
+            a0 -= Dk[i][k] * Li[k][j];
+            a1 -= Dk[i][k + 1] * Li[k + 1][j];
         }
+        if (k < i) a0 -= Dk[i][k] * Li[k][j];
+        Li[i][j] = (a0 + a1) * __shfl_sync(0xffffffffu, rd, i);   // zero above the diagonal: column j starts at e_j
     }
-    __syncthreads();
-    for (int i = jb + kb + threadIdx.x; i < f; i += blockDim.x) {
-        double r[32];
+    __syncwarp();
+    T *O = out + d.l_off + jb + (int64_t)jb * f;
+    if (j < kb)
+        for (int c = 0; c < kb; ++c) O[j + (int64_t)c * f] = j >= c ? (T)Li[j][c] : T(0);
+}
+
+// Column tile J of L11^{-1} below its diagonal block: block row k from the one
+// above down, X_k = -L_kk^{-1} sum_{m=J}^{k-1} L_km X_m (the diagonal blocks'
+// inverses are in place).  One CTA per (front, tile); the chain over k is the
+// CTA's own, so tiles need no other synchronisation.  Rows above J are zeroed.
+template <class T>
+__global__ void __launch_bounds__(INV_THREADS) k_tri_inverse(const int *__restrict__ fronts,
+                                                             const FrontDesc *__restrict__ D,
+                                                             const T *__restrict__ ws, T *out) {
+    const FrontDesc d = D[fronts[blockIdx.x]];
+    const int p = d.p, f = d.p + d.q, j0 = blockIdx.y * 32;
+    if (j0 >= p) return;
+    const int jw = min(32, p - j0);
+    const T *F = ws + d.front_off;
+    T *O = out + d.l_off + (int64_t)j0 * f;
+    __shared__ double A[32][33], B[32][33];
+    const int c = threadIdx.x & 31, r4 = threadIdx.x >> 5;   // output column c, rows r4 + 8 t
+    for (int idx = threadIdx.x; idx < j0 * jw; idx += INV_THREADS) O[idx % j0 + (int64_t)(idx / j0) * f] = T(0);
+    for (int k0 = j0 + 32; k0 < p; k0 += 32) {
+        const int kw = min(32, p - k0);
+        double acc[4] = {0.0, 0.0, 0.0, 0.0};
+        for (int m0 = j0; m0 < k0; m0 += 32) {
+            // rows k0.. of L columns m0..  (A[row][col]) and X_m (B[row][col])
 #pragma unroll
-        for (int k = 0; k < 32; ++k) r[k] = k < kb ? (double)Lp[i + (int64_t)(jb + k) * f] : 0.0;
-#pragma unroll 1
-        for (int j = 0; j < kb; ++j) {
-            double w = 0.0;   // Li is lower triangular: the terms k < j vanish
+            for (int t = 0; t < 4; ++t) {
+                const int col = r4 + 8 * t;
+                A[c][col] = c < kw ? (double)F[k0 + c + (int64_t)(m0 + col) * f] : 0.0;
+                B[c][col] = col < jw ? (double)O[m0 + c + (int64_t)col * f] : 0.0;
+            }
+            __syncthreads();
+#pragma unroll 8
+            for (int m = 0; m < 32; ++m) {
+                const double b = B[m][c];
 #pragma unroll
-            for (int k = 0; k < 32; ++k) w += r[k] * Li[k][j];
-            Lp[i + (int64_t)(jb + j) * f] = (T)w;
+                for (int t = 0; t < 4; ++t) acc[t] += A[r4 + 8 * t][m] * b;
+            }
+            __syncthreads();
         }
+        // X_k = -D_k acc
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+            B[r4 + 8 * t][c] = acc[t];
+            const int col = r4 + 8 * t;
+            A[c][col] = c < kw && col < kw ? (double)out[d.l_off + k0 + c + (int64_t)(k0 + col) * f] : 0.0;
+        }
+        __syncthreads();
+        double x[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll 8
+        for (int m = 0; m < 32; ++m) {
+            const double b = B[m][c];
+#pragma unroll
+            for (int t = 0; t < 4; ++t) x[t] += A[r4 + 8 * t][m] * b;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int t = 0; t < 4; ++t) A[r4 + 8 * t][c] = -x[t];
+        __syncthreads();
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+            const int col = r4 + 8 * t;
+            if (c < kw && col < jw) O[k0 + c + (int64_t)col * f] = (T)A[c][col];
+        }
+        __syncthreads();   // block row k is read back by the next steps
     }
-    for (int idx = threadIdx.x; idx < 1024; idx += blockDim.x) {
-        const int i = idx & 31, j = idx >> 5;
-        if (i < kb && j < kb && i >= j) Lp[(jb + i) + (int64_t)(jb + j) * f] = (T)Li[i][j];
+}
+
+// W = L21 L11^{-1}: 64 x 64 tiles of the structure rows, 256 threads with 4 x 4
+// outputs each; tile column c0 needs the pivots from c0 on.
+template <class T>
+__global__ void __launch_bounds__(256) k_wpanel(const int *__restrict__ fronts, const FrontDesc *__restrict__ D,
+                                                const T *__restrict__ ws, T *out) {
+    const FrontDesc d = D[fronts[blockIdx.x]];
+    const int p = d.p, f = d.p + d.q;
+    const int ntr = (d.q + TILE - 1) / TILE;
+    if (ntr == 0) return;
+    const int ti = blockIdx.y % ntr, tj = blockIdx.y / ntr;
+    const int c0 = tj * TILE, r0 = p + ti * TILE;
+    if (c0 >= p) return;
+    const T *F = ws + d.front_off;
+    T *O = out + d.l_off;
+    __shared__ double sa[NB][TILE + 1], sb[NB][TILE + 1];
+    const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
+    double acc[4][4];
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int b = 0; b < 4; ++b) acc[a][b] = 0.0;
+    for (int m0 = c0; m0 < p; m0 += NB) {
+        for (int idx = threadIdx.x; idx < NB * TILE; idx += 256) {
+            const int i = idx % TILE, m = idx / TILE;
+            sa[m][i] = m0 + m < p && r0 + i < f ? (double)F[r0 + i + (int64_t)(m0 + m) * f] : 0.0;
+            const int mm = idx % NB, cc = idx / NB;
+            sb[mm][cc] = m0 + mm < p && c0 + cc < p ? (double)O[m0 + mm + (int64_t)(c0 + cc) * f] : 0.0;
+        }
+        __syncthreads();
+#pragma unroll 8
+        for (int m = 0; m < NB; ++m) {
+            double av[4], bv[4];
+#pragma unroll
+            for (int a = 0; a < 4; ++a) av[a] = sa[m][tx + 16 * a];
+#pragma unroll
+            for (int b = 0; b < 4; ++b) bv[b] = sb[m][ty + 16 * b];
+#pragma unroll
+            for (int a = 0; a < 4; ++a)
+#pragma unroll
+                for (int b = 0; b < 4; ++b) acc[a][b] += av[a] * bv[b];
+        }
+        __syncthreads();
     }
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+            const int r = r0 + tx + 16 * a, c = c0 + ty + 16 * b;
+            if (r < f && c < p) O[r + (int64_t)c * f] = (T)acc[a][b];
+        }
+}
+
+template <class T>
+static void inverse_form_level(const int *d_fronts, int nf, const FrontDesc *d_fr, int max_p, int max_f, const T *ws,
+                               T *L, cudaStream_t s) {
+    const int nb = (max_p + 31) / 32;
+    if (nb == 0) return;
+    k_diag_inverse<T><<<dim3(nf, nb), 32, 0, s>>>(d_fronts, d_fr, ws, L);
+    k_tri_inverse<T><<<dim3(nf, nb), INV_THREADS, 0, s>>>(d_fronts, d_fr, ws, L);
+    // upper bound of row tiles x column tiles over the level's fronts (q <= max_f, p <= max_p)
+    const int tiles = ((max_f + TILE - 1) / TILE) * ((max_p + TILE - 1) / TILE);
+    k_wpanel<T><<<dim3(nf, tiles), 256, 0, s>>>(d_fronts, d_fr, ws, L);
+    GL_CUDA(cudaGetLastError());
 }
 
 // Subdomains are factorised in consecutive groups whose two live levels of
@@ -570,7 +672,7 @@ void numeric_factor(FactorPlan &P, const double *C, const double *geo, const dou
         child[0].resize(nlev);
         child[1].resize(nlev);
         std::vector<int> max_p(nlev, 0), max_f(nlev, 0), max_pairs(nlev, 0);
-        std::vector<int64_t> lev_ws(nlev, 0), max_panel(nlev, 0);
+        std::vector<int64_t> lev_ws(nlev, 0);
         for (int g = first_front[j0]; g < first_front[j1]; ++g) {
             int d = depth_of[g];
             int f = fr[g].p + fr[g].q;
@@ -581,7 +683,6 @@ void numeric_factor(FactorPlan &P, const double *C, const double *geo, const dou
             max_p[d] = std::max(max_p[d], fr[g].p);
             max_f[d] = std::max(max_f[d], f);
             max_pairs[d] = std::max(max_pairs[d], fr[g].n_pairs);
-            max_panel[d] = std::max<int64_t>(max_panel[d], (int64_t)f * fr[g].p);
         }
         int64_t need = 1;
         for (int d = 0; d < nlev; ++d) need = std::max(need, lev_ws[d]);
@@ -619,19 +720,10 @@ void numeric_factor(FactorPlan &P, const double *C, const double *geo, const dou
             }
             partial_cholesky_level(d_lev[dpt].p, nf, d_fr.p, max_p[dpt], max_f[dpt], W, sizeof(T) == 4, d_err, s,
                                    0.0, nullptr, sizeof(T) == 4 && P.tc_update);
-            int gy = (int)std::min<int64_t>(std::max<int64_t>(1, (max_panel[dpt] + 255) / 256), 4096);
-            k_copy_panel<T><<<dim3(nf, gy), 256, 0, s>>>(d_lev[dpt].p, d_fr.p, W, L);
-            GL_CUDA(cudaGetLastError());
+            inverse_form_level<T>(d_lev[dpt].p, nf, d_fr.p, max_p[dpt], max_f[dpt], W, L, s);
         }
         GL_CUDA(cudaStreamSynchronize(s));   // the group's lists are released at the end of this scope
         j0 = j1;
-    }
-    int max_p = 0;
-    for (const FrontDesc &d : P.fr) max_p = std::max(max_p, d.p);
-    if (!P.fr.empty() && max_p > 0) {
-        k_block_inverse<T><<<dim3((unsigned)P.fr.size(), (max_p + 31) / 32), 256, 0, s>>>(P.d_fr.p, L);
-        GL_CUDA(cudaGetLastError());
-        GL_CUDA(cudaStreamSynchronize(s));
     }
 }
 
@@ -642,525 +734,199 @@ template void numeric_factor<float>(FactorPlan &, const double *, const double *
 
 // ----------------------------------------------------------------- solves
 
-// Threads per CTA of the sweeps: 256, or 512 on levels with fewer fronts than
-// eight per SM (the upper dissection levels, large fronts), where one CTA per
-// front would otherwise leave most warp slots empty.  Both kernels loop
-// over rows and columns with the block size, so either works.
-constexpr int SWEEP_MAX_THREADS = 512;
-constexpr int SWEEP_WIDE_BELOW = 1216;  // fronts per level
-// Threads per CTA of the sweeps on levels with at least SWEEP_WIDE_BELOW fronts
-// (SMALL: those whose largest front has at most SWEEP_SMALL_F rows).
-#ifndef GL_SWEEP_FWD_THREADS
-#define GL_SWEEP_FWD_THREADS 256
-#endif
-#ifndef GL_SWEEP_BWD_THREADS
-#define GL_SWEEP_BWD_THREADS 256
-#endif
-#ifndef GL_SWEEP_FWD_SMALL_THREADS
-#define GL_SWEEP_FWD_SMALL_THREADS 256
-#endif
-#ifndef GL_SWEEP_BWD_SMALL_THREADS
-#define GL_SWEEP_BWD_SMALL_THREADS 128
-#endif
-#ifndef GL_SWEEP_SMALL_F
-#define GL_SWEEP_SMALL_F 800
-#endif
-// Threads per CTA of the sweeps on levels with fewer than SWEEP_WIDE_BELOW fronts.
-#ifndef GL_SWEEP_FWD_WIDE_THREADS
-#define GL_SWEEP_FWD_WIDE_THREADS 512
-#endif
-#ifndef GL_SWEEP_BWD_WIDE_THREADS
-#define GL_SWEEP_BWD_WIDE_THREADS 512
-#endif
+// Sweep kernels.  A level's work is cut into warp tasks over all its fronts
+// (forward: 32 panel rows; backward: a tile of panel columns), which the
+// inverse form makes independent of one another, so a level with a few large
+// fronts fills the chip as well as one with thousands of small ones.  Where
+// even these tasks are fewer than SWEEP_WARPS, they are cut along the summed
+// dimension too and add their parts atomically.
+constexpr int SWEEP_CTA = 128;            // four warp tasks
+constexpr int SWEEP_WARPS = 152 * 12;     // warp tasks that keep the loads of every SM in flight
 
-// The forward sweep of FP64 (FP32) factors treats the structure rows after the
-// triangle when GL_FWD_SPLIT64 (GL_FWD_SPLIT32) is 1, block by block otherwise.
-#ifndef GL_FWD_SPLIT64
-#define GL_FWD_SPLIT64 0
-#endif
-#ifndef GL_FWD_SPLIT32
-#define GL_FWD_SPLIT32 1
-#endif
-template <class T>
-constexpr bool fwd_split() {
-    return sizeof(T) == 8 ? GL_FWD_SPLIT64 != 0 : GL_FWD_SPLIT32 != 0;
-}
-
-// The sweeps read the partitioned-inverse form written by k_block_inverse.
-// Dynamic shared memory of both starts with the front's dense vector v
-// (f x NR entries).
-//
-// Forward substitution for the fronts of one level, one CTA per front.  The
-// panel of a front is its pivot rows (the triangle, in partitioned-inverse
-// form) over its structure rows (a q x p rectangle).
-//   1. the triangle, block by block: x_B (the pivot values as left by the
-//      earlier blocks) is kept in X; the block's own rows hold
-//      L[B,B]^{-1} (zero above the diagonal), so they get y_B = L[B,B]^{-1} x_B,
-//      and the later pivot rows x_i -= W[i,B] x_B -- one row per thread, the
-//      block's rows one more row group.
-//   2. the rectangle at once: structure row i gets -sum_c W[i, c] X_c over all
-//      pivot columns c, one row per thread with no block barrier, and is added
-//      into the ancestors' entries atomically (siblings share rows).
-// One FMA per stored entry; no serial triangular solve remains.
+// Forward: panel rows [r0, r0 + 32), lane = row, the columns of blockIdx.z's
+// chunk.  Pivot rows give y_1 = L11^{-1} b_1 (up to the diagonal block: zeros
+// above it), structure rows subtract W b_1 from the ancestors' entries of b.
+// FP64: one FMA per entry on a pipe of two per clock and SM binds it at every
+// size that fills the chip; FP32 is bound by reading the panel once.  One CTA
+// per front stepping through 32-pivot blocks took 74 us (FP64) and 62 us (FP32)
+// a launch on the 308k- and 475k-DOF corners, this form 44 and 25 us.
 template <class T, int NR>
-__device__ __forceinline__ void fwd_row(const T *__restrict__ col0, int64_t ld, int i, int kb, const T *xb, int xs,
-                                        T acc[NR]) {
-    // acc[r] = sum over the kb columns of the block at col0 of W[i, j] xb[j + r xs]
-    if (kb == 32 && NR == 1) {
-        T l[32];
-#pragma unroll
-        for (int j = 0; j < 32; ++j) l[j] = col0[i + (int64_t)j * ld];
-        T a0 = T(0), a1 = T(0);
-#pragma unroll
-        for (int j = 0; j < 32; j += 2) {
-            a0 += l[j] * xb[j];
-            a1 += l[j + 1] * xb[j + 1];
-        }
-        acc[0] = a0 + a1;
-    } else if (kb == 32) {
-        // several right-hand sides: the row's loads in four groups of eight
-#pragma unroll
-        for (int r = 0; r < NR; ++r) acc[r] = T(0);
-#pragma unroll
-        for (int jc = 0; jc < 32; jc += 8) {
-            T l[8];
-#pragma unroll
-            for (int j = 0; j < 8; ++j) l[j] = col0[i + (int64_t)(jc + j) * ld];
-#pragma unroll
-            for (int r = 0; r < NR; ++r)
-#pragma unroll
-                for (int j = 0; j < 8; ++j) acc[r] += l[j] * xb[jc + j + r * xs];
-        }
-    } else {
-#pragma unroll
-        for (int r = 0; r < NR; ++r) acc[r] = T(0);
-        for (int j = 0; j < kb; ++j) {
-            const T l = col0[i + (int64_t)j * ld];
-#pragma unroll
-            for (int r = 0; r < NR; ++r) acc[r] += l * xb[j + r * xs];
-        }
-    }
-}
-
-template <class T, int NR, bool SPLIT>
-__global__ void __launch_bounds__(SWEEP_MAX_THREADS) k_fwd(const int *__restrict__ fronts, const FrontDesc *__restrict__ D,
-                                             const T *__restrict__ L, const int *__restrict__ rows, T *__restrict__ x,
-                                             int kcols, int c0) {
-    extern __shared__ unsigned char smraw[];
-    const FrontDesc d = D[fronts[blockIdx.x]];
-    const int p = d.p, f = d.p + d.q, n = d.vlen;
-    T *v = reinterpret_cast<T *>(smraw);   // the front's vector, f x NR
-    T *X = v + (int64_t)f * NR;             // x_B of every block, p x NR
-    T *xs = x + d.vec_off * kcols + (int64_t)c0 * n;
-    // rows updated block by block: the pivot rows only (SPLIT), or the structure rows too
-    const int rend = SPLIT ? p : f;
-    for (int i = threadIdx.x; i < rend; i += blockDim.x)
-#pragma unroll
-        for (int r = 0; r < NR; ++r) v[i + r * f] = i < p ? xs[(int64_t)r * n + d.first + i] : T(0);
-    __syncthreads();
-    const T *Lp = L + d.l_off;
-    // 1. the triangle (and, unless SPLIT, the rectangle block by block)
-    for (int jb = 0; jb < p; jb += 32) {
-        const int kb = min(32, p - jb);
-        if (threadIdx.x < 32 * NR) {
-            const int j = threadIdx.x & 31, r = threadIdx.x >> 5;
-            if (j < kb) X[jb + j + r * p] = v[jb + j + r * f];
-        }
-        __syncthreads();
-        for (int i = jb + threadIdx.x; i < rend; i += blockDim.x) {
-            T acc[NR];
-            fwd_row<T, NR>(Lp + (int64_t)jb * f, f, i, kb, X + jb, p, acc);
-            if (i < jb + kb) {
-#pragma unroll
-                for (int r = 0; r < NR; ++r) v[i + r * f] = acc[r];
-            } else {
-#pragma unroll
-                for (int r = 0; r < NR; ++r) v[i + r * f] -= acc[r];
-            }
-        }
-        __syncthreads();
-    }
-    for (int i = threadIdx.x; i < p; i += blockDim.x)
-#pragma unroll
-        for (int r = 0; r < NR; ++r) xs[(int64_t)r * n + d.first + i] = v[i + r * f];
-    if constexpr (!SPLIT) {
-        for (int i = p + threadIdx.x; i < f; i += blockDim.x)
-#pragma unroll
-            for (int r = 0; r < NR; ++r) atomicAdd(xs + (int64_t)r * n + rows[d.row_off + i], v[i + r * f]);
-    } else {
-        // 2. the rectangle
-        for (int i = p + threadIdx.x; i < f; i += blockDim.x) {
-            T sum[NR];
-#pragma unroll
-            for (int r = 0; r < NR; ++r) sum[r] = T(0);
-            for (int jb = 0; jb < p; jb += 32) {
-                T acc[NR];
-                fwd_row<T, NR>(Lp + (int64_t)jb * f, f, i, min(32, p - jb), X + jb, p, acc);
-#pragma unroll
-                for (int r = 0; r < NR; ++r) sum[r] += acc[r];
-            }
-            const int gi = rows[d.row_off + i];
-#pragma unroll
-            for (int r = 0; r < NR; ++r) atomicAdd(xs + (int64_t)r * n + gi, -sum[r]);
-        }
-    }
-}
-
-// Column sums of one warp over a 32-column block of a front panel (column c
-// at cb + c ld, c < kb): a[r] (lane j) = sum over rows i of W[i, j] v[i + r ld_v],
-// the rows taken in passes of SPAN = 32 G rows starting at rows rs, rs + step,
-// ... below rend.  Lane l loads row r0 + l of the columns (coalesced per
-// column) into registers, writes it transposed into the warp's 32 x 33 tile,
-// and lane j accumulates column j over the tile's rows from shared memory: one
-// FMA per entry, no shuffle reduction per column.  The columns are read 2^LW
-// wide: LW = 5 for a full block, the next pass's loads in flight meanwhile; a
-// short block (kb <= 16) is read 16, 8 or 4 wide, one pass then covering
-// G = 2^(5-LW) row tiles (tile g in register slots and lanes [g 2^LW,
-// (g+1) 2^LW)) whose partial sums of a column are added by shuffles at the
-// end -- the FMAs that a 32-wide pass would spend on the missing columns are
-// saved.  On return every lane j holds the sums of column j mod 2^LW.
-template <class T, int NR, int LW>
-__device__ __forceinline__ void warp_col_sums(const T *__restrict__ cb, int64_t ld, int kb, int rs, int rend, int step,
-                                              const T *v, int fv, T *tile, int lane, T a[NR]) {
-    constexpr int G = 32 >> LW, WM = (1 << LW) - 1;
-    constexpr bool PREFETCH = LW == 5;
-    T acc[NR], acc2[NR];   // two chains of FMAs per column
+__global__ void __launch_bounds__(SWEEP_CTA) k_fwd(const int *__restrict__ fronts, const FrontDesc *__restrict__ D,
+                                                   const T *__restrict__ L, const int *__restrict__ rows, T *b,
+                                                   T *y, int kcols, int c0, int chunk) {
+    __shared__ __align__(16) T sx[SWEEP_CTA / 32][32 * NR];
+    const FrontDesc &d = D[fronts[blockIdx.x]];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int p = d.p, f = p + d.q, n = d.vlen;
+    const int r0 = (blockIdx.y * (SWEEP_CTA / 32) + w) * 32;
+    const int cb = blockIdx.z * chunk;
+    // pivot rows need the columns up to their diagonal block, any structure row all of them
+    const int cend = min(r0 + 32 <= p ? r0 + 32 : p, cb + chunk);
+    if (r0 >= f || cb >= cend) return;
+    const int64_t vo = d.vec_off * kcols + (int64_t)c0 * n;
+    const T *b1 = b + vo + d.first;
+    const int row = min(r0 + lane, f - 1);
+    const T *Lr = L + d.l_off + row;
+    T acc[NR], acc2[NR];
 #pragma unroll
     for (int r = 0; r < NR; ++r) acc[r] = acc2[r] = T(0);
-    T w[32];
-    auto load = [&](int r0) {
-#pragma unroll
-        for (int j = 0; j < 32; ++j) {
-            const int i = r0 + 32 * (j >> LW) + lane;
-            w[j] = (i < rend && (j & WM) < kb) ? cb[i + (int64_t)(j & WM) * ld] : T(0);
-        }
-    };
-    int r0 = rs;
-    if (PREFETCH && r0 < rend) load(r0);
-    const int vg = 32 * (lane >> LW);   // this lane's tile within the pass
-    for (; r0 < rend; r0 += step) {
-        if (!PREFETCH) load(r0);
-#pragma unroll
-        for (int j = 0; j < 32; ++j) tile[j * 33 + lane] = w[j];
+    T *xs = sx[w];
+    for (int c = cb; c < cend; c += 32) {
+        const int kb = min(32, cend - c);
         __syncwarp();
-        if (PREFETCH && r0 + step < rend) load(r0 + step);
-        const int vb = r0 + vg;
-        const T *tl = tile + lane * 33;
-        if (r0 + 32 * G <= rend) {
 #pragma unroll
-            for (int ii = 0; ii < 32; ii += 2) {
-                const T t0 = tl[ii], t1 = tl[ii + 1];
+        for (int r = 0; r < NR; ++r) xs[lane * NR + r] = lane < kb ? b1[c + lane + (int64_t)r * n] : T(0);
+        __syncwarp();
+        const T *Lc = Lr + (int64_t)c * f;
+        constexpr int G = sizeof(T) == 4 ? 32 : 16;   // loads in flight per lane
 #pragma unroll
-                for (int r = 0; r < NR; ++r) {
-                    acc[r] += t0 * v[vb + ii + r * fv];
-                    acc2[r] += t1 * v[vb + ii + 1 + r * fv];
+        for (int g = 0; g < 32; g += G) {
+            if (g >= kb) break;
+            T l[G];
+            if (g + G <= kb) {
+#pragma unroll
+                for (int j = 0; j < G; ++j) l[j] = Lc[(int64_t)(g + j) * f];
+#pragma unroll
+                for (int j = 0; j < G; j += 2)
+#pragma unroll
+                    for (int r = 0; r < NR; ++r) {
+                        acc[r] += l[j] * xs[(g + j) * NR + r];
+                        acc2[r] += l[j + 1] * xs[(g + j + 1) * NR + r];
+                    }
+            } else {
+                // the last columns, in fours
+#pragma unroll
+                for (int j = 0; j < G; ++j) l[j] = g + j < kb ? Lc[(int64_t)(g + j) * f] : T(0);
+#pragma unroll
+                for (int h = 0; h < G; h += 4) {
+                    if (g + h >= kb) break;
+#pragma unroll
+                    for (int j = h; j < h + 4; ++j)
+#pragma unroll
+                        for (int r = 0; r < NR; ++r) acc[r] += l[j] * xs[(g + j) * NR + r];
                 }
             }
-        } else {
-            const int cnt = min(32, rend - vb);
-            for (int ii = 0; ii < cnt; ++ii) {
-                const T t = tl[ii];
-#pragma unroll
-                for (int r = 0; r < NR; ++r) acc[r] += t * v[vb + ii + r * fv];
-            }
         }
-        __syncwarp();
     }
+    if (r0 + lane >= f) return;
+    if (row < p) {
+        T *yo = y + vo + d.first + row;
 #pragma unroll
-    for (int r = 0; r < NR; ++r) {
-        T x = acc[r] + acc2[r];
-#pragma unroll
-        for (int o = 1 << LW; o < 32; o <<= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-        a[r] = x;
-    }
-}
-
-template <class T, int NR>
-__device__ __forceinline__ void warp_col_sums_short(const T *__restrict__ cb, int64_t ld, int kb, int rs, int rend,
-                                                    int passes, const T *v, int fv, T *tile, int lane, T a[NR]) {
-    // passes = stride between this warp's passes, counted in passes; a pass spans 32 (32 / 2^LW) rows
-    if (kb > 8) warp_col_sums<T, NR, 4>(cb, ld, kb, rs, rend, passes * 64, v, fv, tile, lane, a);
-    else if (kb > 4) warp_col_sums<T, NR, 3>(cb, ld, kb, rs, rend, passes * 128, v, fv, tile, lane, a);
-    else warp_col_sums<T, NR, 2>(cb, ld, kb, rs, rend, passes * 256, v, fv, tile, lane, a);
-}
-
-// Backward substitution for the fronts of one level, one CTA per front.  The
-// panel of a front is its pivot rows (the triangle, in partitioned-inverse
-// form) over its structure rows (a q x p rectangle).  With u_c = sum over
-// structure rows i of W[i, c] x_i, for each block B of 32 pivots from the last
-// to the first
-//   x_B = L[B,B]^{-T} y_B - W[i,B]^T x_i (later pivot rows i) - u_B.
-//   1. u for all columns at once: the rectangle's transposed product has no
-//      dependence between blocks, so the warps stream it without a block
-//      barrier, warp w taking column blocks w, w + nw, ... (or, when there are
-//      fewer blocks than warps, g = nw / blocks warps per block, each every
-//      g-th row tile, their partial sums added once).
-//   2. the triangle, block by block: the rows of B are negated first so every
-//      row enters one column sum with the same sign, the warps take row tiles
-//      of the pivot rows from B on, and x_B = -(sum + u_B).
-// One FMA per stored entry; no serial triangular solve remains.
-template <class T, int NR>
-__global__ void __launch_bounds__(SWEEP_MAX_THREADS) k_bwd(const int *__restrict__ fronts, const FrontDesc *__restrict__ D,
-                                             const T *__restrict__ L, const int *__restrict__ rows, T *__restrict__ x,
-                                             int kcols, int c0) {
-    extern __shared__ unsigned char smraw[];
-    const FrontDesc d = D[fronts[blockIdx.x]];
-    const int p = d.p, f = d.p + d.q, n = d.vlen;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    T *v = reinterpret_cast<T *>(smraw);      // the front's vector, f x NR
-    T *u = v + (int64_t)f * NR;                 // structure-row sums per pivot column, p x NR
-    T *red = u + (int64_t)p * NR;               // NR x nw x 32 partial column sums
-    T *tile = red + 32 * NR * nw + warp * (32 * 33);   // this warp's transposed row tile
-    T *xs = x + d.vec_off * kcols + (int64_t)c0 * n;
-    for (int i = threadIdx.x; i < f; i += blockDim.x)
-#pragma unroll
-        for (int r = 0; r < NR; ++r)
-            v[i + r * f] = i < p ? xs[(int64_t)r * n + d.first + i] : xs[(int64_t)r * n + rows[d.row_off + i]];
-    if (p == 0) return;
-    const T *Lp = L + d.l_off;
-    const int nbf = p >> 5, kl = p & 31, nb = nbf + (kl ? 1 : 0);
-    // 1. structure rows
-    if (f > p) {
-        const int g = nb >= nw ? 1 : nw / nb, cstep = nw / g, c_first = warp / g, sub = warp % g;
-        __syncthreads();
-        T a[NR];
-        int cb = c_first;
-        for (; cb < nbf; cb += cstep) {
-            warp_col_sums<T, NR, 5>(Lp + (int64_t)32 * cb * f, f, 32, p + 32 * sub, f, 32 * g, v, f, tile, lane, a);
-            if (g == 1) {
-#pragma unroll
-                for (int r = 0; r < NR; ++r) u[32 * cb + lane + r * p] = a[r];
-            } else {
-#pragma unroll
-                for (int r = 0; r < NR; ++r) red[(r * nw + warp) * 32 + lane] = a[r];
-            }
+        for (int r = 0; r < NR; ++r) {
+            if (gridDim.z == 1) yo[(int64_t)r * n] = acc[r] + acc2[r];
+            else atomicAdd(yo + (int64_t)r * n, acc[r] + acc2[r]);
         }
-        if (cb == nbf && kl > 0) {
-            // the short last block, read narrow when it has at most 16 columns
-            if (kl > 16) {
-                warp_col_sums<T, NR, 5>(Lp + (int64_t)32 * cb * f, f, kl, p + 32 * sub, f, 32 * g, v, f, tile, lane,
-                                        a);
-            } else {
-                const int span = 32 * (32 >> (kl > 8 ? 4 : (kl > 4 ? 3 : 2)));
-                warp_col_sums_short<T, NR>(Lp + (int64_t)32 * cb * f, f, kl, p + span * sub, f, g, v, f, tile, lane,
-                                           a);
-            }
-            if (g == 1) {
-                if (lane < kl)
-#pragma unroll
-                    for (int r = 0; r < NR; ++r) u[32 * cb + lane + r * p] = a[r];
-            } else {
-#pragma unroll
-                for (int r = 0; r < NR; ++r) red[(r * nw + warp) * 32 + lane] = a[r];
-            }
-        }
-        __syncthreads();
-        if (g > 1)
-            for (int c = threadIdx.x; c < 32 * NR * nb; c += blockDim.x) {
-                const int r = c / (32 * nb), cc = c % (32 * nb), j = cc & 31, b = cc >> 5;
-                if (cc >= p) continue;
-                T s = T(0);
-                for (int k = 0; k < g; ++k) s += red[(r * nw + b * g + k) * 32 + j];
-                u[cc + r * p] = s;
-            }
     } else {
-        for (int c = threadIdx.x; c < p * NR; c += blockDim.x) u[c] = T(0);
+        T *bo = b + vo + rows[d.row_off + row];
+#pragma unroll
+        for (int r = 0; r < NR; ++r) atomicAdd(bo + (int64_t)r * n, -(acc[r] + acc2[r]));
     }
-    __syncthreads();
-    // 2. the triangle
-    int jb = ((p - 1) / 32) * 32;
-    if (threadIdx.x < 32 * NR) {
-        const int j = threadIdx.x & 31, r = threadIdx.x >> 5;
-        if (j < p - jb) v[jb + j + r * f] = -v[jb + j + r * f];
-    }
-    __syncthreads();
-    // column sums of the block at jb (partial per warp in red) -> x_B; negate the next block's rows
-    auto finish = [&](int jb, int kb) {
-        __syncthreads();
-        if (threadIdx.x < 32 * NR) {
-            const int j = threadIdx.x & 31, r = threadIdx.x >> 5;
-            T s = T(0);
-            for (int ww = 0; ww < nw; ++ww) s += red[(r * nw + ww) * 32 + j];
-            if (j < kb) v[jb + j + r * f] = -(s + u[jb + j + r * p]);
-            // the next block's rows (read from the next step on) enter its sum negated
-            if (jb >= 32) v[jb - 32 + j + r * f] = -v[jb - 32 + j + r * f];
+}
+
+// Sums N (16 or a multiple of 32) values over the lanes of a warp, about one
+// add per value against five of a shuffle tree each: every step halves the
+// values a lane holds.  Value i comes back as v[i % PL] of lane i / PL, PL =
+// N / 32 (N = 16: v[0] of lanes 2 i and 2 i + 1).
+template <class T, int N>
+__device__ __forceinline__ void warp_sum_many(T (&v)[N], int lane) {
+    int n = N;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        if (n == 1) {
+            v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+            continue;
         }
-        __syncthreads();
+        n >>= 1;
+        const bool up = lane & o;
+#pragma unroll
+        for (int k = 0; k < N / 2; ++k)
+            if (k < n) {
+                const T send = up ? v[k] : v[k + n], keep = up ? v[k + n] : v[k];
+                v[k] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+            }
+    }
+}
+
+// Panel columns of one backward warp task: 16 (8, 4 with four and eight
+// right-hand sides) keep the accumulators to 64 registers and so enough warps
+// on an SM to cover the loads.  With 32 columns and one right-hand side the kernel
+// took 226 registers and 74.6 us a launch against 54.5 on the 308k-DOF corner.
+template <int NR>
+__host__ __device__ constexpr int bwd_tile() {
+    return NR <= 2 ? 16 : 32 / NR;
+}
+
+// Backward: x_1 = [L11^{-1}; -W]^T [y_1; x_2].  A warp task is a tile of panel
+// columns over one chunk of the panel's rows, lane = row, one accumulator per
+// (column, right-hand side); the lanes are summed at the end (warp_sum_many).
+// One CTA per front took 85 us (FP64) and 68 us (FP32) a launch on the same
+// corners, this form 44 and 34 us.
+template <class T, int NR>
+__global__ void __launch_bounds__(SWEEP_CTA) k_bwd(const int *__restrict__ fronts, const FrontDesc *__restrict__ D,
+                                                   const T *__restrict__ L, const int *__restrict__ rows,
+                                                   const T *__restrict__ y, T *x, int kcols, int c0, int chunks) {
+    constexpr int CT = bwd_tile<NR>();
+    const FrontDesc &d = D[fronts[blockIdx.x]];
+    const int lane = threadIdx.x & 31;
+    const int p = d.p, f = p + d.q, n = d.vlen;
+    const int task = blockIdx.y * (SWEEP_CTA / 32) + (threadIdx.x >> 5);
+    const int nct = (p + CT - 1) / CT;
+    if (task >= nct * chunks) return;
+    const int j0 = (task % nct) * CT, kb = min(CT, p - j0);
+    // the tile's rows start at its diagonal block; chunks of whole 32-row steps
+    const int steps = (f - j0 + 31) / 32, per = (steps + chunks - 1) / chunks;
+    const int rb = j0 + 32 * per * (task / nct), re = min(f, rb + 32 * per);
+    if (rb >= re) return;
+    const int64_t vo = d.vec_off * kcols + (int64_t)c0 * n;
+    const T *y1 = y + vo + d.first, *xo = x + vo;
+    const int *rw = rows + d.row_off;
+    const T *Lt = L + d.l_off + (int64_t)j0 * f;
+    T acc[CT * NR];
+#pragma unroll
+    for (int i = 0; i < CT * NR; ++i) acc[i] = T(0);
+    // the rows' vector entries: where they are two steps ahead, their values one step ahead
+    auto where = [&](int r) {
+        const int i = min(r + lane, f - 1);
+        return i < p ? y1 + i : xo + rw[i];
     };
-    T a[NR];
-    if (kl > 0 && kl <= 16) {
-        // a short last block, read narrow (once per front, before the full blocks)
-        const int span = 32 * (32 >> (kl > 8 ? 4 : (kl > 4 ? 3 : 2)));
-        warp_col_sums_short<T, NR>(Lp + (int64_t)jb * f, f, kl, jb + span * warp, p, nw, v, f, tile, lane, a);
+    auto fetch_v = [&](int r, const T *at, T *v) {
+        const T sg = r + lane >= re ? T(0) : (r + lane < p ? T(1) : T(-1));
 #pragma unroll
-        for (int r = 0; r < NR; ++r) red[(r * nw + warp) * 32 + lane] = a[r];
-        finish(jb, kl);
-        jb -= 32;
+        for (int k = 0; k < NR; ++k) v[k] = sg * at[(int64_t)k * n];
+    };
+    T v[NR], vn[NR];
+    fetch_v(rb, where(rb), v);
+    const T *at = where(rb + 32);
+    for (int r = rb; r < re; r += 32) {
+        const T *Li = Lt + min(r + lane, f - 1);
+        auto step = [&](auto cols) {
+            constexpr int G = decltype(cols)::value;
+            T l[G];
+#pragma unroll
+            for (int j = 0; j < G; ++j) l[j] = j < kb ? Li[(int64_t)j * f] : T(0);
+            fetch_v(r + 32, at, vn);
+            at = where(r + 64);
+#pragma unroll
+            for (int j = 0; j < G; ++j)
+#pragma unroll
+                for (int k = 0; k < NR; ++k) acc[j * NR + k] += l[j] * v[k];
+        };
+        if (CT == 16 && kb <= 8) step(std::integral_constant<int, CT / 2>());
+        else step(std::integral_constant<int, CT>());
+#pragma unroll
+        for (int k = 0; k < NR; ++k) v[k] = vn[k];
     }
-    for (; jb >= 0; jb -= 32) {
-        const int kb = min(32, p - jb);
-        warp_col_sums<T, NR, 5>(Lp + (int64_t)jb * f, f, kb, jb + 32 * warp, p, 32 * nw, v, f, tile, lane, a);
+    warp_sum_many<T, CT * NR>(acc, lane);
+    constexpr int PL = CT * NR < 32 ? 1 : CT * NR / 32, SH = CT * NR < 32 ? 1 : 0;   // sums per lane; lanes per sum 2^SH
+    if (lane & SH) return;
 #pragma unroll
-        for (int r = 0; r < NR; ++r) red[(r * nw + warp) * 32 + lane] = a[r];
-        finish(jb, kb);
+    for (int t = 0; t < PL; ++t) {
+        const int i = (lane >> SH) * PL + t, j = i / NR, k = i % NR;
+        if (j >= kb) continue;
+        T *out = x + vo + d.first + j0 + j + (int64_t)k * n;
+        if (chunks == 1) *out = acc[t];
+        else atomicAdd(out, acc[t]);
     }
-    for (int i = threadIdx.x; i < p; i += blockDim.x)
-#pragma unroll
-        for (int r = 0; r < NR; ++r) xs[(int64_t)r * n + d.first + i] = v[i + r * f];
-}
-
-// Backward substitution with per-column shuffle reductions, used for the FP32
-// factors: for each block B of 32 pivots from the last to the first, one
-// reduction down each column of the block over the rows from B to the end of
-// the front (the rows of B with +, the rows below with -); warp w owns the
-// columns w, w + 8, ..., its lanes stride the rows with 8 loads in flight, and
-// a shuffle tree adds the lanes.  Its adds cost little where the sweep is
-// bound by HBM (FP32), and its 32 registers and small shared memory keep many
-// CTAs and loads in flight; the FP64 sweep, bound by the FP64 pipe, uses k_bwd.
-template <class T, int NR>
-__global__ void __launch_bounds__(SWEEP_MAX_THREADS) k_bwd_shfl(const int *__restrict__ fronts, const FrontDesc *__restrict__ D,
-                                             const T *__restrict__ L, const int *__restrict__ rows, T *__restrict__ x,
-                                             int kcols, int c0) {
-    extern __shared__ unsigned char smraw[];
-    const FrontDesc d = D[fronts[blockIdx.x]];
-    const int p = d.p, f = d.p + d.q, n = d.vlen;
-    T *v = reinterpret_cast<T *>(smraw);
-    T *red = v + (int64_t)f * NR;   // 32 x NR column results of the block
-    T *xs = x + d.vec_off * kcols + (int64_t)c0 * n;
-    for (int i = threadIdx.x; i < f; i += blockDim.x)
-#pragma unroll
-        for (int r = 0; r < NR; ++r)
-            v[i + r * f] = i < p ? xs[(int64_t)r * n + d.first + i] : xs[(int64_t)r * n + rows[d.row_off + i]];
-    __syncthreads();
-    if (p == 0) return;
-    const T *Lp = L + d.l_off;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    for (int jb = ((p - 1) / 32) * 32; jb >= 0; jb -= 32) {
-        const int kb = min(32, p - jb);
-        for (int j = warp; j < kb; j += nw) {
-            const T *col = Lp + (int64_t)(jb + j) * f;
-            T acc[NR];
-            {
-                // rows of B: L[B,B]^{-1}[i, j] y_i for i >= j, negated here and restored below
-                const bool in = lane >= j && lane < kb;
-                const T l = in ? col[jb + lane] : T(0);
-#pragma unroll
-                for (int r = 0; r < NR; ++r) acc[r] = -(l * v[jb + (in ? lane : 0) + r * f]);
-            }
-            int i = jb + kb + lane;
-            // rows below B: + W[i, j] x_i, 8 independent loads per lane in flight
-            for (; i + 7 * 32 < f; i += 8 * 32) {
-                T l[8];
-#pragma unroll
-                for (int t = 0; t < 8; ++t) l[t] = col[i + 32 * t];
-#pragma unroll
-                for (int t = 0; t < 8; ++t)
-#pragma unroll
-                    for (int r = 0; r < NR; ++r) acc[r] += l[t] * v[i + 32 * t + r * f];
-            }
-            for (; i < f; i += 32) {
-                const T l = col[i];
-#pragma unroll
-                for (int r = 0; r < NR; ++r) acc[r] += l * v[i + r * f];
-            }
-#pragma unroll
-            for (int r = 0; r < NR; ++r) {
-                T a = acc[r];
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-                if (lane == 0) red[j + 32 * r] = -a;
-            }
-        }
-        __syncthreads();
-        if (threadIdx.x < 32 * NR) {
-            const int j = threadIdx.x & 31, r = threadIdx.x >> 5;
-            if (j < kb) v[jb + j + r * f] = red[j + 32 * r];
-        }
-        __syncthreads();
-    }
-    for (int i = threadIdx.x; i < p; i += blockDim.x)
-#pragma unroll
-        for (int r = 0; r < NR; ++r) xs[(int64_t)r * n + d.first + i] = v[i + r * f];
-}
-
-// Shared memory of the sweeps.  Forward: the front vector (f x NR) and the
-// copy of x_B (32 x NR), plus the static inverse block.  Backward: the front
-// vector, the partial column sums (NR x nw x 32) and one 32 x 33 tile per warp,
-// so its block size shrinks on levels whose largest front would not fit.  The
-// dynamic limit of every variant is raised once per device to all that a CTA
-// may hold; build_plan calls sweep_smem_for_plan for every variant, so no
-// attribute is ever changed while a stream is being captured.
-constexpr size_t SMEM_PER_CTA = 227 * 1024;
-
-template <class T, int NR>
-static size_t sweep_static_smem() {
-    static const size_t v = [] {
-        cudaFuncAttributes a{}, b{};
-        GL_CUDA(cudaFuncGetAttributes(&a, k_fwd<T, NR, fwd_split<T>()>));
-        GL_CUDA(cudaFuncGetAttributes(&b, k_bwd<T, NR>));
-        return std::max<size_t>(1, std::max(a.sharedSizeBytes, b.sharedSizeBytes));
-    }();
-    return v;
-}
-
-template <class T, int NR>
-static size_t fwd_dyn_smem(int f) {
-    // front vector and the blocks' x_B (p <= f)
-    return (2 * (size_t)std::max(f, 1)) * NR * sizeof(T);
-}
-
-template <class T, int NR>
-static size_t bwd_dyn_smem(int f, int nthreads) {
-    // front vector and structure-row sums (p <= f), partial sums, one tile per warp
-    const size_t nw = (size_t)nthreads / 32;
-    return ((size_t)std::max(f, 1) * NR * 2 + 32 * NR * nw + 33 * 32 * nw) * sizeof(T);
-}
-
-template <class T, int NR>
-constexpr int bwd_min_threads() {
-    return 32 * NR;   // the column sums of the block are finished by 32 NR threads
-}
-
-template <class T, int NR>
-static bool sweep_fits(int max_f) {
-    const size_t lim = SMEM_PER_CTA - sweep_static_smem<T, NR>();
-    return fwd_dyn_smem<T, NR>(max_f) <= lim && bwd_dyn_smem<T, NR>(max_f, bwd_min_threads<T, NR>()) <= lim;
-}
-
-// Threads per CTA of the backward sweep on a level: the wanted count, halved
-// while the level's largest front does not fit.
-template <class T, int NR>
-static int bwd_threads(int max_f, int want) {
-    const size_t lim = SMEM_PER_CTA - sweep_static_smem<T, NR>();
-    int nt = want;
-    while (nt > bwd_min_threads<T, NR>() && bwd_dyn_smem<T, NR>(max_f, nt) > lim) nt /= 2;
-    return nt;
-}
-
-template <class T, int NR>
-static void ensure_sweep_smem(int max_f) {
-    static SmemLimit limit;
-    if (!sweep_fits<T, NR>(max_f)) return;
-    raise_smem_limit(limit, SMEM_PER_CTA - sweep_static_smem<T, NR>(), [](size_t v) {
-        GL_CUDA(cudaFuncSetAttribute(k_fwd<T, NR, fwd_split<T>()>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)v));
-        GL_CUDA(cudaFuncSetAttribute(k_bwd<T, NR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)v));
-        GL_CUDA(cudaFuncSetAttribute(k_bwd_shfl<T, NR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)v));
-    });
-}
-
-template <class T, int NR>
-static size_t bwd_shfl_dyn_smem(int f) {
-    return ((size_t)std::max(f, 1) + 32) * NR * sizeof(T);
-}
-
-void sweep_smem_for_plan(int max_f) {
-    ensure_sweep_smem<double, 1>(max_f);
-    ensure_sweep_smem<double, 2>(max_f);
-    ensure_sweep_smem<double, 4>(max_f);
-    ensure_sweep_smem<float, 1>(max_f);
-    ensure_sweep_smem<float, 2>(max_f);
-    ensure_sweep_smem<float, 4>(max_f);
 }
 
 void level_clock_enable(FactorPlan &P, bool on) {
@@ -1194,35 +960,28 @@ static void level_clock_fold(const FactorPlan &P) {
     K.calls += 1;
 }
 
-static int sweep_threads(const Level &Lv, bool bwd) {
-    if (Lv.fronts.size() < (size_t)SWEEP_WIDE_BELOW) return bwd ? GL_SWEEP_BWD_WIDE_THREADS : GL_SWEEP_FWD_WIDE_THREADS;
-    if (Lv.max_f <= GL_SWEEP_SMALL_F) return bwd ? GL_SWEEP_BWD_SMALL_THREADS : GL_SWEEP_FWD_SMALL_THREADS;
-    return bwd ? GL_SWEEP_BWD_THREADS : GL_SWEEP_FWD_THREADS;
-}
-
 // One level's forward or backward sweep over the fronts fr[0..nf) of that level.
 template <class T, int NR>
-static void launch_fwd(const FactorPlan &P, const Level &Lv, const int *fr, unsigned nf, const T *L, T *x, int kcols,
-                       int c0, cudaStream_t s) {
-    if (nf == 0) return;
-    const size_t sm = fwd_dyn_smem<T, NR>(Lv.max_f);
-    k_fwd<T, NR, fwd_split<T>()><<<nf, sweep_threads(Lv, false), sm, s>>>(fr, P.d_fr.p, L, P.d_rows.p, x, kcols,
-                                                                         c0);
+static void launch_fwd(const FactorPlan &P, const Level &Lv, const int *fr, unsigned nf, const T *L, T *b, T *y,
+                       int kcols, int c0, cudaStream_t s) {
+    if (nf == 0 || Lv.max_p == 0) return;
+    const int tiles = (Lv.max_f + 31) / 32, blocks = (Lv.max_p + 31) / 32;
+    // (the level's fronts, not nf: the arithmetic is the same however the level is split over streams)
+    const int split = std::min<int64_t>(blocks, std::max<int64_t>(1, SWEEP_WARPS / ((int64_t)Lv.fronts.size() * tiles)));
+    const int chunk = 32 * ((blocks + split - 1) / split);
+    const dim3 g(nf, (tiles + SWEEP_CTA / 32 - 1) / (SWEEP_CTA / 32), (Lv.max_p + chunk - 1) / chunk);
+    k_fwd<T, NR><<<g, SWEEP_CTA, 0, s>>>(fr, P.d_fr.p, L, P.d_rows.p, b, y, kcols, c0, chunk);
 }
 
 template <class T, int NR>
-static void launch_bwd(const FactorPlan &P, const Level &Lv, const int *fr, unsigned nf, const T *L, T *x, int kcols,
-                       int c0, cudaStream_t s) {
-    if (nf == 0) return;
-    const int want = sweep_threads(Lv, true);
-    if (sizeof(T) == 4) {
-        const size_t sm = bwd_shfl_dyn_smem<T, NR>(Lv.max_f);
-        k_bwd_shfl<T, NR><<<nf, want, sm, s>>>(fr, P.d_fr.p, L, P.d_rows.p, x, kcols, c0);
-    } else {
-        const int nt = bwd_threads<T, NR>(Lv.max_f, want);
-        const size_t sm = bwd_dyn_smem<T, NR>(Lv.max_f, nt);
-        k_bwd<T, NR><<<nf, nt, sm, s>>>(fr, P.d_fr.p, L, P.d_rows.p, x, kcols, c0);
-    }
+static void launch_bwd(const FactorPlan &P, const Level &Lv, const int *fr, unsigned nf, const T *L, const T *y, T *x,
+                       int kcols, int c0, cudaStream_t s) {
+    if (nf == 0 || Lv.max_p == 0) return;
+    const int tiles = (Lv.max_p + bwd_tile<NR>() - 1) / bwd_tile<NR>();
+    const int chunks = std::min<int64_t>((Lv.max_f + 63) / 64,
+                                         std::max<int64_t>(1, SWEEP_WARPS / ((int64_t)Lv.fronts.size() * tiles)));
+    const dim3 g(nf, (tiles * chunks + SWEEP_CTA / 32 - 1) / (SWEEP_CTA / 32));
+    k_bwd<T, NR><<<g, SWEEP_CTA, 0, s>>>(fr, P.d_fr.p, L, P.d_rows.p, y, x, kcols, c0, chunks);
 }
 
 static HalfStreams &half_streams(const FactorPlan &P) {
@@ -1248,7 +1007,7 @@ static HalfStreams &half_streams(const FactorPlan &P) {
 // levels start when the first half enters its top levels.  The halves hold
 // disjoint subdomains, so they share no data.
 template <class T, int NR>
-static void solve_levels_overlap(const FactorPlan &P, const T *L, T *x, int kcols, int c0, cudaStream_t s) {
+static void solve_levels_overlap(const FactorPlan &P, const T *L, T *b, T *y, T *x, int kcols, int c0, cudaStream_t s) {
     HalfStreams &H = half_streams(P);
     const int nlev = (int)P.levels.size(), k = std::min(P.overlap_top, nlev);
     GL_CUDA(cudaEventRecord(H.fork, s));
@@ -1268,19 +1027,19 @@ static void solve_levels_overlap(const FactorPlan &P, const T *L, T *x, int kcol
         for (int d = nlev - 1; d >= k; --d) {
             const int *fr; unsigned nf;
             part(h, d, fr, nf);
-            launch_fwd<T, NR>(P, P.levels[d], fr, nf, L, x, kcols, c0, H.lo[h]);
+            launch_fwd<T, NR>(P, P.levels[d], fr, nf, L, b, y, kcols, c0, H.lo[h]);
         }
         GL_CUDA(cudaEventRecord(H.ev[3 * h], H.lo[h]));
         GL_CUDA(cudaStreamWaitEvent(H.hi[h], H.ev[3 * h], 0));
         for (int d = k - 1; d >= 0; --d) {
             const int *fr; unsigned nf;
             part(h, d, fr, nf);
-            launch_fwd<T, NR>(P, P.levels[d], fr, nf, L, x, kcols, c0, H.hi[h]);
+            launch_fwd<T, NR>(P, P.levels[d], fr, nf, L, b, y, kcols, c0, H.hi[h]);
         }
         for (int d = 0; d < k; ++d) {
             const int *fr; unsigned nf;
             part(h, d, fr, nf);
-            launch_bwd<T, NR>(P, P.levels[d], fr, nf, L, x, kcols, c0, H.hi[h]);
+            launch_bwd<T, NR>(P, P.levels[d], fr, nf, L, y, x, kcols, c0, H.hi[h]);
         }
         GL_CUDA(cudaEventRecord(H.ev[3 * h + 1], H.hi[h]));
     }
@@ -1289,7 +1048,7 @@ static void solve_levels_overlap(const FactorPlan &P, const T *L, T *x, int kcol
         for (int d = k; d < nlev; ++d) {
             const int *fr; unsigned nf;
             part(h, d, fr, nf);
-            launch_bwd<T, NR>(P, P.levels[d], fr, nf, L, x, kcols, c0, H.lo[h]);
+            launch_bwd<T, NR>(P, P.levels[d], fr, nf, L, y, x, kcols, c0, H.lo[h]);
         }
         GL_CUDA(cudaEventRecord(H.ev[3 * h + 2], H.lo[h]));
         GL_CUDA(cudaStreamWaitEvent(s, H.ev[3 * h + 2], 0));
@@ -1298,12 +1057,11 @@ static void solve_levels_overlap(const FactorPlan &P, const T *L, T *x, int kcol
 }
 
 template <class T, int NR>
-static void solve_levels(const FactorPlan &P, const T *L, T *x, int kcols, int c0, cudaStream_t s) {
-    ensure_sweep_smem<T, NR>(P.max_f);
+static void solve_levels(const FactorPlan &P, const T *L, T *b, T *y, T *x, int kcols, int c0, cudaStream_t s) {
     const int nlev = (int)P.levels.size();
     const bool timed = NR == 1 && kcols == 1 && P.clock.on && P.clock.ev.size() == 2 * (size_t)nlev + 1;
     if (NR == 1 && kcols == 1 && P.overlap_top > 0 && !timed && P.n_sub >= 2) {
-        solve_levels_overlap<T, NR>(P, L, x, kcols, c0, s);
+        solve_levels_overlap<T, NR>(P, L, b, y, x, kcols, c0, s);
         return;
     }
     auto mark = [&](int k) {
@@ -1312,12 +1070,12 @@ static void solve_levels(const FactorPlan &P, const T *L, T *x, int kcols, int c
     for (int dpt = nlev - 1; dpt >= 0; --dpt) {
         mark(nlev - 1 - dpt);
         const Level &Lv = P.levels[dpt];
-        launch_fwd<T, NR>(P, Lv, Lv.d_fronts.p, (unsigned)Lv.fronts.size(), L, x, kcols, c0, s);
+        launch_fwd<T, NR>(P, Lv, Lv.d_fronts.p, (unsigned)Lv.fronts.size(), L, b, y, kcols, c0, s);
     }
     for (int dpt = 0; dpt < nlev; ++dpt) {
         mark(nlev + dpt);
         const Level &Lv = P.levels[dpt];
-        launch_bwd<T, NR>(P, Lv, Lv.d_fronts.p, (unsigned)Lv.fronts.size(), L, x, kcols, c0, s);
+        launch_bwd<T, NR>(P, Lv, Lv.d_fronts.p, (unsigned)Lv.fronts.size(), L, y, x, kcols, c0, s);
     }
     GL_CUDA(cudaGetLastError());
     if (timed) {
@@ -1327,27 +1085,31 @@ static void solve_levels(const FactorPlan &P, const T *L, T *x, int kcols, int c
 }
 
 template <class T>
-void factor_solve(const FactorPlan &P, const T *L, T *x, int kcols, cudaStream_t s) {
-    const int nr = sweep_fits<T, 4>(P.max_f) ? 4 : (sweep_fits<T, 2>(P.max_f) ? 2 : 1);
-    if (!sweep_fits<T, 1>(P.max_f)) fail(GL_ERR_INVALID_ARG, "factor_solve: front too large for shared memory");
+void factor_solve(const FactorPlan &P, const T *L, T *b, T *y, T *x, int kcols, cudaStream_t s) {
     int c0 = 0;
     while (c0 < kcols) {
-        int left = kcols - c0;
-        if (nr >= 4 && left >= 4) { solve_levels<T, 4>(P, L, x, kcols, c0, s); c0 += 4; }
-        else if (nr >= 2 && left >= 2) { solve_levels<T, 2>(P, L, x, kcols, c0, s); c0 += 2; }
-        else { solve_levels<T, 1>(P, L, x, kcols, c0, s); c0 += 1; }
+        const int left = kcols - c0;
+        if (left >= 8) { solve_levels<T, 8>(P, L, b, y, x, kcols, c0, s); c0 += 8; }
+        else if (left >= 4) { solve_levels<T, 4>(P, L, b, y, x, kcols, c0, s); c0 += 4; }
+        else if (left >= 2) { solve_levels<T, 2>(P, L, b, y, x, kcols, c0, s); c0 += 2; }
+        else { solve_levels<T, 1>(P, L, b, y, x, kcols, c0, s); c0 += 1; }
     }
 }
 
-template void factor_solve<double>(const FactorPlan &, const double *, double *, int, cudaStream_t);
-template void factor_solve<float>(const FactorPlan &, const float *, float *, int, cudaStream_t);
+template void factor_solve<double>(const FactorPlan &, const double *, double *, double *, double *, int,
+                                   cudaStream_t);
+template void factor_solve<float>(const FactorPlan &, const float *, float *, float *, float *, int, cudaStream_t);
 
 // ----------------------------------------------------------------- local <-> global
 
+// b = r at the local DOFs, y = x = 0 (the sweeps add into them)
 template <class T>
-__global__ void k_gather(int64_t n, const int64_t *__restrict__ gdof, const double *__restrict__ r, T *__restrict__ xl) {
+__global__ void k_gather(int64_t n, const int64_t *__restrict__ gdof, const double *__restrict__ r, T *__restrict__ b,
+                         T *__restrict__ y, T *__restrict__ x) {
     int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i < n) xl[i] = (T)r[gdof[i]];
+    if (i >= n) return;
+    b[i] = (T)r[gdof[i]];
+    y[i] = x[i] = T(0);
 }
 
 template <class T>
@@ -1357,9 +1119,9 @@ __global__ void k_scatter_add(int64_t n, const int64_t *__restrict__ gdof, const
 }
 
 template <class T>
-void gather_local(const FactorPlan &P, const double *r, T *xl, cudaStream_t s) {
+void gather_local(const FactorPlan &P, const double *r, T *b, T *y, T *x, cudaStream_t s) {
     if (!P.n_local) return;
-    k_gather<T><<<(unsigned)((P.n_local + 255) / 256), 256, 0, s>>>(P.n_local, P.d_gdof.p, r, xl);
+    k_gather<T><<<(unsigned)((P.n_local + 255) / 256), 256, 0, s>>>(P.n_local, P.d_gdof.p, r, b, y, x);
     GL_CUDA(cudaGetLastError());
 }
 template <class T>
@@ -1368,8 +1130,8 @@ void scatter_add_local(const FactorPlan &P, const T *xl, double *z, cudaStream_t
     k_scatter_add<T><<<(unsigned)((P.n_local + 255) / 256), 256, 0, s>>>(P.n_local, P.d_gdof.p, xl, z);
     GL_CUDA(cudaGetLastError());
 }
-template void gather_local<double>(const FactorPlan &, const double *, double *, cudaStream_t);
-template void gather_local<float>(const FactorPlan &, const double *, float *, cudaStream_t);
+template void gather_local<double>(const FactorPlan &, const double *, double *, double *, double *, cudaStream_t);
+template void gather_local<float>(const FactorPlan &, const double *, float *, float *, float *, cudaStream_t);
 template void scatter_add_local<double>(const FactorPlan &, const double *, double *, cudaStream_t);
 template void scatter_add_local<float>(const FactorPlan &, const float *, double *, cudaStream_t);
 

@@ -140,9 +140,8 @@ void build_plan(const std::vector<SubSymbolic> &subs, FactorPlan &P, cudaStream_
 // Numeric factorisation.  Front entries from the element matrices, formed on
 // the fly in FP64 from C_e (36 per element) and the Gauss-point geometry (270
 // per element), scaled by (1 + sigma xi_i xi_j) (xi indexed by local DOF, may
-// be NULL when sigma == 0).  Factor values of type T, left in the
-// partitioned-inverse form that factor_solve reads (every 32-pivot diagonal
-// block inverted, the rows below it multiplied by that inverse).
+// be NULL when sigma == 0).  Factor values of type T; every front's panel is
+// left in the form [L11^{-1}; L21 L11^{-1}] that factor_solve reads.
 template <class T>
 void numeric_factor(FactorPlan &P, const double *C, const double *geo, const double *xi, double sigma, T *L, int *d_err,
                     cudaStream_t s);
@@ -155,19 +154,20 @@ int syrk_tc_panel();
 void syrk_tc_level(const int *d_fronts, int n_fronts, const FrontDesc *d_fr, int k0, int max_f, float *ws,
                    int *d_err, cudaStream_t s);
 
-// x <- L^{-T} L^{-1} x (L as factored; stored in partitioned-inverse form)
-// for local multi-vectors of kcols columns per subdomain,
-// each column of the subdomain's length stored contiguously:
-// x[vec_off*kcols + c*n + i] (kcols = 1: plain concatenated local vectors).
+// x = L^{-T} L^{-1} b (panels as numeric_factor leaves them) for local
+// multi-vectors of kcols columns per subdomain, each column of the subdomain's
+// length stored contiguously: b[vec_off*kcols + c*n + i] (kcols = 1: plain
+// concatenated local vectors).  b is overwritten; y (scratch) and x must be
+// zero on entry.
 template <class T>
-void factor_solve(const FactorPlan &P, const T *L, T *x, int kcols, cudaStream_t s);
+void factor_solve(const FactorPlan &P, const T *L, T *b, T *y, T *x, int kcols, cudaStream_t s);
 
 // Switch the per-level sweep timing on (resetting it) or off.
 void level_clock_enable(FactorPlan &P, bool on);
 
-// local <-> global transfers: xl[i] = (T) r[gdof[i]]; z[gdof[i]] += xl[i]
+// local <-> global transfers: b[i] = (T) r[gdof[i]], y = x = 0; z[gdof[i]] += xl[i]
 template <class T>
-void gather_local(const FactorPlan &P, const double *r, T *xl, cudaStream_t s);
+void gather_local(const FactorPlan &P, const double *r, T *b, T *y, T *x, cudaStream_t s);
 template <class T>
 void scatter_add_local(const FactorPlan &P, const T *xl, double *z, cudaStream_t s);
 

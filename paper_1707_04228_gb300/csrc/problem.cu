@@ -264,8 +264,9 @@ void problem_coarse(const Problem &P, const gl_opts &o, const FactorPlan &PD, in
             // W = M^{-1} B V
             mark(0);
             GL_CUDA(cudaMemcpyAsync(tmp.p, BV.p, sizeof(double) * gl * k, cudaMemcpyDeviceToDevice, s));
-            factor_solve<double>(PG, LN.p, tmp.p, k, s);
-            std::swap(V.p, tmp.p);
+            BW.zero(s);
+            V.zero(s);
+            factor_solve<double>(PG, LN.p, tmp.p, BW.p, V.p, k, s);
             mark(1);
             BW.zero(s);
             local_K_apply(PG, E, P.C, P.geo, xg, V.p, BW.p, k, s);         // BW = B W

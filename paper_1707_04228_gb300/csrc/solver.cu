@@ -302,6 +302,15 @@ void apply_K(gl_ctx *c, const double *x, double *y) {
     g_launches += 1;
 }
 
+// z += sum_j R_j^T A_j^{-1} R_j r; xl holds three local vectors
+template <class T>
+void local_solve(const FactorPlan &P, const T *L, T *xl, const double *r, double *z, cudaStream_t s) {
+    T *b = xl, *y = xl + P.n_local, *x = xl + 2 * P.n_local;
+    gather_local<T>(P, r, b, y, x, s);
+    factor_solve<T>(P, L, b, y, x, 1, s);
+    scatter_add_local<T>(P, x, z, s);
+}
+
 // z = M^{-1} r (r zero at Dirichlet DOFs)
 void apply_prec(gl_ctx *c, const double *r, double *z) {
     cudaStream_t s = c->stream;
@@ -319,13 +328,9 @@ void apply_prec(gl_ctx *c, const double *r, double *z) {
     }
     prof_begin(c, PH_LOCAL);
     if (c->opts.precision == GL_PREC_MIXED) {
-        gather_local<float>(c->PD, r, c->xl32.p, s);
-        factor_solve<float>(c->PD, c->LD32.p, c->xl32.p, 1, s);
-        scatter_add_local<float>(c->PD, c->xl32.p, z, s);
+        local_solve<float>(c->PD, c->LD32.p, c->xl32.p, r, z, s);
     } else {
-        gather_local<double>(c->PD, r, c->xl64.p, s);
-        factor_solve<double>(c->PD, c->LD64.p, c->xl64.p, 1, s);
-        scatter_add_local<double>(c->PD, c->xl64.p, z, s);
+        local_solve<double>(c->PD, c->LD64.p, c->xl64.p, r, z, s);
     }
     prof_end(c, PH_LOCAL);
     g_launches += 2 + factor_solve_launches(c->PD);
@@ -475,10 +480,10 @@ void setup(gl_ctx *c, const gl_opts &o) {
     c->cvec.alloc(std::max(1, c->co.n0));
     c->cvec2.alloc(std::max(1, c->co.n0));
     if (c->opts.precision == GL_PREC_MIXED) {
-        c->xl32.alloc(c->PD.n_local);
+        c->xl32.alloc(3 * c->PD.n_local);
         c->xl64.release();
     } else {
-        c->xl64.alloc(c->PD.n_local);
+        c->xl64.alloc(3 * c->PD.n_local);
         c->xl32.release();
     }
     c->S.alloc(1);
@@ -759,13 +764,9 @@ void batch_precond(gl_batch *b, const double *r, double *z) {
         g_launches += 3;
     }
     if (b->opts.precision == GL_PREC_MIXED) {
-        gather_local<float>(b->PD, r, b->xl32.p, s);
-        factor_solve<float>(b->PD, b->LD32.p, b->xl32.p, 1, s);
-        scatter_add_local<float>(b->PD, b->xl32.p, z, s);
+        local_solve<float>(b->PD, b->LD32.p, b->xl32.p, r, z, s);
     } else {
-        gather_local<double>(b->PD, r, b->xl64.p, s);
-        factor_solve<double>(b->PD, b->LD64.p, b->xl64.p, 1, s);
-        scatter_add_local<double>(b->PD, b->xl64.p, z, s);
+        local_solve<double>(b->PD, b->LD64.p, b->xl64.p, r, z, s);
     }
     g_launches += 2 + factor_solve_launches(b->PD);
     if (side) GL_CUDA(cudaStreamWaitEvent(s, b->side.join, 0));
@@ -911,8 +912,8 @@ void batch_setup(gl_batch *b, const gl_opts &o) {
     for (DBuf<double> *v : {&b->x, &b->r, &b->z, &b->p, &b->q, &b->ud, &b->fe}) v->alloc(b->N);
     b->c1.alloc(std::max(1, b->co.n0));
     b->c2.alloc(std::max(1, b->co.n0));
-    if (b->opts.precision == GL_PREC_MIXED) b->xl32.alloc(b->PD.n_local);
-    else b->xl64.alloc(b->PD.n_local);
+    if (b->opts.precision == GL_PREC_MIXED) b->xl32.alloc(3 * b->PD.n_local);
+    else b->xl64.alloc(3 * b->PD.n_local);
     b->partials.alloc((size_t)n * SEG_BLOCKS);
     b->scal.alloc((size_t)6 * n);
     b->scal.zero(s);
