@@ -137,10 +137,12 @@ typedef struct {
  *   tol        stop when ||r_k||_2 / ||r_0||_2 <= tol, r_0 = f (x_0 = 0).
  *   sigma      shift of the definite GenEO pencil (eigenvectors do not
  *              depend on it); <= 0 selects 1e-3.
- *   eig_iters  cap on the subspace iterations of the GenEO eigensolver
- *              (<= 0: 100); after at least 4 iterations it stops once the
- *              kept Ritz values of every subdomain change by less than 1e-10
- *              (relative) between iterations.
+ *   eig_iters  cap on the block steps (eight vectors each) of the GenEO
+ *              eigensolver, a block Krylov method (<= 0: 100); it stops once
+ *              the kept Ritz pairs of every subdomain have residuals below
+ *              1e-6 of their value (in the pencil's energy norm), which
+ *              leaves the eigenvalues accurate to about 1e-12, and takes as
+ *              many steps as nev vectors need in any case.
  *   factor_ws_bytes  device workspace per buffer of the numeric
  *              factorisation (two buffers hold the dense fronts of two
  *              adjacent dissection levels); subdomains are factored in
@@ -149,7 +151,7 @@ typedef struct {
  *   eig_group_bytes  device memory for the shifted Neumann factors of one
  *              group of subdomains in the GenEO eigensolver; the subdomains
  *              are processed in consecutive groups that fit it.  <= 0 selects
- *              4e10.  The random start vectors of the subspace iteration are
+ *              4e10.  The random start vectors of the eigensolver are
  *              drawn per group, so another grouping changes the eigenvectors
  *              within the eigensolver's convergence, not the solution of a
  *              converged solve beyond its tolerance.

@@ -25,6 +25,7 @@
 #include "factor.h"
 #include "q2.cuh"
 #include "slaves.h"
+#include "warp.cuh"
 
 namespace gl {
 
@@ -820,30 +821,6 @@ __global__ void __launch_bounds__(SWEEP_CTA) k_fwd(const int *__restrict__ front
         T *bo = b + vo + rows[d.row_off + row];
 #pragma unroll
         for (int r = 0; r < NR; ++r) atomicAdd(bo + (int64_t)r * n, -(acc[r] + acc2[r]));
-    }
-}
-
-// Sums N (16 or a multiple of 32) values over the lanes of a warp, about one
-// add per value against five of a shuffle tree each: every step halves the
-// values a lane holds.  Value i comes back as v[i % PL] of lane i / PL, PL =
-// N / 32 (N = 16: v[0] of lanes 2 i and 2 i + 1).
-template <class T, int N>
-__device__ __forceinline__ void warp_sum_many(T (&v)[N], int lane) {
-    int n = N;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        if (n == 1) {
-            v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
-            continue;
-        }
-        n >>= 1;
-        const bool up = lane & o;
-#pragma unroll
-        for (int k = 0; k < N / 2; ++k)
-            if (k < n) {
-                const T send = up ? v[k] : v[k + n], keep = up ? v[k + n] : v[k];
-                v[k] = keep + __shfl_xor_sync(0xffffffffu, send, o);
-            }
     }
 }
 

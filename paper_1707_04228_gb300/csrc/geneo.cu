@@ -4,11 +4,12 @@
 // of a local generalised eigenproblem are computed and glued with a
 // partition of unity into the coarse space.  The eigenproblem solved here is
 // A_j^N p = lambda B_j p with B_j = Xi_j A_j^N Xi_j, through the definite
-// pencil B p = mu (A^N + sigma B) p (largest mu <-> smallest lambda), by block
-// subspace iteration with Rayleigh-Ritz; these are its batched pieces.
+// pencil B p = mu (A^N + sigma B) p (largest mu <-> smallest lambda), by a block
+// Krylov (Lanczos) method; these are its batched pieces.
 #include <algorithm>
 
 #include "geneo.h"
+#include "warp.cuh"
 
 namespace gl {
 
@@ -16,56 +17,176 @@ constexpr int NV_MAX = 32;
 
 // (local element products: local_K_apply in ku.cu, matrix-free)
 
-// ---------------------------------------------------------------- Gram matrices
+// ---------------------------------------------------------------- block Krylov pieces
 
-constexpr int GRAM_ROWS = 64;
+// G_s[a * ldg + j] += sum_i A_s[i, a] B_s[i, j], a < ma, j < KRY_B, over a chunk
+// of GRAM_ROWS rows.  Warp w takes the columns a = w, w + 8, ... of A (each read
+// once, coalesced), B's chunk sits in shared memory; bound by the FP64 pipe
+// once there are rows enough.
+constexpr int GRAM_ROWS = 512;
 
-__global__ void __launch_bounds__(256) k_gram(const int64_t *__restrict__ voff, const int64_t *__restrict__ vlen,
-                                              const double *__restrict__ A, const double *__restrict__ B, int k,
-                                              double *__restrict__ G) {
+__global__ void __launch_bounds__(256) k_kry_gram(const int64_t *__restrict__ voff, const int64_t *__restrict__ vlen,
+                                                  const double *__restrict__ A, int lda, int ma,
+                                                  const double *__restrict__ B, double *__restrict__ G, int64_t gs,
+                                                  int ldg) {
     const int s = blockIdx.x;
-    const int64_t n = vlen[s], base = voff[s] * k;
+    const int64_t n = vlen[s];
     const int64_t r0 = (int64_t)blockIdx.y * GRAM_ROWS;
     if (r0 >= n) return;
-    const int rows = (n - r0) < GRAM_ROWS ? (int)(n - r0) : GRAM_ROWS;
-    __shared__ double sa[NV_MAX][GRAM_ROWS], sb[NV_MAX][GRAM_ROWS];
-    for (int idx = threadIdx.x; idx < k * GRAM_ROWS; idx += blockDim.x) {
-        int i = idx % GRAM_ROWS, a = idx / GRAM_ROWS;
-        bool ok = i < rows;
-        sa[a][i] = ok ? A[base + a * n + r0 + i] : 0.0;
-        sb[a][i] = ok ? B[base + a * n + r0 + i] : 0.0;
+    const int rows = (int)min((int64_t)GRAM_ROWS, n - r0);
+    __shared__ double sb[KRY_B][GRAM_ROWS];
+    const double *Bs = B + voff[s] * KRY_B + r0, *As = A + voff[s] * lda + r0;
+    for (int idx = threadIdx.x; idx < KRY_B * GRAM_ROWS; idx += 256) {
+        const int i = idx % GRAM_ROWS, j = idx / GRAM_ROWS;
+        sb[j][i] = i < rows ? Bs[(int64_t)j * n + i] : 0.0;
     }
     __syncthreads();
-    for (int idx = threadIdx.x; idx < k * k; idx += blockDim.x) {
-        int a = idx / k, b = idx % k;
-        double acc = 0.0;
-        for (int i = 0; i < rows; ++i) acc += sa[a][i] * sb[b][i];
-        atomicAdd(G + (int64_t)s * k * k + idx, acc);
+    const int lane = threadIdx.x & 31;
+    for (int a = threadIdx.x >> 5; a < ma; a += 8) {
+        const double *Aa = As + (int64_t)a * n;
+        double acc[KRY_B];
+#pragma unroll
+        for (int j = 0; j < KRY_B; ++j) acc[j] = 0.0;
+#pragma unroll 4
+        for (int i = lane; i < GRAM_ROWS; i += 32) {
+            const double v = i < rows ? Aa[i] : 0.0;
+#pragma unroll
+            for (int j = 0; j < KRY_B; ++j) acc[j] += v * sb[j][i];
+        }
+        warp_sum_many<double, KRY_B>(acc, lane);
+        if (lane % (32 / KRY_B) == 0) atomicAdd(G + s * gs + (int64_t)a * ldg + lane / (32 / KRY_B), acc[0]);
     }
 }
 
-void local_gram(const FactorPlan &P, const double *A, const double *B, int k, double *G, cudaStream_t s) {
-    if (k > NV_MAX) fail(GL_ERR_INVALID_ARG, "local_gram: too many vectors");
-    int64_t maxn = 0;
+static unsigned row_chunks(const FactorPlan &P, int rows) {
+    int64_t maxn = 1;
     for (auto v : P.vec_len) maxn = std::max(maxn, v);
-    GL_CUDA(cudaMemsetAsync(G, 0, sizeof(double) * P.n_sub * k * k, s));
-    dim3 g(P.n_sub, (unsigned)((maxn + GRAM_ROWS - 1) / GRAM_ROWS));
-    k_gram<<<g, 256, 0, s>>>(P.d_vec_off.p, P.d_vec_len.p, A, B, k, G);
+    return (unsigned)((maxn + rows - 1) / rows);
+}
+
+void kry_gram(const FactorPlan &P, const double *A, int lda, int ma, const double *B, double *G, int64_t gs, int ldg,
+              cudaStream_t s) {
+    if (ma <= 0) return;
+    k_kry_gram<<<dim3(P.n_sub, row_chunks(P, GRAM_ROWS)), 256, 0, s>>>(P.d_vec_off.p, P.d_vec_len.p, A, lda, ma, B, G,
+                                                                       gs, ldg);
     GL_CUDA(cudaGetLastError());
 }
 
-// ---------------------------------------------------------------- small generalised eigenproblems
+// W_z -= V_z H for the pairs z: one row per thread, H in shared memory.
+__global__ void __launch_bounds__(256) k_kry_project(const int64_t *__restrict__ voff,
+                                                     const int64_t *__restrict__ vlen, KryBlocks K, int ldv, int m,
+                                                     const double *__restrict__ H, int64_t hs, int ldh) {
+    const int s = blockIdx.x;
+    const int64_t n = vlen[s], i = (int64_t)blockIdx.y * 256 + threadIdx.x;
+    if ((int64_t)blockIdx.y * 256 >= n) return;
+    __shared__ double sh[KRY_MAX * KRY_B];
+    for (int idx = threadIdx.x; idx < m * KRY_B; idx += 256)
+        sh[idx] = H[s * hs + (int64_t)(idx / KRY_B) * ldh + idx % KRY_B];
+    __syncthreads();
+    if (i >= n) return;
+    double *out = K.W[blockIdx.z] + voff[s] * KRY_B + i;
+    const double *Vi = K.V[blockIdx.z] + voff[s] * ldv + i;
+    double w[KRY_B];
+#pragma unroll
+    for (int j = 0; j < KRY_B; ++j) w[j] = out[(int64_t)j * n];
+#pragma unroll 4
+    for (int c = 0; c < m; ++c) {
+        const double v = Vi[(int64_t)c * n];
+#pragma unroll
+        for (int j = 0; j < KRY_B; ++j) w[j] -= v * sh[c * KRY_B + j];
+    }
+#pragma unroll
+    for (int j = 0; j < KRY_B; ++j) out[(int64_t)j * n] = w[j];
+}
 
-// One CTA per subdomain, everything in shared memory: Cholesky G_M = L L^T,
-// C = L^{-1} G_B L^{-T}, cyclic Jacobi on C, Y = L^{-T} Q, sort by eigenvalue
-// descending.  The matrices are tiny (k <= 32), so the kernel is a chain of
-// dependent steps and its time is their latency: each Jacobi round applies
-// k/2 disjoint rotations at once (round-robin pairs), every 2 x 2 block of C
-// that a pair of rotations touches by one thread, two barriers per round.
-// One thread per subdomain working in global memory took 10.5 ms a call (k = 20,
-// 10 subdomains); this form takes 10.2 ms less.
+void kry_project(const FactorPlan &P, const KryBlocks &K, int ldv, int m, const double *H, int64_t hs, int ldh,
+                 cudaStream_t s) {
+    if (m <= 0) return;
+    k_kry_project<<<dim3(P.n_sub, row_chunks(P, 256), K.count), 256, 0, s>>>(P.d_vec_off.p, P.d_vec_len.p, K, ldv, m,
+                                                                            H, hs, ldh);
+    GL_CUDA(cudaGetLastError());
+}
+
+// W_z <- W_z R in place; with col >= 0 the columns are also stored at column col of V_z.
+__global__ void __launch_bounds__(256) k_kry_scale(const int64_t *__restrict__ voff, const int64_t *__restrict__ vlen,
+                                                   KryBlocks K, const double *__restrict__ R, int ldv, int col) {
+    const int s = blockIdx.x;
+    const int64_t n = vlen[s], i = (int64_t)blockIdx.y * 256 + threadIdx.x;
+    if ((int64_t)blockIdx.y * 256 >= n) return;
+    __shared__ double sr[KRY_B * KRY_B];
+    if (threadIdx.x < KRY_B * KRY_B) sr[threadIdx.x] = R[(int64_t)s * KRY_B * KRY_B + threadIdx.x];
+    __syncthreads();
+    if (i >= n) return;
+    double *io = K.W[blockIdx.z] + voff[s] * KRY_B + i;
+    double w[KRY_B], o[KRY_B];
+#pragma unroll
+    for (int j = 0; j < KRY_B; ++j) {
+        w[j] = io[(int64_t)j * n];
+        o[j] = 0.0;
+    }
+#pragma unroll
+    for (int c = 0; c < KRY_B; ++c)
+#pragma unroll
+        for (int j = 0; j < KRY_B; ++j) o[j] += w[c] * sr[c * KRY_B + j];
+#pragma unroll
+    for (int j = 0; j < KRY_B; ++j) io[(int64_t)j * n] = o[j];
+    if (col >= 0) {
+        double *dst = K.V[blockIdx.z] + voff[s] * ldv + (int64_t)col * n + i;
+#pragma unroll
+        for (int j = 0; j < KRY_B; ++j) dst[(int64_t)j * n] = o[j];
+    }
+}
+
+void kry_scale(const FactorPlan &P, const KryBlocks &K, const double *R, int ldv, int col, cudaStream_t s) {
+    k_kry_scale<<<dim3(P.n_sub, row_chunks(P, 256), K.count), 256, 0, s>>>(P.d_vec_off.p, P.d_vec_len.p, K, R, ldv,
+                                                                          col);
+    GL_CUDA(cudaGetLastError());
+}
+
+// out[:, 0..k) = V[:, 0..m) Y (row-major m x k, leading dimension ldy), k <= KRY_MAX, eight columns at a time.
+__global__ void __launch_bounds__(256) k_kry_combine(const int64_t *__restrict__ voff,
+                                                     const int64_t *__restrict__ vlen, const double *__restrict__ V,
+                                                     int ldv, int m, const double *__restrict__ Y, int64_t ys, int ldy,
+                                                     int k, double *__restrict__ out, int ldo) {
+    const int s = blockIdx.x, c0 = blockIdx.z * 8;
+    const int64_t n = vlen[s], i = (int64_t)blockIdx.y * 256 + threadIdx.x;
+    if ((int64_t)blockIdx.y * 256 >= n) return;
+    __shared__ double sy[KRY_MAX * 8];
+    for (int idx = threadIdx.x; idx < m * 8; idx += 256)
+        sy[idx] = c0 + idx % 8 < k ? Y[s * ys + (int64_t)(idx / 8) * ldy + c0 + idx % 8] : 0.0;
+    __syncthreads();
+    if (i >= n) return;
+    const double *Vi = V + voff[s] * ldv + i;
+    double w[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) w[j] = 0.0;
+#pragma unroll 4
+    for (int c = 0; c < m; ++c) {
+        const double v = Vi[(int64_t)c * n];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) w[j] += v * sy[c * 8 + j];
+    }
+    double *o = out + voff[s] * ldo + i;
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+        if (c0 + j < k) o[(int64_t)(c0 + j) * n] = w[j];
+}
+
+void kry_combine(const FactorPlan &P, const double *V, int ldv, int m, const double *Y, int64_t ys, int ldy, int k,
+                 double *out, int ldo, cudaStream_t s) {
+    k_kry_combine<<<dim3(P.n_sub, row_chunks(P, 256), (k + 7) / 8), 256, 0, s>>>(P.d_vec_off.p, P.d_vec_len.p, V, ldv,
+                                                                                m, Y, ys, ldy, k, out, ldo);
+    GL_CUDA(cudaGetLastError());
+}
+
+// ---------------------------------------------------------------- small eigenproblems
+
+// The projected problems are tiny (at most KRY_MAX rows), so their kernels are
+// a chain of dependent steps: one CTA per subdomain with everything in shared
+// memory, each Jacobi round applying half as many disjoint rotations as there
+// are rows at once (round-robin pairs), every 2 x 2 block of C that a pair of
+// rotations touches by one thread, two barriers per round.
 constexpr int GENEIG_THREADS = 256;
-constexpr int GENEIG_LD = NV_MAX + 1;
 
 // Pair i of round t in the round-robin tournament of m (even) players.
 __device__ __forceinline__ void jacobi_pair(int m, int t, int i, int &p, int &q) {
@@ -161,107 +282,124 @@ __device__ void cta_jacobi(double *C, double *Q, int ld, int k, double *cs, doub
     __syncthreads();
 }
 
-__global__ void __launch_bounds__(GENEIG_THREADS) k_small_geneig(int k, const double *__restrict__ GB,
-                                                                 const double *__restrict__ GM, double *__restrict__ Y,
-                                                                 double *__restrict__ mu, int *__restrict__ err) {
-    __shared__ double Lm[NV_MAX * GENEIG_LD], C[NV_MAX * GENEIG_LD], Q[NV_MAX * GENEIG_LD];
-    __shared__ double cs[2 * NV_MAX], red[2 * (GENEIG_THREADS / 32)];
-    __shared__ int rank[NV_MAX];
-    const int s = blockIdx.x, kk = k * k, ld = GENEIG_LD, tid = threadIdx.x, nt = blockDim.x;
-    for (int idx = tid; idx < kk; idx += nt) {
-        const int i = idx / k, j = idx % k;
-        const double *gm = GM + (int64_t)s * kk, *gb = GB + (int64_t)s * kk;
-        Lm[i * ld + j] = 0.5 * (gm[idx] + gm[j * k + i]);
-        C[i * ld + j] = 0.5 * (gb[idx] + gb[j * k + i]);
+// R_s with W R_s orthonormal in the M inner product, from G_s = W^T M W: Q
+// Lambda^{-1/2} of G's eigenpairs; directions at or below the noise (drop times
+// the block's squared norm before its projection, H the coefficients it lost)
+// become zero columns and stay zero.
+__global__ void __launch_bounds__(64) k_kry_orth(const double *__restrict__ G, const double *__restrict__ H, int64_t hs,
+                                                 int ldh, int m, double drop, double *__restrict__ R,
+                                                 int *__restrict__ err) {
+    constexpr int ld = KRY_B + 1;
+    __shared__ double C[KRY_B * ld], Q[KRY_B * ld], cs[KRY_B], red[4], sh;
+    const int s = blockIdx.x, tid = threadIdx.x;
+    if (tid == 0) sh = 0.0;
+    for (int idx = tid; idx < KRY_B * KRY_B; idx += 64) {
+        const int i = idx / KRY_B, j = idx % KRY_B;
+        const double *g = G + (int64_t)s * KRY_B * KRY_B;
+        C[i * ld + j] = 0.5 * (g[idx] + g[j * KRY_B + i]);
     }
     __syncthreads();
-    // Cholesky (lower), right-looking
-    for (int j = 0; j < k; ++j) {
-        if (tid == 0) {
-            double d = Lm[j * ld + j];
-            if (!(d > 0.0)) {
-                atomicExch(err, 1);
-                d = 1e-300;
-            }
-            Lm[j * ld + j] = sqrt(d);
-        }
-        __syncthreads();
-        const double djj = Lm[j * ld + j];
-        for (int i = j + 1 + tid; i < k; i += nt) Lm[i * ld + j] /= djj;
-        __syncthreads();
-        const int r = k - j - 1;
-        for (int idx = tid; idx < r * r; idx += nt) {
-            const int i = j + 1 + idx / r, c = j + 1 + idx % r;
-            if (i >= c) Lm[i * ld + c] -= Lm[i * ld + j] * Lm[c * ld + j];
-        }
-        __syncthreads();
+    double lost = 0.0;
+    for (int idx = tid; idx < m * KRY_B; idx += 64) {
+        const double h = H[s * hs + (int64_t)(idx / KRY_B) * ldh + idx % KRY_B];
+        lost += h * h;
     }
-    // C <- L^{-1} C L^{-T}: one thread per column, then one per row
-    for (int pass = 0; pass < 2; ++pass) {
-        if (tid < k) {
-            const int st = pass == 0 ? ld : 1, at = pass == 0 ? tid : tid * ld;   // element i of this line: C[at + i st]
-            for (int i = 0; i < k; ++i) {
-                double v = C[at + i * st];
-                for (int t = 0; t < i; ++t) v -= Lm[i * ld + t] * C[at + t * st];
-                C[at + i * st] = v / Lm[i * ld + i];
-            }
-        }
-        __syncthreads();
+    if (tid < KRY_B) lost += C[tid * ld + tid];
+    atomicAdd(&sh, lost);
+    __syncthreads();
+    const double floor_ = drop * sh;
+    cta_jacobi(C, Q, ld, KRY_B, cs, red);
+    for (int idx = tid; idx < KRY_B * KRY_B; idx += 64) {
+        const int j = idx % KRY_B;
+        const double lam = C[j * ld + j];
+        if (!(fabs(lam) < INFINITY)) atomicExch(err, 1);
+        R[(int64_t)s * KRY_B * KRY_B + idx] = lam > floor_ && lam > 0.0 ? Q[(idx / KRY_B) * ld + j] / sqrt(lam) : 0.0;
     }
-    cta_jacobi(C, Q, ld, k, cs, red);
-    // rank of every eigenvalue, descending (ties by index); Y = L^{-T} Q, one thread per column
-    if (tid < k) {
-        const double me = C[tid * ld + tid];
+}
+
+void kry_orth(int n_sub, const double *G, const double *H, int64_t hs, int ldh, int m, double drop, double *R,
+              int *d_err, cudaStream_t s) {
+    k_kry_orth<<<n_sub, 64, 0, s>>>(G, H, hs, ldh, m, drop, R, d_err);
+    GL_CUDA(cudaGetLastError());
+}
+
+// Ritz pairs of the m x m projected matrix T_s (its upper triangle is read),
+// largest first: keep values mu and vectors Y (row-major m x keep), and the
+// largest relative residual of the first nev, sqrt(y^T G y) / mu with y the
+// vector's part on the last block and G the squared norms of what that block's
+// image has left outside the basis.
+__global__ void __launch_bounds__(GENEIG_THREADS) k_kry_ritz(const double *__restrict__ T, int ldt, int m,
+                                                             const double *__restrict__ G, int nev, int keep,
+                                                             double *__restrict__ Y, int ldy, double *__restrict__ mu,
+                                                             unsigned long long *__restrict__ worst) {
+    extern __shared__ double sm[];
+    const int ld = m + 1, s = blockIdx.x, tid = threadIdx.x, nt = blockDim.x;
+    double *C = sm, *Q = C + m * ld, *cs = Q + m * ld, *red = cs + m + 2;
+    __shared__ int rank[KRY_MAX];
+    const double *Ts = T + (int64_t)s * ldt * ldt;
+    for (int idx = tid; idx < m * m; idx += nt) {
+        const int i = idx / m, j = idx % m;
+        C[i * ld + j] = Ts[(int64_t)min(i, j) * ldt + max(i, j)];
+    }
+    __syncthreads();
+    cta_jacobi(C, Q, ld, m, cs, red);
+    for (int a = tid; a < m; a += nt) {
+        const double me = C[a * ld + a];
         int r = 0;
-        for (int i = 0; i < k; ++i) {
+        for (int i = 0; i < m; ++i) {
             const double v = C[i * ld + i];
-            r += v > me || (v == me && i < tid);
+            r += v > me || (v == me && i < a);
         }
-        rank[tid] = r;
-        mu[(int64_t)s * k + r] = me;
-        for (int i = k - 1; i >= 0; --i) {
-            double v = Q[i * ld + tid];
-            for (int t = i + 1; t < k; ++t) v -= Lm[t * ld + i] * Q[t * ld + tid];
-            Q[i * ld + tid] = v / Lm[i * ld + i];
-        }
+        rank[a] = r;
     }
     __syncthreads();
-    for (int idx = tid; idx < kk; idx += nt) Y[(int64_t)s * kk + (idx / k) * k + rank[idx % k]] = Q[(idx / k) * ld + idx % k];
+    for (int a = tid; a < m; a += nt)
+        if (rank[a] == 0) cs[m] = C[a * ld + a];
+    __syncthreads();
+    for (int idx = tid; idx < m * m; idx += nt) {
+        const int r = rank[idx % m];
+        if (r < keep) Y[((int64_t)s * KRY_MAX + idx / m) * ldy + r] = Q[(idx / m) * ld + idx % m];
+    }
+    for (int a = tid; a < m; a += nt) {
+        const int r = rank[a];
+        const double me = C[a * ld + a];
+        if (r < keep) mu[(int64_t)s * ldy + r] = me;
+        if (r >= nev) continue;
+        const double *g = G + (int64_t)s * KRY_B * KRY_B;
+        double res = 0.0;
+        for (int i = 0; i < KRY_B; ++i)
+            for (int j = 0; j < KRY_B; ++j) res += Q[(m - KRY_B + i) * ld + a] * g[i * KRY_B + j] * Q[(m - KRY_B + j) * ld + a];
+        const double rel = sqrt(fmax(res, 0.0)) / fmax(me, 1e-12 * cs[m]);
+        atomicMax(worst, (unsigned long long)__double_as_longlong(rel));   // rel >= 0: ordered like its bits
+    }
 }
 
-void small_geneig(int n_sub, int k, const double *GB, const double *GM, double *Y, double *mu, int *d_err,
-                  cudaStream_t s) {
-    if (k > NV_MAX) fail(GL_ERR_INVALID_ARG, "small_geneig: k too large");
-    k_small_geneig<<<n_sub, GENEIG_THREADS, 0, s>>>(k, GB, GM, Y, mu, d_err);
+static size_t ritz_smem(int m) { return sizeof(double) * ((size_t)2 * m * (m + 1) + m + 2 + 2 * (GENEIG_THREADS / 32)); }
+
+void kry_ritz(int n_sub, const double *T, int ldt, int m, const double *G, int nev, int keep, double *Y, int ldy,
+              double *mu, unsigned long long *worst, cudaStream_t s) {
+    static SmemLimit limit;
+    raise_smem_limit(limit, ritz_smem(KRY_MAX), [](size_t v) {
+        GL_CUDA(cudaFuncSetAttribute(k_kry_ritz, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)v));
+    });
+    GL_CUDA(cudaMemsetAsync(worst, 0, sizeof(*worst), s));
+    k_kry_ritz<<<n_sub, GENEIG_THREADS, ritz_smem(m), s>>>(T, ldt, m, G, nev, keep, Y, ldy, mu, worst);
     GL_CUDA(cudaGetLastError());
 }
 
-// ---------------------------------------------------------------- rotations, scaling, random
-
-__global__ void k_rotate(const int64_t *__restrict__ voff, const int64_t *__restrict__ vlen, const double *__restrict__ X,
-                         const double *__restrict__ Y, int k, double *__restrict__ out) {
+// T_s = diag(mu_s) (k values), the rest of T_s zero.
+__global__ void k_kry_diag(double *__restrict__ T, int ldt, const double *__restrict__ mu, int ldm, int k) {
     const int s = blockIdx.x;
-    const int64_t n = vlen[s], base = voff[s] * k;
-    __shared__ double sy[NV_MAX * NV_MAX];
-    for (int i = threadIdx.x; i < k * k; i += blockDim.x) sy[i] = Y[(int64_t)s * k * k + i];
-    __syncthreads();
-    for (int64_t i = (int64_t)blockIdx.y * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.y * blockDim.x) {
-        double row[NV_MAX];
-        for (int b = 0; b < k; ++b) row[b] = X[base + b * n + i];
-        for (int a = 0; a < k; ++a) {
-            double v = 0.0;
-            for (int b = 0; b < k; ++b) v += row[b] * sy[b * k + a];
-            out[base + a * n + i] = v;
-        }
-    }
+    for (int idx = threadIdx.x; idx < ldt * ldt; idx += blockDim.x)
+        T[(int64_t)s * ldt * ldt + idx] = idx / ldt == idx % ldt && idx / ldt < k ? mu[(int64_t)s * ldm + idx / ldt] : 0.0;
 }
 
-void local_rotate(const FactorPlan &P, double *X, const double *Y, int k, double *tmp, cudaStream_t s) {
-    dim3 g(P.n_sub, 64);
-    k_rotate<<<g, 256, 0, s>>>(P.d_vec_off.p, P.d_vec_len.p, X, Y, k, tmp);
+void kry_diag(int n_sub, double *T, int ldt, const double *mu, int ldm, int k, cudaStream_t s) {
+    k_kry_diag<<<n_sub, 256, 0, s>>>(T, ldt, mu, ldm, k);
     GL_CUDA(cudaGetLastError());
-    GL_CUDA(cudaMemcpyAsync(X, tmp, sizeof(double) * P.n_local * k, cudaMemcpyDeviceToDevice, s));
 }
+
+// ---------------------------------------------------------------- scaling, random
 
 __global__ void k_scale_rows(const int64_t *__restrict__ voff, const int64_t *__restrict__ vlen, double *__restrict__ X,
                              const double *__restrict__ xi, int k) {

@@ -21,18 +21,36 @@ struct LocalElems {
 void local_K_apply(const FactorPlan &P, const LocalElems &E, const double *C, const double *geo, const double *xi,
                    const double *x, double *y, int nv, cudaStream_t s);
 
-// G_s = A_s^T B_s (k x k per subdomain, row-major k*k block per subdomain), A,
-// B multi-vectors of k columns in the FactorPlan layout.
-void local_gram(const FactorPlan &P, const double *A, const double *B, int k, double *G, cudaStream_t s);
-
-// Per subdomain: solve G_B y = mu G_M y (k x k, G_M SPD), eigenvectors
-// G_M-orthonormal, sorted by mu descending; writes Y (k x k, column a = vector
-// a, row-major [b*k + a]) and mu.
-void small_geneig(int n_sub, int k, const double *GB, const double *GM, double *Y, double *mu, int *d_err,
-                  cudaStream_t s);
-
-// X <- X Y per subdomain (k columns), using tmp of the same size.
-void local_rotate(const FactorPlan &P, double *X, const double *Y, int k, double *tmp, cudaStream_t s);
+// Block Krylov eigensolver of the pencils B p = mu M p (problem.cu), its basis
+// V (with M V and B V) with KRY_MAX columns at most, grown by blocks of KRY_B
+// (the sweeps' widest multi-vector, and more than the six rigid modes, the
+// largest multiple eigenvalue).  V: FactorPlan layout with ldv columns; blocks
+// W: KRY_B columns.
+constexpr int KRY_B = 8, KRY_MAX = 96;
+// Up to three bases and the blocks that go with them.
+struct KryBlocks {
+    int count = 0;
+    double *V[3] = {}, *W[3] = {};
+};
+// G_s[a ldg + j] += A_s[:, a]^T B_s[:, j] for a < ma, j < KRY_B (subdomain stride gs)
+void kry_gram(const FactorPlan &P, const double *A, int lda, int ma, const double *B, double *G, int64_t gs, int ldg,
+              cudaStream_t s);
+// W -= V H for every pair (H_s row-major m x KRY_B, leading dimension ldh)
+void kry_project(const FactorPlan &P, const KryBlocks &K, int ldv, int m, const double *H, int64_t hs, int ldh,
+                 cudaStream_t s);
+// R_s orthonormalising a block with Gram matrix G_s; H, m: what its projection took away
+void kry_orth(int n_sub, const double *G, const double *H, int64_t hs, int ldh, int m, double drop, double *R,
+              int *d_err, cudaStream_t s);
+// W <- W R for every pair; also stored at column col of V unless col < 0
+void kry_scale(const FactorPlan &P, const KryBlocks &K, const double *R, int ldv, int col, cudaStream_t s);
+// Ritz pairs of T_s (leading dimension ldt, m rows), largest first; *worst = the largest relative residual
+// of the first nev (bits of a non-negative double).  Y: KRY_MAX x ldy per subdomain, mu: ldy per subdomain.
+void kry_ritz(int n_sub, const double *T, int ldt, int m, const double *G, int nev, int keep, double *Y, int ldy,
+              double *mu, unsigned long long *worst, cudaStream_t s);
+void kry_diag(int n_sub, double *T, int ldt, const double *mu, int ldm, int k, cudaStream_t s);
+// out_s[:, 0..k) = V_s[:, 0..m) Y_s
+void kry_combine(const FactorPlan &P, const double *V, int ldv, int m, const double *Y, int64_t ys, int ldy, int k,
+                 double *out, int ldo, cudaStream_t s);
 
 // Deterministic pseudo-random fill of a multi-vector (splitmix64 hash of the index).
 void fill_random(double *x, int64_t n, uint64_t seed, cudaStream_t s);

@@ -205,15 +205,16 @@ void problem_coarse(const Problem &P, const gl_opts &o, const FactorPlan &PD, in
     }
     DBuf<double> d_xi;
     d_xi.upload(xi, s);
-    const int k = std::min(32, std::max(nev + 4, ((2 * nev + 3) / 4) * 4));
+    // basis columns: room for about four times nev before a restart, and Ritz vectors kept by one
+    const int mmax = nev <= 12 ? 64 : KRY_MAX, keep = nev + KRY_B;
     const int64_t nl = PN.n_local;
     out.nev = nev;
     out.n0 = nsub * nev;
     out.Z.alloc(nl * nev);
     out.eig.assign((size_t)nsub * nev, 0.0);
     const int iters = o.eig_iters > 0 ? o.eig_iters : 100;
-    // Groups of subdomains: factor of A^N + sigma Xi A^N Xi and block subspace
-    // iteration for the largest mu of B p = mu M p, one group at a time.
+    // Groups of subdomains: factor of M = A^N + sigma B, B = Xi A^N Xi, and the
+    // block Krylov iteration, one group at a time.
     const int64_t budget = (int64_t)((o.eig_group_bytes > 0 ? o.eig_group_bytes : 4e10) / sizeof(double));
     int j0 = 0, max_its = 0;
     while (j0 < nsub) {
@@ -237,100 +238,104 @@ void problem_coarse(const Problem &P, const gl_opts &o, const FactorPlan &PD, in
         P.stamp("Neumann factorisation (group)");
         LocalElems E;
         problem_local_elems(P, j0, j1, PG, E);
-        DBuf<double> V, BV, BW, tmp, GB, GM, Y, mu;
-        V.alloc(gl * k);
-        BV.alloc(gl * k);
-        BW.alloc(gl * k);
-        tmp.alloc(gl * k);
-        GB.alloc((size_t)ng * k * k);
-        GM.alloc((size_t)ng * k * k);
-        Y.alloc((size_t)ng * k * k);
-        mu.alloc((size_t)ng * k);
-        fill_random(V.p, gl * k, 0x1707042280000001ull + (uint64_t)j0, s);
-        BV.zero(s);
-        local_K_apply(PG, E, P.C, P.geo, xg, V.p, BV.p, k, s);            // BV = Xi A^N Xi V
-        std::vector<double> mu_prev((size_t)ng * k, 0.0), mu_now((size_t)ng * k);
-        // optional per-step timing of the iteration (GL_VERBOSE)
-        const bool timed = std::getenv("GL_VERBOSE") != nullptr;
-        cudaEvent_t ev[6] = {};
-        double step_ms[5] = {0, 0, 0, 0, 0};
-        if (timed)
-            for (auto &e : ev) GL_CUDA(cudaEventCreate(&e));
-        auto mark = [&](int i) {
-            if (timed) GL_CUDA(cudaEventRecord(ev[i], s));
+        // Block Krylov (Lanczos) method for the largest mu of B p = mu M p, M = A^N + sigma B factored: the basis
+        // V grows by the block M^{-1} B V_last, made M-orthonormal against all of V, and T = V^T B V gives the Ritz
+        // pairs.  It stops when the residuals |M^{-1} B p - mu p|_M of the kept pairs are below EIG_RESID mu in
+        // every subdomain.  About ten steps of eight solves did for nev = 10 on the corner, where a subspace
+        // iteration with 20 vectors took 20 steps.
+        constexpr double EIG_RESID = 1e-6;
+        DBuf<double> V, MV, BV, W, MW, BW, ysc, T, H, G, R, Y, mu;
+        DBuf<unsigned long long> worst;
+        for (DBuf<double> *v : {&V, &MV, &BV}) v->alloc(gl * mmax);
+        for (DBuf<double> *v : {&W, &MW, &BW, &ysc}) v->alloc(gl * KRY_B);
+        T.alloc((size_t)ng * mmax * mmax);
+        T.zero(s);
+        H.alloc((size_t)ng * mmax * KRY_B);
+        for (DBuf<double> *v : {&G, &R}) v->alloc((size_t)ng * KRY_B * KRY_B);
+        Y.alloc((size_t)ng * KRY_MAX * keep);
+        mu.alloc((size_t)ng * keep);
+        worst.alloc(1);
+        const int64_t ts = (int64_t)mmax * mmax, hs = (int64_t)mmax * KRY_B, ys = (int64_t)KRY_MAX * keep;
+        const KryBlocks first{2, {V.p, MV.p}, {W.p, BW.p}}, all{3, {V.p, MV.p, BV.p}, {W.p, MW.p, BW.p}};
+        const KryBlocks only_w{1, {V.p}, {W.p}};
+        auto gram_block = [&](const double *MWp) {
+            G.zero(s);
+            kry_gram(PG, W.p, KRY_B, KRY_B, MWp, G.p, KRY_B * KRY_B, KRY_B, s);
         };
-        int it = 0;
-        for (; it < iters; ++it) {
-            // W = M^{-1} B V
-            mark(0);
-            GL_CUDA(cudaMemcpyAsync(tmp.p, BV.p, sizeof(double) * gl * k, cudaMemcpyDeviceToDevice, s));
+        auto apply_B = [&]() {
             BW.zero(s);
-            V.zero(s);
-            factor_solve<double>(PG, LN.p, tmp.p, BW.p, V.p, k, s);
-            mark(1);
-            BW.zero(s);
-            local_K_apply(PG, E, P.C, P.geo, xg, V.p, BW.p, k, s);         // BW = B W
-            mark(2);
-            local_gram(PG, V.p, BV.p, k, GM.p, s);                          // W^T M W = W^T (B V)
-            local_gram(PG, V.p, BW.p, k, GB.p, s);                          // W^T B W
-            mark(3);
-            small_geneig(ng, k, GB.p, GM.p, Y.p, mu.p, P.d_err, s);
-            check_err(P, "GenEO Rayleigh-Ritz");
-            mark(4);
-            local_rotate(PG, V.p, Y.p, k, tmp.p, s);
-            local_rotate(PG, BW.p, Y.p, k, tmp.p, s);
-            mark(5);
-            std::swap(BV.p, BW.p);
-            GL_CUDA(cudaMemcpyAsync(mu_now.data(), mu.p, mu_now.size() * sizeof(double), cudaMemcpyDeviceToHost, s));
-            GL_CUDA(cudaStreamSynchronize(s));
-            double change = 0.0;
-            for (int j = 0; j < ng; ++j)
-                for (int a = 0; a < nev; ++a) {
-                    double now = mu_now[(size_t)j * k + a], prev = mu_prev[(size_t)j * k + a];
-                    change = std::max(change, std::fabs(now - prev) / std::fabs(now));
-                }
-            mu_prev = mu_now;
-            if (timed)
-                for (int q = 0; q < 5; ++q) {
-                    float ms = 0.f;
-                    GL_CUDA(cudaEventElapsedTime(&ms, ev[q], ev[q + 1]));
-                    step_ms[q] += ms;
-                }
-            // Ritz values settle like rate^(2 it); a change of 1e-10 leaves the Ritz vectors
-            // accurate to about 1e-5, far below what changes the coarse space's effect on PCG.
-            if (it >= 4 && change < 1e-10) {
-                ++it;
-                break;
+            local_K_apply(PG, E, P.C, P.geo, xg, W.p, BW.p, KRY_B, s);
+        };
+        fill_random(W.p, gl * KRY_B, 0x1707042280000001ull + (uint64_t)j0, s);
+        apply_B();
+        int it = 0, m = 0, kept = 0;
+        double resid = 0.0;
+        for (;;) {
+            // the last block's columns of T; W = M^{-1} B W_last (MW holds the sweeps' right-hand side)
+            if (m > 0) kry_gram(PG, V.p, mmax, m, BW.p, T.p + (m - KRY_B), ts, mmax, s);
+            GL_CUDA(cudaMemcpyAsync(MW.p, BW.p, sizeof(double) * gl * KRY_B, cudaMemcpyDeviceToDevice, s));
+            W.zero(s);
+            ysc.zero(s);
+            factor_solve<double>(PG, LN.p, MW.p, ysc.p, W.p, KRY_B, s);
+            ++it;
+            // first pass: M W = B W_last up to the solve's error, so G is good for the residuals and a first scaling
+            H.zero(s);
+            kry_gram(PG, MV.p, mmax, m, W.p, H.p, hs, KRY_B, s);
+            kry_project(PG, first, mmax, m, H.p, hs, KRY_B, s);
+            gram_block(BW.p);
+            if (m >= nev + KRY_B / 2 || (m >= nev && it > iters)) {
+                kept = std::min(keep, m);
+                kry_ritz(ng, T.p, mmax, m, G.p, nev, kept, Y.p, keep, mu.p, worst.p, s);
+                unsigned long long bits = 0;
+                GL_CUDA(cudaMemcpyAsync(&bits, worst.p, sizeof(bits), cudaMemcpyDeviceToHost, s));
+                check_err(P, "GenEO Rayleigh-Ritz");
+                std::memcpy(&resid, &bits, sizeof(resid));
+                if (resid <= EIG_RESID || it > iters) break;
             }
-        }
-        if (std::getenv("GL_VERBOSE")) {
-            double worst = 0.0, lo = 1e300, hi = 0.0;
-            for (int j = 0; j < ng; ++j) {
-                double lm = 1.0 / mu_now[(size_t)j * k + nev - 1] - sigma, lk = 1.0 / mu_now[(size_t)j * k + k - 1] - sigma;
-                worst = std::max(worst, (lm + sigma) / (lk + sigma));
-                lo = std::min(lo, lm);
-                hi = std::max(hi, lm);
+            kry_orth(ng, G.p, H.p, hs, KRY_B, m, 1e-24, R.p, P.d_err, s);
+            kry_scale(PG, only_w, R.p, mmax, -1, s);
+            if (m + KRY_B > mmax) {
+                // restart from the leading Ritz vectors: V <- V Y, T = diag(mu)
+                DBuf<double> tmp;
+                tmp.alloc(gl * kept);
+                for (DBuf<double> *B : {&V, &MV, &BV}) {
+                    kry_combine(PG, B->p, mmax, m, Y.p, ys, keep, kept, tmp.p, kept, s);
+                    for (int j = 0; j < ng; ++j)
+                        GL_CUDA(cudaMemcpyAsync(B->p + PG.vec_off[j] * mmax, tmp.p + PG.vec_off[j] * kept,
+                                                PG.vec_len[j] * kept * sizeof(double), cudaMemcpyDeviceToDevice, s));
+                }
+                kry_diag(ng, T.p, mmax, mu.p, keep, kept, s);
+                m = kept;
+                GL_CUDA(cudaStreamSynchronize(s));
             }
-            std::fprintf(stderr, "[gl]   group %d-%d: %d iterations, lambda_nev in [%.3g, %.3g], worst rate %.3f\n", j0,
-                         j1 - 1, it, lo, hi, worst);
-            const double nit = std::max(it, 1);
-            std::fprintf(stderr,
-                         "[gl]     per iteration: solve %.1f ms, local K %.1f ms, Gram %.1f ms, Rayleigh-Ritz %.1f ms, "
-                         "rotate %.1f ms (k = %d)\n",
-                         step_ms[0] / nit, step_ms[1] / nit, step_ms[2] / nit, step_ms[3] / nit, step_ms[4] / nit, k);
+            // second pass with the block's own images B W and M W = A^N W + sigma B W: orthonormal to rounding.
+            // (Carrying M W along from the first pass lets the solves' errors grow by the ratio of the largest mu,
+            // 1 / sigma, to the kept ones.)
+            apply_B();
+            MW.zero(s);
+            axpy(MW.p, sigma, BW.p, gl * KRY_B, s);
+            local_K_apply(PG, E, P.C, P.geo, nullptr, W.p, MW.p, KRY_B, s);
+            H.zero(s);
+            kry_gram(PG, V.p, mmax, m, MW.p, H.p, hs, KRY_B, s);
+            kry_project(PG, all, mmax, m, H.p, hs, KRY_B, s);
+            gram_block(MW.p);
+            kry_orth(ng, G.p, H.p, hs, KRY_B, 0, 1e-6, R.p, P.d_err, s);
+            kry_scale(PG, all, R.p, mmax, m, s);
+            m += KRY_B;
         }
-        if (timed)
-            for (auto &e : ev) cudaEventDestroy(e);
+        if (std::getenv("GL_VERBOSE"))
+            std::fprintf(stderr, "[gl]   group %d-%d: %d block steps, basis %d, largest residual %.2e\n", j0, j1 - 1, it, m,
+                         resid);
+        std::vector<double> mu_now((size_t)ng * keep);
+        GL_CUDA(cudaMemcpyAsync(mu_now.data(), mu.p, mu_now.size() * sizeof(double), cudaMemcpyDeviceToHost, s));
+        GL_CUDA(cudaStreamSynchronize(s));
         max_its = std::max(max_its, it);
         for (int j = 0; j < ng; ++j)
-            for (int a = 0; a < nev; ++a) out.eig[(size_t)(j0 + j) * nev + a] = 1.0 / mu_now[(size_t)j * k + a] - sigma;
+            for (int a = 0; a < nev; ++a) out.eig[(size_t)(j0 + j) * nev + a] = 1.0 / mu_now[(size_t)j * keep + a] - sigma;
         // Z columns of these subdomains (whole-problem Neumann layout, nev columns)
-        for (int j = 0; j < ng; ++j) {
-            const int64_t n = PG.vec_len[j];
-            GL_CUDA(cudaMemcpy2DAsync(out.Z.p + PN.vec_off[j0 + j] * nev, n * sizeof(double), V.p + PG.vec_off[j] * k,
-                                      n * sizeof(double), n * sizeof(double), nev, cudaMemcpyDeviceToDevice, s));
-        }
-        P.stamp("GenEO subspace iteration (group)");
+        kry_combine(PG, V.p, mmax, m, Y.p, ys, keep, nev, out.Z.p + goff * nev, nev, s);
+        GL_CUDA(cudaStreamSynchronize(s));
+        P.stamp("GenEO block Krylov (group)");
         j0 = j1;
     }
     out.eig_iters = max_its;

@@ -467,7 +467,7 @@ void setup(gl_ctx *c, const gl_opts &o) {
     c->co = Coarse();
     if (c->opts.nev > 0) problem_coarse(P, c->opts, c->PD, LEAF_NODES, c->co);
     if (std::getenv("GL_VERBOSE"))
-        std::fprintf(stderr, "[gl] GenEO subspace iterations (max over groups): %d\n", c->co.eig_iters);
+        std::fprintf(stderr, "[gl] GenEO block steps (max over groups): %d\n", c->co.eig_iters);
     stamp(c, "GenEO coarse space + K0");
     if (c->co.n_dropped && std::getenv("GL_VERBOSE"))
         std::fprintf(stderr, "[gl]   %d dependent coarse columns dropped\n", c->co.n_dropped);
@@ -693,7 +693,7 @@ namespace {
 // the central subdomain gives factor entries and factorisation flops, scaled
 // by the subdomain count; the predicted time of one solve is
 //   setup = (Dirichlet flops + 2x for the Neumann factor) / F
-//         + 25 subspace iterations x 2 nev vectors x 4 flops x 1.6 nnz / F
+//         + 50 nev eigensolver solves x 4 flops x 1.6 nnz / F
 //         + (2 n0)^3 / 3 / F                     (coarse inverse)
 //   iteration = max(16 nnz / B, 4 nnz / F)       (FP64 sweeps; 8 nnz / B mixed)
 //   total = setup + 40 iterations,
