@@ -126,117 +126,122 @@ void build_plan(const std::vector<SubSymbolic> &subs, FactorPlan &P, cudaStream_
 
 // ----------------------------------------------------------------- numeric kernels
 
-// One block per (front, element): the element stiffness
-// K_e = sum_q w_q |J_q| B_q^T C_e B_q (FP64) is formed in shared memory, then
-// the entries of the front's pivot columns are added into the front.  With
-// sigma != 0 the entry (i, j) is scaled by 1 + sigma xi_i xi_j (the matrix
-// A^N + sigma Xi A^N Xi of the GenEO pencil).
+// One block per (front, element): the entries of K_e = sum_q w_q |J_q| B_q^T C_e B_q
+// (FP64) in the front's pivot columns, added into the front.  With sigma != 0
+// the entry (i, j) is scaled by 1 + sigma xi_i xi_j (the matrix A^N + sigma Xi
+// A^N Xi of the GenEO pencil).  Every DOF is a pivot of one front, so over all
+// fronts only half of the element's 81 x 81 entries are formed: the element's
+// DOFs are sorted by their position in the front (pivots first), a warp takes
+// a pivot column at a time -- its weighted stresses at the 27 Gauss points into
+// shared memory, lane = point -- and its lanes the rows from the diagonal on,
+// 81 FMAs an entry.  Bound by the FP64 pipe.  Forming all 6,561 entries of
+// every pair took 3.5 ms a launch on the 63k-DOF corner.
+constexpr int ASM_THREADS = 256;
+constexpr size_t ASM_SMEM = sizeof(double) * (27 * 27 * 3 + (ASM_THREADS / 32) * 27 * 6);
+
 template <class T>
-__global__ void __launch_bounds__(256) k_assemble(const int *__restrict__ fronts, const FrontDesc *__restrict__ D,
-                                                  const int *__restrict__ pair_elem,
-                                                  const int16_t *__restrict__ pair_pos, const int *__restrict__ rows,
-                                                  const double *__restrict__ C, const double *__restrict__ geo,
-                                                  const double *__restrict__ xi, double sigma, int s20,
-                                                  T *__restrict__ ws) {
-    const FrontDesc d = D[fronts[blockIdx.x]];
+__global__ void __launch_bounds__(ASM_THREADS) k_assemble(const int *__restrict__ fronts,
+                                                          const FrontDesc *__restrict__ D,
+                                                          const int *__restrict__ pair_elem,
+                                                          const int16_t *__restrict__ pair_pos,
+                                                          const int *__restrict__ rows, const double *__restrict__ C,
+                                                          const double *__restrict__ geo,
+                                                          const double *__restrict__ xi, double sigma, int s20,
+                                                          T *__restrict__ ws) {
+    const FrontDesc &d = D[fronts[blockIdx.x]];
     const int pr_i = blockIdx.y;
     if (pr_i >= d.n_pairs) return;
-    extern __shared__ double sK[];   // 81 x 81
-    __shared__ int16_t sp[81];
-    __shared__ double sx[81];
-    __shared__ double sG[27][3];
-    __shared__ double sCB[6][81];
-    __shared__ double sC[36];
-    __shared__ double sw;
-    const int f = d.p + d.q;
+    extern __shared__ double sm[];
+    double (*sG)[27][3] = reinterpret_cast<double (*)[27][3]>(sm);      // [q][node][axis]
+    __shared__ int16_t spos[81], sdof[81];   // positions in the front, ascending; the element DOFs they belong to
+    __shared__ double sx[81], sC[36], sw[27];
+    __shared__ int16_t raw[81];
+    __shared__ int cnt[2];                   // DOFs in the front, pivot columns among them
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int p = d.p, f = d.p + d.q;
     const int64_t e = pair_elem[d.pair_off + pr_i];
-    const int16_t *pos = pair_pos + (d.pair_off + pr_i) * 81;
-    if (threadIdx.x < 81) {
-        int16_t v = pos[threadIdx.x];
-        sp[threadIdx.x] = v;
-        sx[threadIdx.x] = (xi && v >= 0) ? xi[d.vec_off + rows[d.row_off + v]] : 0.0;
+    if (tid < 2) cnt[tid] = 0;
+    if (tid < 81) raw[tid] = pair_pos[(d.pair_off + pr_i) * 81 + tid];
+    if (tid >= 96 && tid < 132) sC[tid - 96] = C[36 * e + tid - 96];
+    if (tid >= 160 && tid < 187) sw[tid - 160] = geo[10 * (e * 27 + tid - 160) + 9];
+    __syncthreads();
+    if (tid < 81 && raw[tid] >= 0) {
+        const int v = raw[tid];
+        int r = 0;
+        for (int i = 0; i < 81; ++i) r += raw[i] >= 0 && raw[i] < v;
+        spos[r] = (int16_t)v;
+        sdof[r] = (int16_t)tid;
+        sx[r] = xi ? xi[d.vec_off + rows[d.row_off + v]] : 0.0;
+        atomicAdd(&cnt[0], 1);
+        if (v < p) atomicAdd(&cnt[1], 1);
     }
-    if (threadIdx.x < 36) sC[threadIdx.x] = C[36 * e + threadIdx.x];
+    // physical gradients of the 27 shape functions at the 27 Gauss points
     Q2Tables Tb;
     Tb.init();
-    double acc[26];
-#pragma unroll
-    for (int i = 0; i < 26; ++i) acc[i] = 0.0;
-    for (int q = 0; q < 27; ++q) {
-        __syncthreads();
-        const int qx = q % 3, qy = (q / 3) % 3, qz = q / 9;
+    for (int idx = tid; idx < 27 * 27; idx += ASM_THREADS) {
+        const int q = idx / 27, a = idx % 27;
+        const int qx = q % 3, qy = (q / 3) % 3, qz = q / 9, i = a % 3, j = (a / 3) % 3, k = a / 9;
         const double *g = geo + 10 * (e * 27 + q);
-        if (threadIdx.x < 27) {
-            int a = threadIdx.x, i = a % 3, j = (a / 3) % 3, k = a / 9;
-            double r0 = Tb.D[qx][i] * Tb.N[qy][j] * Tb.N[qz][k];
-            double r1 = Tb.N[qx][i] * Tb.D[qy][j] * Tb.N[qz][k];
-            double r2 = Tb.N[qx][i] * Tb.N[qy][j] * Tb.D[qz][k];
-            for (int dd = 0; dd < 3; ++dd) sG[a][dd] = r0 * g[0 + dd] + r1 * g[3 + dd] + r2 * g[6 + dd];
-        }
-        if (threadIdx.x == 0) sw = g[9];
-        __syncthreads();
-        for (int idx = threadIdx.x; idx < 6 * 81; idx += blockDim.x) {
-            int I = idx / 81, col = idx % 81, a = col / 3, c = col % 3;
-            double gx = sG[a][0], gy = sG[a][1], gz = sG[a][2], v;
-            if (c == 0) v = sC[6 * I + 0] * gx + sC[6 * I + 4] * gz + sC[6 * I + 5] * gy;
-            else if (c == 1) v = sC[6 * I + 1] * gy + sC[6 * I + 3] * gz + sC[6 * I + 5] * gx;
-            else v = sC[6 * I + 2] * gz + sC[6 * I + 3] * gy + sC[6 * I + 4] * gx;
-            sCB[I][col] = v;
-        }
-        __syncthreads();
-        const double w = sw;
-        int slot = 0;
-        for (int idx = threadIdx.x; idx < 6561; idx += blockDim.x, ++slot) {
-            int r = idx / 81, col = idx % 81, a = r / 3, c = r % 3;
-            double gx = sG[a][0], gy = sG[a][1], gz = sG[a][2], v;
-            if (c == 0) v = gx * sCB[0][col] + gz * sCB[4][col] + gy * sCB[5][col];
-            else if (c == 1) v = gy * sCB[1][col] + gz * sCB[3][col] + gx * sCB[5][col];
-            else v = gz * sCB[2][col] + gy * sCB[3][col] + gx * sCB[4][col];
-            acc[slot] += w * v;
-        }
-    }
-    {
-        int slot = 0;
-        for (int idx = threadIdx.x; idx < 6561; idx += blockDim.x, ++slot) sK[idx] = acc[slot];
+        const double r0 = Tb.D[qx][i] * Tb.N[qy][j] * Tb.N[qz][k];
+        const double r1 = Tb.N[qx][i] * Tb.D[qy][j] * Tb.N[qz][k];
+        const double r2 = Tb.N[qx][i] * Tb.N[qy][j] * Tb.D[qz][k];
+#pragma unroll
+        for (int dd = 0; dd < 3; ++dd) sG[q][a][dd] = r0 * g[0 + dd] + r1 * g[3 + dd] + r2 * g[6 + dd];
     }
     __syncthreads();
     if (s20) {
-        // serendipity element: K <- P^T K P, P the identity on the 20 nodes and the fixed
-        // combinations of them on the 7 face/body centres; first the columns, then the rows
-        // (only master rows and columns are updated; the slaves' are never assembled)
-        for (int idx = threadIdx.x; idx < 6561; idx += blockDim.x) {
-            const int r = idx / 81, col = idx % 81, a = col / 3, cc = col % 3;
+        // serendipity element: the face and body centres follow the 20 nodes, whose shape functions
+        // take their share of the centres' (the centres' DOFs are in no front)
+        for (int idx = tid; idx < 27 * 27; idx += ASM_THREADS) {
+            const int q = idx / 27, a = idx % 27;
             if (s20_is_slave(a)) continue;
-            double v = sK[idx];
+            double v0 = sG[q][a][0], v1 = sG[q][a][1], v2 = sG[q][a][2];
             for (int b = 0; b < 27; ++b)
                 if (s20_is_slave(b)) {
                     const double w = s20_weight(b, a);
-                    if (w != 0.0) v += w * sK[81 * r + 3 * b + cc];
+                    v0 += w * sG[q][b][0];
+                    v1 += w * sG[q][b][1];
+                    v2 += w * sG[q][b][2];
                 }
-            sK[idx] = v;
-        }
-        __syncthreads();
-        for (int idx = threadIdx.x; idx < 6561; idx += blockDim.x) {
-            const int r = idx / 81, col = idx % 81, a = r / 3, cc = r % 3;
-            if (s20_is_slave(a) || s20_is_slave(col / 3)) continue;
-            double v = sK[idx];
-            for (int b = 0; b < 27; ++b)
-                if (s20_is_slave(b)) {
-                    const double w = s20_weight(b, a);
-                    if (w != 0.0) v += w * sK[81 * (3 * b + cc) + col];
-                }
-            sK[idx] = v;
+            sG[q][a][0] = v0;
+            sG[q][a][1] = v1;
+            sG[q][a][2] = v2;
         }
         __syncthreads();
     }
+    const int n = cnt[0], nc = cnt[1];
+    double (*sS)[6] = reinterpret_cast<double (*)[6]>(sm + 27 * 27 * 3 + warp * 27 * 6);
     T *F = ws + d.front_off;
-    for (int idx = threadIdx.x; idx < 6561; idx += blockDim.x) {
-        int c = idx / 81, r = idx % 81;    // column (pivot) c, row r
-        int pc = sp[c], pr = sp[r];
-        if (pc < 0 || pc >= d.p || pr < pc) continue;
-        double v = sK[81 * r + c];
-        if (sigma != 0.0) v *= 1.0 + sigma * sx[r] * sx[c];
-        atomicAdd(F + pr + (int64_t)pc * f, (T)v);
+    for (int j = warp; j < nc; j += ASM_THREADS / 32) {
+        const int dof = sdof[j], node = dof / 3, c = dof % 3;
+        __syncwarp();
+        if (lane < 27) {
+            // w C B_j at Gauss point `lane`: strain of the unit displacement c of the node
+            const double gx = sG[lane][node][0], gy = sG[lane][node][1], gz = sG[lane][node][2], w = sw[lane];
+            const int i0 = c, i1 = c == 0 ? 5 : (c == 1 ? 3 : 4), i2 = c == 0 ? 4 : (c == 1 ? 5 : 3);
+            const double e0 = w * (c == 0 ? gx : (c == 1 ? gy : gz));          // normal strain
+            const double e1 = w * (c == 0 ? gy : (c == 1 ? gz : gx));          // 12, 23, 13
+            const double e2 = w * (c == 0 ? gz : (c == 1 ? gx : gy));          // 13, 12, 23
+#pragma unroll
+            for (int I = 0; I < 6; ++I) sS[lane][I] = sC[6 * I + i0] * e0 + sC[6 * I + i1] * e1 + sC[6 * I + i2] * e2;
+        }
+        __syncwarp();
+        for (int i = j + lane; i < n; i += 32) {
+            const int rd = sdof[i], a = rd / 3, rc = rd % 3;
+            // row rc of the stress: components (rc, x), (rc, y), (rc, z)
+            const int k0 = rc == 0 ? 0 : (rc == 1 ? 5 : 4), k1 = rc == 0 ? 5 : (rc == 1 ? 1 : 3),
+                      k2 = rc == 0 ? 4 : (rc == 1 ? 3 : 2);
+            double v0 = 0.0, v1 = 0.0, v2 = 0.0;
+#pragma unroll 9
+            for (int q = 0; q < 27; ++q) {
+                v0 += sG[q][a][0] * sS[q][k0];
+                v1 += sG[q][a][1] * sS[q][k1];
+                v2 += sG[q][a][2] * sS[q][k2];
+            }
+            double v = v0 + v1 + v2;
+            if (sigma != 0.0) v *= 1.0 + sigma * sx[i] * sx[j];
+            atomicAdd(F + spos[i] + (int64_t)spos[j] * f, (T)v);
+        }
     }
 }
 
@@ -633,10 +638,6 @@ static void inverse_form_level(const int *d_fronts, int nf, const FrontDesc *d_f
 template <class T>
 void numeric_factor(FactorPlan &P, const double *C, const double *geo, const double *xi, double sigma, T *L,
                     int *d_err, cudaStream_t s) {
-    static SmemLimit assemble_smem;
-    raise_smem_limit(assemble_smem, 6561 * 8, [](size_t v) {
-        GL_CUDA(cudaFuncSetAttribute(k_assemble<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)v));
-    });
     const int nlev = (int)P.levels.size();
     const int64_t budget = (int64_t)(P.ws_budget_bytes / sizeof(T));   // entries per workspace buffer
     std::vector<int> depth_of(P.fr.size());
@@ -704,7 +705,7 @@ void numeric_factor(FactorPlan &P, const double *C, const double *geo, const dou
             T *W = ws[dpt & 1].p;
             GL_CUDA(cudaMemsetAsync(W, 0, lev_ws[dpt] * sizeof(T), s));
             if (max_pairs[dpt] > 0) {
-                k_assemble<T><<<dim3(nf, max_pairs[dpt]), 256, 6561 * 8, s>>>(
+                k_assemble<T><<<dim3(nf, max_pairs[dpt]), ASM_THREADS, ASM_SMEM, s>>>(
                     d_lev[dpt].p, d_fr.p, P.d_pair_elem.p, P.d_pair_pos.p, P.d_rows.p, C, geo, xi, sigma, P.s20 ? 1 : 0,
                     W);
                 GL_CUDA(cudaGetLastError());
