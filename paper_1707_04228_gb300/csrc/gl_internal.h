@@ -161,8 +161,9 @@ void launch_ku(const MeshHost &m, const double *C, const double *geo, const doub
                cudaStream_t s);
 void launch_stress(const MeshHost &m, const double *X, const double *C, const double *psi,
                    const double *u, double *s33, double *t13, cudaStream_t s);
+// Failure index; peak[0] = the (F, element) key's bits (element in the low 24), peak[1] = the largest F.
 void launch_failure(const MeshHost &m, const double *X, const double *C, const double *psi_x, const uint8_t *resin,
-                    const double *u, double s33a, double s13a, double *F, unsigned long long *best, cudaStream_t s);
+                    const double *u, double s33a, double s13a, double *F, double *peak, cudaStream_t s);
 // FP64 FMA probe on the current device (probe.cu): flops per second.
 double fp64_probe(int iters, int reps, int *n_sm, double *ms_out);
 // Fails with GL_ERR_INVALID_ARG unless [p, p + bytes) lies inside one device

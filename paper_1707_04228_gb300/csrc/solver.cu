@@ -168,7 +168,7 @@ void require_ctx(gl_ctx *c) {
     GL_CUDA(cudaSetDevice(c->device));
 }
 
-// Copy n doubles from a caller pointer (host or device) into device memory.
+// Copy n doubles between a caller's array (host or device) and device memory.
 void to_device(double *dst, const double *src, int64_t n, cudaStream_t s) {
     if (n) GL_CUDA(cudaMemcpyAsync(dst, src, n * sizeof(double), cudaMemcpyDefault, s));
 }
@@ -186,6 +186,37 @@ void check_err(gl_ctx *c, const char *what) {
         if (h == 2) fail(GL_ERR_TIMEOUT, std::string(what) + ": a tensor-core wait gave up");
         fail(GL_ERR_NOT_SPD, std::string(what) + ": non-positive pivot");
     }
+}
+
+// *dst = v, dst in host or device memory.
+void put_scalar(double *dst, double v) {
+    if (is_device_ptr(dst)) GL_CUDA(cudaMemcpy(dst, &v, sizeof(double), cudaMemcpyDefault));
+    else *dst = v;
+}
+
+// Whether kernels of this context may use the caller's array in place: device
+// memory of the context's device, aligned, and apart from `other` (an input of
+// the same call, which the in-place output must not overwrite early).
+bool in_place(gl_ctx *c, const void *p, int64_t n, const void *other = nullptr, int64_t n_other = 0) {
+    if (!p || (reinterpret_cast<uintptr_t>(p) & 7)) return false;
+    cudaPointerAttributes a{};
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    if (a.type != cudaMemoryTypeDevice || a.device != c->device) return false;
+    const char *b = (const char *)p, *o = (const char *)other;
+    return !o || b + n * sizeof(double) <= o || o + n_other * sizeof(double) <= b;
+}
+
+// A displacement given by the caller as the stress kernels read it: in place,
+// or through the work vector q (host memory, or constrained entries to fill).
+const double *field_in(gl_ctx *c, const double *u) {
+    const MeshHost &m = c->m;
+    if (!has_slaves(m) && in_place(c, u, m.n_dof)) return u;
+    to_device(c->q.p, u, m.n_dof, c->stream);
+    if (has_slaves(m)) slave_fill(m, c->q.p, c->stream);
+    return c->q.p;
 }
 
 // Setup phase timing to stderr when GL_VERBOSE is set (syncs the stream).
@@ -514,7 +545,8 @@ void prepare_rhs(gl_ctx *c, const double *f, bool homogeneous) {
     g_launches += 1 + (nd ? 2 : 0);
 }
 
-// PCG solve of K u = f; homogeneous = zero Dirichlet values (adjoint solves).
+// PCG solve of K u = f into u (or left in c->x when u is that vector);
+// homogeneous = zero Dirichlet values (adjoint solves).
 void solve(gl_ctx *c, const double *f, double *u, gl_info *info, bool homogeneous = false) {
     if (!c->ready) fail(GL_ERR_STATE, "gl_solve before gl_setup");
     cudaStream_t s = c->stream;
@@ -616,7 +648,8 @@ void solve(gl_ctx *c, const double *f, double *u, gl_info *info, bool homogeneou
     }
     for (int ph = 0; ph < PH_N; ++ph) prof_fold(c, ph);
     GL_CUDA(cudaEventRecord(e1, s));
-    from_device(u, c->x.p, N, s);
+    if (u != c->x.p) to_device(u, c->x.p, N, s);
+    GL_CUDA(cudaStreamSynchronize(s));
     float ms = 0;
     GL_CUDA(cudaEventElapsedTime(&ms, e0, e1));
     cudaEventDestroy(e0);
@@ -1329,22 +1362,23 @@ int gl_stress(gl_ctx *c, const double *u, double *s33, double *t13, double *peak
         GL_REQUIRE(u, "null displacement");
         cudaStream_t s = c->stream;
         const MeshHost &m = c->m;
-        DBuf<double> du, d33, d13, dpk;
-        du.alloc(m.n_dof);
-        to_device(du.p, u, m.n_dof, s);
-        if (has_slaves(m)) slave_fill(m, du.p, s);
-        d33.alloc(m.n_elem);
-        d13.alloc(m.n_elem);
-        launch_stress(m, c->d_X.p, c->d_C.p, c->d_psi.p, du.p, d33.p, d13.p, s);
-        g_launches += 1 + (peak ? 1 : 0);
-        if (s33) from_device(s33, d33.p, m.n_elem, s);
-        if (t13) from_device(t13, d13.p, m.n_elem, s);
+        // outputs in host memory (or over u) go through the work vectors z and r
+        const double *du = field_in(c, u);
+        auto out = [&](double *p, DBuf<double> &w, const double *peer) {
+            const bool direct = in_place(c, p, m.n_elem, u, m.n_dof) && in_place(c, p, m.n_elem, peer, m.n_elem);
+            return direct ? p : w.p;
+        };
+        double *d33 = out(s33, c->z, t13), *d13 = out(t13, c->r, s33);
+        launch_stress(m, c->d_X.p, c->d_C.p, c->d_psi.p, du, d33, d13, s);
+        g_launches += 1 + (peak ? 2 : 0);
         if (peak) {
-            dpk.alloc(1);
-            max_where(d33.p, c->d_resin.p, m.n_elem, dpk.p, s);
-            from_device(peak, dpk.p, 1, s);
+            max_where(d33, c->d_resin.p, m.n_elem, c->partials.p, &c->S.p->alpha, s);
+            GL_CUDA(cudaMemcpyAsync(c->h_pin, &c->S.p->alpha, sizeof(double), cudaMemcpyDeviceToHost, s));
         }
+        if (s33 && s33 != d33) to_device(s33, d33, m.n_elem, s);
+        if (t13 && t13 != d13) to_device(t13, d13, m.n_elem, s);
         GL_CUDA(cudaStreamSynchronize(s));
+        if (peak) put_scalar(peak, c->h_pin[0]);
     });
 }
 
@@ -1413,22 +1447,17 @@ int gl_failure_index(gl_ctx *c, const double *u, double s33_allow, double s13_al
         const MeshHost &m = c->m;
         GL_REQUIRE(m.n_elem < (int64_t)1 << 24, "gl_failure_index: at most 16,777,215 elements");
         cudaStream_t s = c->stream;
-        DBuf<double> du, dF;
-        DBuf<unsigned long long> best;
-        du.alloc(m.n_dof);
-        to_device(du.p, u, m.n_dof, s);
-        if (has_slaves(m)) slave_fill(m, du.p, s);
-        dF.alloc(m.n_elem);
-        best.alloc(1);
-        launch_failure(m, c->d_X.p, c->d_C.p, c->d_psi.p, c->d_resin.p, du.p, s33_allow, s13_allow, dF.p, best.p, s);
-        g_launches += 1;
-        unsigned long long key = 0;
-        GL_CUDA(cudaMemcpyAsync(&key, best.p, sizeof(key), cudaMemcpyDeviceToHost, s));
+        const double *du = field_in(c, u);
+        double *dF = in_place(c, F, m.n_elem, u, m.n_dof) ? F : c->z.p;
+        launch_failure(m, c->d_X.p, c->d_C.p, c->d_psi.p, c->d_resin.p, du, s33_allow, s13_allow, dF, c->partials.p, s);
+        g_launches += 2;
+        GL_CUDA(cudaMemcpyAsync(c->h_pin, c->partials.p, 2 * sizeof(double), cudaMemcpyDeviceToHost, s));
+        if (F && F != dF) to_device(F, dF, m.n_elem, s);
         GL_CUDA(cudaStreamSynchronize(s));
-        const int64_t e = (int64_t)(key & 0xFFFFFF);
-        if (peak_elem) *peak_elem = e;
-        if (peak) from_device(peak, dF.p + e, 1, s);
-        if (F) from_device(F, dF.p, m.n_elem, s);
+        int64_t key;
+        std::memcpy(&key, c->h_pin, sizeof(key));
+        if (peak_elem) *peak_elem = key & 0xFFFFFF;
+        if (peak) put_scalar(peak, c->h_pin[1]);
     });
 }
 
@@ -1456,29 +1485,26 @@ int gl_stress_vjp(gl_ctx *c, const double *u, const double *w33, const double *w
         GL_REQUIRE(u, "null displacement");
         cudaStream_t s = c->stream;
         const MeshHost &m = c->m;
-        DBuf<double> du, d33, d13, dgu, dgt;
-        du.alloc(m.n_dof);
-        to_device(du.p, u, m.n_dof, s);
-        if (has_slaves(m)) slave_fill(m, du.p, s);
-        if (w33) {
-            d33.alloc(m.n_elem);
-            to_device(d33.p, w33, m.n_elem, s);
-        }
-        if (w13) {
-            d13.alloc(m.n_elem);
-            to_device(d13.p, w13, m.n_elem, s);
-        }
-        if (dJdu) {
-            dgu.alloc(m.n_dof);
-            dgu.zero(s);
-        }
-        if (dJdth) dgt.alloc(m.n_elem);
+        const int64_t N = m.n_dof, E = m.n_elem;
+        const double *du = field_in(c, u);
+        auto weights = [&](const double *w, DBuf<double> &stage) -> const double * {
+            if (!w || in_place(c, w, E)) return w;
+            to_device(stage.p, w, E, s);
+            return stage.p;
+        };
+        const double *d33 = weights(w33, c->z), *d13 = weights(w13, c->r);
+        auto apart = [&](const double *p, int64_t n) {
+            return in_place(c, p, n, u, N) && in_place(c, p, n, w33, E) && in_place(c, p, n, w13, E);
+        };
+        double *dgu = !dJdu ? nullptr : (apart(dJdu, N) ? dJdu : c->p.p);
+        double *dgt = !dJdth ? nullptr : (apart(dJdth, E) && in_place(c, dJdth, E, dJdu, N) ? dJdth : c->fe.p);
+        if (dgu) GL_CUDA(cudaMemsetAsync(dgu, 0, N * sizeof(double), s));
         launch_stress_vjp(m, c->d_X.p, c->d_C.p, c->d_psi.p, c->d_layer_of_ez.p, c->d_layer_mat.p, c->d_elem_mat.p,
-                          c->d_layer_angle.p, c->d_theta.p, c->d_matC.p, du.p, d33.p, d13.p, dgu.p, dgt.p, s);
+                          c->d_layer_angle.p, c->d_theta.p, c->d_matC.p, du, d33, d13, dgu, dgt, s);
         g_launches += 1;
-        if (dJdu && has_slaves(m)) slave_fold(m, dgu.p, s);   // dJ/du = P^T dJ/du_Q2
-        if (dJdu) from_device(dJdu, dgu.p, m.n_dof, s);
-        if (dJdth) from_device(dJdth, dgt.p, m.n_elem, s);
+        if (dgu && has_slaves(m)) slave_fold(m, dgu, s);   // dJ/du = P^T dJ/du_Q2
+        if (dgu && dgu != dJdu) to_device(dJdu, dgu, N, s);
+        if (dgt && dgt != dJdth) to_device(dJdth, dgt, E, s);
         GL_CUDA(cudaStreamSynchronize(s));
     });
 }
@@ -1490,18 +1516,15 @@ int gl_adjoint(gl_ctx *c, const double *u, const double *dJdu, double *grad, gl_
         GL_REQUIRE(u && dJdu && grad, "null argument");
         cudaStream_t s = c->stream;
         const MeshHost &m = c->m;
-        DBuf<double> lam, du, dg;
-        lam.alloc(m.n_dof);
-        solve(c, dJdu, lam.p, info, true);          // K_ff lambda = (dJ/du)_f, lambda = 0 on Dirichlet DOFs
-        du.alloc(m.n_dof);
-        to_device(du.p, u, m.n_dof, s);
-        if (has_slaves(m)) slave_fill(m, du.p, s);   // lambda comes back filled from solve()
-        dg.alloc(m.n_elem);
+        solve(c, dJdu, c->x.p, info, true);          // K_ff lambda = (dJ/du)_f, lambda = 0 on Dirichlet DOFs
+        const double *du = field_in(c, u);           // lambda comes back filled from solve()
+        double *dg = in_place(c, grad, m.n_elem, u, m.n_dof) ? grad : c->z.p;
         launch_adjoint_contract(m, c->d_geo.p, c->d_layer_of_ez.p, c->d_layer_mat.p, c->d_elem_mat.p,
                                 c->d_layer_angle.p,
-                                c->d_theta.p, c->d_psi.p, c->d_matC.p, du.p, lam.p, dg.p, s);
+                                c->d_theta.p, c->d_psi.p, c->d_matC.p, du, c->x.p, dg, s);
         g_launches += 1;
-        from_device(grad, dg.p, m.n_elem, s);
+        if (dg != grad) to_device(grad, dg, m.n_elem, s);
+        GL_CUDA(cudaStreamSynchronize(s));
     });
 }
 
