@@ -434,36 +434,42 @@ void fill_random(double *x, int64_t n, uint64_t seed, cudaStream_t s) {
 
 // ---------------------------------------------------------------- coarse restrict / prolong
 
+// c = Z^T r: a CTA gathers its chunk of r once, its warps take the columns of Z
+// in turn (contiguous reads, one FMA an entry).  Bound by reading Z; with the
+// column sums of all m columns in one thread (local memory) it took 157 us a
+// launch on the batch of five plates.
+constexpr int RESTRICT_ROWS = 256;
+
 __global__ void __launch_bounds__(256) k_coarse_restrict(const int64_t *__restrict__ voff, const int64_t *__restrict__ vlen,
                                                          const int64_t *__restrict__ gdof, const double *__restrict__ Z,
                                                          int m, const double *__restrict__ r, double *__restrict__ c) {
     const int s = blockIdx.x;
-    const int64_t n = vlen[s], base = voff[s] * m;
-    const int64_t *gd = gdof + voff[s];
-    double acc[NV_MAX];
-    for (int a = 0; a < m; ++a) acc[a] = 0.0;
-    for (int64_t i = (int64_t)blockIdx.y * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.y * blockDim.x) {
-        double ri = r[gd[i]];
-        for (int a = 0; a < m; ++a) acc[a] += Z[base + a * n + i] * ri;
-    }
-    __shared__ double red[8][NV_MAX];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    for (int a = 0; a < m; ++a) {
-        double v = acc[a];
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if (lane == 0) red[w][a] = v;
-    }
+    const int64_t n = vlen[s], r0 = (int64_t)blockIdx.y * RESTRICT_ROWS;
+    if (r0 >= n) return;
+    const int rows = (int)min((int64_t)RESTRICT_ROWS, n - r0);
+    __shared__ double sr[RESTRICT_ROWS];
+    const int64_t *gd = gdof + voff[s] + r0;
+    for (int i = threadIdx.x; i < RESTRICT_ROWS; i += 256) sr[i] = i < rows ? r[gd[i]] : 0.0;
     __syncthreads();
-    if (threadIdx.x < m) {
-        double v = 0.0;
-        for (int i = 0; i < (int)(blockDim.x >> 5); ++i) v += red[i][threadIdx.x];
-        atomicAdd(c + (int64_t)s * m + threadIdx.x, v);
+    const int lane = threadIdx.x & 31;
+    for (int a = threadIdx.x >> 5; a < m; a += 8) {
+        const double *Za = Z + voff[s] * m + (int64_t)a * n + r0;
+        double v0 = 0.0, v1 = 0.0;
+#pragma unroll 8
+        for (int i = lane; i < RESTRICT_ROWS; i += 64) {
+            v0 += (i < rows ? Za[i] : 0.0) * sr[i];
+            v1 += (i + 32 < rows ? Za[i + 32] : 0.0) * sr[i + 32];
+        }
+        double v = v0 + v1;
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (lane == 0) atomicAdd(c + (int64_t)s * m + a, v);
     }
 }
 
 void coarse_restrict(const FactorPlan &P, const double *Z, int m, const double *r, double *c, cudaStream_t s) {
     GL_CUDA(cudaMemsetAsync(c, 0, sizeof(double) * P.n_sub * m, s));
-    k_coarse_restrict<<<dim3(P.n_sub, 32), 256, 0, s>>>(P.d_vec_off.p, P.d_vec_len.p, P.d_gdof.p, Z, m, r, c);
+    k_coarse_restrict<<<dim3(P.n_sub, row_chunks(P, RESTRICT_ROWS)), 256, 0, s>>>(P.d_vec_off.p, P.d_vec_len.p,
+                                                                                 P.d_gdof.p, Z, m, r, c);
     GL_CUDA(cudaGetLastError());
 }
 
@@ -478,6 +484,7 @@ __global__ void k_coarse_prolong(const int64_t *__restrict__ voff, const int64_t
     __syncthreads();
     for (int64_t i = (int64_t)blockIdx.y * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.y * blockDim.x) {
         double v = 0.0;
+#pragma unroll 4
         for (int a = 0; a < m; ++a) v += Z[base + a * n + i] * sy[a];
         atomicAdd(z + gd[i], v);
     }
