@@ -740,10 +740,17 @@ template void numeric_factor<float>(FactorPlan &, const double *, const double *
 // (forward: 32 panel rows; backward: a tile of panel columns), which the
 // inverse form makes independent of one another, so a level with a few large
 // fronts fills the chip as well as one with thousands of small ones.  Where
-// even these tasks are fewer than SWEEP_WARPS, they are cut along the summed
-// dimension too and add their parts atomically.
+// the level has fewer than sweep_warps() tasks they are cut along the summed
+// dimension too (to no less than 32 columns or 64 rows) and add their parts
+// atomically: short tasks hide one another's loads and even out the SMs.  The
+// solve of the 475k-DOF corner (FP32) took 66.9, 64.5, 61.6 and 57.5 ms with
+// 12, 24, 48 and 96 tasks an SM, the 20k-DOF plate 11.3 to 10.4 ms; with
+// several right-hand sides a task has enough work and its atomics cost more.
 constexpr int SWEEP_CTA = 128;            // four warp tasks
-constexpr int SWEEP_WARPS = 152 * 12;     // warp tasks that keep the loads of every SM in flight
+template <int NR>
+constexpr int sweep_warps() {
+    return 152 * (NR == 1 ? 96 : 12);
+}
 
 // Forward: panel rows [r0, r0 + 32), lane = row, the columns of blockIdx.z's
 // chunk.  Pivot rows give y_1 = L11^{-1} b_1 (up to the diagonal block: zeros
@@ -764,11 +771,20 @@ __global__ void __launch_bounds__(SWEEP_CTA) k_fwd(const int *__restrict__ front
     const int cb = blockIdx.z * chunk;
     // pivot rows need the columns up to their diagonal block, any structure row all of them
     const int cend = min(r0 + 32 <= p ? r0 + 32 : p, cb + chunk);
-    if (r0 >= f || cb >= cend) return;
+    if (r0 >= f || cb >= cend) {
+        cudaGridDependencySynchronize();
+        return;
+    }
     const int64_t vo = d.vec_off * kcols + (int64_t)c0 * n;
     const T *b1 = b + vo + d.first;
     const int row = min(r0 + lane, f - 1);
     const T *Lr = L + d.l_off + row;
+    constexpr int G = sizeof(T) == 4 ? 32 : 16;   // loads in flight per lane
+    T l[G];
+    // the panel does not depend on the launches before: its first columns are on their way during the wait
+#pragma unroll
+    for (int j = 0; j < G; ++j) l[j] = cb + j < cend ? Lr[(int64_t)(cb + j) * f] : T(0);
+    cudaGridDependencySynchronize();
     T acc[NR], acc2[NR];
 #pragma unroll
     for (int r = 0; r < NR; ++r) acc[r] = acc2[r] = T(0);
@@ -780,14 +796,15 @@ __global__ void __launch_bounds__(SWEEP_CTA) k_fwd(const int *__restrict__ front
         for (int r = 0; r < NR; ++r) xs[lane * NR + r] = lane < kb ? b1[c + lane + (int64_t)r * n] : T(0);
         __syncwarp();
         const T *Lc = Lr + (int64_t)c * f;
-        constexpr int G = sizeof(T) == 4 ? 32 : 16;   // loads in flight per lane
 #pragma unroll
         for (int g = 0; g < 32; g += G) {
             if (g >= kb) break;
-            T l[G];
+            const bool have = g == 0 && c == cb;
             if (g + G <= kb) {
+                if (!have) {
 #pragma unroll
-                for (int j = 0; j < G; ++j) l[j] = Lc[(int64_t)(g + j) * f];
+                    for (int j = 0; j < G; ++j) l[j] = Lc[(int64_t)(g + j) * f];
+                }
 #pragma unroll
                 for (int j = 0; j < G; j += 2)
 #pragma unroll
@@ -797,8 +814,10 @@ __global__ void __launch_bounds__(SWEEP_CTA) k_fwd(const int *__restrict__ front
                     }
             } else {
                 // the last columns, in fours
+                if (!have) {
 #pragma unroll
-                for (int j = 0; j < G; ++j) l[j] = g + j < kb ? Lc[(int64_t)(g + j) * f] : T(0);
+                    for (int j = 0; j < G; ++j) l[j] = g + j < kb ? Lc[(int64_t)(g + j) * f] : T(0);
+                }
 #pragma unroll
                 for (int h = 0; h < G; h += 4) {
                     if (g + h >= kb) break;
@@ -810,6 +829,7 @@ __global__ void __launch_bounds__(SWEEP_CTA) k_fwd(const int *__restrict__ front
             }
         }
     }
+    cudaTriggerProgrammaticLaunchCompletion();
     if (r0 + lane >= f) return;
     if (row < p) {
         T *yo = y + vo + d.first + row;
@@ -849,12 +869,18 @@ __global__ void __launch_bounds__(SWEEP_CTA) k_bwd(const int *__restrict__ front
     const int p = d.p, f = p + d.q, n = d.vlen;
     const int task = blockIdx.y * (SWEEP_CTA / 32) + (threadIdx.x >> 5);
     const int nct = (p + CT - 1) / CT;
-    if (task >= nct * chunks) return;
+    if (task >= nct * chunks) {
+        cudaGridDependencySynchronize();
+        return;
+    }
     const int j0 = (task % nct) * CT, kb = min(CT, p - j0);
     // the tile's rows start at its diagonal block; chunks of whole 32-row steps
     const int steps = (f - j0 + 31) / 32, per = (steps + chunks - 1) / chunks;
     const int rb = j0 + 32 * per * (task / nct), re = min(f, rb + 32 * per);
-    if (rb >= re) return;
+    if (rb >= re) {
+        cudaGridDependencySynchronize();
+        return;
+    }
     const int64_t vo = d.vec_off * kcols + (int64_t)c0 * n;
     const T *y1 = y + vo + d.first, *xo = x + vo;
     const int *rw = rows + d.row_off;
@@ -872,16 +898,23 @@ __global__ void __launch_bounds__(SWEEP_CTA) k_bwd(const int *__restrict__ front
 #pragma unroll
         for (int k = 0; k < NR; ++k) v[k] = sg * at[(int64_t)k * n];
     };
-    T v[NR], vn[NR];
-    fetch_v(rb, where(rb), v);
-    const T *at = where(rb + 32);
-    for (int r = rb; r < re; r += 32) {
+    T v[NR], vn[NR], l[CT];
+    auto fetch_l = [&](int r) {
         const T *Li = Lt + min(r + lane, f - 1);
+#pragma unroll
+        for (int j = 0; j < CT; ++j) l[j] = j < kb ? Li[(int64_t)j * f] : T(0);
+    };
+    // the panel does not depend on the launches before: its first rows are on their way during the wait
+    fetch_l(rb);
+    const T *at = where(rb);
+    const T *at1 = where(rb + 32);
+    cudaGridDependencySynchronize();
+    fetch_v(rb, at, v);
+    at = at1;
+    for (int r = rb; r < re; r += 32) {
         auto step = [&](auto cols) {
             constexpr int G = decltype(cols)::value;
-            T l[G];
-#pragma unroll
-            for (int j = 0; j < G; ++j) l[j] = j < kb ? Li[(int64_t)j * f] : T(0);
+            if (r != rb) fetch_l(r);
             fetch_v(r + 32, at, vn);
             at = where(r + 64);
 #pragma unroll
@@ -894,6 +927,7 @@ __global__ void __launch_bounds__(SWEEP_CTA) k_bwd(const int *__restrict__ front
 #pragma unroll
         for (int k = 0; k < NR; ++k) v[k] = vn[k];
     }
+    cudaTriggerProgrammaticLaunchCompletion();
     warp_sum_many<T, CT * NR>(acc, lane);
     constexpr int PL = CT * NR < 32 ? 1 : CT * NR / 32, SH = CT * NR < 32 ? 1 : 0;   // sums per lane; lanes per sum 2^SH
     if (lane & SH) return;
@@ -938,6 +972,27 @@ static void level_clock_fold(const FactorPlan &P) {
     K.calls += 1;
 }
 
+// A level's launch may start while the one before it in the stream finishes
+// (programmatic dependent launch): its CTAs read their descriptors and the
+// first part of their panels, then wait for that launch's results.  A launch
+// lets the next one start when its tasks reach their last additions (earlier,
+// the waiting CTAs take the place of running ones: 12.2 instead of 9.0 ms on the
+// 20k-DOF plate).  Every thread waits, also those without work, so that a launch
+// never completes before the ones it follows.
+template <class K, class... A>
+static void launch_chained(K kernel, dim3 grid, cudaStream_t s, A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(SWEEP_CTA);
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    GL_CUDA(cudaLaunchKernelEx(&cfg, kernel, args...));
+}
+
 // One level's forward or backward sweep over the fronts fr[0..nf) of that level.
 template <class T, int NR>
 static void launch_fwd(const FactorPlan &P, const Level &Lv, const int *fr, unsigned nf, const T *L, T *b, T *y,
@@ -945,10 +1000,10 @@ static void launch_fwd(const FactorPlan &P, const Level &Lv, const int *fr, unsi
     if (nf == 0 || Lv.max_p == 0) return;
     const int tiles = (Lv.max_f + 31) / 32, blocks = (Lv.max_p + 31) / 32;
     // (the level's fronts, not nf: the arithmetic is the same however the level is split over streams)
-    const int split = std::min<int64_t>(blocks, std::max<int64_t>(1, SWEEP_WARPS / ((int64_t)Lv.fronts.size() * tiles)));
+    const int split = std::min<int64_t>(blocks, std::max<int64_t>(1, sweep_warps<NR>() / ((int64_t)Lv.fronts.size() * tiles)));
     const int chunk = 32 * ((blocks + split - 1) / split);
     const dim3 g(nf, (tiles + SWEEP_CTA / 32 - 1) / (SWEEP_CTA / 32), (Lv.max_p + chunk - 1) / chunk);
-    k_fwd<T, NR><<<g, SWEEP_CTA, 0, s>>>(fr, P.d_fr.p, L, P.d_rows.p, b, y, kcols, c0, chunk);
+    launch_chained(k_fwd<T, NR>, g, s, fr, (const FrontDesc *)P.d_fr.p, L, (const int *)P.d_rows.p, b, y, kcols, c0, chunk);
 }
 
 template <class T, int NR>
@@ -957,9 +1012,9 @@ static void launch_bwd(const FactorPlan &P, const Level &Lv, const int *fr, unsi
     if (nf == 0 || Lv.max_p == 0) return;
     const int tiles = (Lv.max_p + bwd_tile<NR>() - 1) / bwd_tile<NR>();
     const int chunks = std::min<int64_t>((Lv.max_f + 63) / 64,
-                                         std::max<int64_t>(1, SWEEP_WARPS / ((int64_t)Lv.fronts.size() * tiles)));
+                                         std::max<int64_t>(1, sweep_warps<NR>() / ((int64_t)Lv.fronts.size() * tiles)));
     const dim3 g(nf, (tiles * chunks + SWEEP_CTA / 32 - 1) / (SWEEP_CTA / 32));
-    k_bwd<T, NR><<<g, SWEEP_CTA, 0, s>>>(fr, P.d_fr.p, L, P.d_rows.p, y, x, kcols, c0, chunks);
+    launch_chained(k_bwd<T, NR>, g, s, fr, (const FrontDesc *)P.d_fr.p, L, (const int *)P.d_rows.p, y, x, kcols, c0, chunks);
 }
 
 static HalfStreams &half_streams(const FactorPlan &P) {
