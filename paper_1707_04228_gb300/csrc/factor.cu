@@ -264,63 +264,75 @@ __global__ void k_extend_add(const int *__restrict__ children, const FrontDesc *
     }
 }
 
-// Diagonal block Cholesky (kb <= 32) of each front at pivot offset k0.
+// Diagonal block Cholesky (kb <= 32) of each front at pivot offset k0.  A chain
+// of 32 dependent steps whose FP64 instructions each hold an SM quarter's pipe
+// for 64 clocks, so every step is cut to one reciprocal square root, one
+// product and a quarter of the column updates per warp (the warps compute the
+// column alike, lane = row, and share the updates), and one barrier.  With a
+// square root and divisions in turn it took 53 us a launch, this form 32.
 template <class T>
-__global__ void k_potrf(const int *__restrict__ fronts, const FrontDesc *__restrict__ D, T *__restrict__ ws, int k0,
-                        int *__restrict__ err, T drop, int *__restrict__ drops) {
-    const FrontDesc d = D[fronts[blockIdx.x]];
+__global__ void __launch_bounds__(128) k_potrf(const int *__restrict__ fronts, const FrontDesc *__restrict__ D,
+                                               T *__restrict__ ws, int k0, int *__restrict__ err, T drop,
+                                               int *__restrict__ drops) {
+    const FrontDesc &d = D[fronts[blockIdx.x]];
     if (k0 >= d.p) return;
     const int kb = min(NB, d.p - k0), f = d.p + d.q;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     T *A = ws + d.front_off + k0 + (int64_t)k0 * f;
-    __shared__ T a[NB][NB + 1];
-    for (int idx = threadIdx.x; idx < kb * kb; idx += blockDim.x) {
-        int i = idx % kb, j = idx / kb;
-        a[i][j] = i >= j ? A[i + (int64_t)j * f] : T(0);
-    }
+    __shared__ T a[NB][NB + 1];   // column-major: a[j][i]
+    for (int j = w; j < NB; j += 4) a[j][lane] = j < kb && lane < kb && lane >= j ? A[lane + (int64_t)j * f] : T(0);
     __syncthreads();
     for (int j = 0; j < kb; ++j) {
-        if (threadIdx.x == 0) {
-            T v = a[j][j];
-            if (drop > T(0) && fabs(v) <= drop) {
-                // dependent column (drop mode): zero pivot, the column leaves the factor
-                atomicAdd(drops, 1);
-                a[j][j] = T(0);
+        T v = a[j][j], l;
+        if (drop > T(0) && fabs(v) <= drop) {
+            // dependent column (drop mode): zero pivot, the column leaves the factor
+            if (threadIdx.x == 0) atomicAdd(drops, 1);
+            l = T(0);
+        } else {
+            if (!(v > T(0))) {
+                if (threadIdx.x == 0) atomicExch(err, 1);
+                v = T(1);
+            }
+            if (sizeof(T) == 8) {
+                const T r = (T)rsqrt((double)v);
+                l = lane == j ? v * r : a[j][lane] * r;
             } else {
-                if (!(v > T(0))) {
-                    atomicExch(err, 1);
-                    v = T(1);
-                }
-                a[j][j] = sqrt(v);
+                const T r = (T)sqrtf((float)v);
+                l = lane == j ? r : a[j][lane] / r;
             }
         }
-        __syncthreads();
-        T djj = a[j][j];
-        for (int i = j + 1 + threadIdx.x; i < kb; i += blockDim.x) a[i][j] = djj != T(0) ? a[i][j] / djj : T(0);
-        __syncthreads();
-        for (int idx = threadIdx.x; idx < kb * kb; idx += blockDim.x) {
-            int i = idx % kb, k = idx / kb;
-            if (k > j && i >= k) a[i][k] -= a[i][j] * a[k][j];
+        if (lane < j) l = T(0);
+        for (int k = j + 1 + w; k < kb; k += 4) {
+            const T lk = __shfl_sync(0xffffffffu, l, k);
+            if (lane >= k) a[k][lane] -= l * lk;
         }
-        __syncthreads();
+        __syncthreads();          // every warp has read column j; its updates are in place
+        if (w == 0) a[j][lane] = l;
     }
-    for (int idx = threadIdx.x; idx < kb * kb; idx += blockDim.x) {
-        int i = idx % kb, j = idx / kb;
-        if (i >= j) A[i + (int64_t)j * f] = a[i][j];
-    }
+    __syncthreads();
+    for (int j = w; j < kb; j += 4)
+        if (lane < kb && lane >= j) A[lane + (int64_t)j * f] = a[j][lane];
 }
 
-// Panel below the diagonal block: rows r in [k0+kb, f) <- row * L_kk^{-T}.
+// Panel below the diagonal block: rows r in [k0+kb, f) <- row * L_kk^{-T}, one
+// row per thread.  The pivots' reciprocals are formed once per CTA (FP64): a
+// division per entry, 32 of them against 500 FMAs, took most of the time (69
+// us a launch on the 63k-DOF corner, now 48).
 template <class T>
-__global__ void k_trsm(const int *__restrict__ fronts, const FrontDesc *__restrict__ D, T *__restrict__ ws, int k0) {
-    const FrontDesc d = D[fronts[blockIdx.x]];
+__global__ void __launch_bounds__(128) k_trsm(const int *__restrict__ fronts, const FrontDesc *__restrict__ D,
+                                              T *__restrict__ ws, int k0) {
+    const FrontDesc &d = D[fronts[blockIdx.x]];
     if (k0 >= d.p) return;
     const int kb = min(NB, d.p - k0), f = d.p + d.q;
+    if (k0 + kb + (int)(blockIdx.y * blockDim.x) >= f) return;
     const int r = k0 + kb + blockIdx.y * blockDim.x + threadIdx.x;
-    __shared__ T l[NB][NB + 1];
+    __shared__ T l[NB][NB + 1];   // l[j][i] = L[j, i], i < j; the diagonal holds the reciprocal (FP64) or the pivot
     T *F = ws + d.front_off;
-    for (int idx = threadIdx.x; idx < kb * kb; idx += blockDim.x) {
-        int i = idx % kb, j = idx / kb;
-        l[i][j] = i >= j ? F[(k0 + i) + (int64_t)(k0 + j) * f] : T(0);
+    for (int idx = threadIdx.x; idx < NB * NB; idx += blockDim.x) {
+        const int j = idx % NB, i = idx / NB;
+        T v = j < kb && i <= j ? F[(k0 + j) + (int64_t)(k0 + i) * f] : T(0);
+        if (sizeof(T) == 8 && i == j) v = v != T(0) ? T(1) / v : T(0);
+        l[j][i] = v;
     }
     __syncthreads();
     if (r >= f) return;
@@ -331,11 +343,16 @@ __global__ void k_trsm(const int *__restrict__ fronts, const FrontDesc *__restri
 #pragma unroll
     for (int j = 0; j < NB; ++j) {
         if (j < kb) {
-            T v = x[j];
+            T v = x[j], v1 = T(0);   // two chains
 #pragma unroll
             for (int i = 0; i < NB; ++i)
-                if (i < j) v -= x[i] * l[j][i];
-            x[j] = l[j][j] != T(0) ? v / l[j][j] : T(0);   // zero pivot: a dropped column
+                if (i < j) {
+                    if (i & 1) v1 -= x[i] * l[j][i];
+                    else v -= x[i] * l[j][i];
+                }
+            v += v1;
+            if (sizeof(T) == 8) x[j] = v * l[j][j];                        // zero pivot: a dropped column
+            else x[j] = l[j][j] != T(0) ? v / l[j][j] : T(0);
         }
     }
 #pragma unroll
