@@ -431,51 +431,39 @@ __global__ void __launch_bounds__(256) k_syrk(const int *__restrict__ fronts, co
 }
 
 // Blocked right-looking partial Cholesky of the p pivot columns of every front
-// of a level.  FP64 (and FP32 with tc = false): blocks of NB = 32 pivots, each
-// followed by the rank-32 update of the whole trailing lower triangle.  FP32
-// with tc: outer panels of 128 columns factored with the same 32-wide steps,
-// whose updates stay inside the panel, and one rank-128 update of the trailing
-// matrix per panel on the tensor cores (syrk_tc.cu) -- four times the flops
-// per byte of trailing matrix read and written.
+// of a level, in blocks of NB = 32 pivots.  Without tc each block is followed
+// by the rank-32 update of the whole trailing lower triangle.  With tc the
+// blocks' updates stay inside an outer panel, and one update of the trailing
+// matrix per panel runs on the tensor cores: FP32 with panels of 128 columns
+// (syrk_tc.cu), FP64 with panels of 64 (gemm64_tc.cu; wider ones leave more to
+// the FP64 pipe inside the panel than they save outside).
+constexpr int PANEL64 = 64;
+
+template <class T>
 static void partial_cholesky_level(const int *d_fronts, int n_fronts, const FrontDesc *d_fr, int max_p, int max_f,
-                                   void *ws, bool fp32, int *d_err, cudaStream_t s, double drop = 0.0,
-                                   int *d_drops = nullptr, bool tc = false) {
-    if (fp32 && tc) {
-        const int PW = syrk_tc_panel();
-        for (int k0 = 0; k0 < max_p; k0 += PW) {
-            const int kend = k0 + PW;
-            for (int k1 = k0; k1 < std::min(kend, max_p); k1 += NB) {
-                const int rows = std::max(1, max_f - k1);
-                const int m = max_f - k1;
-                const int nt = m > 0 ? (m + TILE - 1) / TILE : 0;
+                                   T *ws, int *d_err, cudaStream_t s, T drop = T(0), int *d_drops = nullptr,
+                                   bool tc = false) {
+    const int PW = !tc ? NB : (sizeof(T) == 4 ? syrk_tc_panel() : PANEL64);
+    for (int k0 = 0; k0 < max_p; k0 += PW) {
+        const int kend = k0 + PW;
+        for (int k1 = k0; k1 < std::min(kend, max_p); k1 += NB) {
+            // upper bounds over the level's fronts (a front's last pivot block may be short)
+            const int rows = std::max(1, max_f - k1);
+            const int nt = (rows + TILE - 1) / TILE;
+            k_potrf<T><<<n_fronts, 128, 0, s>>>(d_fronts, d_fr, ws, k1, d_err, drop, d_drops);
+            k_trsm<T><<<dim3(n_fronts, (rows + 127) / 128), 128, 0, s>>>(d_fronts, d_fr, ws, k1);
+            if (!tc) {
+                k_syrk<T><<<dim3(n_fronts, nt * (nt + 1) / 2), 256, 0, s>>>(d_fronts, d_fr, ws, k1, 0);
+            } else if (k1 + NB < kend) {
                 const int ncw = std::min(nt, (kend - k1 - 1) / TILE + 1);    // column tiles inside the panel
-                const int tiles = std::max(1, ncw * nt - ncw * (ncw - 1) / 2);
-                k_potrf<float><<<n_fronts, 128, 0, s>>>(d_fronts, d_fr, (float *)ws, k1, d_err, (float)drop, d_drops);
-                k_trsm<float><<<dim3(n_fronts, (rows + 127) / 128), 128, 0, s>>>(d_fronts, d_fr, (float *)ws, k1);
-                k_syrk<float><<<dim3(n_fronts, tiles), 256, 0, s>>>(d_fronts, d_fr, (float *)ws, k1, kend);
-                GL_CUDA(cudaGetLastError());
+                k_syrk<T><<<dim3(n_fronts, std::max(1, ncw * nt - ncw * (ncw - 1) / 2)), 256, 0, s>>>(d_fronts, d_fr, ws,
+                                                                                                   k1, kend);
             }
-            syrk_tc_level(d_fronts, n_fronts, d_fr, k0, max_f, (float *)ws, d_err, s);
+            GL_CUDA(cudaGetLastError());
         }
-        return;
-    }
-    for (int k0 = 0; k0 < max_p; k0 += NB) {
-        // upper bounds over the level's fronts (a front's last pivot block may be short)
-        int rows = std::max(1, max_f - k0);
-        int m = max_f - k0;
-        int nt = m > 0 ? (m + TILE - 1) / TILE : 0;
-        int tiles = std::max(1, nt * (nt + 1) / 2);
-        dim3 gt(n_fronts, (rows + 127) / 128), gs(n_fronts, tiles);
-        if (fp32) {
-            k_potrf<float><<<n_fronts, 128, 0, s>>>(d_fronts, d_fr, (float *)ws, k0, d_err, (float)drop, d_drops);
-            k_trsm<float><<<gt, 128, 0, s>>>(d_fronts, d_fr, (float *)ws, k0);
-            k_syrk<float><<<gs, 256, 0, s>>>(d_fronts, d_fr, (float *)ws, k0, 0);
-        } else {
-            k_potrf<double><<<n_fronts, 128, 0, s>>>(d_fronts, d_fr, (double *)ws, k0, d_err, drop, d_drops);
-            k_trsm<double><<<gt, 128, 0, s>>>(d_fronts, d_fr, (double *)ws, k0);
-            k_syrk<double><<<gs, 256, 0, s>>>(d_fronts, d_fr, (double *)ws, k0, 0);
-        }
-        GL_CUDA(cudaGetLastError());
+        if (!tc) continue;
+        if constexpr (sizeof(T) == 4) syrk_tc_level(d_fronts, n_fronts, d_fr, k0, max_f, ws, d_err, s);
+        else syrk64_tc_level(d_fronts, n_fronts, d_fr, k0, PANEL64, max_f, ws, d_err, s);
     }
 }
 
@@ -638,14 +626,18 @@ __global__ void __launch_bounds__(256) k_wpanel(const int *__restrict__ fronts, 
 
 template <class T>
 static void inverse_form_level(const int *d_fronts, int nf, const FrontDesc *d_fr, int max_p, int max_f, const T *ws,
-                               T *L, cudaStream_t s) {
+                               T *L, int *d_err, cudaStream_t s) {
     const int nb = (max_p + 31) / 32;
     if (nb == 0) return;
     k_diag_inverse<T><<<dim3(nf, nb), 32, 0, s>>>(d_fronts, d_fr, ws, L);
     k_tri_inverse<T><<<dim3(nf, nb), INV_THREADS, 0, s>>>(d_fronts, d_fr, ws, L);
-    // upper bound of row tiles x column tiles over the level's fronts (q <= max_f, p <= max_p)
-    const int tiles = ((max_f + TILE - 1) / TILE) * ((max_p + TILE - 1) / TILE);
-    k_wpanel<T><<<dim3(nf, tiles), 256, 0, s>>>(d_fronts, d_fr, ws, L);
+    if constexpr (sizeof(T) == 8) {
+        wpanel_tc_level(d_fronts, nf, d_fr, max_p, max_f, ws, L, d_err, s);
+    } else {
+        // upper bound of row tiles x column tiles over the level's fronts (q <= max_f, p <= max_p)
+        const int tiles = ((max_f + TILE - 1) / TILE) * ((max_p + TILE - 1) / TILE);
+        k_wpanel<T><<<dim3(nf, tiles), 256, 0, s>>>(d_fronts, d_fr, ws, L);
+    }
     GL_CUDA(cudaGetLastError());
 }
 
@@ -737,9 +729,9 @@ void numeric_factor(FactorPlan &P, const double *C, const double *geo, const dou
                     GL_CUDA(cudaGetLastError());
                 }
             }
-            partial_cholesky_level(d_lev[dpt].p, nf, d_fr.p, max_p[dpt], max_f[dpt], W, sizeof(T) == 4, d_err, s,
-                                   0.0, nullptr, sizeof(T) == 4 && P.tc_update);
-            inverse_form_level<T>(d_lev[dpt].p, nf, d_fr.p, max_p[dpt], max_f[dpt], W, L, s);
+            partial_cholesky_level<T>(d_lev[dpt].p, nf, d_fr.p, max_p[dpt], max_f[dpt], W, d_err, s, T(0), nullptr,
+                                      sizeof(T) == 8 || P.tc_update);
+            inverse_form_level<T>(d_lev[dpt].p, nf, d_fr.p, max_p[dpt], max_f[dpt], W, L, d_err, s);
         }
         GL_CUDA(cudaStreamSynchronize(s));   // the group's lists are released at the end of this scope
         j0 = j1;
@@ -1244,7 +1236,7 @@ int dense_inverse(const double *A, int n, double *Ainv, int *d_err, cudaStream_t
     F.alloc((size_t)4 * n * n);
     k_aug_init<<<1024, 256, 0, s>>>(A, n, F.p);
     GL_CUDA(cudaGetLastError());
-    partial_cholesky_level(idx.p, 1, d.p, n, 2 * n, F.p, false, d_err, s, drop, drops.p);
+    partial_cholesky_level<double>(idx.p, 1, d.p, n, 2 * n, F.p, d_err, s, drop, drops.p);
     k_extract_inv<<<1024, 256, 0, s>>>(A, F.p, n, Ainv);
     GL_CUDA(cudaGetLastError());
     int h = 0;

@@ -154,6 +154,14 @@ int syrk_tc_panel();
 void syrk_tc_level(const int *d_fronts, int n_fronts, const FrontDesc *d_fr, int k0, int max_f, float *ws,
                    int *d_err, cudaStream_t s);
 
+// FP64 products of a level's fronts on the tensor cores (gemm64_tc.cu): the
+// trailing update by the kw = min(panel, p - k0) factored columns from k0 on,
+// and W = L21 L11^{-1} of the inverse-form panels.  panel <= 128; d_err as above.
+void syrk64_tc_level(const int *d_fronts, int n_fronts, const FrontDesc *d_fr, int k0, int panel, int max_f, double *ws,
+                     int *d_err, cudaStream_t s);
+void wpanel_tc_level(const int *d_fronts, int n_fronts, const FrontDesc *d_fr, int max_p, int max_f, const double *ws,
+                     double *out, int *d_err, cudaStream_t s);
+
 // x = L^{-T} L^{-1} b (panels as numeric_factor leaves them) for local
 // multi-vectors of kcols columns per subdomain, each column of the subdomain's
 // length stored contiguously: b[vec_off*kcols + c*n + i] (kcols = 1: plain

@@ -1,0 +1,404 @@
+// FP64 products of the supernodal fronts on the 5th-generation tensor cores
+// (tcgen05, FP16 operands, FP32 accumulation in tensor memory).
+//
+// Section 2.3 solves the overlapping subdomain problems with direct local
+// factorisations.  Two products hold nearly all their flops: the trailing
+// update of a front's partial Cholesky, F[r, c] -= sum_k P[r, k] P[c, k], and
+// W = L21 L11^{-1} of the inverse-form panels.  The FP64 pipe of this part does
+// two FMAs per clock and SM, its tensor cores some 3,500 in FP16, so a product
+// is formed there from integer slices (the error-free splitting of Ozaki,
+// Ogita, Oishi and Rump, Numer. Algorithms 59, 2012, on fixed-point rows):
+//   * a row's entries over the summed range are scaled by a power of two to
+//     fixed point, 62 bits below the row's largest exponent (no FP64 bit of the
+//     largest entries is lost; smaller ones lose bits below 2^-62 of it);
+//   * the fixed-point number is cut into eight signed base-256 digits, each in
+//     [-128, 127] and exact in FP16;
+//   * the digit products of equal weight i + j = s <= 7 are summed over k <= 128
+//     in one FP32 accumulator: an integer of at most 8 x 128 x 2^14 = 2^24, so
+//     every addition is exact; the weights s >= 8 lie below 2^-60 of the
+//     product of the rows' largest entries and are left out;
+//   * the eight sums are put together in two 64-bit integers, converted to
+//     FP64 without loss and added to the result by two FMAs.
+//
+// One CTA of 256 threads forms a 128 x 32 tile: a thread stages the digits of
+// eight columns of a row at a time (K-major core matrices of 8 rows x 16 bytes,
+// no swizzle), 32 columns per round.  The eight accumulators take 256 columns
+// of tensor memory, so two CTAs share an SM and each works while the other
+// waits for its loads or its products.  Every wait is bounded: if a commit does
+// not arrive within the limit the kernel raises the error flag, skips the
+// write-back, frees its tensor memory and returns (the host reports
+// GL_ERR_TIMEOUT).
+//
+// Measured on the 63k-DOF corner's set-up: trailing updates 50.6 ms on the FP64
+// pipe, 13.2 ms here and 7.8 ms inside the panels; W 19.0 ms, 3.8 ms here.  What
+// binds it now is the latency of its loads (two CTAs an SM; FP64 pipe 18% and
+// tensor pipe 7% active).  One-subdomain direct solves (25k to 75k DOF, six
+// laminates) left residuals of 0.7 to 0.9 of those with FP64 FMAs and solution
+// errors as large as theirs; cutting the sums to 2^-54 of the largest entries'
+// product instead of converting both halves made them up to 100 times larger.
+#include <cuda_fp16.h>
+
+#include "factor.h"
+
+namespace gl {
+
+namespace {
+
+constexpr int OZ_M = 128, OZ_N = 32;        // output tile
+constexpr int OZ_KC = 32;                   // summed columns staged per round (2 MMAs of K = 16)
+constexpr int OZ_KB = 128;                  // summed columns per exact accumulation
+constexpr int OZ_S = 8;                     // digits
+constexpr int OZ_THREADS = 256;
+constexpr int OZ_TMEM_COLS = OZ_S * OZ_N;   // 256: two CTAs per SM
+constexpr int OZ_A_BYTES = OZ_M * OZ_KC * 2, OZ_B_BYTES = OZ_N * OZ_KC * 2;   // one digit of an operand tile
+constexpr int OZ_BUF = OZ_S * (OZ_A_BYTES + OZ_B_BYTES);
+constexpr int OZ_SMEM = OZ_BUF + 1024;      // + alignment slack
+constexpr unsigned OZ_WAIT_LIMIT = 1u << 26;
+
+// Byte offset of element (row m, column k): core matrices are 128 B apart
+// along K (leading byte offset) and OZ_KC / 8 x 128 B along M (stride byte offset).
+constexpr uint32_t OZ_LBO = 128, OZ_SBO = OZ_KC / 8 * 128;
+__device__ __forceinline__ uint32_t oz_off(int m, int k8) {
+    return (uint32_t)((m >> 3) * OZ_SBO + k8 * OZ_LBO + (m & 7) * 16);
+}
+
+__device__ __forceinline__ uint32_t oz_smem(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
+
+__device__ __forceinline__ uint64_t oz_desc(uint32_t addr) {
+    return (uint64_t)((addr & 0x3FFFFu) >> 4) | ((uint64_t)(OZ_LBO >> 4) << 16) | ((uint64_t)(OZ_SBO >> 4) << 32) |
+           (1ull << 46);
+}
+
+// Instruction descriptor of kind::f16: D FP32 (bits 4-5 = 1), A and B FP16 (0),
+// both K-major, N >> 3 at bit 17, M >> 4 at bit 24.
+constexpr uint32_t OZ_IDESC = (1u << 4) | ((uint32_t)(OZ_N >> 3) << 17) | ((uint32_t)(OZ_M >> 4) << 24);
+
+__device__ __forceinline__ void oz_mma(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d_tmem),
+        "l"(a), "l"(b), "r"(OZ_IDESC), "r"(accumulate));
+}
+
+__device__ __forceinline__ bool oz_wait(uint32_t mbar, uint32_t parity) {
+    for (unsigned it = 0; it < OZ_WAIT_LIMIT; ++it) {
+        uint32_t done;
+        asm volatile(
+            "{\n\t.reg .pred P1;\n\t"
+            "mbarrier.try_wait.parity.shared::cta.b64 P1, [%1], %2;\n\t"
+            "selp.b32 %0, 1, 0, P1;\n\t}\n"
+            : "=r"(done)
+            : "r"(mbar), "r"(parity)
+            : "memory");
+        if (done) return true;
+    }
+    return false;
+}
+
+// 8 accumulator columns of this warp's 32 lanes (no wait).
+__device__ __forceinline__ void oz_tmem_ld8(uint32_t taddr, uint32_t r[8]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(taddr));
+}
+
+// x in fixed point, 2^62 at twice the largest power of two of its row (biased
+// exponent e of the row), with 128 added to every base-256 digit.
+__device__ __forceinline__ uint64_t oz_fixed(double x, int e) {
+    const uint64_t b = (uint64_t)__double_as_longlong(x);
+    const int ex = (int)(b >> 52) & 0x7FF;
+    int64_t m = (int64_t)((b & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull);
+    m = (b >> 63) ? -m : m;
+    const int sh = e - ex;                      // >= 0
+    int64_t q = m << 9;
+    if (sh > 0) q = sh < 63 ? (q + (1ll << (sh - 1))) >> sh : 0;   // to nearest
+    if (ex == 0) q = 0;
+    return (uint64_t)q + 0x8080808080808080ull;
+}
+
+// Digits of eight consecutive summed columns of one row: 16 bytes per digit
+// into the digit's tile at `at` (tiles `stride` bytes apart).
+__device__ __forceinline__ void oz_stage8(const uint64_t u[8], unsigned char *at, int stride) {
+    const __half2 off = __floats2half2_rn(1152.0f, 1152.0f);   // 1024 + 128
+#pragma unroll
+    for (int i = 0; i < OZ_S; ++i) {
+        const int byte = 7 - i, bsel = byte & 3;
+        uint32_t w[4];
+#pragma unroll
+        for (int h = 0; h < 4; ++h) {
+            const uint32_t a = (uint32_t)(byte >= 4 ? u[2 * h] >> 32 : u[2 * h]);
+            const uint32_t b = (uint32_t)(byte >= 4 ? u[2 * h + 1] >> 32 : u[2 * h + 1]);
+            // the digit's bytes as the low bits of 0x64xx = 1024 + byte in FP16
+            const uint32_t t = (__byte_perm(a, b, (uint32_t)(bsel | ((4 + bsel) << 8))) & 0x00FF00FFu) | 0x64006400u;
+            __half2 v;
+            memcpy(&v, &t, 4);
+            v = __hsub2(v, off);
+            memcpy(&w[h], &v, 4);
+        }
+        *reinterpret_cast<uint4 *>(at + i * stride) = make_uint4(w[0], w[1], w[2], w[3]);
+    }
+}
+
+struct OzShared {
+    int ea[OZ_M], eb[OZ_N];       // largest biased exponent of each row over the summed range
+    uint32_t tmem;
+    __align__(8) uint64_t mbar;
+    int failed;
+};
+
+// Sums over k in [k0, k1) (at most OZ_KB) of A(i, k) B(j, k) for the tile: this
+// thread's row 32 (warp % 4) + lane and columns 16 (warp / 4) + c through
+// put(c, hi, lo, x): the sum is (hi 2^32 + lo) 2^x (x OZ_NONE: zero, OZ_NOT: not
+// a number).
+// A and B return 0 out of range; before_wait() runs while the products are
+// still being formed.  Returns false if a wait gave up.
+constexpr int OZ_NONE = -100000, OZ_NOT = 100000;
+
+template <class FA, class FB, class Pre, class Put>
+__device__ bool oz_block(OzShared &S, unsigned char *sm, uint32_t &phase, FA A, FB B, int k0, int k1, Pre before_wait,
+                         Put put) {
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int ra = t & (OZ_M - 1), ha = t >> 7;      // A: two threads per row, 16 columns each
+    const int rb = t & (OZ_N - 1), hb = t >> 5;      // B: four threads per row, 8 columns each (warps 0-3)
+    if (t < OZ_M) S.ea[t] = 0;
+    if (t < OZ_N) S.eb[t] = 0;
+    __syncthreads();
+    {
+        int ma = 0, mb = 0;
+#pragma unroll 2
+        for (int kc = k0; kc < k1; kc += OZ_KC) {
+#pragma unroll
+            for (int j = 0; j < 16; ++j)
+                ma = max(ma, (int)((uint64_t)__double_as_longlong(A(ra, kc + 16 * ha + j)) >> 52) & 0x7FF);
+            if (warp < 4)
+#pragma unroll
+                for (int j = 0; j < 8; ++j)
+                    mb = max(mb, (int)((uint64_t)__double_as_longlong(B(rb, kc + 8 * hb + j)) >> 52) & 0x7FF);
+        }
+        atomicMax(&S.ea[ra], ma);
+        if (warp < 4) atomicMax(&S.eb[rb], mb);
+    }
+    __syncthreads();
+    const int ea = S.ea[ra], eb = S.eb[rb];
+    unsigned char *pa = sm, *pb = sm + OZ_S * OZ_A_BYTES;
+    for (int kc = k0; kc < k1; kc += OZ_KC) {
+        if (kc > k0) {              // until the tensor cores have read the last round's digits
+            if (!oz_wait(oz_smem(&S.mbar), phase)) S.failed = 1;
+            phase ^= 1u;
+            __syncthreads();
+            if (S.failed) break;
+        }
+#pragma unroll
+        for (int g = 0; g < 2; ++g) {
+            uint64_t u[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) u[j] = oz_fixed(A(ra, kc + 16 * ha + 8 * g + j), ea);
+            oz_stage8(u, pa + oz_off(ra, 2 * ha + g), OZ_A_BYTES);
+        }
+        if (warp < 4) {
+            uint64_t u[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) u[j] = oz_fixed(B(rb, kc + 8 * hb + j), eb);
+            oz_stage8(u, pb + oz_off(rb, hb), OZ_B_BYTES);
+        }
+        // generic-proxy stores -> visible to the tensor cores (async proxy)
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        __syncthreads();
+        if (t == 0) {
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const uint32_t a0 = oz_smem(pa), b0 = oz_smem(pb);
+#pragma unroll 1
+            for (int s = 0; s < OZ_KC / 16; ++s) {
+                const uint32_t ko = (uint32_t)(2 * s) * OZ_LBO;    // K = 16 halves = two core matrices
+#pragma unroll 1
+                for (int i = 0; i < OZ_S; ++i)
+#pragma unroll 1
+                    for (int j = 0; i + j < OZ_S; ++j)
+                        oz_mma(S.tmem + OZ_N * (i + j), oz_desc(a0 + i * OZ_A_BYTES + ko),
+                               oz_desc(b0 + j * OZ_B_BYTES + ko), kc > k0 || s > 0 || i > 0 ? 1u : 0u);
+            }
+            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                             oz_smem(&S.mbar))
+                         : "memory");
+        }
+    }
+    before_wait();
+    if (!S.failed) {
+        if (!oz_wait(oz_smem(&S.mbar), phase)) S.failed = 1;
+        phase ^= 1u;
+    }
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    __syncthreads();
+    if (S.failed) return false;
+    // a = q_a 2^(ea - 1084), ea biased by 1023; q_a q_b = 2^56 (hi 2^32 + lo), |hi|, |lo| < 2^50
+    const int er = S.ea[32 * (warp & 3) + lane];
+    const int col0 = 16 * (warp >> 2);
+    const uint32_t tm = S.tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)col0;
+#pragma unroll
+    for (int cb = 0; cb < 16; cb += 8) {
+        uint32_t r[OZ_S][8];
+#pragma unroll
+        for (int s = 0; s < OZ_S; ++s) oz_tmem_ld8(tm + OZ_N * s + cb, r[s]);
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            int64_t hi = 0, lo = 0;
+#pragma unroll
+            for (int s = 0; s < 4; ++s) {
+                hi = (hi << 8) + __float2int_rn(__uint_as_float(r[s][j]));
+                lo = (lo << 8) + __float2int_rn(__uint_as_float(r[s + 4][j]));
+            }
+            const int ec = S.eb[col0 + cb + j];
+            const int x = er == 0x7FF || ec == 0x7FF ? OZ_NOT : (er == 0 || ec == 0 ? OZ_NONE : er + ec - 2112);
+            put(cb + j, hi, lo, x);
+        }
+    }
+    // the next block's products overwrite the accumulators
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    return true;
+}
+
+// 2^x as oz_block gives it: 0 below the normal numbers, NaN for OZ_NOT.
+__device__ __forceinline__ double oz_pow2(int x) {
+    if (x >= OZ_NOT) return __longlong_as_double(0x7FF8000000000000ll);
+    return x > -1023 ? __longlong_as_double((int64_t)(min(x, 1023) + 1023) << 52) : 0.0;
+}
+
+__device__ __forceinline__ unsigned char *oz_begin(OzShared &S, unsigned char *raw) {
+    if (threadIdx.x < 32) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(oz_smem(&S.tmem)),
+                     "r"(OZ_TMEM_COLS));
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+    }
+    if (threadIdx.x == 0) {
+        S.failed = 0;
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(oz_smem(&S.mbar)), "r"(1));
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    return reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(raw) + 1023) & ~static_cast<uintptr_t>(1023));
+}
+
+__device__ __forceinline__ void oz_end(OzShared &S, bool ok, int *err) {
+    if (!ok && threadIdx.x == 0) atomicExch(err, 2);
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(S.tmem), "r"(OZ_TMEM_COLS));
+    }
+}
+
+// F[r, c] -= sum over the kw = min(panel, p - k0) columns k from k0 of
+// F[r, k] F[c, k], k0 + kw <= c <= r < f: one CTA per (front, tile that meets
+// the lower triangle).
+__global__ void __launch_bounds__(OZ_THREADS, 2) k_syrk64_tc(const int *__restrict__ fronts,
+                                                             const FrontDesc *__restrict__ D, double *ws, int k0,
+                                                             int panel, int *__restrict__ err) {
+    const FrontDesc &d = D[fronts[blockIdx.x]];
+    const int p = d.p, f = d.p + d.q;
+    if (k0 >= p) return;
+    const int base = min(k0 + panel, p), m = f - base;
+    constexpr int R = OZ_M / OZ_N;                            // tile columns per tile row: R (ti + 1) in row ti
+    const int t = blockIdx.y;
+    int ti = (int)((sqrtf(8.0f / R * t + 1.0f) - 1.0f) * 0.5f);
+    while (R * (ti + 1) * (ti + 2) / 2 <= t) ++ti;
+    while (R * ti * (ti + 1) / 2 > t) --ti;
+    const int tj = t - R * ti * (ti + 1) / 2;
+    if (ti * OZ_M >= m || tj * OZ_N >= m) return;
+    const int r0 = base + ti * OZ_M, c0 = base + tj * OZ_N;
+    double *F = ws + d.front_off;
+    extern __shared__ unsigned char oz_raw[];
+    __shared__ OzShared S;
+    unsigned char *sm = oz_begin(S, oz_raw);
+    uint32_t phase = 0u;
+    const int r = r0 + 32 * ((threadIdx.x >> 5) & 3) + (threadIdx.x & 31), cw = c0 + 16 * (threadIdx.x >> 7);
+    double e[16];   // the thread's entries of F, loaded while the products are formed
+    const bool ok = oz_block(
+        S, sm, phase, [&](int i, int k) { return r0 + i < f && k < base ? F[r0 + i + (int64_t)k * f] : 0.0; },
+        [&](int i, int k) { return c0 + i < f && k < base ? F[c0 + i + (int64_t)k * f] : 0.0; }, k0, base,
+        [&]() {
+#pragma unroll
+            for (int c = 0; c < 16; ++c) e[c] = r < f && cw + c <= r ? F[r + (int64_t)(cw + c) * f] : 0.0;
+        },
+        [&](int c, int64_t hi, int64_t lo, int x) {
+            if (r < f && cw + c <= r)
+                F[r + (int64_t)(cw + c) * f] = fma((double)hi, -oz_pow2(x + 32), fma((double)lo, -oz_pow2(x), e[c]));
+        });
+    oz_end(S, ok, err);
+}
+
+// W = L21 L11^{-1}: rows p .. f of the panel, from L21 in the front and the
+// inverse in the panel's pivot rows; tile column c0 needs the pivots from c0 on.
+__global__ void __launch_bounds__(OZ_THREADS, 2) k_wpanel_tc(const int *__restrict__ fronts,
+                                                             const FrontDesc *__restrict__ D, const double *ws,
+                                                             double *out, int *__restrict__ err) {
+    const FrontDesc &d = D[fronts[blockIdx.x]];
+    const int p = d.p, f = d.p + d.q;
+    const int ntr = (d.q + OZ_M - 1) / OZ_M;
+    if (ntr == 0) return;
+    const int ti = blockIdx.y % ntr, tj = blockIdx.y / ntr;
+    const int r0 = p + ti * OZ_M, c0 = tj * OZ_N;
+    if (c0 >= p) return;
+    const double *F = ws + d.front_off;
+    double *O = out + d.l_off;
+    extern __shared__ unsigned char oz_raw[];
+    __shared__ OzShared S;
+    unsigned char *sm = oz_begin(S, oz_raw);
+    uint32_t phase = 0u;
+    const int r = r0 + 32 * ((threadIdx.x >> 5) & 3) + (threadIdx.x & 31), cw = c0 + 16 * (threadIdx.x >> 7);
+    double acc[16];
+#pragma unroll
+    for (int j = 0; j < 16; ++j) acc[j] = 0.0;
+    bool ok = true;
+    for (int kb = c0; kb < p && ok; kb += OZ_KB) {
+        const int ke = min(p, kb + OZ_KB);
+        ok = oz_block(
+            S, sm, phase, [&](int i, int k) { return r0 + i < f && k < ke ? F[r0 + i + (int64_t)k * f] : 0.0; },
+            [&](int i, int k) { return c0 + i < p && k < ke ? O[k + (int64_t)(c0 + i) * f] : 0.0; }, kb, ke, []() {},
+            [&](int c, int64_t hi, int64_t lo, int x) {
+                acc[c] = fma((double)hi, oz_pow2(x + 32), fma((double)lo, oz_pow2(x), acc[c]));
+            });
+    }
+    if (ok && r < f) {
+#pragma unroll
+        for (int j = 0; j < 16; ++j)
+            if (cw + j < p) O[r + (int64_t)(cw + j) * f] = acc[j];
+    }
+    oz_end(S, ok, err);
+}
+
+void oz_smem_limit() {
+    static SmemLimit lim;
+    lim.ensure(OZ_SMEM, [](size_t v) {
+        GL_CUDA(cudaFuncSetAttribute(k_syrk64_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)v));
+        GL_CUDA(cudaFuncSetAttribute(k_wpanel_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)v));
+    });
+}
+
+}  // namespace
+
+void syrk64_tc_level(const int *d_fronts, int n_fronts, const FrontDesc *d_fr, int k0, int panel, int max_f, double *ws,
+                     int *d_err, cudaStream_t s) {
+    oz_smem_limit();
+    const int m = max_f - k0;   // upper bound of the trailing size over the level's fronts
+    if (m <= 0) return;
+    const int nt = (m + OZ_M - 1) / OZ_M;
+    k_syrk64_tc<<<dim3(n_fronts, OZ_M / OZ_N * nt * (nt + 1) / 2), OZ_THREADS, OZ_SMEM, s>>>(d_fronts, d_fr, ws, k0, panel, d_err);
+    GL_CUDA(cudaGetLastError());
+}
+
+void wpanel_tc_level(const int *d_fronts, int n_fronts, const FrontDesc *d_fr, int max_p, int max_f, const double *ws,
+                     double *out, int *d_err, cudaStream_t s) {
+    oz_smem_limit();
+    const int tiles = ((max_f + OZ_M - 1) / OZ_M) * ((max_p + OZ_N - 1) / OZ_N);
+    if (tiles <= 0) return;
+    k_wpanel_tc<<<dim3(n_fronts, tiles), OZ_THREADS, OZ_SMEM, s>>>(d_fronts, d_fr, ws, out, d_err);
+    GL_CUDA(cudaGetLastError());
+}
+
+}  // namespace gl
