@@ -195,17 +195,38 @@ __device__ __forceinline__ void jacobi_pair(int m, int t, int i, int &p, int &q)
     q = max(a, b);
 }
 
-// Eigenvectors of the symmetric k x k matrix C by cyclic Jacobi: on return the
-// diagonal of C holds the eigenvalues and the columns of Q the vectors.  All
-// threads of the CTA take part; cs holds 2 doubles per pair, red one per warp + 1.
-__device__ void cta_jacobi(double *C, double *Q, int ld, int k, double *cs, double *red) {
+// Rotation (c, s) that annihilates apq between the diagonal entries app and
+// aqq.  Only the angle may be rough (it leaves its error times apq, which the
+// next sweep takes), so it is computed in FP32; c^2 + s^2 = 1 holds to T.
+template <class T>
+__device__ __forceinline__ void jacobi_rotation(T app, T aqq, T apq, T &c, T &s) {
+    const float b = (float)apq;
+    if (b == 0.0f) {
+        c = T(1);
+        s = T(0);
+        return;
+    }
+    const float tau = (float)(aqq - app) / (2.0f * b);
+    const T t = (T)(copysignf(1.0f, tau) / (fabsf(tau) + sqrtf(1.0f + tau * tau)));
+    c = rsqrt(T(1) + t * t);
+    s = t * c;
+}
+
+// Eigenvectors of the symmetric k x k matrix C by cyclic Jacobi, until the
+// squares of the off-diagonal entries sum to at most tol of all: on return the
+// diagonal of C holds the eigenvalues and Q the vectors as columns (times what
+// it held, unless init).  All threads of the CTA take part; cs holds 2 numbers
+// and pairs one per pair, red two per warp.
+template <class T>
+__device__ void cta_jacobi(T *C, T *Q, int ld, int k, T *cs, int *pairs, T *red, T tol, bool init) {
     const int m = k + (k & 1), np = m / 2, nt = blockDim.x, tid = threadIdx.x;
-    for (int idx = tid; idx < k * k; idx += nt) Q[(idx / k) * ld + idx % k] = idx / k == idx % k ? 1.0 : 0.0;
+    if (init)
+        for (int idx = tid; idx < k * k; idx += nt) Q[(idx / k) * ld + idx % k] = idx / k == idx % k ? T(1) : T(0);
     __syncthreads();
     for (int sweep = 0; sweep < 60; ++sweep) {
-        double off = 0.0, tot = 0.0;
+        T off = T(0), tot = T(0);
         for (int idx = tid; idx < k * k; idx += nt) {
-            const double v = C[(idx / k) * ld + idx % k];
+            const T v = C[(idx / k) * ld + idx % k];
             tot += v * v;
             if (idx / k != idx % k) off += v * v;
         }
@@ -218,67 +239,133 @@ __device__ void cta_jacobi(double *C, double *Q, int ld, int k, double *cs, doub
             red[2 * (tid >> 5) + 1] = tot;
         }
         __syncthreads();
-        off = tot = 0.0;
+        off = tot = T(0);
         for (int w = 0; w < nt / 32; ++w) {
             off += red[2 * w];
             tot += red[2 * w + 1];
         }
         __syncthreads();
-        if (!(off > 1e-30 * tot)) break;   // uniform: every thread adds the same numbers
+        if (!(off > tol * tot)) break;   // uniform: every thread adds the same numbers
         for (int t = 0; t < m - 1; ++t) {
-            if (tid < np) {
+            for (int i = tid; i < np; i += nt) {
                 int p, q;
-                jacobi_pair(m, t, tid, p, q);
-                double c = 1.0, sn = 0.0;
-                if (q < k) {
-                    const double apq = C[p * ld + q];
-                    if (!(fabs(apq) < 1e-300)) {
-                        const double tau = (C[q * ld + q] - C[p * ld + p]) / (2.0 * apq);
-                        const double tt = (tau >= 0 ? 1.0 : -1.0) / (fabs(tau) + sqrt(1.0 + tau * tau));
-                        c = 1.0 / sqrt(1.0 + tt * tt);
-                        sn = tt * c;
-                    }
-                }
-                cs[2 * tid] = c;
-                cs[2 * tid + 1] = sn;
+                jacobi_pair(m, t, i, p, q);
+                T c = T(1), sn = T(0);
+                if (q < k) jacobi_rotation(C[p * ld + p], C[q * ld + q], C[p * ld + q], c, sn);
+                cs[2 * i] = c;
+                cs[2 * i + 1] = sn;
+                pairs[i] = p | (q << 16);
             }
             __syncthreads();
-            for (int idx = tid; idx < np * np; idx += nt) {
-                const int i = idx / np, j = idx % np;
-                int p, q, u, v;
-                jacobi_pair(m, t, i, p, q);
-                jacobi_pair(m, t, j, u, v);
-                const double ci = cs[2 * i], si = cs[2 * i + 1], cj = cs[2 * j], sj = cs[2 * j + 1];
-                if (q < k && v < k) {
-                    const double a = C[p * ld + u], b = C[p * ld + v], c = C[q * ld + u], d = C[q * ld + v];
-                    const double a1 = cj * a - sj * b, b1 = sj * a + cj * b;
-                    const double c1 = cj * c - sj * d, d1 = sj * c + cj * d;
-                    C[p * ld + u] = ci * a1 - si * c1;
-                    C[p * ld + v] = ci * b1 - si * d1;
-                    C[q * ld + u] = si * a1 + ci * c1;
-                    C[q * ld + v] = si * b1 + ci * d1;
-                } else if (q < k) {   // odd k: the player without a partner (u) is not rotated
-                    const double a = C[p * ld + u], c = C[q * ld + u];
-                    C[p * ld + u] = ci * a - si * c;
-                    C[q * ld + u] = si * a + ci * c;
-                } else if (v < k) {
-                    const double a = C[p * ld + u], b = C[p * ld + v];
-                    C[p * ld + u] = cj * a - sj * b;
-                    C[p * ld + v] = sj * a + cj * b;
+            // a warp per pair of rows (C) or row (Q), a lane per pair of columns
+            for (int j = tid & 31; j < np; j += 32) {
+                const int u = pairs[j] & 0xFFFF, v = pairs[j] >> 16;
+                const T cj = cs[2 * j], sj = cs[2 * j + 1];
+                for (int i = tid >> 5; i < np; i += nt >> 5) {
+                    const int p = pairs[i] & 0xFFFF, q = pairs[i] >> 16;
+                    const T ci = cs[2 * i], si = cs[2 * i + 1];
+                    if (q < k && v < k) {
+                        const T a = C[p * ld + u], b = C[p * ld + v], c = C[q * ld + u], d = C[q * ld + v];
+                        const T a1 = cj * a - sj * b, b1 = sj * a + cj * b;
+                        const T c1 = cj * c - sj * d, d1 = sj * c + cj * d;
+                        C[p * ld + u] = ci * a1 - si * c1;
+                        C[p * ld + v] = ci * b1 - si * d1;
+                        C[q * ld + u] = si * a1 + ci * c1;
+                        C[q * ld + v] = si * b1 + ci * d1;
+                    } else if (q < k) {   // odd k: the player without a partner (u) is not rotated
+                        const T a = C[p * ld + u], c = C[q * ld + u];
+                        C[p * ld + u] = ci * a - si * c;
+                        C[q * ld + u] = si * a + ci * c;
+                    } else if (v < k) {
+                        const T a = C[p * ld + u], b = C[p * ld + v];
+                        C[p * ld + u] = cj * a - sj * b;
+                        C[p * ld + v] = sj * a + cj * b;
+                    }
                 }
-            }
-            for (int idx = tid; idx < k * np; idx += nt) {
-                const int r = idx / np, j = idx % np;
-                int u, v;
-                jacobi_pair(m, t, j, u, v);
-                if (v >= k) continue;
-                const double cj = cs[2 * j], sj = cs[2 * j + 1], a = Q[r * ld + u], b = Q[r * ld + v];
-                Q[r * ld + u] = cj * a - sj * b;
-                Q[r * ld + v] = sj * a + cj * b;
+                if (v < k)
+                    for (int r = tid >> 5; r < k; r += nt >> 5) {
+                        const T a = Q[r * ld + u], b = Q[r * ld + v];
+                        Q[r * ld + u] = cj * a - sj * b;
+                        Q[r * ld + v] = sj * a + cj * b;
+                    }
             }
             __syncthreads();
         }
     }
+    __syncthreads();
+}
+
+// out = A^T B (at) or A B, m x m, leading dimension ld.
+__device__ void cta_product(const double *A, const double *B, double *out, int ld, int m, bool at) {
+    for (int idx = threadIdx.x; idx < m * m; idx += blockDim.x) {
+        const int i = idx / m, j = idx % m;
+        double v = 0.0;
+        if (at)
+            for (int k = 0; k < m; ++k) v += A[k * ld + i] * B[k * ld + j];
+        else
+            for (int k = 0; k < m; ++k) v += A[i * ld + k] * B[k * ld + j];
+        out[i * ld + j] = v;
+    }
+    __syncthreads();
+}
+
+// Eigenpairs of the symmetric m x m matrix C in FP64: Jacobi in FP32 first,
+// whose vectors, made orthonormal to FP64 rounding by two Newton-Schulz steps
+// Q (3 - Q^T Q) / 2, leave C nearly diagonal, so that the FP64 sweeps (each
+// some 6 m^3 FMAs at two per clock) are two or three instead of about nine.
+// tmp: m x ld doubles.
+__device__ void cta_eig(double *C, double *Q, double *tmp, int ld, int m, double *cs, int *pairs, double *red) {
+    const int nt = blockDim.x, tid = threadIdx.x;
+    float *Cf = reinterpret_cast<float *>(tmp), *Qf = Cf + m * ld;
+    // C scaled by a power of two to FP32's range
+    double big = 0.0;
+    for (int idx = tid; idx < m * m; idx += nt) big = fmax(big, fabs(C[(idx / m) * ld + idx % m]));
+    for (int o = 16; o > 0; o >>= 1) big = fmax(big, __shfl_xor_sync(0xffffffffu, big, o));
+    if ((tid & 31) == 0) red[tid >> 5] = big;
+    __syncthreads();
+    big = 0.0;
+    for (int w = 0; w < nt / 32; ++w) big = fmax(big, red[w]);
+    __syncthreads();
+    const int e = big > 0.0 && big < INFINITY ? -ilogb(big) : 0;
+    for (int idx = tid; idx < m * m; idx += nt) {
+        const int at = (idx / m) * ld + idx % m;
+        C[at] = scalbn(C[at], e);
+        Cf[at] = (float)C[at];
+    }
+    __syncthreads();
+    cta_jacobi<float>(Cf, Qf, ld, m, reinterpret_cast<float *>(cs), pairs, reinterpret_cast<float *>(red), 1e-11f,
+                      true);
+    for (int idx = tid; idx < m * m; idx += nt) {
+        const int at = (idx / m) * ld + idx % m;
+        Q[at] = (double)Qf[at];
+    }
+    __syncthreads();
+    for (int step = 0; step < 2; ++step) {
+        cta_product(Q, Q, tmp, ld, m, true);
+        // Q <- Q (3 I - tmp) / 2, nt / m rows at a time
+        const int rows = max(1, nt / m);
+        for (int r0 = 0; r0 < m; r0 += rows) {
+            const int i = r0 + tid / m, j = tid % m;
+            const bool on = tid < rows * m && i < m;
+            double v = 0.0;
+            if (on) {
+                for (int k = 0; k < m; ++k) v -= Q[i * ld + k] * tmp[k * ld + j];
+                v = 0.5 * (3.0 * Q[i * ld + j] + v);
+            }
+            __syncthreads();
+            if (on) Q[i * ld + j] = v;
+            __syncthreads();
+        }
+    }
+    cta_product(C, Q, tmp, ld, m, false);
+    cta_product(Q, tmp, C, ld, m, true);
+    for (int idx = tid; idx < m * m; idx += nt) {
+        const int i = idx / m, j = idx % m;
+        if (i < j) C[i * ld + j] = C[j * ld + i] = 0.5 * (C[i * ld + j] + C[j * ld + i]);
+    }
+    __syncthreads();
+    cta_jacobi<double>(C, Q, ld, m, cs, pairs, red, 1e-30, false);
+    for (int i = tid; i < m; i += nt) C[i * ld + i] = scalbn(C[i * ld + i], -e);
     __syncthreads();
 }
 
@@ -291,6 +378,7 @@ __global__ void __launch_bounds__(64) k_kry_orth(const double *__restrict__ G, c
                                                  int *__restrict__ err) {
     constexpr int ld = KRY_B + 1;
     __shared__ double C[KRY_B * ld], Q[KRY_B * ld], cs[KRY_B], red[4], sh;
+    __shared__ int pairs[KRY_B / 2];
     const int s = blockIdx.x, tid = threadIdx.x;
     if (tid == 0) sh = 0.0;
     for (int idx = tid; idx < KRY_B * KRY_B; idx += 64) {
@@ -308,10 +396,17 @@ __global__ void __launch_bounds__(64) k_kry_orth(const double *__restrict__ G, c
     atomicAdd(&sh, lost);
     __syncthreads();
     const double floor_ = drop * sh;
-    cta_jacobi(C, Q, ld, KRY_B, cs, red);
+    // scaled by a power of two to the range of the rotations' FP32 angles
+    double big = 0.0;
+    for (int idx = 0; idx < KRY_B * KRY_B; ++idx) big = fmax(big, fabs(C[(idx / KRY_B) * ld + idx % KRY_B]));
+    const int e = big > 0.0 && big < INFINITY ? -ilogb(big) : 0;
+    __syncthreads();
+    C[(tid / KRY_B) * ld + tid % KRY_B] = scalbn(C[(tid / KRY_B) * ld + tid % KRY_B], e);   // 64 threads, 64 entries
+    __syncthreads();
+    cta_jacobi<double>(C, Q, ld, KRY_B, cs, pairs, red, 1e-30, true);
     for (int idx = tid; idx < KRY_B * KRY_B; idx += 64) {
         const int j = idx % KRY_B;
-        const double lam = C[j * ld + j];
+        const double lam = scalbn(C[j * ld + j], -e);
         if (!(fabs(lam) < INFINITY)) atomicExch(err, 1);
         R[(int64_t)s * KRY_B * KRY_B + idx] = lam > floor_ && lam > 0.0 ? Q[(idx / KRY_B) * ld + j] / sqrt(lam) : 0.0;
     }
@@ -334,7 +429,7 @@ __global__ void __launch_bounds__(GENEIG_THREADS) k_kry_ritz(const double *__res
                                                              unsigned long long *__restrict__ worst) {
     extern __shared__ double sm[];
     const int ld = m + 1, s = blockIdx.x, tid = threadIdx.x, nt = blockDim.x;
-    double *C = sm, *Q = C + m * ld, *cs = Q + m * ld, *red = cs + m + 2;
+    double *C = sm, *Q = C + m * ld, *tmp = Q + m * ld, *cs = tmp + m * ld, *red = cs + m + 2;
     __shared__ int rank[KRY_MAX];
     const double *Ts = T + (int64_t)s * ldt * ldt;
     for (int idx = tid; idx < m * m; idx += nt) {
@@ -342,7 +437,7 @@ __global__ void __launch_bounds__(GENEIG_THREADS) k_kry_ritz(const double *__res
         C[i * ld + j] = Ts[(int64_t)min(i, j) * ldt + max(i, j)];
     }
     __syncthreads();
-    cta_jacobi(C, Q, ld, m, cs, red);
+    cta_eig(C, Q, tmp, ld, m, cs, rank, red);   // rank is free until the pairs are known
     for (int a = tid; a < m; a += nt) {
         const double me = C[a * ld + a];
         int r = 0;
@@ -374,7 +469,7 @@ __global__ void __launch_bounds__(GENEIG_THREADS) k_kry_ritz(const double *__res
     }
 }
 
-static size_t ritz_smem(int m) { return sizeof(double) * ((size_t)2 * m * (m + 1) + m + 2 + 2 * (GENEIG_THREADS / 32)); }
+static size_t ritz_smem(int m) { return sizeof(double) * ((size_t)3 * m * (m + 1) + m + 2 + 2 * (GENEIG_THREADS / 32)); }
 
 void kry_ritz(int n_sub, const double *T, int ldt, int m, const double *G, int nev, int keep, double *Y, int ldy,
               double *mu, unsigned long long *worst, cudaStream_t s) {

@@ -268,7 +268,7 @@ void problem_coarse(const Problem &P, const gl_opts &o, const FactorPlan &PD, in
         };
         fill_random(W.p, gl * KRY_B, 0x1707042280000001ull + (uint64_t)j0, s);
         apply_B();
-        int it = 0, m = 0, kept = 0;
+        int it = 0, m = 0, kept = 0, next_check = 0;
         double resid = 0.0;
         for (;;) {
             // the last block's columns of T; W = M^{-1} B W_last (MW holds the sweeps' right-hand side)
@@ -283,14 +283,18 @@ void problem_coarse(const Problem &P, const gl_opts &o, const FactorPlan &PD, in
             kry_gram(PG, MV.p, mmax, m, W.p, H.p, hs, KRY_B, s);
             kry_project(PG, first, mmax, m, H.p, hs, KRY_B, s);
             gram_block(BW.p);
-            if (m >= nev + KRY_B / 2 || (m >= nev && it > iters)) {
+            // The Ritz pairs when they are needed: to restart, at the end, and as soon as the residuals can have got
+            // there -- they fall by less than 30 a step (3 to 10 as a rule).
+            const bool last = it > iters && m >= nev;
+            if (last || (m >= nev && m + KRY_B > mmax) || (m >= nev + KRY_B / 2 && it >= next_check)) {
                 kept = std::min(keep, m);
                 kry_ritz(ng, T.p, mmax, m, G.p, nev, kept, Y.p, keep, mu.p, worst.p, s);
                 unsigned long long bits = 0;
                 GL_CUDA(cudaMemcpyAsync(&bits, worst.p, sizeof(bits), cudaMemcpyDeviceToHost, s));
                 check_err(P, "GenEO Rayleigh-Ritz");
                 std::memcpy(&resid, &bits, sizeof(resid));
-                if (resid <= EIG_RESID || it > iters) break;
+                if (resid <= EIG_RESID || last) break;
+                next_check = it + 1 + std::max(0, std::min(8, (int)(std::log(resid / EIG_RESID) / std::log(30.0))));
             }
             kry_orth(ng, G.p, H.p, hs, KRY_B, m, 1e-24, R.p, P.d_err, s);
             kry_scale(PG, only_w, R.p, mmax, -1, s);
