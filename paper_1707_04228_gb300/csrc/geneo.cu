@@ -592,8 +592,6 @@ void coarse_prolong(const FactorPlan &P, const double *Z, int m, const double *y
 
 // ---------------------------------------------------------------- PCG vector kernels
 
-constexpr int RED_BLOCKS = 1024;
-
 __device__ __forceinline__ double block_sum(double v) {
     __shared__ double red[32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -609,62 +607,101 @@ __device__ __forceinline__ double block_sum(double v) {
     return t;
 }
 
-__global__ void __launch_bounds__(256) k_dot_partial(const double *__restrict__ a, const double *__restrict__ b, int64_t n,
-                                                     double *__restrict__ partials) {
-    double v = 0.0;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        v += a[i] * b[i];
+// Blocks of a reduction over n entries: four a thread at least.  (1,024 blocks
+// whatever n took 8.7 us on 20k entries, most of it their 8,192 divisions.)
+static int red_blocks(int64_t n) { return (int)std::min<int64_t>(RED_BLOCKS, std::max<int64_t>(1, (n + 1023) / 1024)); }
+
+// Sum over the grid of the blocks' v: the block that finishes last adds the
+// partial sums in block order and returns true with the total in its thread 0
+// -- a second launch for it cost 3 us and a gap.
+__device__ __forceinline__ bool grid_sum(double v, double *partials, double &total) {
+    __shared__ bool last;
+    unsigned int *done = reinterpret_cast<unsigned int *>(partials + RED_BLOCKS);
     v = block_sum(v);
-    if (threadIdx.x == 0) partials[blockIdx.x] = v;
+    if (threadIdx.x == 0) {
+        partials[blockIdx.x] = v;
+        __threadfence();
+        last = atomicAdd(done, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!last) return false;
+    __threadfence();
+    double t = 0.0;
+    for (int i = threadIdx.x; i < gridDim.x; i += blockDim.x) t += __ldcg(partials + i);
+    total = block_sum(t);
+    if (threadIdx.x == 0) *done = 0u;
+    return true;
 }
 
-__global__ void __launch_bounds__(1024) k_reduce_final(const double *__restrict__ partials, int n, double *__restrict__ out) {
-    double v = 0.0;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) v += partials[i];
-    v = block_sum(v);
-    if (threadIdx.x == 0) *out = v;
+__global__ void __launch_bounds__(256) k_dot(const double *__restrict__ a, const double *__restrict__ b, int64_t n,
+                                             double *partials, double *__restrict__ out) {
+    double v = 0.0, t;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+        v += a[i] * b[i];
+    if (grid_sum(v, partials, t) && threadIdx.x == 0) *out = t;
 }
 
 void dot(const double *a, const double *b, int64_t n, double *partials, double *out, cudaStream_t s) {
-    k_dot_partial<<<RED_BLOCKS, 256, 0, s>>>(a, b, n, partials);
-    k_reduce_final<<<1, 1024, 0, s>>>(partials, RED_BLOCKS, out);
+    k_dot<<<red_blocks(n), 256, 0, s>>>(a, b, n, partials, out);
     GL_CUDA(cudaGetLastError());
 }
 
 __global__ void __launch_bounds__(256) k_update_xr(double *__restrict__ x, double *__restrict__ r,
-                                                   const double *__restrict__ p, const double *__restrict__ q, int64_t n,
-                                                   CGScalars *__restrict__ S, double *__restrict__ partials) {
-    const double alpha = S->rho / S->pq;
-    double v = 0.0;
+                                                   const double *__restrict__ p, const double *__restrict__ q,
+                                                   const uint8_t *__restrict__ mask, double *__restrict__ z, int64_t n,
+                                                   CGScalars *__restrict__ S, double *partials) {
+    __shared__ double sa;
+    if (threadIdx.x == 0) sa = S->rho / S->pq;
+    __syncthreads();
+    const double alpha = sa;
+    double v = 0.0, t;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         x[i] += alpha * p[i];
-        double ri = r[i] - alpha * q[i];
+        const double ri = mask[i] ? 0.0 : r[i] - alpha * q[i];
         r[i] = ri;
+        if (z) z[i] = 0.0;
         v += ri * ri;
     }
-    v = block_sum(v);
-    if (threadIdx.x == 0) partials[blockIdx.x] = v;
-    if (blockIdx.x == 0 && threadIdx.x == 0) S->alpha = alpha;
+    if (grid_sum(v, partials, t) && threadIdx.x == 0) {
+        S->rr = t;
+        S->alpha = alpha;
+    }
 }
 
-void cg_update_xr(double *x, double *r, const double *p, const double *q, int64_t n, CGScalars *S, double *partials,
-                  cudaStream_t s) {
-    k_update_xr<<<RED_BLOCKS, 256, 0, s>>>(x, r, p, q, n, S, partials);
-    k_reduce_final<<<1, 1024, 0, s>>>(partials, RED_BLOCKS, &S->rr);
+void cg_update_xr(double *x, double *r, const double *p, const double *q, const uint8_t *mask, double *z, int64_t n,
+                  CGScalars *S, double *partials, cudaStream_t s) {
+    k_update_xr<<<red_blocks(n), 256, 0, s>>>(x, r, p, q, mask, z, n, S, partials);
     GL_CUDA(cudaGetLastError());
 }
 
-// beta = (rho_new - rz_old) / rho  (rz_old = 0 gives the standard recurrence)
-__global__ void __launch_bounds__(256) k_update_p(double *__restrict__ p, const double *__restrict__ z, int64_t n,
-                                                  CGScalars *__restrict__ S) {
-    const double beta = (S->rho_new - S->rz_old) / S->rho;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+// beta = (rho_new - rz_old) / rho  (rz_old = 0 gives the standard recurrence);
+// the block that finishes last moves rho on
+__global__ void __launch_bounds__(256) k_update_p(double *__restrict__ p, const double *__restrict__ z,
+                                                  double *__restrict__ q, int64_t n, CGScalars *S, double *partials) {
+    __shared__ double sb;
+    __shared__ bool last;
+    if (threadIdx.x == 0) sb = (S->rho_new - S->rz_old) / S->rho;
+    __syncthreads();
+    const double beta = sb;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         p[i] = z[i] + beta * p[i];
+        q[i] = 0.0;
+    }
+    if (threadIdx.x == 0) {
+        unsigned int *done = reinterpret_cast<unsigned int *>(partials + RED_BLOCKS);
+        __threadfence();
+        last = atomicAdd(done, 1u) == gridDim.x - 1;
+        if (last) {
+            S->beta = beta;
+            S->rho = S->rho_new;
+            *done = 0u;
+        }
+    }
 }
 
-__global__ void k_finish_p(CGScalars *S) {
-    S->beta = (S->rho_new - S->rz_old) / S->rho;
-    S->rho = S->rho_new;
+void cg_update_p(double *p, const double *z, double *q, int64_t n, CGScalars *S, double *partials, cudaStream_t s) {
+    k_update_p<<<red_blocks(n), 256, 0, s>>>(p, z, q, n, S, partials);
+    GL_CUDA(cudaGetLastError());
 }
 
 // ---- per-part (segmented) versions for many laminates solved together
@@ -779,12 +816,6 @@ __global__ void k_seg_confirm(SegScalars S, int n, double tol2, int max_iter, in
 void seg_confirm(SegScalars S, int n, double tol, int max_iter, int *n_active, cudaStream_t s) {
     GL_CUDA(cudaMemsetAsync(n_active, 0, sizeof(int), s));
     k_seg_confirm<<<(n + 127) / 128, 128, 0, s>>>(S, n, tol * tol, max_iter, n_active);
-    GL_CUDA(cudaGetLastError());
-}
-
-void cg_update_p(double *p, const double *z, int64_t n, CGScalars *S, cudaStream_t s) {
-    k_update_p<<<RED_BLOCKS, 256, 0, s>>>(p, z, n, S);
-    k_finish_p<<<1, 1, 0, s>>>(S);
     GL_CUDA(cudaGetLastError());
 }
 

@@ -97,14 +97,18 @@ void seg_confirm(SegScalars S, int n, double tol, int max_iter, int *n_active, c
 struct CGScalars {
     double rho, rho_new, pq, rr, rz_old, alpha, beta, ff;
 };
+// Partial sums of a reduction, one per block, and the count of blocks done
+// (zero between launches: the last block of each resets it).
+constexpr int RED_BLOCKS = 1024, RED_SCRATCH = RED_BLOCKS + 1;
 
-// out = sum a_i b_i (deterministic two-stage reduction) written to *out (device).
+// out = sum a_i b_i written to *out (device); the order of the sum depends on n only.
+// partials: RED_SCRATCH entries, the last one zero.
 void dot(const double *a, const double *b, int64_t n, double *partials, double *out, cudaStream_t s);
-// x += alpha p; r -= alpha q, alpha = S->rho / S->pq; partial sums of r.r -> S->rr
-void cg_update_xr(double *x, double *r, const double *p, const double *q, int64_t n, CGScalars *S,
-                  double *partials, cudaStream_t s);
-// beta = rho_new / rho (or flexible), p = z + beta p, rho = rho_new
-void cg_update_p(double *p, const double *z, int64_t n, CGScalars *S, cudaStream_t s);
+// x += alpha p; r -= alpha q (0 where mask), alpha = S->rho / S->pq; r.r -> S->rr; z = 0 unless z is NULL
+void cg_update_xr(double *x, double *r, const double *p, const double *q, const uint8_t *mask, double *z, int64_t n,
+                  CGScalars *S, double *partials, cudaStream_t s);
+// beta = rho_new / rho (or flexible), p = z + beta p, q = 0, rho = rho_new
+void cg_update_p(double *p, const double *z, double *q, int64_t n, CGScalars *S, double *partials, cudaStream_t s);
 // y[dof[i]] = val (val = 0 or from array)
 void set_entries(double *y, const int64_t *dof, int64_t n, const double *vals, cudaStream_t s);
 // y = a - b

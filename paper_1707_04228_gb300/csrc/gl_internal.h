@@ -157,8 +157,9 @@ void launch_elem_material(int64_t n_elem, int nx, int ny, const int *layer_of_ez
 void launch_elem_geometry(const MeshHost &m, const double *X, double *geo, cudaStream_t s);
 void launch_traction(const MeshHost &m, const double *X, int face, const double t[3], double *f,
                      cudaStream_t s);
+// y = K x (zeroed: y is zero already)
 void launch_ku(const MeshHost &m, const double *C, const double *geo, const double *x, double *y,
-               cudaStream_t s);
+               cudaStream_t s, bool zeroed = false);
 void launch_stress(const MeshHost &m, const double *X, const double *C, const double *psi,
                    const double *u, double *s33, double *t13, cudaStream_t s);
 // Failure index; peak[0] = the (F, element) key's bits (element in the low 24), peak[1] = the largest F.

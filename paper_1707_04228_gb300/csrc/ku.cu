@@ -191,8 +191,9 @@ __global__ void __launch_bounds__(32 * KU_EPB) k_ku(int64_t n_elem, int nx, int 
     }
 }
 
-void launch_ku(const MeshHost &m, const double *C, const double *geo, const double *x, double *y, cudaStream_t s) {
-    GL_CUDA(cudaMemsetAsync(y, 0, m.n_dof * sizeof(double), s));
+void launch_ku(const MeshHost &m, const double *C, const double *geo, const double *x, double *y, cudaStream_t s,
+               bool zeroed) {
+    if (!zeroed) GL_CUDA(cudaMemsetAsync(y, 0, m.n_dof * sizeof(double), s));
     int64_t nb = (m.n_elem + KU_EPB - 1) / KU_EPB;
     k_ku<<<(unsigned)nb, 32 * KU_EPB, 0, s>>>(m.n_elem, m.nx, m.ny, m.NX, m.NY, C, geo, x, y);
     GL_CUDA(cudaGetLastError());

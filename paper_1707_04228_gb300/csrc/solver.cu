@@ -112,7 +112,7 @@ struct gl_ctx {
     // device mesh data
     DBuf<double> d_tn, d_ln, d_rn, d_dr, d_X, d_C, d_geo, d_psi, d_theta, d_layer_angle, d_matC;
     DBuf<int> d_layer_of_ez, d_layer_mat, d_elem_mat;
-    DBuf<uint8_t> d_resin;
+    DBuf<uint8_t> d_resin, d_mask;   // resin elements; eliminated DOFs
     // boundary data
     std::vector<int64_t> dir_dof;
     std::vector<double> dir_val;
@@ -136,12 +136,14 @@ struct gl_ctx {
     DBuf<CGScalars> S;
     DBuf<int> err;
     double *h_pin = nullptr;
+    cudaEvent_t ev_scalar = nullptr;
     double ms_setup = 0;
     int64_t n_free = 0;
     SideStream side;
 
     ~gl_ctx() {
         if (h_pin) cudaFreeHost(h_pin);
+        if (ev_scalar) cudaEventDestroy(ev_scalar);
     }
 };
 
@@ -316,18 +318,18 @@ int64_t factor_solve_launches(const FactorPlan &P) {
     return n;
 }
 
-void apply_K(gl_ctx *c, const double *x, double *y) {
+void apply_K(gl_ctx *c, const double *x, double *y, bool zeroed = false) {
     prof_begin(c, PH_KU);
     if (has_slaves(c->m)) {
         // constrained DOFs (serendipity, periodic width): y = P^T K_Q2 P x, the slave entries of x
         // filled in a copy and folded out of y
         GL_CUDA(cudaMemcpyAsync(c->ks.p, x, c->m.n_dof * sizeof(double), cudaMemcpyDeviceToDevice, c->stream));
         slave_fill(c->m, c->ks.p, c->stream);
-        launch_ku(c->m, c->d_C.p, c->d_geo.p, c->ks.p, y, c->stream);
+        launch_ku(c->m, c->d_C.p, c->d_geo.p, c->ks.p, y, c->stream, zeroed);
         slave_fold(c->m, y, c->stream);
         g_launches += 2;
     } else {
-        launch_ku(c->m, c->d_C.p, c->d_geo.p, x, y, c->stream);
+        launch_ku(c->m, c->d_C.p, c->d_geo.p, x, y, c->stream, zeroed);
     }
     prof_end(c, PH_KU);
     g_launches += 1;
@@ -342,10 +344,10 @@ void local_solve(const FactorPlan &P, const T *L, T *xl, const double *r, double
     scatter_add_local<T>(P, x, z, s);
 }
 
-// z = M^{-1} r (r zero at Dirichlet DOFs)
-void apply_prec(gl_ctx *c, const double *r, double *z) {
+// z = M^{-1} r (r zero at Dirichlet DOFs; zeroed: z is zero already)
+void apply_prec(gl_ctx *c, const double *r, double *z, bool zeroed = false) {
     cudaStream_t s = c->stream;
-    GL_CUDA(cudaMemsetAsync(z, 0, c->m.n_dof * sizeof(double), s));
+    if (!zeroed) GL_CUDA(cudaMemsetAsync(z, 0, c->m.n_dof * sizeof(double), s));
     // the coarse correction overlaps the local sweeps (whose upper dissection
     // levels leave SMs idle) unless the phases are being timed separately
     const bool side = c->co.n0 > 0 && !c->prof.on;
@@ -437,6 +439,8 @@ void setup(gl_ctx *c, const gl_opts &o) {
         c->d_dir_dof.upload(dd, s);
         c->d_dir_val.upload(dv, s);
         c->n_dir = (int64_t)dd.size();
+        c->d_mask.upload(is_dir, s);
+        GL_CUDA(cudaStreamSynchronize(s));   // the lists are released at the end of this scope
     }
     c->n_free = m.n_dof - (int64_t)std::count(is_dir.begin(), is_dir.end(), (uint8_t)1);
     // the laminate as a one-part problem
@@ -507,7 +511,8 @@ void setup(gl_ctx *c, const gl_opts &o) {
     if (has_slaves(m)) c->ks.alloc(N);
     else c->ks.release();
     for (DBuf<double> *b : {&c->x, &c->r, &c->z, &c->p, &c->q, &c->ud, &c->fe}) b->alloc(N);
-    c->partials.alloc(1024);
+    c->partials.alloc(RED_SCRATCH);
+    c->partials.zero(s);
     c->cvec.alloc(std::max(1, c->co.n0));
     c->cvec2.alloc(std::max(1, c->co.n0));
     if (c->opts.precision == GL_PREC_MIXED) {
@@ -519,10 +524,22 @@ void setup(gl_ctx *c, const gl_opts &o) {
     }
     c->S.alloc(1);
     if (!c->h_pin) GL_CUDA(cudaMallocHost(&c->h_pin, 8 * sizeof(double)));
+    if (!c->ev_scalar) GL_CUDA(cudaEventCreateWithFlags(&c->ev_scalar, cudaEventDisableTiming));
     GL_CUDA(cudaStreamSynchronize(s));
     if (c->prof.levels) level_clock_enable(c->PD, true);
     c->ready = true;
     c->ms_setup = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
+}
+
+// The scalar's way to the host, and the host's wait for it; what is enqueued in
+// between runs meanwhile.
+void send_scalar(gl_ctx *c, const double *d) {
+    GL_CUDA(cudaMemcpyAsync(c->h_pin, d, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
+    GL_CUDA(cudaEventRecord(c->ev_scalar, c->stream));
+}
+double await_scalar(gl_ctx *c) {
+    GL_CUDA(cudaEventSynchronize(c->ev_scalar));
+    return c->h_pin[0];
 }
 
 double read_scalar(gl_ctx *c, const double *d) {
@@ -545,6 +562,15 @@ void prepare_rhs(gl_ctx *c, const double *f, bool homogeneous) {
     g_launches += 1 + (nd ? 2 : 0);
 }
 
+// r = fe - K x on the free DOFs in FP64, r.r -> S->rr
+void true_residual(gl_ctx *c, CGScalars *S) {
+    apply_K(c, c->x.p, c->q.p);
+    set_entries(c->q.p, c->d_dir_dof.p, c->n_dir, nullptr, c->stream);
+    sub(c->r.p, c->fe.p, c->q.p, c->m.n_dof, c->stream);
+    dot(c->r.p, c->r.p, c->m.n_dof, c->partials.p, &S->rr, c->stream);
+    g_launches += (c->n_dir ? 1 : 0) + 2;
+}
+
 // PCG solve of K u = f into u (or left in c->x when u is that vector);
 // homogeneous = zero Dirichlet values (adjoint solves).
 void solve(gl_ctx *c, const double *f, double *u, gl_info *info, bool homogeneous = false) {
@@ -560,7 +586,7 @@ void solve(gl_ctx *c, const double *f, double *u, gl_info *info, bool homogeneou
     c->S.zero(s);
     dot(c->fe.p, c->fe.p, N, c->partials.p, &S->ff, s);
     const int nds = nd ? 1 : 0;   // set_entries launches a kernel only for a non-empty list
-    g_launches += 2;
+    g_launches += 1;
     const double ff = read_scalar(c, &S->ff);
     if (!std::isfinite(ff)) {
         GL_CUDA(cudaEventDestroy(e0));
@@ -575,16 +601,33 @@ void solve(gl_ctx *c, const double *f, double *u, gl_info *info, bool homogeneou
     if (ff > 0.0) {
         apply_prec(c, c->r.p, c->z.p);
         dot(c->r.p, c->z.p, N, c->partials.p, &S->rho, s);
-        g_launches += 2;
+        g_launches += 1;
         GL_CUDA(cudaMemcpyAsync(c->p.p, c->z.p, N * sizeof(double), cudaMemcpyDeviceToDevice, s));
         rel = 1.0;
+        // z = M r, beta and the next direction (q zeroed for the next K p)
+        auto next_direction = [&]() {
+            if (mixed) {
+                dot(c->r.p, c->z.p, N, c->partials.p, &S->rz_old, s);   // flexible beta
+                g_launches += 1;
+            }
+            apply_prec(c, c->r.p, c->z.p, !mixed);
+            dot(c->r.p, c->z.p, N, c->partials.p, &S->rho_new, s);
+            cg_update_p(c->p.p, c->z.p, c->q.p, N, S, c->partials.p, s);
+            g_launches += 2;
+        };
         for (int it = 1; it <= c->opts.max_iter; ++it) {
-            apply_K(c, c->p.p, c->q.p);
-            set_entries(c->q.p, c->d_dir_dof.p, nd, nullptr, s);
-            dot(c->p.p, c->q.p, N, c->partials.p, &S->pq, s);
-            cg_update_xr(c->x.p, c->r.p, c->p.p, c->q.p, N, S, c->partials.p, s);
-            g_launches += nds + 4;
-            const double rr = read_scalar(c, &S->rr);
+            apply_K(c, c->p.p, c->q.p, it > 1);
+            dot(c->p.p, c->q.p, N, c->partials.p, &S->pq, s);   // p is zero at the eliminated DOFs
+            cg_update_xr(c->x.p, c->r.p, c->p.p, c->q.p, c->d_mask.p, mixed ? nullptr : c->z.p, N, S, c->partials.p, s);
+            g_launches += 2;
+            // The host waits for ||r||; as long as the last one was far from the tolerance the next direction is
+            // enqueued first and the device does not wait with it (if the iteration does end here after all, that
+            // direction is not used).
+            const bool special = mixed && it % c->opts.resid_period == 0;
+            const bool ahead = rel > 100.0 * c->opts.tol && it < c->opts.max_iter && !special;
+            send_scalar(c, &S->rr);
+            if (ahead) next_direction();
+            const double rr = await_scalar(c);
             iters = it;
             if (!std::isfinite(rr)) {
                 status = GL_ERR_NAN;
@@ -599,11 +642,7 @@ void solve(gl_ctx *c, const double *f, double *u, gl_info *info, bool homogeneou
             bool replaced = false;
             if (rel <= c->opts.tol) {
                 if (!mixed) break;
-                apply_K(c, c->x.p, c->q.p);
-                set_entries(c->q.p, c->d_dir_dof.p, nd, nullptr, s);
-                sub(c->r.p, c->fe.p, c->q.p, N, s);
-                dot(c->r.p, c->r.p, N, c->partials.p, &S->rr, s);
-                g_launches += nds + 3;
+                true_residual(c, S);
                 const double rt = read_scalar(c, &S->rr);
                 if (!std::isfinite(rt)) {
                     status = GL_ERR_NAN;
@@ -617,31 +656,31 @@ void solve(gl_ctx *c, const double *f, double *u, gl_info *info, bool homogeneou
                 status = GL_ERR_NOT_CONVERGED;
                 break;
             }
-            if (mixed && !replaced && it % c->opts.resid_period == 0) {
+            if (special && !replaced) {
                 // residual replacement: r = fe - K x in FP64
                 apply_K(c, c->x.p, c->q.p);
                 set_entries(c->q.p, c->d_dir_dof.p, nd, nullptr, s);
                 sub(c->r.p, c->fe.p, c->q.p, N, s);
                 g_launches += nds + 1;
             }
-            if (mixed) {
-                dot(c->r.p, c->z.p, N, c->partials.p, &S->rz_old, s);   // flexible beta
-                g_launches += 2;
+            if (replaced && ahead) {
+                // a fall by more than 100 onto a residual that does not hold: z, p and rho are those of the
+                // recurrence's next step, so the directions start anew from the true residual
+                apply_prec(c, c->r.p, c->z.p);
+                dot(c->r.p, c->z.p, N, c->partials.p, &S->rho, s);
+                GL_CUDA(cudaMemcpyAsync(c->p.p, c->z.p, N * sizeof(double), cudaMemcpyDeviceToDevice, s));
+                c->q.zero(s);
+                g_launches += 1;
+            } else if (!ahead) {
+                next_direction();
             }
-            apply_prec(c, c->r.p, c->z.p);
-            dot(c->r.p, c->z.p, N, c->partials.p, &S->rho_new, s);
-            cg_update_p(c->p.p, c->z.p, N, S, s);
-            g_launches += 4;
         }
     }
     // true residual and the full displacement
-    apply_K(c, c->x.p, c->q.p);
-    set_entries(c->q.p, c->d_dir_dof.p, nd, nullptr, s);
-    sub(c->r.p, c->fe.p, c->q.p, N, s);
-    dot(c->r.p, c->r.p, N, c->partials.p, &S->rr, s);
+    true_residual(c, S);
     const double rt = read_scalar(c, &S->rr);
     axpy(c->x.p, 1.0, c->ud.p, N, s);
-    g_launches += nds + 4;
+    g_launches += 1;
     if (has_slaves(c->m)) {
         slave_fill(c->m, c->x.p, s);   // the constrained entries carry the field's values
         g_launches += 1;
