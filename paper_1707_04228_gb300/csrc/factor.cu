@@ -902,10 +902,18 @@ __global__ void __launch_bounds__(SWEEP_CTA) k_bwd(const int *__restrict__ front
         const int i = min(r + lane, f - 1);
         return i < p ? y1 + i : xo + rw[i];
     };
+    // y_1 or -x_2, zero past the chunk; by the bits, not by the FP64 pipe that binds the kernel
     auto fetch_v = [&](int r, const T *at, T *v) {
-        const T sg = r + lane >= re ? T(0) : (r + lane < p ? T(1) : T(-1));
+        const bool in = r + lane < re;
+        const unsigned flip = r + lane < p ? 0u : 0x80000000u;
 #pragma unroll
-        for (int k = 0; k < NR; ++k) v[k] = sg * at[(int64_t)k * n];
+        for (int k = 0; k < NR; ++k) {
+            const T t = at[(int64_t)k * n];
+            if constexpr (sizeof(T) == 8)
+                v[k] = in ? (T)__hiloint2double(__double2hiint(t) ^ (int)flip, __double2loint(t)) : T(0);
+            else
+                v[k] = in ? (T)__int_as_float(__float_as_int(t) ^ (int)flip) : T(0);
+        }
     };
     T v[NR], vn[NR], l[CT];
     auto fetch_l = [&](int r) {
