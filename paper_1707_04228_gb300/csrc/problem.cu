@@ -2,12 +2,10 @@
 // decomposition, symbolic analysis with global numbering, local element maps
 // and the GenEO coarse space (Section 2.3, Fig. eig).
 #include <algorithm>
-#include <atomic>
 #include <cmath>
 #include <cstdio>
-#include <mutex>
-#include <thread>
 
+#include "host_parallel.h"
 #include "problem.h"
 
 namespace gl {
@@ -20,31 +18,6 @@ namespace {
 // this happens when two subdomains coincide (a box grown by the overlap to the
 // whole extent of a narrow laminate) or when Xi_j p vanishes.
 constexpr double COARSE_DROP_TOL = 1e-10;
-
-template <class F>
-void parallel_for(int n, F fn) {
-    int nt = std::max(1u, std::min(std::thread::hardware_concurrency(), 32u));
-    nt = std::min(nt, n);
-    std::atomic<int> next(0);
-    std::vector<std::thread> th;
-    std::vector<Error> errs;
-    std::mutex mu;
-    for (int t = 0; t < nt; ++t)
-        th.emplace_back([&]() {
-            for (;;) {
-                int i = next++;
-                if (i >= n) break;
-                try {
-                    fn(i);
-                } catch (const Error &e) {
-                    std::lock_guard<std::mutex> g(mu);
-                    errs.push_back(e);
-                }
-            }
-        });
-    for (auto &t : th) t.join();
-    if (!errs.empty()) throw errs.front();
-}
 
 std::vector<std::pair<int, int>> split_range(int n, int p) {
     std::vector<std::pair<int, int>> out;
@@ -129,12 +102,17 @@ void problem_symbolic(const Problem &P, bool neumann, int leaf_nodes, std::vecto
 }
 
 void problem_local_elems(const Problem &P, int s0, int s1, const FactorPlan &plan, LocalElems &E) {
-    std::vector<int> elem, sub, loc;
+    std::vector<int64_t> at(s1 - s0 + 1, 0);   // first pair of each subdomain
     for (int j = s0; j < s1; ++j) {
+        const int *e = P.boxes[j].ebox;
+        at[j - s0 + 1] = at[j - s0] + (int64_t)(e[1] - e[0]) * (e[3] - e[2]) * (e[5] - e[4]);
+    }
+    std::vector<int> elem(at.back()), sub(at.back()), loc(81 * at.back());
+    parallel_for(s1 - s0, [&](int jl) {
+        const int j = s0 + jl;
         const Part &pt = P.parts[P.sub_part[j]];
         const MeshHost &m = *pt.m;
         const SubBox &b = P.boxes[j];
-        const int jl = j - s0;
         const int nbx = b.nbox[1] - b.nbox[0] + 1, nby = b.nbox[3] - b.nbox[2] + 1, nbz = b.nbox[5] - b.nbox[4] + 1;
         std::vector<int> map((size_t)nbx * nby * nbz * 3, -1);
         const int64_t off = plan.vec_off[jl];
@@ -146,20 +124,22 @@ void problem_local_elems(const Problem &P, int s0, int s1, const FactorPlan &pla
             map[3 * ((size_t)(x - b.nbox[0]) + (size_t)nbx * ((y - b.nbox[2]) + (size_t)nby * (z - b.nbox[4]))) + comp] =
                 (int)i;
         }
+        int64_t k = at[jl];
         for (int ez = b.ebox[4]; ez < b.ebox[5]; ++ez)
             for (int ey = b.ebox[2]; ey < b.ebox[3]; ++ey)
-                for (int ex = b.ebox[0]; ex < b.ebox[1]; ++ex) {
-                    elem.push_back((int)(pt.elem_off + ex + (int64_t)m.nx * (ey + (int64_t)m.ny * ez)));
-                    sub.push_back(jl);
+                for (int ex = b.ebox[0]; ex < b.ebox[1]; ++ex, ++k) {
+                    elem[k] = (int)(pt.elem_off + ex + (int64_t)m.nx * (ey + (int64_t)m.ny * ez));
+                    sub[k] = jl;
+                    int *l = &loc[81 * k];
                     for (int a = 0; a < 27; ++a) {
                         int yg = 2 * ey + (a / 3) % 3;
                         if (m.periodic && yg == m.NY - 1) yg = 0;   // the first-plane partner carries the DOFs
                         int x = 2 * ex + a % 3 - b.nbox[0], y = yg - b.nbox[2], z = 2 * ez + a / 9 - b.nbox[4];
                         for (int cc = 0; cc < 3; ++cc)
-                            loc.push_back(map[3 * ((size_t)x + (size_t)nbx * (y + (size_t)nby * z)) + cc]);
+                            l[3 * a + cc] = map[3 * ((size_t)x + (size_t)nbx * (y + (size_t)nby * z)) + cc];
                     }
                 }
-    }
+    });
     E.n_pairs = (int64_t)elem.size();
     E.elem.upload(elem, P.stream);
     E.sub.upload(sub, P.stream);
@@ -167,16 +147,23 @@ void problem_local_elems(const Problem &P, int s0, int s1, const FactorPlan &pla
     GL_CUDA(cudaStreamSynchronize(P.stream));
 }
 
-void problem_coarse(const Problem &P, const gl_opts &o, const FactorPlan &PD, int leaf_nodes, Coarse &out) {
+std::future<std::vector<SubSymbolic>> neumann_symbolic(const Problem &P, int leaf_nodes) {
+    return std::async(std::launch::async, [&P, leaf_nodes] {
+        std::vector<SubSymbolic> syms;
+        problem_symbolic(P, true, leaf_nodes, syms);
+        return syms;
+    });
+}
+
+void problem_coarse(const Problem &P, const gl_opts &o, const FactorPlan &PD, std::vector<SubSymbolic> syms,
+                    Coarse &out) {
     cudaStream_t s = P.stream;
     const int nev = o.nev;
     const double sigma = o.sigma > 0 ? o.sigma : 1e-3;
     const int nsub = (int)P.boxes.size();
-    std::vector<SubSymbolic> syms;
-    problem_symbolic(P, true, leaf_nodes, syms);
     build_plan(syms, out.PN, s);
     out.PN.s20 = PD.s20;
-    P.stamp("Neumann symbolic");
+    P.stamp("Neumann plan");
     FactorPlan &PN = out.PN;
     for (int j = 0; j < nsub; ++j)
         if (PN.vec_len[j] < nev) fail(GL_ERR_INVALID_ARG, "subdomain has fewer DOFs than nev");
@@ -184,7 +171,7 @@ void problem_coarse(const Problem &P, const gl_opts &o, const FactorPlan &PD, in
     std::vector<int> mult(P.n_dof, 0);
     for (int64_t g : PD.h_gdof) mult[g] += 1;
     std::vector<double> xi(PN.n_local, 0.0);
-    for (int j = 0; j < nsub; ++j) {
+    parallel_for(nsub, [&](int j) {
         const Part &pt = P.parts[P.sub_part[j]];
         const MeshHost &m = *pt.m;
         const SubBox &b = P.boxes[j];
@@ -202,7 +189,7 @@ void problem_coarse(const Problem &P, const gl_opts &o, const FactorPlan &PD, in
                 xi[PN.vec_off[j] + i] = 1.0 / mult[g];
             }
         }
-    }
+    });
     DBuf<double> d_xi;
     d_xi.upload(xi, s);
     // basis columns: room for about four times nev before a restart, and Ritz vectors kept by one
@@ -217,18 +204,21 @@ void problem_coarse(const Problem &P, const gl_opts &o, const FactorPlan &PD, in
     // block Krylov iteration, one group at a time.
     const int64_t budget = (int64_t)((o.eig_group_bytes > 0 ? o.eig_group_bytes : 4e10) / sizeof(double));
     int j0 = 0, max_its = 0;
+    LocalElems E;
     while (j0 < nsub) {
         int j1 = j0;
         int64_t acc = 0;
         while (j1 < nsub && (j1 == j0 || acc + syms[j1].l_size <= budget)) acc += syms[j1++].l_size;
         const int ng = j1 - j0;
         ++out.n_groups;
-        std::vector<SubSymbolic> gs(syms.begin() + j0, syms.begin() + j1);
-        FactorPlan PG;
-        build_plan(gs, PG, s);
+        // a group of all subdomains is the whole problem's plan
+        FactorPlan group;
+        if (ng < nsub) {
+            build_plan(std::vector<SubSymbolic>(syms.begin() + j0, syms.begin() + j1), group, s);
+            group.s20 = PD.s20;
+        }
+        FactorPlan &PG = ng < nsub ? group : PN;
         PG.ws_budget_bytes = PD.ws_budget_bytes;
-        PG.s20 = PD.s20;
-        gs.clear();
         const int64_t goff = PN.vec_off[j0], gl = PG.n_local;
         DBuf<double> LN;
         LN.alloc(PG.l_size);
@@ -236,7 +226,6 @@ void problem_coarse(const Problem &P, const gl_opts &o, const FactorPlan &PD, in
         numeric_factor<double>(PG, P.C, P.geo, xg, sigma, LN.p, P.d_err, s);
         check_err(P, "GenEO shifted Neumann factorisation");
         P.stamp("Neumann factorisation (group)");
-        LocalElems E;
         problem_local_elems(P, j0, j1, PG, E);
         // Block Krylov (Lanczos) method for the largest mu of B p = mu M p, M = A^N + sigma B factored: the basis
         // V grows by the block M^{-1} B V_last, made M-orthonormal against all of V, and T = V^T B V gives the Ritz
@@ -345,8 +334,7 @@ void problem_coarse(const Problem &P, const gl_opts &o, const FactorPlan &PD, in
     out.eig_iters = max_its;
     syms.clear();
     scale_rows(PN, out.Z.p, d_xi.p, nev, s);                        // Z = Xi p
-    LocalElems E;
-    problem_local_elems(P, 0, nsub, PN, E);
+    if (out.n_groups > 1) problem_local_elems(P, 0, nsub, PN, E);
     // K_0 = Z^T K Z per part: Y_j = A^N_j Z_j, then blocks against the overlapping subdomains of the part
     DBuf<double> KZ;
     KZ.alloc(nl * nev);

@@ -6,6 +6,7 @@
 #pragma once
 
 #include <functional>
+#include <future>
 
 #include "factor.h"
 #include "geneo.h"
@@ -57,7 +58,10 @@ struct Coarse {
     DBuf<int> d_kvoff, d_kn;
 };
 
-void problem_coarse(const Problem &P, const gl_opts &o, const FactorPlan &PD, int leaf_nodes, Coarse &out);
+// The subdomains' Neumann symbolic factorisation on host threads of its own
+// (P must outlive it); problem_coarse takes its result.
+std::future<std::vector<SubSymbolic>> neumann_symbolic(const Problem &P, int leaf_nodes);
+void problem_coarse(const Problem &P, const gl_opts &o, const FactorPlan &PD, std::vector<SubSymbolic> syms, Coarse &out);
 
 // z += Z K_0^{-1} Z^T r (per part blocks); c1, c2 scratch of n0 entries.
 void coarse_apply(const Coarse &Cs, const double *r, double *z, double *c1, double *c2, cudaStream_t s);

@@ -16,6 +16,7 @@
 #include <mutex>
 #include <thread>
 
+#include "host_parallel.h"
 #include "problem.h"
 #include "slaves.h"
 
@@ -488,6 +489,9 @@ void setup(gl_ctx *c, const gl_opts &o) {
                          Lv.fronts.size(), ent, emax, Lv.max_f);
         }
     }
+    // the Neumann matrices' symbolic phase runs on host threads while the device factors the Dirichlet ones
+    std::future<std::vector<SubSymbolic>> neumann;
+    if (c->opts.nev > 0) neumann = neumann_symbolic(P, LEAF_NODES);
     if (c->opts.precision == GL_PREC_MIXED) {
         c->LD64.release();
         c->LD32.alloc(c->PD.l_size);
@@ -500,7 +504,7 @@ void setup(gl_ctx *c, const gl_opts &o) {
     check_err(c, "local Dirichlet factorisation");
     stamp(c, "Dirichlet factorisation");
     c->co = Coarse();
-    if (c->opts.nev > 0) problem_coarse(P, c->opts, c->PD, LEAF_NODES, c->co);
+    if (c->opts.nev > 0) problem_coarse(P, c->opts, c->PD, neumann.get(), c->co);
     if (std::getenv("GL_VERBOSE"))
         std::fprintf(stderr, "[gl] GenEO block steps (max over groups): %d\n", c->co.eig_iters);
     stamp(c, "GenEO coarse space + K0");
@@ -771,13 +775,8 @@ namespace {
 //   total = setup + 40 iterations,
 // with F = 0.8e12 flop/s (FP64) and B = 4.5e12 B/s (sustained HBM); the ratios
 // Neumann/Dirichlet (1.6x entries, 2x flops) were measured on the corner laminate.
-std::array<int, 2> autotune_grid(const MeshHost &m, const std::vector<uint8_t> &is_dir, int overlap, int nev,
-                                 bool mixed) {
-    const double F = 0.8e12, B = 4.5e12;
-    struct Cand {
-        int px, py;
-    };
-    std::vector<Cand> cands, all;
+std::vector<std::array<int, 2>> autotune_candidates(const MeshHost &m) {
+    std::vector<std::array<int, 2>> cands, all;
     for (int px = 1; px <= std::min(64, m.nx); ++px)
         for (int py = 1; py <= std::min(64, m.ny); ++py) {
             const int ns = px * py;
@@ -787,31 +786,55 @@ std::array<int, 2> autotune_grid(const MeshHost &m, const std::vector<uint8_t> &
             if (ax <= 2 * ay && ay <= 2 * ax) cands.push_back({px, py});
         }
     if (cands.empty()) cands = all;
-    if (cands.empty()) return {std::min(m.nx, 2), std::min(m.ny, 2)};
-    double best = 1e300;
-    std::array<int, 2> pick = {cands[0].px, cands[0].py};
-    for (const Cand &cd : cands) {
-        std::vector<SubBox> boxes;
-        part_boxes(m, cd.px, cd.py, 1, overlap, boxes);
-        SubSymbolic S;
-        build_symbolic(m, boxes[(cd.py / 2) * cd.px + cd.px / 2], is_dir, false, LEAF_NODES, S);
-        const int ns = cd.px * cd.py;
-        double fl = 0.0;
-        for (const Supernode &sn : S.sn) {
-            const double f = sn.p + sn.q;
-            for (int j = 0; j < sn.p; ++j) fl += (f - j) * (f - j);
-        }
-        const double nnz = (double)S.l_size * ns, flops = fl * ns, n0 = (double)ns * nev;
-        const double setup = (mixed ? 0.1 : 1.0) * flops / F + 2.0 * flops / F + 25.0 * 2 * nev * 4.0 * 1.6 * nnz / F +
-                             8.0 * n0 * n0 * n0 / 3.0 / F;
-        const double iter = mixed ? 8.0 * nnz / B : std::max(16.0 * nnz / B, 4.0 * nnz / F);
-        const double cost = setup + 40.0 * iter;
-        if (cost < best) {
-            best = cost;
-            pick = {cd.px, cd.py};
-        }
+    return cands;
+}
+
+double autotune_cost(const MeshHost &m, const std::vector<uint8_t> &is_dir, int overlap, int nev, bool mixed,
+                     std::array<int, 2> cd) {
+    const double F = 0.8e12, B = 4.5e12;
+    const int px = cd[0], py = cd[1];
+    std::vector<SubBox> boxes;
+    part_boxes(m, px, py, 1, overlap, boxes);
+    SubSymbolic S;
+    build_symbolic(m, boxes[(py / 2) * px + px / 2], is_dir, false, LEAF_NODES, S);
+    const int ns = px * py;
+    double fl = 0.0;
+    for (const Supernode &sn : S.sn) {
+        const double f = sn.p + sn.q;
+        for (int j = 0; j < sn.p; ++j) fl += (f - j) * (f - j);
     }
-    return pick;
+    const double nnz = (double)S.l_size * ns, flops = fl * ns, n0 = (double)ns * nev;
+    const double setup = (mixed ? 0.1 : 1.0) * flops / F + 2.0 * flops / F + 25.0 * 2 * nev * 4.0 * 1.6 * nnz / F +
+                         8.0 * n0 * n0 * n0 / 3.0 / F;
+    const double iter = mixed ? 8.0 * nnz / B : std::max(16.0 * nnz / B, 4.0 * nnz / F);
+    return setup + 40.0 * iter;
+}
+
+// The grid of every laminate: its candidates' costs on all host threads, the
+// first of the cheapest taken.
+void autotune_grids(const std::vector<gl_ctx *> &items, const std::vector<std::vector<uint8_t>> &is_dir, int overlap,
+                    int nev, bool mixed, std::vector<std::array<int, 2>> &grid) {
+    const int n = (int)items.size();
+    std::vector<std::vector<std::array<int, 2>>> cands(n);
+    std::vector<std::pair<int, int>> jobs;
+    for (int i = 0; i < n; ++i) {
+        cands[i] = autotune_candidates(items[i]->m);
+        for (int k = 0; k < (int)cands[i].size(); ++k) jobs.push_back({i, k});
+    }
+    std::vector<double> cost(jobs.size());
+    parallel_for((int)jobs.size(), [&](int q) {
+        const int i = jobs[q].first;
+        cost[q] = autotune_cost(items[i]->m, is_dir[i], overlap, nev, mixed, cands[i][jobs[q].second]);
+    });
+    std::vector<double> best(n, 1e300);
+    for (int i = 0; i < n; ++i)
+        grid[i] = cands[i].empty() ? std::array<int, 2>{std::min(items[i]->m.nx, 2), std::min(items[i]->m.ny, 2)}
+                                   : cands[i][0];
+    for (size_t q = 0; q < jobs.size(); ++q)
+        if (cost[q] < best[jobs[q].first]) {
+            best[jobs[q].first] = cost[q];
+            grid[jobs[q].first] = cands[jobs[q].first][jobs[q].second];
+        }
 }
 
 __global__ void k_seg_init(SegScalars S, int n) {
@@ -919,16 +942,7 @@ void batch_setup(gl_batch *b, const gl_opts &o) {
     // decomposition: given grid, or the autotuner per laminate
     b->grid.assign(n, {o.px, o.py});
     if (o.px <= 0 || o.py <= 0) {
-        std::vector<std::thread> th;
-        std::atomic<int> next(0);
-        const int nt = std::max(1, std::min(n, (int)std::thread::hardware_concurrency()));
-        for (int t = 0; t < nt; ++t)
-            th.emplace_back([&]() {
-                for (int i = next++; i < n; i = next++)
-                    b->grid[i] = autotune_grid(b->items[i]->m, is_dir[i], o.overlap, o.nev,
-                                               o.precision == GL_PREC_MIXED);
-            });
-        for (auto &t : th) t.join();
+        autotune_grids(b->items, is_dir, o.overlap, o.nev, o.precision == GL_PREC_MIXED, b->grid);
     }
     Problem &P = b->prob;
     P = Problem();
@@ -960,6 +974,8 @@ void batch_setup(gl_batch *b, const gl_opts &o) {
         b->PD.ws_budget_bytes = b->opts.factor_ws_bytes > 0 ? b->opts.factor_ws_bytes : 6e9;
         b->PD.tc_update = b->opts.fp32_update == 0;
     }
+    std::future<std::vector<SubSymbolic>> neumann;
+    if (b->opts.nev > 0) neumann = neumann_symbolic(P, LEAF_NODES);
     if (b->opts.precision == GL_PREC_MIXED) {
         b->LD64.release();
         b->LD32.alloc(b->PD.l_size);
@@ -980,7 +996,7 @@ void batch_setup(gl_batch *b, const gl_opts &o) {
         }
     }
     b->co = Coarse();
-    if (b->opts.nev > 0) problem_coarse(P, b->opts, b->PD, LEAF_NODES, b->co);
+    if (b->opts.nev > 0) problem_coarse(P, b->opts, b->PD, neumann.get(), b->co);
     for (DBuf<double> *v : {&b->x, &b->r, &b->z, &b->p, &b->q, &b->ud, &b->fe}) v->alloc(b->N);
     b->c1.alloc(std::max(1, b->co.n0));
     b->c2.alloc(std::max(1, b->co.n0));
