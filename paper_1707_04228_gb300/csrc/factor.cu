@@ -749,17 +749,14 @@ template void numeric_factor<float>(FactorPlan &, const double *, const double *
 // (forward: 32 panel rows; backward: a tile of panel columns), which the
 // inverse form makes independent of one another, so a level with a few large
 // fronts fills the chip as well as one with thousands of small ones.  Where
-// the level has fewer than sweep_warps() tasks they are cut along the summed
+// the level has fewer than SWEEP_WARPS tasks they are cut along the summed
 // dimension too (to no less than 32 columns or 64 rows) and add their parts
 // atomically: short tasks hide one another's loads and even out the SMs.  The
 // solve of the 475k-DOF corner (FP32) took 66.9, 64.5, 61.6 and 57.5 ms with
-// 12, 24, 48 and 96 tasks an SM, the 20k-DOF plate 11.3 to 10.4 ms; with
-// several right-hand sides a task has enough work and its atomics cost more.
+// 12, 24, 48 and 96 tasks an SM, the 20k-DOF plate 11.3 to 10.4 ms, and k_fwd
+// with eight right-hand sides 169 to 147 us a launch on the 63k-DOF corner.
 constexpr int SWEEP_CTA = 128;            // four warp tasks
-template <int NR>
-constexpr int sweep_warps() {
-    return 152 * (NR == 1 ? 96 : 12);
-}
+constexpr int SWEEP_WARPS = 152 * 96;
 
 // Forward: panel rows [r0, r0 + 32), lane = row, the columns of blockIdx.z's
 // chunk.  Pivot rows give y_1 = L11^{-1} b_1 (up to the diagonal block: zeros
@@ -1017,7 +1014,7 @@ static void launch_fwd(const FactorPlan &P, const Level &Lv, const int *fr, unsi
     if (nf == 0 || Lv.max_p == 0) return;
     const int tiles = (Lv.max_f + 31) / 32, blocks = (Lv.max_p + 31) / 32;
     // (the level's fronts, not nf: the arithmetic is the same however the level is split over streams)
-    const int split = std::min<int64_t>(blocks, std::max<int64_t>(1, sweep_warps<NR>() / ((int64_t)Lv.fronts.size() * tiles)));
+    const int split = std::min<int64_t>(blocks, std::max<int64_t>(1, SWEEP_WARPS / ((int64_t)Lv.fronts.size() * tiles)));
     const int chunk = 32 * ((blocks + split - 1) / split);
     const dim3 g(nf, (tiles + SWEEP_CTA / 32 - 1) / (SWEEP_CTA / 32), (Lv.max_p + chunk - 1) / chunk);
     launch_chained(k_fwd<T, NR>, g, s, fr, (const FrontDesc *)P.d_fr.p, L, (const int *)P.d_rows.p, b, y, kcols, c0, chunk);
@@ -1029,7 +1026,7 @@ static void launch_bwd(const FactorPlan &P, const Level &Lv, const int *fr, unsi
     if (nf == 0 || Lv.max_p == 0) return;
     const int tiles = (Lv.max_p + bwd_tile<NR>() - 1) / bwd_tile<NR>();
     const int chunks = std::min<int64_t>((Lv.max_f + 63) / 64,
-                                         std::max<int64_t>(1, sweep_warps<NR>() / ((int64_t)Lv.fronts.size() * tiles)));
+                                         std::max<int64_t>(1, SWEEP_WARPS / ((int64_t)Lv.fronts.size() * tiles)));
     const dim3 g(nf, (tiles * chunks + SWEEP_CTA / 32 - 1) / (SWEEP_CTA / 32));
     launch_chained(k_bwd<T, NR>, g, s, fr, (const FrontDesc *)P.d_fr.p, L, (const int *)P.d_rows.p, y, x, kcols, c0, chunks);
 }

@@ -1473,9 +1473,16 @@ int gl_apply_K(gl_ctx *c, const double *x, double *y) {
         if (!c->ready) fail(GL_ERR_STATE, "gl_apply_K before gl_setup");
         GL_REQUIRE(x && y, "null vector");
         cudaStream_t s = c->stream;
-        to_device(c->p.p, x, c->m.n_dof, s);
-        apply_K(c, c->p.p, c->q.p);
-        from_device(y, c->q.p, c->m.n_dof, s);
+        const int64_t N = c->m.n_dof;
+        const double *dx = x;
+        if (!in_place(c, x, N)) {
+            to_device(c->p.p, x, N, s);
+            dx = c->p.p;
+        }
+        double *dy = in_place(c, y, N, x, N) ? y : c->q.p;
+        apply_K(c, dx, dy);
+        if (dy != y) to_device(y, dy, N, s);
+        GL_CUDA(cudaStreamSynchronize(s));
     });
 }
 
