@@ -49,14 +49,20 @@ __global__ void k_scatter_cols(const int64_t *__restrict__ gdof, int64_t off, in
     }
 }
 
-// K0[(row0 + a) + (col0 + b) * n0] = sum_i Z_l[i, a] G[gdof_l[i] - gshift, b]
-__global__ void __launch_bounds__(256) k_coarse_block(const int64_t *__restrict__ gdof, int64_t off, int64_t n,
-                                                      const double *__restrict__ Z, int64_t zoff, int m,
-                                                      const double *__restrict__ G, int64_t N, int64_t gshift,
-                                                      double *__restrict__ K0, int64_t n0, int row0, int col0) {
-    const int a = blockIdx.x / m, b = blockIdx.x % m;
+// Blocks (l, j) of K0 for the neighbours l = nbr[blockIdx.y] of subdomain j:
+// K0[((l - sub0) m + a) + (col0 + b) n0] = sum_i Z_l[i, a] G[gdof_l[i] - gshift, b].
+__global__ void __launch_bounds__(256) k_coarse_block(const int *__restrict__ nbr, const int64_t *__restrict__ voff,
+                                                      const int64_t *__restrict__ vlen,
+                                                      const int64_t *__restrict__ gdof, const double *__restrict__ Z,
+                                                      int m, const double *__restrict__ G, int64_t N, int64_t gshift,
+                                                      double *__restrict__ K0, int64_t n0, int sub0, int col0) {
+    const int a = blockIdx.x / m, b = blockIdx.x % m, l = nbr[blockIdx.y];
+    const int64_t n = vlen[l];
+    const double *Za = Z + voff[l] * m + a * n, *Gb = G + b * N - gshift;
+    const int64_t *gd = gdof + voff[l];
     double v = 0.0;
-    for (int64_t i = threadIdx.x; i < n; i += blockDim.x) v += Z[zoff + a * n + i] * G[b * N + gdof[off + i] - gshift];
+#pragma unroll 4
+    for (int64_t i = threadIdx.x; i < n; i += blockDim.x) v += Za[i] * Gb[gd[i]];
     __shared__ double red[256];
     red[threadIdx.x] = v;
     __syncthreads();
@@ -64,7 +70,7 @@ __global__ void __launch_bounds__(256) k_coarse_block(const int64_t *__restrict_
         if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
         __syncthreads();
     }
-    if (threadIdx.x == 0) K0[(row0 + a) + (int64_t)(col0 + b) * n0] = red[0];
+    if (threadIdx.x == 0) K0[((int64_t)(l - sub0) * m + a) + (int64_t)(col0 + b) * n0] = red[0];
 }
 
 }  // namespace
@@ -364,20 +370,28 @@ void problem_coarse(const Problem &P, const gl_opts &o, const FactorPlan &PD, st
         G.zero(s);
         K0.alloc((size_t)n0p * n0p);
         K0.zero(s);
+        // the neighbours of every subdomain (boxes that meet), one launch for all of one's blocks
+        std::vector<int> nbr, at(1, 0);
         for (int j = pt.sub0; j < pt.sub1; ++j) {
-            int64_t nj = PN.vec_len[j], oj = PN.vec_off[j];
-            k_scatter_cols<<<256, 256, 0, s>>>(PN.d_gdof.p, oj, nj, KZ.p, oj * nev, nev, G.p, Np, pt.dof_off, 0);
             for (int l = pt.sub0; l < pt.sub1; ++l) {
                 bool overlap = true;
                 for (int d = 0; d < 3; ++d)
                     if (P.boxes[l].nbox[2 * d] > P.boxes[j].nbox[2 * d + 1] ||
                         P.boxes[j].nbox[2 * d] > P.boxes[l].nbox[2 * d + 1])
                         overlap = false;
-                if (!overlap) continue;
-                k_coarse_block<<<nev * nev, 256, 0, s>>>(PN.d_gdof.p, PN.vec_off[l], PN.vec_len[l], out.Z.p,
-                                                         PN.vec_off[l] * nev, nev, G.p, Np, pt.dof_off, K0.p, n0p,
-                                                         (l - pt.sub0) * nev, (j - pt.sub0) * nev);
+                if (overlap) nbr.push_back(l);
             }
+            at.push_back((int)nbr.size());
+        }
+        DBuf<int> d_nbr;
+        d_nbr.upload(nbr, s);
+        for (int j = pt.sub0; j < pt.sub1; ++j) {
+            const int64_t nj = PN.vec_len[j], oj = PN.vec_off[j];
+            const int k = j - pt.sub0;
+            k_scatter_cols<<<256, 256, 0, s>>>(PN.d_gdof.p, oj, nj, KZ.p, oj * nev, nev, G.p, Np, pt.dof_off, 0);
+            k_coarse_block<<<dim3(nev * nev, at[k + 1] - at[k]), 256, 0, s>>>(
+                d_nbr.p + at[k], PN.d_vec_off.p, PN.d_vec_len.p, PN.d_gdof.p, out.Z.p, nev, G.p, Np, pt.dof_off, K0.p,
+                n0p, pt.sub0, k * nev);
             k_scatter_cols<<<256, 256, 0, s>>>(PN.d_gdof.p, oj, nj, KZ.p, oj * nev, nev, G.p, Np, pt.dof_off, 1);
             GL_CUDA(cudaGetLastError());
         }
