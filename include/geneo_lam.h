@@ -169,8 +169,8 @@ typedef struct {
  *              large top fronts leave idle.  0 selects the default, every
  *              level counted as top (the halves sweep concurrently, both at
  *              high priority); < 0 sweeps sequentially.  Same arithmetic
- *              either way.  Single laminates (gl_setup) only; timed phases
- *              (gl_profile) sweep sequentially. */
+ *              either way, in gl_setup and gl_batch_setup; with the levels timed
+ *              (gl_profile 2) they sweep sequentially. */
 typedef struct {
     int px, py, pz, overlap, nev, max_iter, precision, resid_period;
     double tol, sigma;

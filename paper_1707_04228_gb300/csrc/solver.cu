@@ -973,6 +973,7 @@ void batch_setup(gl_batch *b, const gl_opts &o) {
         build_plan(syms, b->PD, s);
         b->PD.ws_budget_bytes = b->opts.factor_ws_bytes > 0 ? b->opts.factor_ws_bytes : 6e9;
         b->PD.tc_update = b->opts.fp32_update == 0;
+        b->PD.overlap_top = sweep_overlap_top(b->opts);
     }
     std::future<std::vector<SubSymbolic>> neumann;
     if (b->opts.nev > 0) neumann = neumann_symbolic(P, LEAF_NODES);
