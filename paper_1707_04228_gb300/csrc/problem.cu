@@ -36,6 +36,7 @@ void check_err(const Problem &P, const char *what) {
     GL_CUDA(cudaStreamSynchronize(P.stream));
     if (h) {
         GL_CUDA(cudaMemsetAsync(P.d_err, 0, sizeof(int), P.stream));
+        if (h == 2) fail(GL_ERR_TIMEOUT, std::string(what) + ": a tensor-core wait gave up");
         fail(GL_ERR_NOT_SPD, std::string(what) + ": non-positive pivot");
     }
 }
