@@ -753,8 +753,7 @@ template void numeric_factor<float>(FactorPlan &, const double *, const double *
 // dimension too (to no less than 32 columns or 64 rows) and add their parts
 // atomically: short tasks hide one another's loads and even out the SMs.  The
 // solve of the 475k-DOF corner (FP32) took 66.9, 64.5, 61.6 and 57.5 ms with
-// 12, 24, 48 and 96 tasks an SM, the 20k-DOF plate 11.3 to 10.4 ms, and k_fwd
-// with eight right-hand sides 169 to 147 us a launch on the 63k-DOF corner.
+// 12, 24, 48 and 96 tasks an SM, the 20k-DOF plate 11.3 to 10.4 ms.
 constexpr int SWEEP_CTA = 128;            // four warp tasks
 constexpr int SWEEP_WARPS = 152 * 96;
 
@@ -765,14 +764,14 @@ constexpr int SWEEP_WARPS = 152 * 96;
 // size that fills the chip; FP32 is bound by reading the panel once.  One CTA
 // per front stepping through 32-pivot blocks took 74 us (FP64) and 62 us (FP32)
 // a launch on the 308k- and 475k-DOF corners, this form 44 and 25 us.
-template <class T, int NR>
+template <class T>
 __global__ void __launch_bounds__(SWEEP_CTA) k_fwd(const int *__restrict__ fronts, const FrontDesc *__restrict__ D,
                                                    const T *__restrict__ L, const int *__restrict__ rows, T *b,
-                                                   T *y, int kcols, int c0, int chunk) {
-    __shared__ __align__(16) T sx[SWEEP_CTA / 32][32 * NR];
+                                                   T *y, int chunk) {
+    __shared__ __align__(16) T sx[SWEEP_CTA / 32][32];
     const FrontDesc &d = D[fronts[blockIdx.x]];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int p = d.p, f = p + d.q, n = d.vlen;
+    const int p = d.p, f = p + d.q;
     const int r0 = (blockIdx.y * (SWEEP_CTA / 32) + w) * 32;
     const int cb = blockIdx.z * chunk;
     // pivot rows need the columns up to their diagonal block, any structure row all of them
@@ -781,8 +780,7 @@ __global__ void __launch_bounds__(SWEEP_CTA) k_fwd(const int *__restrict__ front
         cudaGridDependencySynchronize();
         return;
     }
-    const int64_t vo = d.vec_off * kcols + (int64_t)c0 * n;
-    const T *b1 = b + vo + d.first;
+    const T *b1 = b + d.vec_off + d.first;
     const int row = min(r0 + lane, f - 1);
     const T *Lr = L + d.l_off + row;
     constexpr int G = sizeof(T) == 4 ? 32 : 16;   // loads in flight per lane
@@ -791,15 +789,12 @@ __global__ void __launch_bounds__(SWEEP_CTA) k_fwd(const int *__restrict__ front
 #pragma unroll
     for (int j = 0; j < G; ++j) l[j] = cb + j < cend ? Lr[(int64_t)(cb + j) * f] : T(0);
     cudaGridDependencySynchronize();
-    T acc[NR], acc2[NR];
-#pragma unroll
-    for (int r = 0; r < NR; ++r) acc[r] = acc2[r] = T(0);
+    T acc = T(0), acc2 = T(0);
     T *xs = sx[w];
     for (int c = cb; c < cend; c += 32) {
         const int kb = min(32, cend - c);
         __syncwarp();
-#pragma unroll
-        for (int r = 0; r < NR; ++r) xs[lane * NR + r] = lane < kb ? b1[c + lane + (int64_t)r * n] : T(0);
+        xs[lane] = lane < kb ? b1[c + lane] : T(0);
         __syncwarp();
         const T *Lc = Lr + (int64_t)c * f;
 #pragma unroll
@@ -812,12 +807,10 @@ __global__ void __launch_bounds__(SWEEP_CTA) k_fwd(const int *__restrict__ front
                     for (int j = 0; j < G; ++j) l[j] = Lc[(int64_t)(g + j) * f];
                 }
 #pragma unroll
-                for (int j = 0; j < G; j += 2)
-#pragma unroll
-                    for (int r = 0; r < NR; ++r) {
-                        acc[r] += l[j] * xs[(g + j) * NR + r];
-                        acc2[r] += l[j + 1] * xs[(g + j + 1) * NR + r];
-                    }
+                for (int j = 0; j < G; j += 2) {
+                    acc += l[j] * xs[g + j];
+                    acc2 += l[j + 1] * xs[g + j + 1];
+                }
             } else {
                 // the last columns, in fours
                 if (!have) {
@@ -828,9 +821,7 @@ __global__ void __launch_bounds__(SWEEP_CTA) k_fwd(const int *__restrict__ front
                 for (int h = 0; h < G; h += 4) {
                     if (g + h >= kb) break;
 #pragma unroll
-                    for (int j = h; j < h + 4; ++j)
-#pragma unroll
-                        for (int r = 0; r < NR; ++r) acc[r] += l[j] * xs[(g + j) * NR + r];
+                    for (int j = h; j < h + 4; ++j) acc += l[j] * xs[g + j];
                 }
             }
         }
@@ -838,41 +829,31 @@ __global__ void __launch_bounds__(SWEEP_CTA) k_fwd(const int *__restrict__ front
     cudaTriggerProgrammaticLaunchCompletion();
     if (r0 + lane >= f) return;
     if (row < p) {
-        T *yo = y + vo + d.first + row;
-#pragma unroll
-        for (int r = 0; r < NR; ++r) {
-            if (gridDim.z == 1) yo[(int64_t)r * n] = acc[r] + acc2[r];
-            else atomicAdd(yo + (int64_t)r * n, acc[r] + acc2[r]);
-        }
+        T *yo = y + d.vec_off + d.first + row;
+        if (gridDim.z == 1) *yo = acc + acc2;
+        else atomicAdd(yo, acc + acc2);
     } else {
-        T *bo = b + vo + rows[d.row_off + row];
-#pragma unroll
-        for (int r = 0; r < NR; ++r) atomicAdd(bo + (int64_t)r * n, -(acc[r] + acc2[r]));
+        atomicAdd(b + d.vec_off + rows[d.row_off + row], -(acc + acc2));
     }
 }
 
-// Panel columns of one backward warp task: 16 (8, 4 with four and eight
-// right-hand sides) keep the accumulators to 64 registers and so enough warps
-// on an SM to cover the loads.  With 32 columns and one right-hand side the kernel
-// took 226 registers and 74.6 us a launch against 54.5 on the 308k-DOF corner.
-template <int NR>
-__host__ __device__ constexpr int bwd_tile() {
-    return NR <= 2 ? 16 : 32 / NR;
-}
-
-// Backward: x_1 = [L11^{-1}; -W]^T [y_1; x_2].  A warp task is a tile of panel
-// columns over one chunk of the panel's rows, lane = row, one accumulator per
-// (column, right-hand side); the lanes are summed at the end (warp_sum_many).
-// One CTA per front took 85 us (FP64) and 68 us (FP32) a launch on the same
+// Backward: x_1 = [L11^{-1}; -W]^T [y_1; x_2].  A warp task is a tile of 16
+// panel columns over one chunk of the panel's rows, lane = row, one accumulator
+// per column; the lanes are summed at the end (warp_sum_many).  With 32 columns
+// the kernel took 226 registers and 74.6 us a launch against 54.5 on the
+// 308k-DOF corner: too few warps on an SM to cover the loads.  One CTA per
+// front took 85 us (FP64) and 68 us (FP32) a launch on the 308k- and 475k-DOF
 // corners, this form 44 and 34 us.
-template <class T, int NR>
+constexpr int BWD_TILE = 16;
+
+template <class T>
 __global__ void __launch_bounds__(SWEEP_CTA) k_bwd(const int *__restrict__ fronts, const FrontDesc *__restrict__ D,
                                                    const T *__restrict__ L, const int *__restrict__ rows,
-                                                   const T *__restrict__ y, T *x, int kcols, int c0, int chunks) {
-    constexpr int CT = bwd_tile<NR>();
+                                                   const T *__restrict__ y, T *x, int chunks) {
+    constexpr int CT = BWD_TILE;
     const FrontDesc &d = D[fronts[blockIdx.x]];
     const int lane = threadIdx.x & 31;
-    const int p = d.p, f = p + d.q, n = d.vlen;
+    const int p = d.p, f = p + d.q;
     const int task = blockIdx.y * (SWEEP_CTA / 32) + (threadIdx.x >> 5);
     const int nct = (p + CT - 1) / CT;
     if (task >= nct * chunks) {
@@ -887,32 +868,28 @@ __global__ void __launch_bounds__(SWEEP_CTA) k_bwd(const int *__restrict__ front
         cudaGridDependencySynchronize();
         return;
     }
-    const int64_t vo = d.vec_off * kcols + (int64_t)c0 * n;
-    const T *y1 = y + vo + d.first, *xo = x + vo;
+    const T *y1 = y + d.vec_off + d.first, *xo = x + d.vec_off;
     const int *rw = rows + d.row_off;
     const T *Lt = L + d.l_off + (int64_t)j0 * f;
-    T acc[CT * NR];
+    T acc[CT];
 #pragma unroll
-    for (int i = 0; i < CT * NR; ++i) acc[i] = T(0);
+    for (int i = 0; i < CT; ++i) acc[i] = T(0);
     // the rows' vector entries: where they are two steps ahead, their values one step ahead
     auto where = [&](int r) {
         const int i = min(r + lane, f - 1);
         return i < p ? y1 + i : xo + rw[i];
     };
     // y_1 or -x_2, zero past the chunk; by the bits, not by the FP64 pipe that binds the kernel
-    auto fetch_v = [&](int r, const T *at, T *v) {
+    auto fetch_v = [&](int r, const T *at) {
         const bool in = r + lane < re;
-        const unsigned flip = r + lane < p ? 0u : 0x80000000u;
-#pragma unroll
-        for (int k = 0; k < NR; ++k) {
-            const T t = at[(int64_t)k * n];
-            if constexpr (sizeof(T) == 8)
-                v[k] = in ? (T)__hiloint2double(__double2hiint(t) ^ (int)flip, __double2loint(t)) : T(0);
-            else
-                v[k] = in ? (T)__int_as_float(__float_as_int(t) ^ (int)flip) : T(0);
-        }
+        const int flip = r + lane < p ? 0 : (int)0x80000000u;
+        const T t = *at;
+        if constexpr (sizeof(T) == 8)
+            return in ? (T)__hiloint2double(__double2hiint(t) ^ flip, __double2loint(t)) : T(0);
+        else
+            return in ? (T)__int_as_float(__float_as_int(t) ^ flip) : T(0);
     };
-    T v[NR], vn[NR], l[CT];
+    T v, vn, l[CT];
     auto fetch_l = [&](int r) {
         const T *Li = Lt + min(r + lane, f - 1);
 #pragma unroll
@@ -923,36 +900,28 @@ __global__ void __launch_bounds__(SWEEP_CTA) k_bwd(const int *__restrict__ front
     const T *at = where(rb);
     const T *at1 = where(rb + 32);
     cudaGridDependencySynchronize();
-    fetch_v(rb, at, v);
+    v = fetch_v(rb, at);
     at = at1;
     for (int r = rb; r < re; r += 32) {
         auto step = [&](auto cols) {
             constexpr int G = decltype(cols)::value;
             if (r != rb) fetch_l(r);
-            fetch_v(r + 32, at, vn);
+            vn = fetch_v(r + 32, at);
             at = where(r + 64);
 #pragma unroll
-            for (int j = 0; j < G; ++j)
-#pragma unroll
-                for (int k = 0; k < NR; ++k) acc[j * NR + k] += l[j] * v[k];
+            for (int j = 0; j < G; ++j) acc[j] += l[j] * v;
         };
-        if (CT == 16 && kb <= 8) step(std::integral_constant<int, CT / 2>());
+        if (kb <= CT / 2) step(std::integral_constant<int, CT / 2>());
         else step(std::integral_constant<int, CT>());
-#pragma unroll
-        for (int k = 0; k < NR; ++k) v[k] = vn[k];
+        v = vn;
     }
     cudaTriggerProgrammaticLaunchCompletion();
-    warp_sum_many<T, CT * NR>(acc, lane);
-    constexpr int PL = CT * NR < 32 ? 1 : CT * NR / 32, SH = CT * NR < 32 ? 1 : 0;   // sums per lane; lanes per sum 2^SH
-    if (lane & SH) return;
-#pragma unroll
-    for (int t = 0; t < PL; ++t) {
-        const int i = (lane >> SH) * PL + t, j = i / NR, k = i % NR;
-        if (j >= kb) continue;
-        T *out = x + vo + d.first + j0 + j + (int64_t)k * n;
-        if (chunks == 1) *out = acc[t];
-        else atomicAdd(out, acc[t]);
-    }
+    warp_sum_many<T, CT>(acc, lane);
+    const int j = lane >> 1;      // two lanes hold each sum
+    if ((lane & 1) || j >= kb) return;
+    T *out = x + d.vec_off + d.first + j0 + j;
+    if (chunks == 1) *out = acc[0];
+    else atomicAdd(out, acc[0]);
 }
 
 void level_clock_enable(FactorPlan &P, bool on) {
@@ -1008,27 +977,27 @@ static void launch_chained(K kernel, dim3 grid, cudaStream_t s, A... args) {
 }
 
 // One level's forward or backward sweep over the fronts fr[0..nf) of that level.
-template <class T, int NR>
+template <class T>
 static void launch_fwd(const FactorPlan &P, const Level &Lv, const int *fr, unsigned nf, const T *L, T *b, T *y,
-                       int kcols, int c0, cudaStream_t s) {
+                       cudaStream_t s) {
     if (nf == 0 || Lv.max_p == 0) return;
     const int tiles = (Lv.max_f + 31) / 32, blocks = (Lv.max_p + 31) / 32;
     // (the level's fronts, not nf: the arithmetic is the same however the level is split over streams)
     const int split = std::min<int64_t>(blocks, std::max<int64_t>(1, SWEEP_WARPS / ((int64_t)Lv.fronts.size() * tiles)));
     const int chunk = 32 * ((blocks + split - 1) / split);
     const dim3 g(nf, (tiles + SWEEP_CTA / 32 - 1) / (SWEEP_CTA / 32), (Lv.max_p + chunk - 1) / chunk);
-    launch_chained(k_fwd<T, NR>, g, s, fr, (const FrontDesc *)P.d_fr.p, L, (const int *)P.d_rows.p, b, y, kcols, c0, chunk);
+    launch_chained(k_fwd<T>, g, s, fr, (const FrontDesc *)P.d_fr.p, L, (const int *)P.d_rows.p, b, y, chunk);
 }
 
-template <class T, int NR>
+template <class T>
 static void launch_bwd(const FactorPlan &P, const Level &Lv, const int *fr, unsigned nf, const T *L, const T *y, T *x,
-                       int kcols, int c0, cudaStream_t s) {
+                       cudaStream_t s) {
     if (nf == 0 || Lv.max_p == 0) return;
-    const int tiles = (Lv.max_p + bwd_tile<NR>() - 1) / bwd_tile<NR>();
+    const int tiles = (Lv.max_p + BWD_TILE - 1) / BWD_TILE;
     const int chunks = std::min<int64_t>((Lv.max_f + 63) / 64,
                                          std::max<int64_t>(1, SWEEP_WARPS / ((int64_t)Lv.fronts.size() * tiles)));
     const dim3 g(nf, (tiles * chunks + SWEEP_CTA / 32 - 1) / (SWEEP_CTA / 32));
-    launch_chained(k_bwd<T, NR>, g, s, fr, (const FrontDesc *)P.d_fr.p, L, (const int *)P.d_rows.p, y, x, kcols, c0, chunks);
+    launch_chained(k_bwd<T>, g, s, fr, (const FrontDesc *)P.d_fr.p, L, (const int *)P.d_rows.p, y, x, chunks);
 }
 
 static HalfStreams &half_streams(const FactorPlan &P) {
@@ -1053,8 +1022,8 @@ static HalfStreams &half_streams(const FactorPlan &P) {
 // then its deep backward levels on lo[h].  The second half's deep forward
 // levels start when the first half enters its top levels.  The halves hold
 // disjoint subdomains, so they share no data.
-template <class T, int NR>
-static void solve_levels_overlap(const FactorPlan &P, const T *L, T *b, T *y, T *x, int kcols, int c0, cudaStream_t s) {
+template <class T>
+static void solve_levels_overlap(const FactorPlan &P, const T *L, T *b, T *y, T *x, cudaStream_t s) {
     HalfStreams &H = half_streams(P);
     const int nlev = (int)P.levels.size(), k = std::min(P.overlap_top, nlev);
     GL_CUDA(cudaEventRecord(H.fork, s));
@@ -1074,19 +1043,19 @@ static void solve_levels_overlap(const FactorPlan &P, const T *L, T *b, T *y, T 
         for (int d = nlev - 1; d >= k; --d) {
             const int *fr; unsigned nf;
             part(h, d, fr, nf);
-            launch_fwd<T, NR>(P, P.levels[d], fr, nf, L, b, y, kcols, c0, H.lo[h]);
+            launch_fwd<T>(P, P.levels[d], fr, nf, L, b, y, H.lo[h]);
         }
         GL_CUDA(cudaEventRecord(H.ev[3 * h], H.lo[h]));
         GL_CUDA(cudaStreamWaitEvent(H.hi[h], H.ev[3 * h], 0));
         for (int d = k - 1; d >= 0; --d) {
             const int *fr; unsigned nf;
             part(h, d, fr, nf);
-            launch_fwd<T, NR>(P, P.levels[d], fr, nf, L, b, y, kcols, c0, H.hi[h]);
+            launch_fwd<T>(P, P.levels[d], fr, nf, L, b, y, H.hi[h]);
         }
         for (int d = 0; d < k; ++d) {
             const int *fr; unsigned nf;
             part(h, d, fr, nf);
-            launch_bwd<T, NR>(P, P.levels[d], fr, nf, L, y, x, kcols, c0, H.hi[h]);
+            launch_bwd<T>(P, P.levels[d], fr, nf, L, y, x, H.hi[h]);
         }
         GL_CUDA(cudaEventRecord(H.ev[3 * h + 1], H.hi[h]));
     }
@@ -1095,7 +1064,7 @@ static void solve_levels_overlap(const FactorPlan &P, const T *L, T *b, T *y, T 
         for (int d = k; d < nlev; ++d) {
             const int *fr; unsigned nf;
             part(h, d, fr, nf);
-            launch_bwd<T, NR>(P, P.levels[d], fr, nf, L, y, x, kcols, c0, H.lo[h]);
+            launch_bwd<T>(P, P.levels[d], fr, nf, L, y, x, H.lo[h]);
         }
         GL_CUDA(cudaEventRecord(H.ev[3 * h + 2], H.lo[h]));
         GL_CUDA(cudaStreamWaitEvent(s, H.ev[3 * h + 2], 0));
@@ -1103,12 +1072,12 @@ static void solve_levels_overlap(const FactorPlan &P, const T *L, T *b, T *y, T 
     GL_CUDA(cudaGetLastError());
 }
 
-template <class T, int NR>
-static void solve_levels(const FactorPlan &P, const T *L, T *b, T *y, T *x, int kcols, int c0, cudaStream_t s) {
+template <class T>
+void factor_solve(const FactorPlan &P, const T *L, T *b, T *y, T *x, cudaStream_t s) {
     const int nlev = (int)P.levels.size();
-    const bool timed = NR == 1 && kcols == 1 && P.clock.on && P.clock.ev.size() == 2 * (size_t)nlev + 1;
-    if (NR == 1 && kcols == 1 && P.overlap_top > 0 && !timed && P.n_sub >= 2) {
-        solve_levels_overlap<T, NR>(P, L, b, y, x, kcols, c0, s);
+    const bool timed = P.clock.on && P.clock.ev.size() == 2 * (size_t)nlev + 1;
+    if (P.overlap_top > 0 && !timed && P.n_sub >= 2) {
+        solve_levels_overlap<T>(P, L, b, y, x, s);
         return;
     }
     auto mark = [&](int k) {
@@ -1117,12 +1086,12 @@ static void solve_levels(const FactorPlan &P, const T *L, T *b, T *y, T *x, int 
     for (int dpt = nlev - 1; dpt >= 0; --dpt) {
         mark(nlev - 1 - dpt);
         const Level &Lv = P.levels[dpt];
-        launch_fwd<T, NR>(P, Lv, Lv.d_fronts.p, (unsigned)Lv.fronts.size(), L, b, y, kcols, c0, s);
+        launch_fwd<T>(P, Lv, Lv.d_fronts.p, (unsigned)Lv.fronts.size(), L, b, y, s);
     }
     for (int dpt = 0; dpt < nlev; ++dpt) {
         mark(nlev + dpt);
         const Level &Lv = P.levels[dpt];
-        launch_bwd<T, NR>(P, Lv, Lv.d_fronts.p, (unsigned)Lv.fronts.size(), L, y, x, kcols, c0, s);
+        launch_bwd<T>(P, Lv, Lv.d_fronts.p, (unsigned)Lv.fronts.size(), L, y, x, s);
     }
     GL_CUDA(cudaGetLastError());
     if (timed) {
@@ -1131,21 +1100,20 @@ static void solve_levels(const FactorPlan &P, const T *L, T *b, T *y, T *x, int 
     }
 }
 
-template <class T>
-void factor_solve(const FactorPlan &P, const T *L, T *b, T *y, T *x, int kcols, cudaStream_t s) {
-    int c0 = 0;
-    while (c0 < kcols) {
-        const int left = kcols - c0;
-        if (left >= 8) { solve_levels<T, 8>(P, L, b, y, x, kcols, c0, s); c0 += 8; }
-        else if (left >= 4) { solve_levels<T, 4>(P, L, b, y, x, kcols, c0, s); c0 += 4; }
-        else if (left >= 2) { solve_levels<T, 2>(P, L, b, y, x, kcols, c0, s); c0 += 2; }
-        else { solve_levels<T, 1>(P, L, b, y, x, kcols, c0, s); c0 += 1; }
+template void factor_solve<double>(const FactorPlan &, const double *, double *, double *, double *, cudaStream_t);
+template void factor_solve<float>(const FactorPlan &, const float *, float *, float *, float *, cudaStream_t);
+
+void factor_solve8(const FactorPlan &P, const double *L, double *b, double *y, double *x, int *d_err, cudaStream_t s) {
+    const int nlev = (int)P.levels.size();
+    for (int d = nlev - 1; d >= 0; --d) {
+        const Level &Lv = P.levels[d];
+        fwd_tc_level(Lv.d_fronts.p, (int)Lv.fronts.size(), P.d_fr.p, Lv.max_p, Lv.max_f, L, P.d_rows.p, b, y, d_err, s);
+    }
+    for (int d = 0; d < nlev; ++d) {
+        const Level &Lv = P.levels[d];
+        bwd_tc_level(Lv.d_fronts.p, (int)Lv.fronts.size(), P.d_fr.p, Lv.max_p, Lv.max_f, L, P.d_rows.p, y, x, d_err, s);
     }
 }
-
-template void factor_solve<double>(const FactorPlan &, const double *, double *, double *, double *, int,
-                                   cudaStream_t);
-template void factor_solve<float>(const FactorPlan &, const float *, float *, float *, float *, int, cudaStream_t);
 
 // ----------------------------------------------------------------- local <-> global
 

@@ -168,7 +168,16 @@ void wpanel_tc_level(const int *d_fronts, int n_fronts, const FrontDesc *d_fr, i
 // concatenated local vectors).  b is overwritten; y (scratch) and x must be
 // zero on entry.
 template <class T>
-void factor_solve(const FactorPlan &P, const T *L, T *b, T *y, T *x, int kcols, cudaStream_t s);
+void factor_solve(const FactorPlan &P, const T *L, T *b, T *y, T *x, cudaStream_t s);
+// The same for eight vectors per subdomain, each of the subdomain's length and
+// stored one after the other: b[vec_off*8 + v*n + i].  d_err is set to 2 if a
+// wait on the tensor cores gave up.
+void factor_solve8(const FactorPlan &P, const double *L, double *b, double *y, double *x, int *d_err, cudaStream_t s);
+// One level's forward and backward step of factor_solve8 on the tensor cores (gemm64_tc.cu).
+void fwd_tc_level(const int *d_fronts, int n_fronts, const FrontDesc *d_fr, int max_p, int max_f, const double *L,
+                  const int *rows, double *b, double *y, int *d_err, cudaStream_t s);
+void bwd_tc_level(const int *d_fronts, int n_fronts, const FrontDesc *d_fr, int max_p, int max_f, const double *L,
+                  const int *rows, const double *y, double *x, int *d_err, cudaStream_t s);
 
 // Switch the per-level sweep timing on (resetting it) or off.
 void level_clock_enable(FactorPlan &P, bool on);

@@ -38,6 +38,8 @@
 // product instead of converting both halves made them up to 100 times larger.
 #include <cuda_fp16.h>
 
+#include <algorithm>
+
 #include "factor.h"
 
 namespace gl {
@@ -73,12 +75,13 @@ __device__ __forceinline__ uint64_t oz_desc(uint32_t addr) {
 // both K-major, N >> 3 at bit 17, M >> 4 at bit 24.
 constexpr uint32_t OZ_IDESC = (1u << 4) | ((uint32_t)(OZ_N >> 3) << 17) | ((uint32_t)(OZ_M >> 4) << 24);
 
-__device__ __forceinline__ void oz_mma(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t accumulate) {
+__device__ __forceinline__ void oz_mma(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t accumulate,
+                                       uint32_t idesc = OZ_IDESC) {
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
         "setp.ne.b32 p, %4, 0;\n\t"
         "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d_tmem),
-        "l"(a), "l"(b), "r"(OZ_IDESC), "r"(accumulate));
+        "l"(a), "l"(b), "r"(idesc), "r"(accumulate));
 }
 
 __device__ __forceinline__ bool oz_wait(uint32_t mbar, uint32_t parity) {
@@ -100,6 +103,12 @@ __device__ __forceinline__ bool oz_wait(uint32_t mbar, uint32_t parity) {
 __device__ __forceinline__ void oz_tmem_ld8(uint32_t taddr, uint32_t r[8]) {
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(taddr));
+}
+
+__device__ __forceinline__ void oz_tmem_ld4(uint32_t taddr, uint32_t r[4]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
                  : "r"(taddr));
 }
 
@@ -266,10 +275,11 @@ __device__ __forceinline__ double oz_pow2(int x) {
     return x > -1023 ? __longlong_as_double((int64_t)(min(x, 1023) + 1023) << 52) : 0.0;
 }
 
-__device__ __forceinline__ unsigned char *oz_begin(OzShared &S, unsigned char *raw) {
+template <int COLS, class Sh>
+__device__ __forceinline__ unsigned char *oz_begin(Sh &S, unsigned char *raw) {
     if (threadIdx.x < 32) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(oz_smem(&S.tmem)),
-                     "r"(OZ_TMEM_COLS));
+                     "r"(COLS));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
     if (threadIdx.x == 0) {
@@ -283,13 +293,14 @@ __device__ __forceinline__ unsigned char *oz_begin(OzShared &S, unsigned char *r
     return reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(raw) + 1023) & ~static_cast<uintptr_t>(1023));
 }
 
-__device__ __forceinline__ void oz_end(OzShared &S, bool ok, int *err) {
+template <int COLS, class Sh>
+__device__ __forceinline__ void oz_end(Sh &S, bool ok, int *err) {
     if (!ok && threadIdx.x == 0) atomicExch(err, 2);
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     if (threadIdx.x < 32) {
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(S.tmem), "r"(OZ_TMEM_COLS));
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(S.tmem), "r"(COLS));
     }
 }
 
@@ -314,7 +325,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 2) k_syrk64_tc(const int *__restri
     double *F = ws + d.front_off;
     extern __shared__ unsigned char oz_raw[];
     __shared__ OzShared S;
-    unsigned char *sm = oz_begin(S, oz_raw);
+    unsigned char *sm = oz_begin<OZ_TMEM_COLS>(S, oz_raw);
     uint32_t phase = 0u;
     const int r = r0 + 32 * ((threadIdx.x >> 5) & 3) + (threadIdx.x & 31), cw = c0 + 16 * (threadIdx.x >> 7);
     double e[16];   // the thread's entries of F, loaded while the products are formed
@@ -329,7 +340,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 2) k_syrk64_tc(const int *__restri
             if (r < f && cw + c <= r)
                 F[r + (int64_t)(cw + c) * f] = fma((double)hi, -oz_pow2(x + 32), fma((double)lo, -oz_pow2(x), e[c]));
         });
-    oz_end(S, ok, err);
+    oz_end<OZ_TMEM_COLS>(S, ok, err);
 }
 
 // W = L21 L11^{-1}: rows p .. f of the panel, from L21 in the front and the
@@ -348,7 +359,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 2) k_wpanel_tc(const int *__restri
     double *O = out + d.l_off;
     extern __shared__ unsigned char oz_raw[];
     __shared__ OzShared S;
-    unsigned char *sm = oz_begin(S, oz_raw);
+    unsigned char *sm = oz_begin<OZ_TMEM_COLS>(S, oz_raw);
     uint32_t phase = 0u;
     const int r = r0 + 32 * ((threadIdx.x >> 5) & 3) + (threadIdx.x & 31), cw = c0 + 16 * (threadIdx.x >> 7);
     double acc[16];
@@ -369,7 +380,254 @@ __global__ void __launch_bounds__(OZ_THREADS, 2) k_wpanel_tc(const int *__restri
         for (int j = 0; j < 16; ++j)
             if (cw + j < p) O[r + (int64_t)(cw + j) * f] = acc[j];
     }
-    oz_end(S, ok, err);
+    oz_end<OZ_TMEM_COLS>(S, ok, err);
+}
+
+// ---------------------------------------------------------------- sweeps with eight right-hand sides
+
+// The panel times OZ_V vectors: the digits of the vectors are the columns of
+// one operand (row 8 j + v: digit j of vector v), so that digit i of the panel
+// times its digit groups, added 8 i columns further in tensor memory, collects
+// every weight i + j <= 7 of a vector in one column.  (The columns of D and N
+// stay multiples of 16: odd digits have accumulators of their own.)  A CTA takes
+// 128 panel rows (forward) or columns (backward) and a chunk of the summed ones,
+// 64 at a time, held in registers while their largest exponents are found.
+// With eight accumulators a lane on the FP64 pipe (8 of its FMAs an entry, 512
+// pipe clocks a warp and 32 entries) a launch took 138 us forward and 131 us
+// backward on the 63k-DOF corner's eigensolver, this form 73 and 94 us, about
+// 50 integer instructions an entry for its digits, which now bind it together
+// with reading the panel; backward its 64-byte lane stride costs the rest.  The
+// small levels gain too (20k-DOF plate: 42 to 23 and 44 to 27 us), so there is
+// no second form.
+constexpr int OZ_V = 8;
+constexpr int OZ_VK = 64;                   // summed entries held in registers per accumulation
+constexpr int OZ_MV_CTAS = 152 * 16;        // wanted per level (4 and 8 an SM: 3% and 2% slower over a sweep)
+constexpr int OZ_MV_COLS = 128;             // of tensor memory
+constexpr int OZ_MV_SMEM = OZ_S * OZ_A_BYTES + OZ_S * OZ_V * OZ_KC * 2 + 1024;
+
+struct OzMvShared {
+    int ea[2][OZ_M], eb[2][OZ_V];           // largest exponents, alternating between accumulations
+    uint32_t tmem;
+    __align__(8) uint64_t mbar;
+    int failed;
+};
+
+// out[v] = sum over k in [k0, k1) of A(i, k) X(k, 4 (warp / 4) + v), v < 4, for
+// row i = 32 (warp % 4) + lane of the tile.  unit(pass) = the (row, group of
+// eight columns) this thread stages, 2 passes per round; rows from `used` on are
+// left out.  A and X return 0 out of range.  Returns false if a wait gave up.
+template <class FA, class FX, class Unit>
+__device__ bool oz_mv(OzMvShared &S, unsigned char *sm, FA A, FX X, Unit unit, int used, int k0, int k1,
+                      double out[4]) {
+    constexpr int R = OZ_VK / OZ_KC;
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int xv = lane & 7, xg = lane >> 3;          // warps 0 .. R-1, a round each: vector, group of eight
+    int row[2], grp[2];
+    unit(0, row[0], grp[0]);
+    unit(1, row[1], grp[1]);
+    double a[R][2][8], xr[8];
+    auto load = [&](int kb) {
+#pragma unroll
+        for (int h = 0; h < R; ++h)
+#pragma unroll
+            for (int q = 0; q < 2; ++q)
+#pragma unroll
+                for (int j = 0; j < 8; ++j)
+                    a[h][q][j] = row[q] < used ? A(row[q], kb + OZ_KC * h + 8 * grp[q] + j) : 0.0;
+        if (warp < R)
+#pragma unroll
+            for (int j = 0; j < 8; ++j) xr[j] = X(kb + OZ_KC * warp + 8 * xg + j, xv);
+    };
+    auto expo = [](double x) { return (int)((uint64_t)__double_as_longlong(x) >> 52) & 0x7FF; };
+#pragma unroll
+    for (int j = 0; j < 4; ++j) out[j] = 0.0;
+    for (int i = t; i < 2 * OZ_M; i += OZ_THREADS) S.ea[i / OZ_M][i % OZ_M] = 0;
+    if (t < 2 * OZ_V) S.eb[t / OZ_V][t % OZ_V] = 0;
+    load(k0);
+    __syncthreads();
+    unsigned char *pa = sm, *pb = sm + OZ_S * OZ_A_BYTES;
+    uint32_t phase = 0u;
+    int w = 0;
+    for (int kb = k0; kb < k1; kb += OZ_VK, w ^= 1) {
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            int e = 0;
+#pragma unroll
+            for (int h = 0; h < R; ++h)
+#pragma unroll
+                for (int j = 0; j < 8; ++j) e = max(e, expo(a[h][q][j]));
+            if (e) atomicMax(&S.ea[w][row[q]], e);
+        }
+        if (warp < R) {
+            int e = 0;
+#pragma unroll
+            for (int j = 0; j < 8; ++j) e = max(e, expo(xr[j]));
+            if (e) atomicMax(&S.eb[w][xv], e);
+        }
+        __syncthreads();
+        if (t < OZ_M) S.ea[w ^ 1][t] = 0;
+        if (t < OZ_V) S.eb[w ^ 1][t] = 0;
+#pragma unroll
+        for (int h = 0; h < R; ++h) {
+            if (kb + OZ_KC * h >= k1) break;
+            if (h > 0) {            // until the tensor cores have read the last round's digits
+                if (!oz_wait(oz_smem(&S.mbar), phase)) S.failed = 1;
+                phase ^= 1u;
+                __syncthreads();
+                if (S.failed) return false;
+            }
+#pragma unroll
+            for (int q = 0; q < 2; ++q)
+                if (row[q] < used) {
+                    const int e = S.ea[w][row[q]];
+                    uint64_t u[8];
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) u[j] = oz_fixed(a[h][q][j], e);
+                    oz_stage8(u, pa + oz_off(row[q], grp[q]), OZ_A_BYTES);
+                }
+            if (warp == h) {
+                const int e = S.eb[w][xv];
+                uint64_t u[8];
+#pragma unroll
+                for (int j = 0; j < 8; ++j) u[j] = oz_fixed(xr[j], e);
+                oz_stage8(u, pb + oz_off(xv, xg), OZ_SBO);
+            }
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            __syncthreads();
+            if (t == 0) {
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                const uint32_t a0 = oz_smem(pa), b0 = oz_smem(pb);
+#pragma unroll 1
+                for (int s = 0; s < OZ_KC / 16; ++s) {
+                    const uint32_t ko = (uint32_t)(2 * s) * OZ_LBO;
+#pragma unroll 1
+                    for (int i = 0; i < OZ_S; ++i) {
+                        // even digits into columns 0-63, odd ones, one weight lower, into 64-127
+                        const int n = OZ_S * OZ_V - OZ_V * (i & ~1);
+                        const uint32_t idesc = (1u << 4) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(OZ_M >> 4) << 24);
+                        oz_mma(S.tmem + (i & 1) * OZ_S * OZ_V + OZ_V * (i & ~1), oz_desc(a0 + i * OZ_A_BYTES + ko),
+                               oz_desc(b0 + ko), h > 0 || s > 0 || i > 1 ? 1u : 0u, idesc);
+                    }
+                }
+                asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                                 oz_smem(&S.mbar))
+                             : "memory");
+            }
+        }
+        if (kb + OZ_VK < k1) load(kb + OZ_VK);
+        if (!oz_wait(oz_smem(&S.mbar), phase)) S.failed = 1;
+        phase ^= 1u;
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        __syncthreads();
+        if (S.failed) return false;
+        const int er = S.ea[w][32 * (warp & 3) + lane], v0 = 4 * (warp >> 2);
+        const uint32_t tm = S.tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)v0;
+        int64_t hi[4] = {0, 0, 0, 0}, lo[4] = {0, 0, 0, 0};
+#pragma unroll
+        for (int s4 = 0; s4 < 2; ++s4) {
+            uint32_t r[4][4], o[4][4];
+#pragma unroll
+            for (int s = 0; s < 4; ++s) {
+                oz_tmem_ld4(tm + OZ_V * (4 * s4 + s), r[s]);
+                if (s4 + s > 0) oz_tmem_ld4(tm + OZ_V * (OZ_S + 4 * s4 + s - 1), o[s]);
+                else o[s][0] = o[s][1] = o[s][2] = o[s][3] = 0u;
+            }
+            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+            for (int s = 0; s < 4; ++s)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    int64_t &z = s4 ? lo[j] : hi[j];
+                    z = (z << 8) + __float2int_rn(__uint_as_float(r[s][j])) + __float2int_rn(__uint_as_float(o[s][j]));
+                }
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int ec = S.eb[w][v0 + j];
+            const int x = er == 0x7FF || ec == 0x7FF ? OZ_NOT : (er == 0 || ec == 0 ? OZ_NONE : er + ec - 2112);
+            out[j] = fma((double)hi[j], oz_pow2(x + 32), fma((double)lo[j], oz_pow2(x), out[j]));
+        }
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");   // the next products overwrite them
+    }
+    return true;
+}
+
+// Forward step (k_fwd of the single sweep) with eight vectors: panel rows
+// [128 blockIdx.y, ...), pivots [chunk blockIdx.z, ...).
+__global__ void __launch_bounds__(OZ_THREADS, 2) k_fwd_tc(const int *__restrict__ fronts,
+                                                          const FrontDesc *__restrict__ D,
+                                                          const double *__restrict__ L, const int *__restrict__ rows,
+                                                          double *b, double *y, int chunk, int *__restrict__ err) {
+    const FrontDesc &d = D[fronts[blockIdx.x]];
+    const int p = d.p, f = p + d.q, n = d.vlen;
+    const int r0 = blockIdx.y * OZ_M, k0 = blockIdx.z * chunk;
+    // pivot rows need the pivots up to their own tile, structure rows all
+    const int k1 = min(k0 + chunk, r0 + OZ_M <= p ? r0 + OZ_M : p);
+    if (r0 >= f || k0 >= k1) return;
+    extern __shared__ unsigned char oz_raw[];
+    __shared__ OzMvShared S;
+    unsigned char *sm = oz_begin<OZ_MV_COLS>(S, oz_raw);
+    const double *Lr = L + d.l_off + r0;
+    const int64_t vo = d.vec_off * OZ_V;
+    const double *b1 = b + vo + d.first;
+    const int used = min(OZ_M, f - r0), t = threadIdx.x;
+    double out[4];
+    const bool ok = oz_mv(
+        S, sm, [&](int i, int k) { return k < k1 && k <= r0 + i ? Lr[i + (int64_t)k * f] : 0.0; },
+        [&](int k, int v) { return k < k1 ? b1[k + (int64_t)v * n] : 0.0; },
+        [&](int pass, int &row, int &grp) {
+            row = t & (OZ_M - 1);
+            grp = (t >> 7) + 2 * pass;
+        },
+        used, k0, k1, out);
+    const int i = 32 * ((t >> 5) & 3) + (t & 31), row = r0 + i, v0 = 4 * (t >> 7);
+    if (ok && i < used) {
+        double *o = row < p ? y + vo + d.first + row : b + vo + rows[d.row_off + row];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) atomicAdd(o + (int64_t)(v0 + j) * n, row < p ? out[j] : -out[j]);
+    }
+    oz_end<OZ_MV_COLS>(S, ok, err);
+}
+
+// Backward step with eight vectors: panel columns [128 blockIdx.y, ...), panel
+// rows [chunk blockIdx.z, ...).
+__global__ void __launch_bounds__(OZ_THREADS, 2) k_bwd_tc(const int *__restrict__ fronts,
+                                                          const FrontDesc *__restrict__ D,
+                                                          const double *__restrict__ L, const int *__restrict__ rows,
+                                                          const double *__restrict__ y, double *x,
+                                                          int chunk, int *__restrict__ err) {
+    const FrontDesc &d = D[fronts[blockIdx.x]];
+    const int p = d.p, f = p + d.q, n = d.vlen;
+    const int j0 = blockIdx.y * OZ_M, k1 = min((int)(blockIdx.z + 1) * chunk, f);
+    const int k0 = max((int)blockIdx.z * chunk, j0);   // zeros above the diagonal
+    if (j0 >= p || k0 >= k1) return;
+    extern __shared__ unsigned char oz_raw[];
+    __shared__ OzMvShared S;
+    unsigned char *sm = oz_begin<OZ_MV_COLS>(S, oz_raw);
+    const double *Lt = L + d.l_off + (int64_t)j0 * f;
+    const int64_t vo = d.vec_off * OZ_V;
+    const double *y1 = y + vo + d.first, *xo = x + vo;
+    const int *rw = rows + d.row_off;
+    const int used = min(OZ_M, p - j0), t = threadIdx.x;
+    double out[4];
+    const bool ok = oz_mv(
+        S, sm, [&](int i, int k) { return k < k1 && k >= j0 + i ? Lt[k + (int64_t)i * f] : 0.0; },
+        [&](int k, int v) {
+            if (k >= k1) return 0.0;
+            return k < p ? y1[k + (int64_t)v * n] : -xo[rw[k] + (int64_t)v * n];
+        },
+        [&](int pass, int &row, int &grp) {   // four threads a column: 256 contiguous bytes
+            row = (t >> 2) + 64 * pass;
+            grp = t & 3;
+        },
+        used, k0, k1, out);
+    const int i = 32 * ((t >> 5) & 3) + (t & 31), v0 = 4 * (t >> 7);
+    if (ok && i < used) {
+        double *o = x + vo + d.first + j0 + i;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) atomicAdd(o + (int64_t)(v0 + j) * n, out[j]);
+    }
+    oz_end<OZ_MV_COLS>(S, ok, err);
 }
 
 void oz_smem_limit() {
@@ -377,6 +635,8 @@ void oz_smem_limit() {
     lim.ensure(OZ_SMEM, [](size_t v) {
         GL_CUDA(cudaFuncSetAttribute(k_syrk64_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)v));
         GL_CUDA(cudaFuncSetAttribute(k_wpanel_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)v));
+        GL_CUDA(cudaFuncSetAttribute(k_fwd_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, OZ_MV_SMEM));
+        GL_CUDA(cudaFuncSetAttribute(k_bwd_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, OZ_MV_SMEM));
     });
 }
 
@@ -398,6 +658,33 @@ void wpanel_tc_level(const int *d_fronts, int n_fronts, const FrontDesc *d_fr, i
     const int tiles = ((max_f + OZ_M - 1) / OZ_M) * ((max_p + OZ_N - 1) / OZ_N);
     if (tiles <= 0) return;
     k_wpanel_tc<<<dim3(n_fronts, tiles), OZ_THREADS, OZ_SMEM, s>>>(d_fronts, d_fr, ws, out, d_err);
+    GL_CUDA(cudaGetLastError());
+}
+
+// Summed entries per CTA: whole accumulations, cut finer while the level has too few CTAs.
+static int oz_chunk(int64_t ctas, int n) {
+    const int blocks = (n + OZ_VK - 1) / OZ_VK;
+    const int split = (int)std::min<int64_t>(blocks, std::max<int64_t>(1, OZ_MV_CTAS / ctas));
+    return OZ_VK * ((blocks + split - 1) / split);
+}
+
+void fwd_tc_level(const int *d_fronts, int n_fronts, const FrontDesc *d_fr, int max_p, int max_f, const double *L,
+                  const int *rows, double *b, double *y, int *d_err, cudaStream_t s) {
+    if (n_fronts == 0 || max_p == 0) return;
+    oz_smem_limit();
+    const int tiles = (max_f + OZ_M - 1) / OZ_M, chunk = oz_chunk((int64_t)n_fronts * tiles, max_p);
+    k_fwd_tc<<<dim3(n_fronts, tiles, (max_p + chunk - 1) / chunk), OZ_THREADS, OZ_MV_SMEM, s>>>(d_fronts, d_fr, L, rows,
+                                                                                              b, y, chunk, d_err);
+    GL_CUDA(cudaGetLastError());
+}
+
+void bwd_tc_level(const int *d_fronts, int n_fronts, const FrontDesc *d_fr, int max_p, int max_f, const double *L,
+                  const int *rows, const double *y, double *x, int *d_err, cudaStream_t s) {
+    if (n_fronts == 0 || max_p == 0) return;
+    oz_smem_limit();
+    const int tiles = (max_p + OZ_M - 1) / OZ_M, chunk = oz_chunk((int64_t)n_fronts * tiles, max_f);
+    k_bwd_tc<<<dim3(n_fronts, tiles, (max_f + chunk - 1) / chunk), OZ_THREADS, OZ_MV_SMEM, s>>>(d_fronts, d_fr, L, rows,
+                                                                                              y, x, chunk, d_err);
     GL_CUDA(cudaGetLastError());
 }
 

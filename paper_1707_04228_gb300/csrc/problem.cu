@@ -272,7 +272,7 @@ void problem_coarse(const Problem &P, const gl_opts &o, const FactorPlan &PD, st
             GL_CUDA(cudaMemcpyAsync(MW.p, BW.p, sizeof(double) * gl * KRY_B, cudaMemcpyDeviceToDevice, s));
             W.zero(s);
             ysc.zero(s);
-            factor_solve<double>(PG, LN.p, MW.p, ysc.p, W.p, KRY_B, s);
+            factor_solve8(PG, LN.p, MW.p, ysc.p, W.p, P.d_err, s);
             ++it;
             // first pass: M W = B W_last up to the solve's error, so G is good for the residuals and a first scaling
             H.zero(s);

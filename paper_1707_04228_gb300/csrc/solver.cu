@@ -341,7 +341,7 @@ template <class T>
 void local_solve(const FactorPlan &P, const T *L, T *xl, const double *r, double *z, cudaStream_t s) {
     T *b = xl, *y = xl + P.n_local, *x = xl + 2 * P.n_local;
     gather_local<T>(P, r, b, y, x, s);
-    factor_solve<T>(P, L, b, y, x, 1, s);
+    factor_solve<T>(P, L, b, y, x, s);
     scatter_add_local<T>(P, x, z, s);
 }
 
