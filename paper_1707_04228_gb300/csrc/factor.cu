@@ -511,6 +511,7 @@ __global__ void __launch_bounds__(32) k_diag_inverse(const int *__restrict__ fro
 // above down, X_k = -L_kk^{-1} sum_{m=J}^{k-1} L_km X_m (the diagonal blocks'
 // inverses are in place).  One CTA per (front, tile); the chain over k is the
 // CTA's own, so tiles need no other synchronisation.  Rows above J are zeroed.
+// (FP32 storage; FP64 on the tensor cores, k_trinv_tc.)
 template <class T>
 __global__ void __launch_bounds__(INV_THREADS) k_tri_inverse(const int *__restrict__ fronts,
                                                              const FrontDesc *__restrict__ D,
@@ -625,15 +626,16 @@ __global__ void __launch_bounds__(256) k_wpanel(const int *__restrict__ fronts, 
 }
 
 template <class T>
-static void inverse_form_level(const int *d_fronts, int nf, const FrontDesc *d_fr, int max_p, int max_f, const T *ws,
+static void inverse_form_level(const int *d_fronts, int nf, const FrontDesc *d_fr, int max_p, int max_f, T *ws,
                                T *L, int *d_err, cudaStream_t s) {
     const int nb = (max_p + 31) / 32;
     if (nb == 0) return;
     k_diag_inverse<T><<<dim3(nf, nb), 32, 0, s>>>(d_fronts, d_fr, ws, L);
-    k_tri_inverse<T><<<dim3(nf, nb), INV_THREADS, 0, s>>>(d_fronts, d_fr, ws, L);
     if constexpr (sizeof(T) == 8) {
+        trinv_tc_level(d_fronts, nf, d_fr, max_p, ws, L, d_err, s);
         wpanel_tc_level(d_fronts, nf, d_fr, max_p, max_f, ws, L, d_err, s);
     } else {
+        k_tri_inverse<T><<<dim3(nf, nb), INV_THREADS, 0, s>>>(d_fronts, d_fr, ws, L);
         // upper bound of row tiles x column tiles over the level's fronts (q <= max_f, p <= max_p)
         const int tiles = ((max_f + TILE - 1) / TILE) * ((max_p + TILE - 1) / TILE);
         k_wpanel<T><<<dim3(nf, tiles), 256, 0, s>>>(d_fronts, d_fr, ws, L);

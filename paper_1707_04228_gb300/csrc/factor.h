@@ -156,9 +156,13 @@ void syrk_tc_level(const int *d_fronts, int n_fronts, const FrontDesc *d_fr, int
 
 // FP64 products of a level's fronts on the tensor cores (gemm64_tc.cu): the
 // trailing update by the kw = min(panel, p - k0) factored columns from k0 on,
-// and W = L21 L11^{-1} of the inverse-form panels.  panel <= 128; d_err as above.
+// L11^{-1} from its inverted 32 x 32 diagonal blocks (overwrites the fronts'
+// upper triangles) and W = L21 L11^{-1} of the inverse-form panels.  panel <=
+// 128; d_err as above.
 void syrk64_tc_level(const int *d_fronts, int n_fronts, const FrontDesc *d_fr, int k0, int panel, int max_f, double *ws,
                      int *d_err, cudaStream_t s);
+void trinv_tc_level(const int *d_fronts, int n_fronts, const FrontDesc *d_fr, int max_p, double *ws, double *out,
+                    int *d_err, cudaStream_t s);
 void wpanel_tc_level(const int *d_fronts, int n_fronts, const FrontDesc *d_fr, int max_p, int max_f, const double *ws,
                      double *out, int *d_err, cudaStream_t s);
 

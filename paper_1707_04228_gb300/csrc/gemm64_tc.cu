@@ -160,15 +160,18 @@ struct OzShared {
 // thread's row 32 (warp % 4) + lane and columns 16 (warp / 4) + c through
 // put(c, hi, lo, x): the sum is (hi 2^32 + lo) 2^x (x OZ_NONE: zero, OZ_NOT: not
 // a number).
-// A and B return 0 out of range; before_wait() runs while the products are
+// PART: rows from `used` on (whole warps of them) are left out; a row of the
+// result needs no other row of A.  (Always testing it cost the trailing updates
+// 15%.)  A and B return 0 out of range; before_wait() runs while the products are
 // still being formed.  Returns false if a wait gave up.
 constexpr int OZ_NONE = -100000, OZ_NOT = 100000;
 
-template <class FA, class FB, class Pre, class Put>
-__device__ bool oz_block(OzShared &S, unsigned char *sm, uint32_t &phase, FA A, FB B, int k0, int k1, Pre before_wait,
-                         Put put) {
+template <bool PART, class FA, class FB, class Pre, class Put>
+__device__ bool oz_block(OzShared &S, unsigned char *sm, uint32_t &phase, int used, FA A, FB B, int k0, int k1,
+                         Pre before_wait, Put put) {
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const int ra = t & (OZ_M - 1), ha = t >> 7;      // A: two threads per row, 16 columns each
+    const bool live = !PART || (ra & ~31) < used;
     const int rb = t & (OZ_N - 1), hb = t >> 5;      // B: four threads per row, 8 columns each (warps 0-3)
     if (t < OZ_M) S.ea[t] = 0;
     if (t < OZ_N) S.eb[t] = 0;
@@ -179,7 +182,7 @@ __device__ bool oz_block(OzShared &S, unsigned char *sm, uint32_t &phase, FA A, 
         for (int kc = k0; kc < k1; kc += OZ_KC) {
 #pragma unroll
             for (int j = 0; j < 16; ++j)
-                ma = max(ma, (int)((uint64_t)__double_as_longlong(A(ra, kc + 16 * ha + j)) >> 52) & 0x7FF);
+                if (live) ma = max(ma, (int)((uint64_t)__double_as_longlong(A(ra, kc + 16 * ha + j)) >> 52) & 0x7FF);
             if (warp < 4)
 #pragma unroll
                 for (int j = 0; j < 8; ++j)
@@ -200,6 +203,7 @@ __device__ bool oz_block(OzShared &S, unsigned char *sm, uint32_t &phase, FA A, 
         }
 #pragma unroll
         for (int g = 0; g < 2; ++g) {
+            if (!live) break;
             uint64_t u[8];
 #pragma unroll
             for (int j = 0; j < 8; ++j) u[j] = oz_fixed(A(ra, kc + 16 * ha + 8 * g + j), ea);
@@ -246,6 +250,7 @@ __device__ bool oz_block(OzShared &S, unsigned char *sm, uint32_t &phase, FA A, 
     const uint32_t tm = S.tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)col0;
 #pragma unroll
     for (int cb = 0; cb < 16; cb += 8) {
+        if (PART && 32 * (warp & 3) >= used) break;
         uint32_t r[OZ_S][8];
 #pragma unroll
         for (int s = 0; s < OZ_S; ++s) oz_tmem_ld8(tm + OZ_N * s + cb, r[s]);
@@ -329,8 +334,8 @@ __global__ void __launch_bounds__(OZ_THREADS, 2) k_syrk64_tc(const int *__restri
     uint32_t phase = 0u;
     const int r = r0 + 32 * ((threadIdx.x >> 5) & 3) + (threadIdx.x & 31), cw = c0 + 16 * (threadIdx.x >> 7);
     double e[16];   // the thread's entries of F, loaded while the products are formed
-    const bool ok = oz_block(
-        S, sm, phase, [&](int i, int k) { return r0 + i < f && k < base ? F[r0 + i + (int64_t)k * f] : 0.0; },
+    const bool ok = oz_block<false>(
+        S, sm, phase, OZ_M, [&](int i, int k) { return r0 + i < f && k < base ? F[r0 + i + (int64_t)k * f] : 0.0; },
         [&](int i, int k) { return c0 + i < f && k < base ? F[c0 + i + (int64_t)k * f] : 0.0; }, k0, base,
         [&]() {
 #pragma unroll
@@ -368,8 +373,8 @@ __global__ void __launch_bounds__(OZ_THREADS, 2) k_wpanel_tc(const int *__restri
     bool ok = true;
     for (int kb = c0; kb < p && ok; kb += OZ_KB) {
         const int ke = min(p, kb + OZ_KB);
-        ok = oz_block(
-            S, sm, phase, [&](int i, int k) { return r0 + i < f && k < ke ? F[r0 + i + (int64_t)k * f] : 0.0; },
+        ok = oz_block<false>(
+            S, sm, phase, OZ_M, [&](int i, int k) { return r0 + i < f && k < ke ? F[r0 + i + (int64_t)k * f] : 0.0; },
             [&](int i, int k) { return c0 + i < p && k < ke ? O[k + (int64_t)(c0 + i) * f] : 0.0; }, kb, ke, []() {},
             [&](int c, int64_t hi, int64_t lo, int x) {
                 acc[c] = fma((double)hi, oz_pow2(x + 32), fma((double)lo, oz_pow2(x), acc[c]));
@@ -379,6 +384,66 @@ __global__ void __launch_bounds__(OZ_THREADS, 2) k_wpanel_tc(const int *__restri
 #pragma unroll
         for (int j = 0; j < 16; ++j)
             if (cw + j < p) O[r + (int64_t)(cw + j) * f] = acc[j];
+    }
+    oz_end<OZ_TMEM_COLS>(S, ok, err);
+}
+
+// L11^{-1} from its inverted 32 x 32 diagonal blocks by doubling: with the
+// inverses X11, X22 of two neighbouring blocks of b pivots in place, the block
+// below the diagonal is X21 = -X22 (L21 X11).  STEP 0 forms the bracket, kept
+// transposed in the front's unused upper triangle, STEP 1 the product; one CTA
+// per (front, pair, 128 x 32 tile), two launches per doubling.  Block column by
+// block column in one CTA each, the FP64 pipe of one SM held a chain of up to
+// (p / 32)^2 / 2 block products: 443 us a level on the 63k-DOF corner, 294 us
+// in this form (about six launches), which the latency of a tile binds.
+template <int STEP>
+__global__ void __launch_bounds__(OZ_THREADS, 2) k_trinv_tc(const int *__restrict__ fronts,
+                                                            const FrontDesc *__restrict__ D, double *ws, double *out,
+                                                            int b, int *__restrict__ err) {
+    const FrontDesc &d = D[fronts[blockIdx.x]];
+    const int p = d.p, f = d.p + d.q;
+    const int ct = b / OZ_N, tiles = ct * ((b + OZ_M - 1) / OZ_M), pair = blockIdx.y / tiles, t = blockIdx.y % tiles;
+    const int base = 2 * b * pair, mid = base + b, end = min(p, mid + b);
+    const int r0 = mid + OZ_M * (t / ct), c0 = base + OZ_N * (t % ct);
+    if (r0 >= end) return;
+    double *F = ws + d.front_off, *O = out + d.l_off;
+    extern __shared__ unsigned char oz_raw[];
+    __shared__ OzShared S;
+    unsigned char *sm = oz_begin<OZ_TMEM_COLS>(S, oz_raw);
+    uint32_t phase = 0u;
+    const int r = r0 + 32 * ((threadIdx.x >> 5) & 3) + (threadIdx.x & 31), cw = c0 + 16 * (threadIdx.x >> 7);
+    double acc[16];
+#pragma unroll
+    for (int j = 0; j < 16; ++j) acc[j] = 0.0;
+    bool ok = true;
+    // summed pivots: block 1 from the tile's columns on, block 2 up to the tile's rows
+    const int k0 = STEP == 0 ? c0 : mid, k1 = STEP == 0 ? mid : min(end, r0 + OZ_M);
+    for (int kb = k0; kb < k1 && ok; kb += OZ_KB) {
+        const int ke = min(k1, kb + OZ_KB);
+        ok = oz_block<true>(
+            S, sm, phase, end - r0,
+            [&](int i, int k) {
+                if (r0 + i >= end || k >= ke) return 0.0;
+                if (STEP == 0) return F[r0 + i + (int64_t)k * f];
+                return k <= r0 + i ? O[r0 + i + (int64_t)k * f] : 0.0;
+            },
+            [&](int i, int k) {
+                if (k >= ke) return 0.0;
+                if (STEP == 0) return k >= c0 + i ? O[k + (int64_t)(c0 + i) * f] : 0.0;
+                return F[c0 + i + (int64_t)k * f];
+            },
+            kb, ke, []() {},
+            [&](int c, int64_t hi, int64_t lo, int x) {
+                acc[c] = fma((double)hi, oz_pow2(x + 32), fma((double)lo, oz_pow2(x), acc[c]));
+            });
+    }
+    if (ok && r < end) {
+        double *up = (STEP == 0 ? F : O) + (int64_t)r * f;      // the mirror entries: the bracket; zeros
+#pragma unroll
+        for (int j = 0; j < 16; ++j) {
+            up[cw + j] = STEP == 0 ? acc[j] : 0.0;
+            if (STEP == 1) O[r + (int64_t)(cw + j) * f] = -acc[j];
+        }
     }
     oz_end<OZ_TMEM_COLS>(S, ok, err);
 }
@@ -635,6 +700,8 @@ void oz_smem_limit() {
     lim.ensure(OZ_SMEM, [](size_t v) {
         GL_CUDA(cudaFuncSetAttribute(k_syrk64_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)v));
         GL_CUDA(cudaFuncSetAttribute(k_wpanel_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)v));
+        GL_CUDA(cudaFuncSetAttribute(k_trinv_tc<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)v));
+        GL_CUDA(cudaFuncSetAttribute(k_trinv_tc<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)v));
         GL_CUDA(cudaFuncSetAttribute(k_fwd_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, OZ_MV_SMEM));
         GL_CUDA(cudaFuncSetAttribute(k_bwd_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, OZ_MV_SMEM));
     });
@@ -649,6 +716,18 @@ void syrk64_tc_level(const int *d_fronts, int n_fronts, const FrontDesc *d_fr, i
     if (m <= 0) return;
     const int nt = (m + OZ_M - 1) / OZ_M;
     k_syrk64_tc<<<dim3(n_fronts, OZ_M / OZ_N * nt * (nt + 1) / 2), OZ_THREADS, OZ_SMEM, s>>>(d_fronts, d_fr, ws, k0, panel, d_err);
+    GL_CUDA(cudaGetLastError());
+}
+
+void trinv_tc_level(const int *d_fronts, int n_fronts, const FrontDesc *d_fr, int max_p, double *ws, double *out,
+                    int *d_err, cudaStream_t s) {
+    oz_smem_limit();
+    for (int b = 32; b < max_p; b *= 2) {
+        const int pairs = (max_p - b + 2 * b - 1) / (2 * b);     // pairs with a second block
+        const dim3 g(n_fronts, pairs * (b / OZ_N) * ((b + OZ_M - 1) / OZ_M));
+        k_trinv_tc<0><<<g, OZ_THREADS, OZ_SMEM, s>>>(d_fronts, d_fr, ws, out, b, d_err);
+        k_trinv_tc<1><<<g, OZ_THREADS, OZ_SMEM, s>>>(d_fronts, d_fr, ws, out, b, d_err);
+    }
     GL_CUDA(cudaGetLastError());
 }
 
