@@ -279,8 +279,9 @@ void problem_coarse(const Problem &P, const gl_opts &o, const FactorPlan &PD, st
             kry_gram(PG, MV.p, mmax, m, W.p, H.p, hs, KRY_B, s);
             kry_project(PG, first, mmax, m, H.p, hs, KRY_B, s);
             gram_block(BW.p);
-            // The Ritz pairs when they are needed: to restart, at the end, and as soon as the residuals can have got
-            // there -- they fall by less than 30 a step (3 to 10 as a rule).
+            // The Ritz pairs when they are needed: to restart, at the end, and when the residuals should have got
+            // there at 10 a step, the fastest they were seen to fall (3 to 10).  A pair costs 1.5 to 2 ms, a step 1 to
+            // 6; with 30 a step for the estimate two of six times were in vain.
             const bool last = it > iters && m >= nev;
             if (last || (m >= nev && m + KRY_B > mmax) || (m >= nev + KRY_B / 2 && it >= next_check)) {
                 kept = std::min(keep, m);
@@ -290,7 +291,7 @@ void problem_coarse(const Problem &P, const gl_opts &o, const FactorPlan &PD, st
                 check_err(P, "GenEO Rayleigh-Ritz");
                 std::memcpy(&resid, &bits, sizeof(resid));
                 if (resid <= EIG_RESID || last) break;
-                next_check = it + 1 + std::max(0, std::min(8, (int)(std::log(resid / EIG_RESID) / std::log(30.0))));
+                next_check = it + 1 + std::max(0, std::min(8, (int)(std::log10(resid / EIG_RESID))));
             }
             kry_orth(ng, G.p, H.p, hs, KRY_B, m, 1e-24, R.p, P.d_err, s);
             kry_scale(PG, only_w, R.p, mmax, -1, s);
