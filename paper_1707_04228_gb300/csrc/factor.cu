@@ -759,13 +759,20 @@ template void numeric_factor<float>(FactorPlan &, const double *, const double *
 constexpr int SWEEP_CTA = 128;            // four warp tasks
 constexpr int SWEEP_WARPS = 152 * 96;
 
-// Forward: panel rows [r0, r0 + 32), lane = row, the columns of blockIdx.z's
+// Forward: panel rows [r0, r0 + 32 R), lane = row (R rows), the columns of blockIdx.z's
 // chunk.  Pivot rows give y_1 = L11^{-1} b_1 (up to the diagonal block: zeros
 // above it), structure rows subtract W b_1 from the ancestors' entries of b.
 // FP64: one FMA per entry on a pipe of two per clock and SM binds it at every
 // size that fills the chip; FP32 is bound by reading the panel once.  One CTA
 // per front stepping through 32-pivot blocks took 74 us (FP64) and 62 us (FP32)
 // a launch on the 308k- and 475k-DOF corners, this form 44 and 25 us.
+// Rows per lane of a forward task: two in FP32, 256 contiguous bytes a column,
+// which HBM likes better: 9.74 to 8.78 ms for all levels of the 12.2M-DOF corner
+// (one level after another), and no slower on the 475k-DOF one.  Four gained 2%
+// more there and cost 4% here.
+template <class T>
+constexpr int FWD_ROWS = sizeof(T) == 4 ? 2 : 1;
+
 template <class T>
 __global__ void __launch_bounds__(SWEEP_CTA) k_fwd(const int *__restrict__ fronts, const FrontDesc *__restrict__ D,
                                                    const T *__restrict__ L, const int *__restrict__ rows, T *b,
@@ -774,31 +781,37 @@ __global__ void __launch_bounds__(SWEEP_CTA) k_fwd(const int *__restrict__ front
     const FrontDesc &d = D[fronts[blockIdx.x]];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int p = d.p, f = p + d.q;
-    const int r0 = (blockIdx.y * (SWEEP_CTA / 32) + w) * 32;
+    constexpr int R = FWD_ROWS<T>, RT = 32 * R;      // rows per lane, per warp task
+    const int r0 = (blockIdx.y * (SWEEP_CTA / 32) + w) * RT;
     const int cb = blockIdx.z * chunk;
     // pivot rows need the columns up to their diagonal block, any structure row all of them
-    const int cend = min(r0 + 32 <= p ? r0 + 32 : p, cb + chunk);
+    const int cend = min(r0 + RT <= p ? r0 + RT : p, cb + chunk);
     if (r0 >= f || cb >= cend) {
         cudaGridDependencySynchronize();
         return;
     }
     const T *b1 = b + d.vec_off + d.first;
-    const int row = min(r0 + lane, f - 1);
-    const T *Lr = L + d.l_off + row;
-    constexpr int G = sizeof(T) == 4 ? 32 : 16;   // loads in flight per lane
-    T l[G];
+    const T *Lr[R];
+#pragma unroll
+    for (int q = 0; q < R; ++q) Lr[q] = L + d.l_off + min(r0 + lane + 32 * q, f - 1);
+    constexpr int G = sizeof(T) == 4 ? 32 / R : 16;   // columns in flight per lane
+    T l[R][G];
     // the panel does not depend on the launches before: its first columns are on their way during the wait
 #pragma unroll
-    for (int j = 0; j < G; ++j) l[j] = cb + j < cend ? Lr[(int64_t)(cb + j) * f] : T(0);
+    for (int j = 0; j < G; ++j)
+#pragma unroll
+        for (int q = 0; q < R; ++q) l[q][j] = cb + j < cend ? Lr[q][(int64_t)(cb + j) * f] : T(0);
     cudaGridDependencySynchronize();
-    T acc = T(0), acc2 = T(0);
+    T acc[R], acc2[R];
+#pragma unroll
+    for (int q = 0; q < R; ++q) acc[q] = acc2[q] = T(0);
     T *xs = sx[w];
     for (int c = cb; c < cend; c += 32) {
         const int kb = min(32, cend - c);
         __syncwarp();
         xs[lane] = lane < kb ? b1[c + lane] : T(0);
         __syncwarp();
-        const T *Lc = Lr + (int64_t)c * f;
+        const int64_t cf = (int64_t)c * f;
 #pragma unroll
         for (int g = 0; g < 32; g += G) {
             if (g >= kb) break;
@@ -806,36 +819,49 @@ __global__ void __launch_bounds__(SWEEP_CTA) k_fwd(const int *__restrict__ front
             if (g + G <= kb) {
                 if (!have) {
 #pragma unroll
-                    for (int j = 0; j < G; ++j) l[j] = Lc[(int64_t)(g + j) * f];
+                    for (int j = 0; j < G; ++j)
+#pragma unroll
+                        for (int q = 0; q < R; ++q) l[q][j] = Lr[q][cf + (int64_t)(g + j) * f];
                 }
 #pragma unroll
-                for (int j = 0; j < G; j += 2) {
-                    acc += l[j] * xs[g + j];
-                    acc2 += l[j + 1] * xs[g + j + 1];
-                }
+                for (int j = 0; j < G; j += 2)
+#pragma unroll
+                    for (int q = 0; q < R; ++q) {
+                        acc[q] += l[q][j] * xs[g + j];
+                        acc2[q] += l[q][j + 1] * xs[g + j + 1];
+                    }
             } else {
                 // the last columns, in fours
                 if (!have) {
 #pragma unroll
-                    for (int j = 0; j < G; ++j) l[j] = g + j < kb ? Lc[(int64_t)(g + j) * f] : T(0);
+                    for (int j = 0; j < G; ++j)
+#pragma unroll
+                        for (int q = 0; q < R; ++q) l[q][j] = g + j < kb ? Lr[q][cf + (int64_t)(g + j) * f] : T(0);
                 }
 #pragma unroll
                 for (int h = 0; h < G; h += 4) {
                     if (g + h >= kb) break;
 #pragma unroll
-                    for (int j = h; j < h + 4; ++j) acc += l[j] * xs[g + j];
+                    for (int j = h; j < h + 4; ++j)
+#pragma unroll
+                        for (int q = 0; q < R; ++q) acc[q] += l[q][j] * xs[g + j];
                 }
             }
         }
     }
     cudaTriggerProgrammaticLaunchCompletion();
-    if (r0 + lane >= f) return;
-    if (row < p) {
-        T *yo = y + d.vec_off + d.first + row;
-        if (gridDim.z == 1) *yo = acc + acc2;
-        else atomicAdd(yo, acc + acc2);
-    } else {
-        atomicAdd(b + d.vec_off + rows[d.row_off + row], -(acc + acc2));
+#pragma unroll
+    for (int q = 0; q < R; ++q) {
+        const int row = r0 + lane + 32 * q;
+        if (row >= f) break;
+        const T sum = acc[q] + acc2[q];
+        if (row < p) {
+            T *yo = y + d.vec_off + d.first + row;
+            if (gridDim.z == 1) *yo = sum;
+            else atomicAdd(yo, sum);
+        } else {
+            atomicAdd(b + d.vec_off + rows[d.row_off + row], -sum);
+        }
     }
 }
 
@@ -983,7 +1009,7 @@ template <class T>
 static void launch_fwd(const FactorPlan &P, const Level &Lv, const int *fr, unsigned nf, const T *L, T *b, T *y,
                        cudaStream_t s) {
     if (nf == 0 || Lv.max_p == 0) return;
-    const int tiles = (Lv.max_f + 31) / 32, blocks = (Lv.max_p + 31) / 32;
+    const int tiles = (Lv.max_f + 32 * FWD_ROWS<T> - 1) / (32 * FWD_ROWS<T>), blocks = (Lv.max_p + 31) / 32;
     // (the level's fronts, not nf: the arithmetic is the same however the level is split over streams)
     const int split = std::min<int64_t>(blocks, std::max<int64_t>(1, SWEEP_WARPS / ((int64_t)Lv.fronts.size() * tiles)));
     const int chunk = 32 * ((blocks + split - 1) / split);

@@ -1,13 +1,12 @@
 // Stress recovery whose peak reduction needs no device allocation.
 //
-// gl_stress accepts host or device arrays and allocates device staging
-// buffers on every call.  Some callers cannot allow that: a host framework
-// that has reserved nearly all device memory for its own caching pool (after
-// the local factors, little is left), a latency-bound loop where cudaMalloc
-// and cudaFree would synchronise the device and stall other streams, or a
-// deployment whose device footprint must be fixed once the library is loaded.
-// gl_stress_noalloc serves them: the caller passes device buffers for every
-// input and output, and the only scratch -- the per-block partial maxima of
+// gl_stress accepts host or device arrays, stages what it cannot use in place
+// in the context's work vectors and waits for its result.  Some callers need
+// more: a host framework that has reserved nearly all device memory for its own
+// caching pool (after the local factors, little is left), a latency-bound loop
+// that must not wait, or a deployment whose device footprint must be fixed once
+// the library is loaded.  gl_stress_noalloc serves them: the caller passes
+// device buffers for every input and output, nothing waits, and the only scratch -- the per-block partial maxima of
 // the resin peak -- lives in the file-scope device array below.
 #include <mutex>
 
