@@ -13,7 +13,8 @@
 //      diagonal block (POTRF), panel below (TRSM), trailing lower triangle
 //      (SYRK/GEMM) -- the trailing update also forms the update matrix;
 //   5. write the front's panel to the factor array in inverse form:
-//      L11^{-1} over W = L21 L11^{-1} (k_diag_inverse, k_tri_inverse, k_wpanel).
+//      L11^{-1} over W = L21 L11^{-1} (k_diag_inverse; FP32: k_tri_inverse,
+//      k_wpanel; FP64: k_trinv_tc, k_wpanel_tc in gemm64_tc.cu).
 // The solves walk the same levels, forward (leaves to root) and backward.  With
 // the pivot block's inverse stored, a front's step is one product with its
 // panel and no row of it waits for another.

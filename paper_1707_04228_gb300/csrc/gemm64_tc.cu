@@ -20,6 +20,9 @@
 //   * the eight sums are put together in two 64-bit integers, converted to
 //     FP64 without loss and added to the result by two FMAs.
 //
+// The inverse of the pivot block (k_trinv_tc) and the eigensolver's sweeps with
+// eight vectors (k_fwd_tc, k_bwd_tc) are formed the same way.
+//
 // One CTA of 256 threads forms a 128 x 32 tile: a thread stages the digits of
 // eight columns of a row at a time (K-major core matrices of 8 rows x 16 bytes,
 // no swizzle), 32 columns per round.  The eight accumulators take 256 columns
