@@ -769,8 +769,8 @@ constexpr int SWEEP_WARPS = 152 * 96;
 // a launch on the 308k- and 475k-DOF corners, this form 44 and 25 us.
 // Rows per lane of a forward task: two in FP32, 256 contiguous bytes a column,
 // which HBM likes better: 9.74 to 8.78 ms for all levels of the 12.2M-DOF corner
-// (one level after another), and no slower on the 475k-DOF one.  Four gained 2%
-// more there and cost 4% here.
+// (one level after another), 50.9 to 50.5 ms a solve on the 475k-DOF one.  Four
+// rows gained 2% more on the former and cost 3% on the latter.
 template <class T>
 constexpr int FWD_ROWS = sizeof(T) == 4 ? 2 : 1;
 
