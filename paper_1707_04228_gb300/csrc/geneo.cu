@@ -107,9 +107,24 @@ void kry_project(const FactorPlan &P, const KryBlocks &K, int ldv, int m, const 
     GL_CUDA(cudaGetLastError());
 }
 
-// W_z <- W_z R in place; with col >= 0 the columns are also stored at column col of V_z.
+// Uniform in [-1, 1): splitmix64 of the seed and an index.
+__device__ __forceinline__ double hash_uniform(uint64_t seed, int64_t i) {
+    uint64_t z = seed + 0x9E3779B97F4A7C15ull * (uint64_t)(i + 1);
+    z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
+    z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
+    z = z ^ (z >> 31);
+    return (double)(z >> 11) * (2.0 / 9007199254740992.0) - 1.0;
+}
+
+// W_z <- W_z R in place; with col >= 0 the columns are also stored at column col
+// of V_z.  With refill != 0 the columns that R drops become random ones: the
+// block's image lies in the basis there, and without new directions an
+// eigenvalue with more copies than the block has columns would come out with
+// KRY_B of them only (Xi constant over the whole subdomain: every eigenvalue
+// is the same one).
 __global__ void __launch_bounds__(256) k_kry_scale(const int64_t *__restrict__ voff, const int64_t *__restrict__ vlen,
-                                                   KryBlocks K, const double *__restrict__ R, int ldv, int col) {
+                                                   KryBlocks K, const double *__restrict__ R, int ldv, int col,
+                                                   uint64_t refill) {
     const int s = blockIdx.x;
     const int64_t n = vlen[s], i = (int64_t)blockIdx.y * 256 + threadIdx.x;
     if ((int64_t)blockIdx.y * 256 >= n) return;
@@ -128,6 +143,15 @@ __global__ void __launch_bounds__(256) k_kry_scale(const int64_t *__restrict__ v
     for (int c = 0; c < KRY_B; ++c)
 #pragma unroll
         for (int j = 0; j < KRY_B; ++j) o[j] += w[c] * sr[c * KRY_B + j];
+    if (refill) {
+#pragma unroll
+        for (int j = 0; j < KRY_B; ++j) {
+            bool dropped = true;
+#pragma unroll
+            for (int c = 0; c < KRY_B; ++c) dropped = dropped && sr[c * KRY_B + j] == 0.0;
+            if (dropped) o[j] = hash_uniform(refill, (voff[s] + i) * KRY_B + j);
+        }
+    }
 #pragma unroll
     for (int j = 0; j < KRY_B; ++j) io[(int64_t)j * n] = o[j];
     if (col >= 0) {
@@ -137,9 +161,10 @@ __global__ void __launch_bounds__(256) k_kry_scale(const int64_t *__restrict__ v
     }
 }
 
-void kry_scale(const FactorPlan &P, const KryBlocks &K, const double *R, int ldv, int col, cudaStream_t s) {
+void kry_scale(const FactorPlan &P, const KryBlocks &K, const double *R, int ldv, int col, cudaStream_t s,
+               uint64_t refill) {
     k_kry_scale<<<dim3(P.n_sub, row_chunks(P, 256), K.count), 256, 0, s>>>(P.d_vec_off.p, P.d_vec_len.p, K, R, ldv,
-                                                                          col);
+                                                                          col, refill);
     GL_CUDA(cudaGetLastError());
 }
 
@@ -370,51 +395,63 @@ __device__ void cta_eig(double *C, double *Q, double *tmp, int ld, int m, double
 }
 
 // R_s with W R_s orthonormal in the M inner product, from G_s = W^T M W: Q
-// Lambda^{-1/2} of G's eigenpairs; directions at or below the noise (drop times
-// the block's squared norm before its projection, H the coefficients it lost)
-// become zero columns and stay zero.
+// Lambda^{-1/2} of G's eigenpairs; directions at or below the noise become zero
+// columns.  H holds the coefficients that W's projection took away.  FIRST:
+// noise is drop times the block's squared norm before the projection.  Else (a
+// block of near-unit columns and random ones of any length) every column is held
+// to drop times its own, and those that stay are brought to a length near one
+// by a power of two.
+template <bool FIRST>
 __global__ void __launch_bounds__(64) k_kry_orth(const double *__restrict__ G, const double *__restrict__ H, int64_t hs,
                                                  int ldh, int m, double drop, double *__restrict__ R,
                                                  int *__restrict__ err) {
     constexpr int ld = KRY_B + 1;
-    __shared__ double C[KRY_B * ld], Q[KRY_B * ld], cs[KRY_B], red[4], sh;
+    __shared__ double C[KRY_B * ld], Q[KRY_B * ld], cs[KRY_B], red[4], lost[KRY_B], scale[KRY_B];
     __shared__ int pairs[KRY_B / 2];
     const int s = blockIdx.x, tid = threadIdx.x;
-    if (tid == 0) sh = 0.0;
+    if (tid < KRY_B) lost[tid] = 0.0;
     for (int idx = tid; idx < KRY_B * KRY_B; idx += 64) {
         const int i = idx / KRY_B, j = idx % KRY_B;
         const double *g = G + (int64_t)s * KRY_B * KRY_B;
         C[i * ld + j] = 0.5 * (g[idx] + g[j * KRY_B + i]);
     }
     __syncthreads();
-    double lost = 0.0;
+    double h2 = 0.0;                                         // of column tid % KRY_B
     for (int idx = tid; idx < m * KRY_B; idx += 64) {
         const double h = H[s * hs + (int64_t)(idx / KRY_B) * ldh + idx % KRY_B];
-        lost += h * h;
+        h2 += h * h;
     }
-    if (tid < KRY_B) lost += C[tid * ld + tid];
-    atomicAdd(&sh, lost);
+    if (tid < KRY_B) h2 += C[tid * ld + tid];
+    atomicAdd(&lost[tid % KRY_B], h2);
     __syncthreads();
-    const double floor_ = drop * sh;
+    if (tid < KRY_B) {
+        const double g = C[tid * ld + tid];
+        if (FIRST || !(fabs(g) < INFINITY)) scale[tid] = 1.0;
+        else scale[tid] = g > drop * lost[tid] ? scalbn(1.0, -(ilogb(g) / 2)) : 0.0;
+    }
+    __syncthreads();
+    const int ci = tid / KRY_B, cj = tid % KRY_B;            // 64 threads, 64 entries
+    if (!FIRST) C[ci * ld + cj] *= scale[ci] * scale[cj];
+    __syncthreads();
+    double sum = 0.0, big = 0.0;
+    for (int j = 0; j < KRY_B; ++j) sum += FIRST ? lost[j] : C[j * ld + j];
+    const double floor_ = drop * sum;
     // scaled by a power of two to the range of the rotations' FP32 angles
-    double big = 0.0;
     for (int idx = 0; idx < KRY_B * KRY_B; ++idx) big = fmax(big, fabs(C[(idx / KRY_B) * ld + idx % KRY_B]));
     const int e = big > 0.0 && big < INFINITY ? -ilogb(big) : 0;
     __syncthreads();
-    C[(tid / KRY_B) * ld + tid % KRY_B] = scalbn(C[(tid / KRY_B) * ld + tid % KRY_B], e);   // 64 threads, 64 entries
+    C[ci * ld + cj] = scalbn(C[ci * ld + cj], e);
     __syncthreads();
     cta_jacobi<double>(C, Q, ld, KRY_B, cs, pairs, red, 1e-30, true);
-    for (int idx = tid; idx < KRY_B * KRY_B; idx += 64) {
-        const int j = idx % KRY_B;
-        const double lam = scalbn(C[j * ld + j], -e);
-        if (!(fabs(lam) < INFINITY)) atomicExch(err, 1);
-        R[(int64_t)s * KRY_B * KRY_B + idx] = lam > floor_ && lam > 0.0 ? Q[(idx / KRY_B) * ld + j] / sqrt(lam) : 0.0;
-    }
+    const double lam = scalbn(C[cj * ld + cj], -e);
+    if (!(fabs(lam) < INFINITY)) atomicExch(err, 1);
+    R[(int64_t)s * KRY_B * KRY_B + tid] = lam > floor_ && lam > 0.0 ? scale[ci] * Q[ci * ld + cj] / sqrt(lam) : 0.0;
 }
 
-void kry_orth(int n_sub, const double *G, const double *H, int64_t hs, int ldh, int m, double drop, double *R,
-              int *d_err, cudaStream_t s) {
-    k_kry_orth<<<n_sub, 64, 0, s>>>(G, H, hs, ldh, m, drop, R, d_err);
+void kry_orth(int n_sub, bool first, const double *G, const double *H, int64_t hs, int ldh, int m, double drop,
+              double *R, int *d_err, cudaStream_t s) {
+    if (first) k_kry_orth<true><<<n_sub, 64, 0, s>>>(G, H, hs, ldh, m, drop, R, d_err);
+    else k_kry_orth<false><<<n_sub, 64, 0, s>>>(G, H, hs, ldh, m, drop, R, d_err);
     GL_CUDA(cudaGetLastError());
 }
 
@@ -422,8 +459,10 @@ void kry_orth(int n_sub, const double *G, const double *H, int64_t hs, int ldh, 
 // largest first: keep values mu and vectors Y (row-major m x keep), and the
 // largest relative residual of the first nev, sqrt(y^T G y) / mu with y the
 // vector's part on the last block and G the squared norms of what that block's
-// image has left outside the basis.
-__global__ void __launch_bounds__(GENEIG_THREADS) k_kry_ritz(const double *__restrict__ T, int ldt, int m,
+// image has left outside the basis.  A value of exactly zero is that of a zero
+// column: no pair yet, unless the basis holds the whole space of the subdomain.
+__global__ void __launch_bounds__(GENEIG_THREADS) k_kry_ritz(const int64_t *__restrict__ vlen,
+                                                             const double *__restrict__ T, int ldt, int m,
                                                              const double *__restrict__ G, int nev, int keep,
                                                              double *__restrict__ Y, int ldy, double *__restrict__ mu,
                                                              unsigned long long *__restrict__ worst) {
@@ -464,21 +503,21 @@ __global__ void __launch_bounds__(GENEIG_THREADS) k_kry_ritz(const double *__res
         double res = 0.0;
         for (int i = 0; i < KRY_B; ++i)
             for (int j = 0; j < KRY_B; ++j) res += Q[(m - KRY_B + i) * ld + a] * g[i * KRY_B + j] * Q[(m - KRY_B + j) * ld + a];
-        const double rel = sqrt(fmax(res, 0.0)) / fmax(me, 1e-12 * cs[m]);
+        const double rel = me > 0.0 || m >= vlen[s] ? sqrt(fmax(res, 0.0)) / fmax(me, 1e-12 * cs[m]) : INFINITY;
         atomicMax(worst, (unsigned long long)__double_as_longlong(rel));   // rel >= 0: ordered like its bits
     }
 }
 
 static size_t ritz_smem(int m) { return sizeof(double) * ((size_t)3 * m * (m + 1) + m + 2 + 2 * (GENEIG_THREADS / 32)); }
 
-void kry_ritz(int n_sub, const double *T, int ldt, int m, const double *G, int nev, int keep, double *Y, int ldy,
-              double *mu, unsigned long long *worst, cudaStream_t s) {
+void kry_ritz(const FactorPlan &P, const double *T, int ldt, int m, const double *G, int nev, int keep, double *Y,
+              int ldy, double *mu, unsigned long long *worst, cudaStream_t s) {
     static SmemLimit limit;
     raise_smem_limit(limit, ritz_smem(KRY_MAX), [](size_t v) {
         GL_CUDA(cudaFuncSetAttribute(k_kry_ritz, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)v));
     });
     GL_CUDA(cudaMemsetAsync(worst, 0, sizeof(*worst), s));
-    k_kry_ritz<<<n_sub, GENEIG_THREADS, ritz_smem(m), s>>>(T, ldt, m, G, nev, keep, Y, ldy, mu, worst);
+    k_kry_ritz<<<P.n_sub, GENEIG_THREADS, ritz_smem(m), s>>>(P.d_vec_len.p, T, ldt, m, G, nev, keep, Y, ldy, mu, worst);
     GL_CUDA(cudaGetLastError());
 }
 
@@ -513,12 +552,7 @@ void scale_rows(const FactorPlan &P, double *X, const double *xi, int k, cudaStr
 
 __global__ void k_fill_random(double *x, int64_t n, uint64_t seed) {
     int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    uint64_t z = seed + 0x9E3779B97F4A7C15ull * (uint64_t)(i + 1);
-    z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
-    z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
-    z = z ^ (z >> 31);
-    x[i] = (double)(z >> 11) * (2.0 / 9007199254740992.0) - 1.0;
+    if (i < n) x[i] = hash_uniform(seed, i);
 }
 
 void fill_random(double *x, int64_t n, uint64_t seed, cudaStream_t s) {

@@ -23,9 +23,10 @@ void local_K_apply(const FactorPlan &P, const LocalElems &E, const double *C, co
 
 // Block Krylov eigensolver of the pencils B p = mu M p (problem.cu), its basis
 // V (with M V and B V) with KRY_MAX columns at most, grown by blocks of KRY_B
-// (the sweeps' widest multi-vector, and more than the six rigid modes, the
-// largest multiple eigenvalue).  V: FactorPlan layout with ldv columns; blocks
-// W: KRY_B columns.
+// (the sweeps' widest multi-vector, and more than the six rigid modes; where an
+// eigenvalue has more copies, random columns take the place of those that the
+// basis already holds).  V: FactorPlan layout with ldv columns; blocks W: KRY_B
+// columns.
 constexpr int KRY_B = 8, KRY_MAX = 96;
 // Up to three bases and the blocks that go with them.
 struct KryBlocks {
@@ -39,14 +40,16 @@ void kry_gram(const FactorPlan &P, const double *A, int lda, int ma, const doubl
 void kry_project(const FactorPlan &P, const KryBlocks &K, int ldv, int m, const double *H, int64_t hs, int ldh,
                  cudaStream_t s);
 // R_s orthonormalising a block with Gram matrix G_s; H, m: what its projection took away
-void kry_orth(int n_sub, const double *G, const double *H, int64_t hs, int ldh, int m, double drop, double *R,
-              int *d_err, cudaStream_t s);
-// W <- W R for every pair; also stored at column col of V unless col < 0
-void kry_scale(const FactorPlan &P, const KryBlocks &K, const double *R, int ldv, int col, cudaStream_t s);
+void kry_orth(int n_sub, bool first, const double *G, const double *H, int64_t hs, int ldh, int m, double drop,
+              double *R, int *d_err, cudaStream_t s);
+// W <- W R for every pair; also stored at column col of V unless col < 0.  refill != 0: the columns that
+// R leaves zero are random ones instead (refill: their seed)
+void kry_scale(const FactorPlan &P, const KryBlocks &K, const double *R, int ldv, int col, cudaStream_t s,
+               uint64_t refill = 0);
 // Ritz pairs of T_s (leading dimension ldt, m rows), largest first; *worst = the largest relative residual
 // of the first nev (bits of a non-negative double).  Y: KRY_MAX x ldy per subdomain, mu: ldy per subdomain.
-void kry_ritz(int n_sub, const double *T, int ldt, int m, const double *G, int nev, int keep, double *Y, int ldy,
-              double *mu, unsigned long long *worst, cudaStream_t s);
+void kry_ritz(const FactorPlan &P, const double *T, int ldt, int m, const double *G, int nev, int keep, double *Y,
+              int ldy, double *mu, unsigned long long *worst, cudaStream_t s);
 void kry_diag(int n_sub, double *T, int ldt, const double *mu, int ldm, int k, cudaStream_t s);
 // out_s[:, 0..k) = V_s[:, 0..m) Y_s
 void kry_combine(const FactorPlan &P, const double *V, int ldv, int m, const double *Y, int64_t ys, int ldy, int k,

@@ -285,16 +285,16 @@ void problem_coarse(const Problem &P, const gl_opts &o, const FactorPlan &PD, st
             const bool last = it > iters && m >= nev;
             if (last || (m >= nev && m + KRY_B > mmax) || (m >= nev + KRY_B / 2 && it >= next_check)) {
                 kept = std::min(keep, m);
-                kry_ritz(ng, T.p, mmax, m, G.p, nev, kept, Y.p, keep, mu.p, worst.p, s);
+                kry_ritz(PG, T.p, mmax, m, G.p, nev, kept, Y.p, keep, mu.p, worst.p, s);
                 unsigned long long bits = 0;
                 GL_CUDA(cudaMemcpyAsync(&bits, worst.p, sizeof(bits), cudaMemcpyDeviceToHost, s));
                 check_err(P, "GenEO Rayleigh-Ritz");
                 std::memcpy(&resid, &bits, sizeof(resid));
                 if (resid <= EIG_RESID || last) break;
-                next_check = it + 1 + std::max(0, std::min(8, (int)(std::log10(resid / EIG_RESID))));
+                next_check = it + 1 + (int)std::max(0.0, std::min(8.0, std::log10(resid / EIG_RESID)));
             }
-            kry_orth(ng, G.p, H.p, hs, KRY_B, m, 1e-24, R.p, P.d_err, s);
-            kry_scale(PG, only_w, R.p, mmax, -1, s);
+            kry_orth(ng, true, G.p, H.p, hs, KRY_B, m, 1e-24, R.p, P.d_err, s);
+            kry_scale(PG, only_w, R.p, mmax, -1, s, 0x1707042280000000ull + ((uint64_t)it << 40) + (uint64_t)j0);
             if (m + KRY_B > mmax) {
                 // restart from the leading Ritz vectors: V <- V Y, T = diag(mu)
                 DBuf<double> tmp;
@@ -320,7 +320,7 @@ void problem_coarse(const Problem &P, const gl_opts &o, const FactorPlan &PD, st
             kry_gram(PG, V.p, mmax, m, MW.p, H.p, hs, KRY_B, s);
             kry_project(PG, all, mmax, m, H.p, hs, KRY_B, s);
             gram_block(MW.p);
-            kry_orth(ng, G.p, H.p, hs, KRY_B, 0, 1e-6, R.p, P.d_err, s);
+            kry_orth(ng, false, G.p, H.p, hs, KRY_B, m, 1e-6, R.p, P.d_err, s);
             kry_scale(PG, all, R.p, mmax, m, s);
             m += KRY_B;
         }
