@@ -167,6 +167,9 @@ void launch_failure(const MeshHost &m, const double *X, const double *C, const d
                     const double *u, double s33a, double s13a, double *F, double *peak, cudaStream_t s);
 // FP64 FMA probe on the current device (probe.cu): flops per second.
 double fp64_probe(int iters, int reps, int *n_sm, double *ms_out);
+// Whether [p, p + bytes) lies inside one device allocation (false also where
+// the driver cannot tell).
+bool in_device_span(const void *p, size_t bytes);
 // Fails with GL_ERR_INVALID_ARG unless [p, p + bytes) lies inside one device
 // allocation (cuMemGetAddressRange; no allocation is made).
 void require_device_span(const void *p, size_t bytes, const char *what);

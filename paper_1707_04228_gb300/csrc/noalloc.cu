@@ -98,6 +98,14 @@ AddressRangeFn address_range_fn() {
 
 }  // namespace
 
+bool in_device_span(const void *p, size_t bytes) {
+    AddressRangeFn fn = address_range_fn();
+    unsigned long long base = 0;
+    size_t size = 0;
+    const unsigned long long a = reinterpret_cast<unsigned long long>(p);
+    return fn && fn(&base, &size, a) == 0 && a >= base && a - base <= size && size - (a - base) >= bytes;
+}
+
 void require_device_span(const void *p, size_t bytes, const char *what) {
     AddressRangeFn fn = address_range_fn();
     if (!fn) fail(GL_ERR_CUDA, "cuMemGetAddressRange is not available from the driver");

@@ -13,6 +13,7 @@
 #include <cmath>
 #include <cstdio>
 #include <functional>
+#include <initializer_list>
 #include <mutex>
 #include <thread>
 
@@ -197,26 +198,34 @@ void put_scalar(double *dst, double v) {
     else *dst = v;
 }
 
+// An array of a caller: n doubles at p (p may be null).
+struct Span {
+    const double *p;
+    int64_t n;
+};
+
 // Whether kernels of this context may use the caller's array in place: device
-// memory of the context's device, aligned, and apart from `other` (an input of
-// the same call, which the in-place output must not overwrite early).
-bool in_place(gl_ctx *c, const void *p, int64_t n, const void *other = nullptr, int64_t n_other = 0) {
-    if (!p || (reinterpret_cast<uintptr_t>(p) & 7)) return false;
-    cudaPointerAttributes a{};
-    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+// memory of the context's device, aligned, all of it inside its allocation, and
+// apart from the other arrays of the call (inputs that an in-place output must
+// not overwrite early).  What may not goes through the work vectors by a copy,
+// which refuses an array that is too short.
+bool in_place(gl_ctx *c, Span a, std::initializer_list<Span> others = {}) {
+    if (!a.p || (reinterpret_cast<uintptr_t>(a.p) & 7)) return false;
+    for (const Span &o : others)
+        if (o.p && a.p < o.p + o.n && o.p < a.p + a.n) return false;
+    cudaPointerAttributes at{};
+    if (cudaPointerGetAttributes(&at, a.p) != cudaSuccess) {
         cudaGetLastError();
         return false;
     }
-    if (a.type != cudaMemoryTypeDevice || a.device != c->device) return false;
-    const char *b = (const char *)p, *o = (const char *)other;
-    return !o || b + n * sizeof(double) <= o || o + n_other * sizeof(double) <= b;
+    return at.type == cudaMemoryTypeDevice && at.device == c->device && in_device_span(a.p, a.n * sizeof(double));
 }
 
 // A displacement given by the caller as the stress kernels read it: in place,
 // or through the work vector q (host memory, or constrained entries to fill).
 const double *field_in(gl_ctx *c, const double *u) {
     const MeshHost &m = c->m;
-    if (!has_slaves(m) && in_place(c, u, m.n_dof)) return u;
+    if (!has_slaves(m) && in_place(c, {u, m.n_dof})) return u;
     to_device(c->q.p, u, m.n_dof, c->stream);
     if (has_slaves(m)) slave_fill(m, c->q.p, c->stream);
     return c->q.p;
@@ -1421,8 +1430,7 @@ int gl_stress(gl_ctx *c, const double *u, double *s33, double *t13, double *peak
         // outputs in host memory (or over u) go through the work vectors z and r
         const double *du = field_in(c, u);
         auto out = [&](double *p, DBuf<double> &w, const double *peer) {
-            const bool direct = in_place(c, p, m.n_elem, u, m.n_dof) && in_place(c, p, m.n_elem, peer, m.n_elem);
-            return direct ? p : w.p;
+            return in_place(c, {p, m.n_elem}, {{u, m.n_dof}, {peer, m.n_elem}}) ? p : w.p;
         };
         double *d33 = out(s33, c->z, t13), *d13 = out(t13, c->r, s33);
         launch_stress(m, c->d_X.p, c->d_C.p, c->d_psi.p, du, d33, d13, s);
@@ -1476,11 +1484,11 @@ int gl_apply_K(gl_ctx *c, const double *x, double *y) {
         cudaStream_t s = c->stream;
         const int64_t N = c->m.n_dof;
         const double *dx = x;
-        if (!in_place(c, x, N)) {
+        if (!in_place(c, {x, N})) {
             to_device(c->p.p, x, N, s);
             dx = c->p.p;
         }
-        double *dy = in_place(c, y, N, x, N) ? y : c->q.p;
+        double *dy = in_place(c, {y, N}, {{x, N}}) ? y : c->q.p;
         apply_K(c, dx, dy);
         if (dy != y) to_device(y, dy, N, s);
         GL_CUDA(cudaStreamSynchronize(s));
@@ -1511,7 +1519,7 @@ int gl_failure_index(gl_ctx *c, const double *u, double s33_allow, double s13_al
         GL_REQUIRE(m.n_elem < (int64_t)1 << 24, "gl_failure_index: at most 16,777,215 elements");
         cudaStream_t s = c->stream;
         const double *du = field_in(c, u);
-        double *dF = in_place(c, F, m.n_elem, u, m.n_dof) ? F : c->z.p;
+        double *dF = in_place(c, {F, m.n_elem}, {{u, m.n_dof}}) ? F : c->z.p;
         launch_failure(m, c->d_X.p, c->d_C.p, c->d_psi.p, c->d_resin.p, du, s33_allow, s13_allow, dF, c->partials.p, s);
         g_launches += 2;
         GL_CUDA(cudaMemcpyAsync(c->h_pin, c->partials.p, 2 * sizeof(double), cudaMemcpyDeviceToHost, s));
@@ -1551,16 +1559,15 @@ int gl_stress_vjp(gl_ctx *c, const double *u, const double *w33, const double *w
         const int64_t N = m.n_dof, E = m.n_elem;
         const double *du = field_in(c, u);
         auto weights = [&](const double *w, DBuf<double> &stage) -> const double * {
-            if (!w || in_place(c, w, E)) return w;
+            if (!w || in_place(c, {w, E})) return w;
             to_device(stage.p, w, E, s);
             return stage.p;
         };
         const double *d33 = weights(w33, c->z), *d13 = weights(w13, c->r);
-        auto apart = [&](const double *p, int64_t n) {
-            return in_place(c, p, n, u, N) && in_place(c, p, n, w33, E) && in_place(c, p, n, w13, E);
-        };
-        double *dgu = !dJdu ? nullptr : (apart(dJdu, N) ? dJdu : c->p.p);
-        double *dgt = !dJdth ? nullptr : (apart(dJdth, E) && in_place(c, dJdth, E, dJdu, N) ? dJdth : c->fe.p);
+        const Span in[3] = {{u, N}, {w33, E}, {w13, E}};
+        double *dgu = !dJdu ? nullptr : (in_place(c, {dJdu, N}, {in[0], in[1], in[2]}) ? dJdu : c->p.p);
+        double *dgt = !dJdth ? nullptr
+                             : (in_place(c, {dJdth, E}, {in[0], in[1], in[2], {dJdu, N}}) ? dJdth : c->fe.p);
         if (dgu) GL_CUDA(cudaMemsetAsync(dgu, 0, N * sizeof(double), s));
         launch_stress_vjp(m, c->d_X.p, c->d_C.p, c->d_psi.p, c->d_layer_of_ez.p, c->d_layer_mat.p, c->d_elem_mat.p,
                           c->d_layer_angle.p, c->d_theta.p, c->d_matC.p, du, d33, d13, dgu, dgt, s);
@@ -1581,7 +1588,7 @@ int gl_adjoint(gl_ctx *c, const double *u, const double *dJdu, double *grad, gl_
         const MeshHost &m = c->m;
         solve(c, dJdu, c->x.p, info, true);          // K_ff lambda = (dJ/du)_f, lambda = 0 on Dirichlet DOFs
         const double *du = field_in(c, u);           // lambda comes back filled from solve()
-        double *dg = in_place(c, grad, m.n_elem, u, m.n_dof) ? grad : c->z.p;
+        double *dg = in_place(c, {grad, m.n_elem}, {{u, m.n_dof}}) ? grad : c->z.p;
         launch_adjoint_contract(m, c->d_geo.p, c->d_layer_of_ez.p, c->d_layer_mat.p, c->d_elem_mat.p,
                                 c->d_layer_angle.p,
                                 c->d_theta.p, c->d_psi.p, c->d_matC.p, du, c->x.p, dg, s);
