@@ -155,7 +155,7 @@ void problem_local_elems(const Problem &P, int s0, int s1, const FactorPlan &pla
 }
 
 std::future<std::vector<SubSymbolic>> neumann_symbolic(const Problem &P, int leaf_nodes) {
-    return std::async(std::launch::async, [&P, leaf_nodes] {
+    return in_background([&P, leaf_nodes] {
         std::vector<SubSymbolic> syms;
         problem_symbolic(P, true, leaf_nodes, syms);
         return syms;
