@@ -149,9 +149,11 @@ typedef struct {
  *              adjacent dissection levels); subdomains are factored in
  *              consecutive groups that fit it.  <= 0 selects 6e9.  A smaller
  *              value only adds groups (more launches), never changes results.
- *   eig_group_bytes  device memory for the shifted Neumann factors of one
- *              group of subdomains in the GenEO eigensolver; the subdomains
- *              are processed in consecutive groups that fit it.  <= 0 selects
+ *   eig_group_bytes  device memory of one group of subdomains in the GenEO
+ *              eigensolver: their shifted Neumann factors, and the Krylov
+ *              basis with its images (up to 1,952 bytes per local DOF for nev
+ *              <= 12, 2,848 above); the subdomains are processed in
+ *              consecutive groups that fit it (one at least).  <= 0 selects
  *              4e10.  The random start vectors of the eigensolver are
  *              drawn per group, so another grouping changes the eigenvectors
  *              within the eigensolver's convergence, not the solution of a

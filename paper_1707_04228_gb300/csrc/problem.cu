@@ -208,14 +208,21 @@ void problem_coarse(const Problem &P, const gl_opts &o, const FactorPlan &PD, st
     out.eig.assign((size_t)nsub * nev, 0.0);
     const int iters = o.eig_iters > 0 ? o.eig_iters : 100;
     // Groups of subdomains: factor of M = A^N + sigma B, B = Xi A^N Xi, and the
-    // block Krylov iteration, one group at a time.
+    // block Krylov iteration, one group at a time.  Beside the factors a local DOF
+    // holds a row of the basis and its two images, of the four blocks and of a
+    // restart's copy.
     const int64_t budget = (int64_t)((o.eig_group_bytes > 0 ? o.eig_group_bytes : 4e10) / sizeof(double));
+    const int64_t per_dof = 3 * mmax + 4 * KRY_B + keep;
     int j0 = 0, max_its = 0;
     LocalElems E;
     while (j0 < nsub) {
         int j1 = j0;
         int64_t acc = 0;
-        while (j1 < nsub && (j1 == j0 || acc + syms[j1].l_size <= budget)) acc += syms[j1++].l_size;
+        for (; j1 < nsub; ++j1) {
+            const int64_t need = syms[j1].l_size + per_dof * syms[j1].n;
+            if (j1 > j0 && acc + need > budget) break;
+            acc += need;
+        }
         const int ng = j1 - j0;
         ++out.n_groups;
         // a group of all subdomains is the whole problem's plan
