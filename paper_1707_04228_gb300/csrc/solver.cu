@@ -192,10 +192,13 @@ void check_err(gl_ctx *c, const char *what) {
     }
 }
 
-// *dst = v, dst in host or device memory.
-void put_scalar(double *dst, double v) {
-    if (is_device_ptr(dst)) GL_CUDA(cudaMemcpy(dst, &v, sizeof(double), cudaMemcpyDefault));
-    else *dst = v;
+// *dst = *d (d in device memory), dst in host or device memory: what is enqueued
+// so far is waited for, *pin is *d by then.
+void finish_scalar(gl_ctx *c, double *dst, const double *d, const double *pin) {
+    const bool on_device = dst && is_device_ptr(dst);
+    if (on_device) to_device(dst, d, 1, c->stream);
+    GL_CUDA(cudaStreamSynchronize(c->stream));
+    if (dst && !on_device) *dst = *pin;
 }
 
 // An array of a caller: n doubles at p (p may be null).
@@ -1441,8 +1444,7 @@ int gl_stress(gl_ctx *c, const double *u, double *s33, double *t13, double *peak
         }
         if (s33 && s33 != d33) to_device(s33, d33, m.n_elem, s);
         if (t13 && t13 != d13) to_device(t13, d13, m.n_elem, s);
-        GL_CUDA(cudaStreamSynchronize(s));
-        if (peak) put_scalar(peak, c->h_pin[0]);
+        finish_scalar(c, peak, &c->S.p->alpha, c->h_pin);
     });
 }
 
@@ -1524,11 +1526,10 @@ int gl_failure_index(gl_ctx *c, const double *u, double s33_allow, double s13_al
         g_launches += 2;
         GL_CUDA(cudaMemcpyAsync(c->h_pin, c->partials.p, 2 * sizeof(double), cudaMemcpyDeviceToHost, s));
         if (F && F != dF) to_device(F, dF, m.n_elem, s);
-        GL_CUDA(cudaStreamSynchronize(s));
+        finish_scalar(c, peak, c->partials.p + 1, c->h_pin + 1);
         int64_t key;
         std::memcpy(&key, c->h_pin, sizeof(key));
         if (peak_elem) *peak_elem = key & 0xFFFFFF;
-        if (peak) put_scalar(peak, c->h_pin[1]);
     });
 }
 
