@@ -47,9 +47,10 @@ sys.path.insert(0, ROOT)
 METRIC = "PCG DOF-iterations/s at 1e-10 rel. residual; K*u HBM GB/s vs peak"
 # DRAM bytes (ncu dram__bytes_read.sum + dram__bytes_write.sum) of one FP64
 # local-solve application per algorithmic byte, measured over the 20 launches
-# of one application on the 151,011-DOF 32x8x23 corner; every panel is read
-# once, so it scales with the panels to the full-size workload.
-FP64_LOCAL_TRAFFIC_PER_ALG_BYTE = 1.076
+# of one application of the present sweeps on the 151,011-DOF 32x8x23 corner;
+# every panel is read once, so it scales with the panels to the full-size
+# workload.  A constant of the panels' layout, not measured by the run.
+FP64_LOCAL_TRAFFIC_PER_ALG_BYTE = 1.075
 UNIT = "DOF-iterations/s"
 FP64_FMA_PER_SM_CLK = 2        # nominal FP64 FMA rate per SM and clock of this part (context only)
 
@@ -502,8 +503,9 @@ def main():
     if fp64:
         roof = {"bound": "alu", "achieved": loc_tf, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
                 "frac": loc_tf / FP64_PEAK_TFLOPS, "traffic": FP64_LOCAL_TRAFFIC_PER_ALG_BYTE * loc_bytes,
-                "traffic_note": "bytes per application: the ratio of DRAM to algorithmic bytes measured by ncu "
-                                "on the 32x8x23 corner times this workload's algorithmic bytes",
+                "traffic_note": "bytes per application, not measured in this run: the ratio of DRAM to algorithmic "
+                                "bytes measured by ncu on the 32x8x23 corner with the present sweeps (1.075) times "
+                                "this workload's algorithmic bytes",
                 "kernel": "local forward/backward supernodal sweeps (all levels) + gather/scatter",
                 "hbm_gbs": loc_bytes / (loc_ms / 1e3) / 1e9, "hbm_frac": loc_bytes / (loc_ms / 1e3) / 1e9 / hbm,
                 "peak_note": f"FP64 peak measured in this run by the FMA probe ({probe['n_sm']} SMs, nominal "

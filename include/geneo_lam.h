@@ -141,9 +141,10 @@ typedef struct {
  *              eigensolver, a block Krylov method (<= 0: 100); it stops once
  *              the kept Ritz pairs of every subdomain have residuals below
  *              1e-6 of their value (in the pencil's energy norm), which
- *              leaves the eigenvalues accurate to about 1e-12 (to 1e-6 at
- *              worst inside a cluster), and takes as many steps as nev
- *              vectors need in any case.
+ *              leaves the eigenvalues as accurate as the matrices' rounding
+ *              does (1e-12 to 1e-9 on laminates; to 1e-6 at worst inside a
+ *              cluster), and takes as many steps as nev vectors need in any
+ *              case.
  *   factor_ws_bytes  device workspace per buffer of the numeric
  *              factorisation (two buffers hold the dense fronts of two
  *              adjacent dissection levels); subdomains are factored in

@@ -9,14 +9,16 @@
 // is formed there from integer slices (the error-free splitting of Ozaki,
 // Ogita, Oishi and Rump, Numer. Algorithms 59, 2012, on fixed-point rows):
 //   * a row's entries over the summed range are scaled by a power of two to
-//     fixed point, 62 bits below the row's largest exponent (no FP64 bit of the
-//     largest entries is lost; smaller ones lose bits below 2^-62 of it);
+//     fixed point, 62 bits below the row's largest exponent (entries down to
+//     2^-9 of the largest keep all FP64 bits, smaller ones what lies above
+//     2^-62 of it);
 //   * the fixed-point number is cut into eight signed base-256 digits, each in
 //     [-128, 127] and exact in FP16;
 //   * the digit products of equal weight i + j = s <= 7 are summed over k <= 128
 //     in one FP32 accumulator: an integer of at most 8 x 128 x 2^14 = 2^24, so
-//     every addition is exact; the weights s >= 8 lie below 2^-60 of the
-//     product of the rows' largest entries and are left out;
+//     every addition is exact; the weights s >= 8 (28 of the 64 digit products)
+//     are left out: at most 2^-57 of the product of the two rows' largest
+//     entries per column, 2^-50 over 128 columns;
 //   * the eight sums are put together in two 64-bit integers, converted to
 //     FP64 without loss and added to the result by two FMAs.
 //
@@ -35,10 +37,22 @@
 // Measured on the 63k-DOF corner's set-up: trailing updates 50.6 ms on the FP64
 // pipe, 13.2 ms here and 7.8 ms inside the panels; W 19.0 ms, 3.8 ms here.  What
 // binds it now is the latency of its loads (two CTAs an SM; FP64 pipe 18% and
-// tensor pipe 7% active).  One-subdomain direct solves (25k to 75k DOF, six
-// laminates) left residuals of 0.7 to 0.9 of those with FP64 FMAs and solution
-// errors as large as theirs; cutting the sums to 2^-54 of the largest entries'
-// product instead of converting both halves made them up to 100 times larger.
+// tensor pipe 7% active).
+//
+// Accuracy: better than FP64 sums where the entries of a row are of one size,
+// not so where two rows are large in different columns and their products small,
+// since the error is relative to the rows' largest entries.  For the Cholesky
+// that is the usual bound (a row of L is at most the root of the diagonal entry
+// of A), not the entry by entry one.  Residuals of one-subdomain direct solves
+// against the same program with FP64 FMAs: 0.75 to 1.0 on laminates and blocks of
+// one material (50 to 17,000 DOF), 0.65 to 1.3 with random stiffnesses up to 1e4
+// apart, up to 1.7 with a checkerboard 1e4 apart, 60 (2.7e-12 for 4.4e-14) with
+// one 1e6 apart; W and L11^{-1} lose that, the trailing updates 0.83 to 1.15
+// everywhere.  Solution errors are as large as with FMAs (0.8 to 1.5).  Taking
+// the pivots' sizes out of the columns of L21 and the rows of L11^{-1} first (by
+// the exponents) gave 44 instead of 60 and made first calls 2% slower; cutting the
+// sums to 2^-54 of the largest entries' product instead of converting both halves
+// made errors up to 100 times larger.
 #include <cuda_fp16.h>
 
 #include <algorithm>

@@ -787,6 +787,10 @@ namespace {
 //   total = setup + 40 iterations,
 // with F = 0.8e12 flop/s (FP64) and B = 4.5e12 B/s (sustained HBM); the ratios
 // Neumann/Dirichlet (1.6x entries, 2x flops) were measured on the corner laminate.
+// The set-up terms are those of products on the FP64 pipe and of a subspace
+// iteration.  The products run on the tensor cores now and the block Krylov
+// method takes some 14 steps of eight solves, so set-up is priced too high and
+// the choice leans to smaller factors than the fastest total would have.
 std::vector<std::array<int, 2>> autotune_candidates(const MeshHost &m) {
     std::vector<std::array<int, 2>> cands, all;
     for (int px = 1; px <= std::min(64, m.nx); ++px)
